@@ -53,16 +53,55 @@ Allocator current_allocator()
     return Allocator{g_alloc, g_free, g_alloc_ctx};
 }
 
+namespace {
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+
+// The scratch pool of the current device, made on first use; nullptr if there is none.
+cudaMemPool_t device_pool()
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        uint64_t keeps = kPoolKeeps;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keeps) != cudaSuccess) {
+            cudaGetLastError();
+            if (pool) cudaMemPoolDestroy(pool);
+            return nullptr;
+        }
+        g_pool[dev] = pool;
+    }
+    return g_pool[dev];
+}
+
+// Gives back what the pools of all devices keep unused.
+void trim_pools()
+{
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (cudaMemPool_t p : g_pool)
+        if (p) cudaMemPoolTrimTo(p, 0);
+}
+}  // namespace
+
 void *Allocator::allocate(size_t bytes, cudaStream_t s) const
 {
     if (bytes == 0) bytes = 16;
     if (alloc) return alloc(bytes, (void *)s, ctx);
     void *p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
         cudaGetLastError();  // clear the (non-sticky) allocation error
-        return nullptr;
+        if (attempt == 0) trim_pools();
     }
-    return p;
+    return nullptr;
 }
 
 void Allocator::release(void *p, cudaStream_t s) const
@@ -72,6 +111,25 @@ void Allocator::release(void *p, cudaStream_t s) const
         free_fn(p, (void *)s, ctx);
     else
         cudaFree(p);
+}
+
+void *Allocator::scratch(size_t bytes, cudaStream_t s) const
+{
+    if (alloc) return allocate(bytes, s);
+    const cudaMemPool_t pool = device_pool();
+    void *p = nullptr;
+    if (pool && cudaMallocFromPoolAsync(&p, bytes ? bytes : 16, pool, s) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+}
+
+void Allocator::release_scratch(void *p, cudaStream_t s) const
+{
+    if (!p) return;
+    if (free_fn)
+        free_fn(p, (void *)s, ctx);
+    else
+        cudaFreeAsync(p, s);
 }
 
 // ------------------------------------------------------------ thresholds ---
@@ -357,7 +415,7 @@ ising_status ising_create(const ising_params *params, void *cuda_stream, ising_l
         break;
     case ISING_FROM_BUFFER: {
         const size_t n = (size_t)(h->L * h->L);
-        int8_t *tmp = (int8_t *)h->alloc.allocate(n, h->stream);
+        int8_t *tmp = (int8_t *)h->alloc.scratch(n, h->stream);
         if (!tmp) return bail(fail(ISING_ERR_OOM, "cannot allocate %zu bytes of staging", n));
         e = cudaMemsetAsync(h->d_acc, 0, 16, h->stream);
         if (e == cudaSuccess)
@@ -367,7 +425,7 @@ ising_status ising_create(const ising_params *params, void *cuda_stream, ising_l
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(h->h_acc, h->d_acc, 16, cudaMemcpyDeviceToHost, h->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-        h->alloc.release(tmp, h->stream);
+        h->alloc.release_scratch(tmp, h->stream);
         if (e == cudaSuccess && ((unsigned int *)h->h_acc)[0] != 0)
             return bail(fail(ISING_ERR_INVALID, "init_data holds %u values that are not +1/-1",
                              ((unsigned int *)h->h_acc)[0]));
@@ -608,12 +666,12 @@ ising_status ising_get_spins(ising_lattice *h, uint64_t row0, uint64_t nrows, in
     if (nrows == 0) return ISING_OK;
     if ((st = harvest(h)) != ISING_OK) return st;
     const size_t n = (size_t)(nrows * h->L);
-    int8_t *tmp = (int8_t *)h->alloc.allocate(n, h->stream);
+    int8_t *tmp = (int8_t *)h->alloc.scratch(n, h->stream);
     if (!tmp) return fail(ISING_ERR_OOM, "cannot allocate %zu bytes of staging", n);
     cudaError_t e = launch_unpack(h->d_spins, h->L, h->word_bits, row0, nrows, tmp, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, tmp, n, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    h->alloc.release(tmp, h->stream);
+    h->alloc.release_scratch(tmp, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "get_spins");
     return ISING_OK;
 }

@@ -32,7 +32,14 @@ struct Allocator {
     void *ctx = nullptr;
     void *allocate(size_t bytes, cudaStream_t s) const;
     void release(void *p, cudaStream_t s) const;
+    // Scratch and staging memory, used in the order of stream s: from the hook, or
+    // from a pool per device that keeps at most kPoolKeeps bytes of what was
+    // released (and gives them back when an allocation of the library fails), so
+    // that a handle that comes and goes does not map and unmap its scratch.
+    void *scratch(size_t bytes, cudaStream_t s) const;
+    void release_scratch(void *p, cudaStream_t s) const;
 };
+constexpr size_t kPoolKeeps = 256ull << 20;
 Allocator current_allocator();
 
 // floor(2^32 exp(-dE / T)), clamped to [0, 2^32 - 1].
