@@ -260,6 +260,16 @@ ISING_API const char *ising_last_error(void);
  * and B instead of a kernel boundary; for lattices the autotuner's scratch holds
  * whole (L <= 65536).  In a field the field step kernel runs instead.
  * persistent = 0 otherwise.
+ *
+ * The draw-ahead form.  A handle whose configuration was not set runs calls of
+ * enough sweeps (200 at L = 64, 100 at 128, 10 at 256, 3 below 2048, 5 up to 8192)
+ * on a lattice of L <= 8192 without a field in another form: the acceptance masks of
+ * a block of sweeps are drawn by the whole GPU one launch before the tiles of the
+ * lattice are updated with them.  It needs scratch memory (three blocks of masks,
+ * a second lattice: 3 MB at L = 512, 103 MB at 4096, 210 MB at 8192), which the handle
+ * allocates on its first such call and keeps; where the allocator refuses, or while
+ * the stream is captured, the configuration's form runs.  Results are the same.
+ * ising_set_launch switches it off for the handle.
  */
 typedef struct {
     uint32_t proc_bits, regcap, block, rows_per_item, grid, insert;
@@ -276,8 +286,9 @@ ISING_API uint32_t ising_launch_candidates(uint64_t L, ising_launch *out, uint32
 /*
  * Times every candidate (reps timed step pairs each, after one untimed pair;
  * a one-CTA candidate: one launch of 8 reps sweeps after a one-sweep launch)
- * on a scratch copy of up to 256 MiB of the handle's rows, installs the
- * fastest on the handle, remembers it for later handles of the same L and
+ * and the draw-ahead form, on a scratch copy of up to 256 MiB of the handle's rows,
+ * installs the fastest candidate on the handle (and keeps the draw-ahead form in
+ * use only where that is faster still), remembers it for later handles of the same L and
  * word width on this device, and returns it with its mean time per step in
  * microseconds.  The lattice itself is not changed.  Waits for the GPU.
  */

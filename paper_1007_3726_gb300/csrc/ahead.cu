@@ -1,0 +1,757 @@
+// Draw-ahead form of a sweep call: the acceptance masks of a block of steps are
+// drawn by the whole GPU one launch ahead of the update that uses them.
+//
+// The draws of Sec. 5.3's role do not depend on the spins (the random-number
+// contract fixes them by site and step), and they are nearly all of a sweep's
+// work: about 13 of its 14 instructions per attempt.  A step of a lattice that
+// does not fill the GPU is bound by something else, the synchronisation between
+// the steps.  So one launch holds two roles:
+//   update  the first CTAs: each holds a tile of rows (all columns) with `halo`
+//           rows on either side and runs the block's steps on it without any
+//           other CTA; a step spoils one more row at either end of the tile, so
+//           that a block of `halo` steps leaves the tile's own rows right.  The
+//           redundant rows cost only bit logic (8 operations per 32 sites);
+//   draw    all other CTAs: the masks of the next block, into another buffer.
+// The next launch updates what this one drew; a launch boundary is the only
+// synchronisation between CTAs.
+//
+// Bound: draws at 1.75 per ns on the whole GPU (below); where the lattice is small,
+// the chain of steps of a tile (80 ns a step at L = 64, 110 .. 220 ns above) and 2 to
+// 3 us per launch.  Measured, one call, before (step launches or one-launch forms)
+// and with this form: L = 64, 1000 sweeps 239 -> 179 us; 256, 1000: 1072 -> 342;
+// 320, 500: 2996 -> 299; 512, 1000: 4887 -> 470; 1024, 500: 2766 -> 443; 2048, 200:
+// 1446 -> 606; 4096, 200: 3548 -> 2332 (1.44 attempts per ns of 0.95).  Persistent
+// CTAs that wait for one another on flags instead of launches were no faster (a
+// block's hand-over costs them 3.4 us).
+//
+// Layout of a tile: the two checkerboard colours of a row are kept apart, 32
+// sites of one colour per word, so that a step works on full words: bit k of
+// word w of colour p in row y is the site x = 64 w + 2 k + o, o = (y + p) & 1.
+// The neighbours of a site of colour p are of the other colour q: the bit at
+// the same place in rows y - 1 and y + 1, and in row y the bit at the same
+// place and the one before (o = 0) or behind it (o = 1).  With a the site's spin
+// and n1 .. n4 its neighbours, S3 = n1 ^ n2 ^ n3 and M3 = maj(n1, n2, n3):
+//   two or more anti-aligned  (a ^ M3) | ((a ^ S3) & (a ^ n4))
+//   one or three              S3 ^ n4
+// and since a draw below thr8 is below thr4 too, Eq. 5 of Sec. 4 is
+//   flip = two or more | (P4 & one or three) | P8.
+#include "ahead.h"
+#include "handle.h"
+#include "sweep_device.cuh"
+
+#include <algorithm>
+#include <atomic>
+
+namespace ising {
+
+namespace {
+
+// Steps whose masks an update thread holds or has on the way: their latency (about
+// a microsecond with the L2 busy) against the time of a step, within 128 KiB.
+__host__ __device__ constexpr uint32_t stages_of(uint32_t kw) { return kw == 8 ? 4 : 8; }
+
+constexpr uint32_t kThreads = 512;  // per CTA; one CTA per SM, so that an update has an SM to itself
+
+constexpr uint32_t kChunk = 8;     // steps of a stage of the one-warp form
+constexpr uint32_t kWarpStages = 8;
+constexpr uint32_t kBuffers = 3;   // mask buffers, used in turn
+constexpr uint32_t kWaitLimit = 1u << 22;  // polls of a wait for masks on their way into shared memory
+
+template <int V>
+struct Parity {
+    static constexpr int value = V;
+};
+
+__device__ __forceinline__ uint32_t shared_addr(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+
+// Bits 0, 2, .. 62 of v as one word.
+__device__ __forceinline__ uint32_t even_bits(uint64_t v)
+{
+    uint32_t h[2] = {(uint32_t)v & 0x55555555u, (uint32_t)(v >> 32) & 0x55555555u};
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        h[i] = (h[i] | (h[i] >> 1)) & 0x33333333u;
+        h[i] = (h[i] | (h[i] >> 2)) & 0x0F0F0F0Fu;
+        h[i] = (h[i] | (h[i] >> 4)) & 0x00FF00FFu;
+    }
+    return __byte_perm(h[0], h[1], 0x6420);
+}
+// The inverse: bit k of v at bit 2 k.
+__device__ __forceinline__ uint64_t spread_bits(uint32_t v)
+{
+    uint32_t h[2] = {__byte_perm(v, 0u, 0x4140), __byte_perm(v, 0u, 0x4342)};
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        h[i] = (h[i] | (h[i] << 4)) & 0x0F0F0F0Fu;
+        h[i] = (h[i] | (h[i] << 2)) & 0x33333333u;
+        h[i] = (h[i] | (h[i] << 1)) & 0x55555555u;
+    }
+    return (uint64_t)h[0] | ((uint64_t)h[1] << 32);
+}
+
+// ------------------------------------------------------------------ draw --
+// One item: the masks of one word of one colour for K sweeps from the block's sweep sw.
+// A widening multiplication keeps its pipe for 4 cycles and the ALU for 2 of them, so
+// a call of 4 draws (16.4 multiplications, 27 ALU operations, 8 insertions) takes 86
+// cycles of a sub-partition at best; 92 measured: 1756 draws per ns with K = 4, 1616
+// with K = 1.  16 warps a SM are enough for that.  (Insertions kept off the multiply
+// pipe, carry chains, funnel shifts, keys in registers: no faster or slower.)
+// The first Philox round, and the half of the second that works on its result,
+// depend on the site and the colour only: they are done once for the K steps.
+template <int K>
+__device__ __forceinline__ void draw_item(const AheadArgs &a, uint32_t p, uint32_t sw, uint32_t idx)
+{
+    const uint32_t t = a.d_t0 + sw;
+    // mask order: pair of rows, word, row of the pair
+    const uint32_t pair = a.by_wc.quotient(idx >> 1), w = (idx >> 1) - pair * a.wc;
+    const uint32_t g0 = (2u * pair + (idx & 1u)) * (a.L >> 3) + w * 8u;
+    const uint32_t x2k = (a.c3base | p) ^ a.key.k1[0];
+    uint32_t c0[K], c2[K], c3[K], m4[K], m8[K];
+    {
+        // the step's uniform values, lane k those of sweep t + k % K
+        const uint64_t pb = (uint64_t)(t + (threadIdx.x & (K - 1u))) * kPhiloxMulB;
+        const uint64_t pa = (uint64_t)((uint32_t)(pb >> 32) ^ a.key.k0[0]) * kPhiloxMulA;
+        const uint32_t v0 = (uint32_t)pb ^ a.key.k0[1], v2 = (uint32_t)(pa >> 32) ^ a.key.k1[1];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            c0[k] = K == 1 ? v0 : __shfl_sync(0xFFFFFFFFu, v0, k);
+            c2[k] = K == 1 ? v2 : __shfl_sync(0xFFFFFFFFu, v2, k);
+            c3[k] = K == 1 ? (uint32_t)pa : __shfl_sync(0xFFFFFFFFu, (uint32_t)pa, k);
+            m4[k] = m8[k] = 0u;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const uint64_t pa = (uint64_t)(g0 + q) * kPhiloxMulA;
+        const uint64_t pb = (uint64_t)((uint32_t)(pa >> 32) ^ x2k) * kPhiloxMulB;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            uint32_t u[4] = {(uint32_t)(pb >> 32) ^ c0[k], (uint32_t)pb, (uint32_t)pa ^ c2[k], c3[k]};
+            philox_rounds_from<2>(u[0], u[1], u[2], u[3], a.key);
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
+                    : "+r"(m4[k])
+                    : "r"(u[l]), "r"(a.thr4), "r"(1u << (4 * q + l)));
+                asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
+                    : "+r"(m8[k])
+                    : "r"(u[l]), "r"(a.thr8), "r"(1u << (4 * q + l)));
+            }
+        }
+    }
+    uint2 *out = a.d_masks + (size_t)(2u * sw + p) * a.nwords + idx;
+#pragma unroll
+    for (int k = 0; k < K; ++k) out[(size_t)(2 * k) * a.nwords] = make_uint2(m4[k], m8[k]);
+}
+
+// The warps of the launch take tickets for 32 items each (consecutive words of
+// one colour and group of sweeps: nwords is a multiple of 64).
+__device__ __forceinline__ void draw_role(const AheadArgs &a)
+{
+    const uint32_t lane = threadIdx.x & 31u, per_group = a.nwords / 32u;
+    uint32_t next = lane == 0 ? atomicAdd(a.d_ticket, 1u) : 0u;
+    for (;;) {
+        const uint32_t it = __shfl_sync(0xFFFFFFFFu, next, 0);
+        if (it >= a.d_tickets) return;
+        if (lane == 0) next = atomicAdd(a.d_ticket, 1u);  // back before this item is done
+        const uint32_t gp = a.by_group.quotient(it), idx = (it - gp * per_group) * 32u + lane;
+        if (a.d_four)
+            draw_item<4>(a, gp & 1u, (gp >> 1) * 4u, idx);
+        else
+            draw_item<1>(a, gp & 1u, gp >> 1, idx);
+    }
+}
+
+// ---------------------------------------------------------------- update --
+// Asynchronous copies to shared memory: each thread fetches only what it reads
+// itself, so that waiting for its own copies is enough.
+__device__ __forceinline__ void copy_async16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+__device__ __forceinline__ void mbar_init(uint64_t *bar)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(shared_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(shared_addr(bar)) : "memory");
+}
+// A bounded wait for the phase of the given parity; false when it runs out.
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32_t limit)
+{
+    for (uint32_t n = 0; n < limit; ++n) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(shared_addr(bar)), "r"(parity)
+                     : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+// Announces `bytes` on the barrier of a stage; the copy then completes it.
+__device__ __forceinline__ void copy_bulk(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(shared_addr(bar)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(shared_addr(dst)),
+                 "l"(src), "r"(bytes), "r"(shared_addr(bar))
+                 : "memory");
+}
+
+// The words of a run of KW rows of one column, both colours, from the rows' 64-bit
+// words and back (KW is even and runs start at even rows: a row's parity is k's).
+template <int KW>
+__device__ __forceinline__ void load_run(const uint64_t *p, uint32_t wc, uint32_t (&v)[2][KW])
+{
+#pragma unroll
+    for (int k = 0; k < KW; ++k) {
+        const uint64_t word = __ldcg(p + k * wc);
+        const uint32_t e = even_bits(word), o = even_bits(word >> 1);
+        v[0][k] = (k & 1) ? o : e;
+        v[1][k] = (k & 1) ? e : o;
+    }
+}
+template <int KW>
+__device__ __forceinline__ void store_run(uint64_t *p, uint32_t wc, const uint32_t (&v)[2][KW])
+{
+#pragma unroll
+    for (int k = 0; k < KW; ++k) {
+        const uint32_t e = (k & 1) ? v[1][k] : v[0][k], o = (k & 1) ? v[0][k] : v[1][k];
+        __stcg(p + k * wc, spread_bits(e) | (spread_bits(o) << 1));
+    }
+}
+
+// One step of parity P on a run: hz the horizontal neighbours' words, up / dn the
+// words above and below the run, m the masks.
+template <int KW, int P>
+__device__ __forceinline__ void step_run(uint32_t (&v)[2][KW], const uint32_t (&hz)[KW], uint32_t up, uint32_t dn,
+                                         const uint4 (&m)[KW / 2])
+{
+#pragma unroll
+    for (int k = 0; k < KW; ++k) {
+        const uint32_t p4 = (k & 1) ? m[k / 2].z : m[k / 2].x, p8 = (k & 1) ? m[k / 2].w : m[k / 2].y;
+        const uint32_t n1 = v[1 - P][k];
+        const uint32_t n2 = ((k + P) & 1) ? __funnelshift_r(n1, hz[k], 1) : __funnelshift_l(hz[k], n1, 1);
+        const uint32_t n3 = k == 0 ? up : v[1 - P][k - 1], n4 = k == KW - 1 ? dn : v[1 - P][k + 1];
+        const uint32_t s3 = n1 ^ n2 ^ n3, m3 = (n1 & n2) | (n3 & (n1 | n2));
+        uint32_t x = v[P][k];
+        x ^= (x ^ m3) | ((x ^ s3) & (x ^ n4)) | ((s3 ^ n4) & p4) | p8;
+        v[P][k] = x;
+    }
+}
+// After the step of parity 1: +1 spins of the run, and the anti-aligned bonds of
+// its sites of parity 1 (every bond of the lattice once), by the bit-sliced sum
+// b0 + 2 b1 + 4 b2 of a site's four.
+template <int KW>
+__device__ __forceinline__ void count_run(const uint32_t (&v)[2][KW], const uint32_t (&hz)[KW], uint32_t up, uint32_t dn,
+                                          uint32_t &cu, uint32_t &ca)
+{
+    cu = ca = 0u;
+#pragma unroll
+    for (int k = 0; k < KW; ++k) {
+        const uint32_t n1 = v[0][k], x = v[1][k];
+        const uint32_t n2 = ((k + 1) & 1) ? __funnelshift_r(n1, hz[k], 1) : __funnelshift_l(hz[k], n1, 1);
+        const uint32_t n3 = k == 0 ? up : v[0][k - 1], n4 = k == KW - 1 ? dn : v[0][k + 1];
+        const uint32_t s3 = n1 ^ n2 ^ n3, m3 = (n1 & n2) | (n3 & (n1 | n2));
+        const uint32_t t = (x ^ s3) & (x ^ n4), h = x ^ m3;
+        cu += __popc(x) + __popc(n1);
+        ca += __popc(s3 ^ n4) + 2 * __popc(h ^ t) + 4 * __popc(h & t);
+    }
+}
+
+// A sweep is counted when it is recorded, and the call's last one always.
+struct Counting {
+    uint32_t phase, slot;
+    __device__ __forceinline__ bool next(const AheadArgs &a, bool last)
+    {
+        const bool rec = a.record_every != 0u && phase + 1 == a.record_every;
+        if (a.record_every) phase = rec ? 0u : phase + 1;
+        return rec || last;
+    }
+};
+
+// The state of a run after a counted sweep, for the counting CTAs of the next
+// launch: row k of colour q of run c at [(q KW + k) runs + c].
+template <int KW>
+__device__ __forceinline__ void store_snapshot(const AheadArgs &a, uint32_t slot, uint32_t c, uint32_t nthr, const uint32_t (&v)[2][KW])
+{
+    uint32_t *const p = a.u_snaps + (size_t)slot * (2u * a.nwords) + c;
+#pragma unroll
+    for (int k = 0; k < 2 * KW; ++k) p[k * nthr] = v[k / KW][k % KW];
+}
+
+// One tile through the block: threads hold KW rows of one column each (a run).
+template <int KW>
+__device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, unsigned char *smem)
+{
+    constexpr uint32_t ST = stages_of(KW);
+    const uint32_t tid = threadIdx.x, wc = a.wc, L = a.L;
+    const uint32_t nruns = (a.tile_rows + 2 * a.halo) / KW, nthr = nruns * wc;  // threads with a run
+    const uint32_t nbar = (nthr + 31u) & ~31u;
+    uint4 *const ring = reinterpret_cast<uint4 *>(smem);          // [ST][KW / 2][kThreads]: (P4, P8) of two rows
+    uint32_t *const X = reinterpret_cast<uint32_t *>(ring + ST * (KW / 2) * kThreads);  // [2][KW][kThreads]: the two colours
+    uint32_t *const cnt = X + 2 * KW * kThreads;                   // [samples of the block, last state][2]
+    const bool whole = a.halo == 0u;                              // the tile is the lattice
+    if (!whole) {
+        for (uint32_t k = tid; k < 2 * a.u_slots; k += kThreads) cnt[k] = 0u;
+        __syncthreads();
+    }
+    if (tid < nbar) {
+        // (a thread past the last run repeats the last one's work)
+        const uint32_t c = min(tid, nthr - 1u), run = a.by_wc.quotient(c), w = c - run * wc;
+        const uint32_t groups = L / KW;                           // row groups of the lattice
+        uint32_t group = (tile * a.tile_rows + L - a.halo) / KW + run;  // the run's row group
+        while (group >= groups) group -= groups;
+        const bool mine = tid < nthr && run >= a.halo / KW && run < (a.halo + a.tile_rows) / KW;
+        const uint32_t xl = c - w + (w == 0 ? wc - 1u : w - 1u), xr = c - w + (w + 1u == wc ? 0u : w + 1u);
+        const uint32_t xu = (KW - 1) * kThreads + (run == 0 ? nthr - wc + w : c - wc);
+        const uint32_t xd = c + wc >= nthr ? w : c + wc;
+        // the steps after which this warp's rows are of no more use: a step spoils a
+        // row at either end of the tile
+        uint32_t useful = a.u_steps;
+        if (!whole) useful = min(useful, __reduce_max_sync(0xFFFFFFFFu, (min(run, nruns - 1u - run) + 1u) * KW - 1u));
+
+        // the masks of the next step not yet asked for, into its stage
+        const uint4 *msrc = reinterpret_cast<const uint4 *>(a.u_masks) + (size_t)(group * (KW / 2)) * wc + w;
+        const uint32_t mdst = shared_addr(ring + c);
+        uint32_t fetched = 0;
+        auto fetch = [&]() {
+            if (fetched < useful) {
+#pragma unroll
+                for (int k = 0; k < KW / 2; ++k)
+                    copy_async16(mdst + ((fetched & (ST - 1u)) * (KW / 2) + k) * kThreads * 16u, msrc + k * wc);
+            }
+            copy_commit();
+            msrc += a.nwords / 2;
+            ++fetched;
+        };
+#pragma unroll
+        for (uint32_t s = 0; s < ST; ++s) fetch();
+
+        uint32_t v[2][KW];
+        load_run<KW>(a.src + (size_t)(group * KW) * wc + w, wc, v);
+#pragma unroll
+        for (int k = 0; k < KW; ++k) {
+            X[k * kThreads + c] = v[0][k];
+            X[(KW + k) * kThreads + c] = v[1][k];
+        }
+        Counting cn{a.u_phase, 0u};
+        uint4 m[KW / 2];
+        copy_wait<ST - 1>();
+#pragma unroll
+        for (int k = 0; k < KW / 2; ++k) m[k] = ring[k * kThreads + c];
+        asm volatile("bar.sync 1, %0;" ::"r"(nbar) : "memory");
+
+        auto step = [&](auto parity, uint32_t s, bool count) {
+            constexpr int P = decltype(parity)::value;
+            if (s < useful) {
+                const uint32_t *const B = X + (1 - P) * KW * kThreads;
+                uint32_t hz[KW];
+#pragma unroll
+                for (int k = 0; k < KW; ++k) hz[k] = B[k * kThreads + (((k + P) & 1) ? xr : xl)];
+                const uint32_t up = B[xu], dn = B[xd];
+                step_run<KW, P>(v, hz, up, dn, m);
+#pragma unroll
+                for (int k = 0; k < KW; ++k) X[(P * KW + k) * kThreads + c] = v[P][k];
+                // the next step's masks, while the others reach the barrier
+                fetch();  // into the stage of this step, whose masks are in registers
+                copy_wait<ST - 1>();
+#pragma unroll
+                for (int k = 0; k < KW / 2; ++k) m[k] = ring[(((s + 1u) & (ST - 1u)) * (KW / 2) + k) * kThreads + c];
+                if (P == 1 && count) {
+                    if (whole) {
+                        if (tid < nthr) store_snapshot<KW>(a, cn.slot, c, nthr, v);
+                    } else {
+                        uint32_t cu, ca;
+                        count_run<KW>(v, hz, up, dn, cu, ca);
+                        cu = __reduce_add_sync(0xFFFFFFFFu, mine ? cu : 0u);
+                        ca = __reduce_add_sync(0xFFFFFFFFu, mine ? ca : 0u);
+                        if ((tid & 31u) == 0) {
+                            atomicAdd(&cnt[2 * cn.slot], cu);
+                            atomicAdd(&cnt[2 * cn.slot + 1], ca);
+                        }
+                    }
+                }
+            }
+            asm volatile("bar.sync 1, %0;" ::"r"(nbar) : "memory");
+        };
+        for (uint32_t s = 0; s < a.u_steps; s += 2) {
+            const bool count = cn.next(a, a.u_last != 0u && s + 2 == a.u_steps);
+            step(Parity<0>{}, s, false);
+            step(Parity<1>{}, s + 1u, count);
+            if (count) ++cn.slot;
+        }
+        copy_wait<0>();
+        // the block's samples (the last counter, if it is none, is the state after the call)
+        for (uint32_t k = tid; !whole && k < a.u_slots; k += nbar) {
+            const unsigned long long up = cnt[2 * k], anti = cnt[2 * k + 1];
+            if (k < a.u_recs) {
+                atomicAdd(a.acc + 2 * (size_t)(a.u_slot0 + k), up);
+                atomicAdd(a.acc + 2 * (size_t)(a.u_slot0 + k) + 1, anti);
+            }
+            if (a.u_last != 0u && k + 1 == a.u_slots) {
+                atomicAdd(a.final_acc, up);
+                atomicAdd(a.final_acc + 1, anti);
+            }
+        }
+        if (mine) store_run<KW>(a.dst + (size_t)(group * KW) * wc + w, wc, v);
+    }
+    __syncthreads();  // the tile's shared memory is free again
+}
+
+// L = 64: one warp holds the lattice, two rows a lane; the rows above and below come by
+// shuffles and a step has no barrier.  Another warp fetches the masks, in chunks
+// of several steps.
+__device__ __forceinline__ void update_warp(const AheadArgs &a, unsigned char *smem)
+{
+    __shared__ __align__(8) uint64_t full[kWarpStages], empty[kWarpStages];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    uint4 *const ring = reinterpret_cast<uint4 *>(smem);          // [kWarpStages][kChunk][lane]
+    if (tid == 0) {
+        for (uint32_t k = 0; k < kWarpStages; ++k) {
+            mbar_init(&full[k]);
+            mbar_init(&empty[k]);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const uint32_t limit = a.hold_step ? 1u << 12 : kWaitLimit;
+    if (tid == 32) {
+        uint32_t f = 0;  // chunks asked for
+        const uint4 *from = reinterpret_cast<const uint4 *>(a.u_masks);
+        for (uint32_t s = 0; s < a.u_steps; s += kChunk, ++f, from += kChunk * 32) {
+            const uint32_t st = f % kWarpStages;
+            if (f >= kWarpStages && !mbar_wait(&empty[st], (f / kWarpStages - 1u) & 1u, 4 * limit)) break;
+            // (failure testing: the held step's chunk and those behind it never arrive)
+            if (a.hold_step != 0u && a.hold_step - 1u < a.u_step0 + s + kChunk) break;
+            copy_bulk(ring + st * kChunk * 32, from, min(kChunk, a.u_steps - s) * 512u, &full[st]);
+        }
+        // no copy is on its way when the CTA goes on
+        for (uint32_t k = f > kWarpStages ? f - kWarpStages : 0u; k < f; ++k)
+            (void)mbar_wait(&full[k % kWarpStages], k / kWarpStages & 1u, limit);
+    } else if (tid < 32) {
+        uint32_t v[2][2];
+        load_run<2>(a.src + lane * 2, 1u, v);
+        Counting cn{a.u_phase, 0u};
+        bool good = true;
+        for (uint32_t s0 = 0, f = 0; s0 < a.u_steps; s0 += kChunk, ++f) {
+            const uint32_t st = f % kWarpStages, n = min(kChunk, a.u_steps - s0);
+            good = __all_sync(0xFFFFFFFFu, mbar_wait(&full[st], f / kWarpStages & 1u, limit));
+            if (!good) break;
+            const uint4 *mp = ring + st * kChunk * 32 + lane;
+            uint4 m[1] = {mp[0]};
+            auto step = [&](auto parity, bool more) {
+                constexpr int P = decltype(parity)::value;
+                mp += 32;
+                const uint4 next = more ? *mp : m[0];
+                const uint32_t up = __shfl_sync(0xFFFFFFFFu, v[1 - P][1], lane - 1u);
+                const uint32_t dn = __shfl_sync(0xFFFFFFFFu, v[1 - P][0], lane + 1u);
+                // a row is one word: its horizontal neighbours are its own bits
+                const uint32_t hz[2] = {v[1 - P][0], v[1 - P][1]};
+                step_run<2, P>(v, hz, up, dn, m);
+                m[0] = next;
+            };
+            for (uint32_t s = 0; s < n; s += 2) {
+                step(Parity<0>{}, true);
+                step(Parity<1>{}, s + 2 < n);
+                if (cn.next(a, a.u_last != 0u && s0 + s + 2 == a.u_steps)) store_snapshot<2>(a, cn.slot++, lane, 32u, v);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[st]);
+        }
+        if (!good && lane == 0 && a.err) atomicExch(a.err, 1u);
+        store_run<2>(a.dst + lane * 2, 1u, v);
+    }
+    __syncthreads();
+}
+
+// M and E of the snapshots of the launch before, a thread a run.
+template <int KW>
+__device__ __forceinline__ void count_role(const AheadArgs &a, uint32_t cta)
+{
+    const uint32_t wc = a.wc, nthr = a.nwords / KW, per = (nthr + 31u) & ~31u;  // threads a snapshot: whole warps
+    for (uint32_t i = cta * kThreads + threadIdx.x; i < a.c_slots * per; i += a.count_ctas * kThreads) {
+        const uint32_t slot = i / per, t = i - slot * per;
+        const uint32_t c = min(t, nthr - 1u), run = a.by_wc.quotient(c), w = c - run * wc;
+        const uint32_t *const B = a.c_snaps + (size_t)slot * (2u * a.nwords);
+        uint32_t v[2][KW], hz[KW], cu, ca;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) {
+            v[0][k] = B[k * nthr + c];
+            v[1][k] = B[(KW + k) * nthr + c];
+            hz[k] = B[k * nthr + c - w + (((k + 1) & 1) ? (w + 1u == wc ? 0u : w + 1u) : (w == 0 ? wc - 1u : w - 1u))];
+        }
+        const uint32_t up = B[(KW - 1) * nthr + (run == 0 ? nthr - wc + w : c - wc)], dn = B[c + wc >= nthr ? w : c + wc];
+        count_run<KW>(v, hz, up, dn, cu, ca);
+        cu = __reduce_add_sync(0xFFFFFFFFu, t < nthr ? cu : 0u);
+        ca = __reduce_add_sync(0xFFFFFFFFu, t < nthr ? ca : 0u);
+        if ((threadIdx.x & 31u) == 0u) {
+            if (slot < a.c_recs) {
+                atomicAdd(a.acc + 2 * (size_t)(a.c_slot0 + slot), (unsigned long long)cu);
+                atomicAdd(a.acc + 2 * (size_t)(a.c_slot0 + slot) + 1, (unsigned long long)ca);
+            }
+            if (a.c_last != 0u && slot + 1 == a.c_slots) {
+                atomicAdd(a.final_acc, (unsigned long long)cu);
+                atomicAdd(a.final_acc + 1, (unsigned long long)ca);
+            }
+        }
+    }
+}
+
+template <int KW, bool WARP>
+__global__ void __launch_bounds__(kThreads, 1) k_ahead(const __grid_constant__ AheadArgs a)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    // The first launch of a call (it only draws) starts after all work before it.
+    // A later one draws into a buffer, and takes tickets from a counter, that no
+    // launch still running uses (three and four in turn), so its draws need not
+    // wait; updates and counts need what the launch before wrote.
+    const uint32_t early = a.update_ctas + a.count_ctas;
+    if (blockIdx.x < early || early == 0u) dependent_launch_wait();
+    dependent_launch_trigger();
+    if (blockIdx.x < a.update_ctas) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *a.next_ticket = 0u;
+        if constexpr (WARP)
+            update_warp(a, smem);
+        else
+            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<KW>(a, t, smem);
+    } else if (blockIdx.x < early) {
+        count_role<KW>(a, blockIdx.x - a.update_ctas);
+    }
+    if (a.d_tickets != 0u) draw_role(a);
+}
+
+using AheadKernel = void (*)(AheadArgs);
+
+AheadKernel pick_kernel(const AheadPlan &p)
+{
+    if (p.warp) return k_ahead<2, true>;
+    return p.kw == 2 ? k_ahead<2, false> : p.kw == 4 ? k_ahead<4, false> : p.kw == 8 ? k_ahead<8, false> : nullptr;
+}
+
+constexpr int kMaxDevices = 64;
+constexpr int kMaxSmem = 200 * 1024;
+constexpr size_t kTicketBytes = 256;  // the ticket counters at the start of the scratch
+
+FastDiv fast_div(uint32_t d)
+{
+    FastDiv f{};
+    f.shift = 24;
+    while ((1u << (f.shift - 24)) < d) ++f.shift;
+    f.mul = (uint32_t)(((1ull << f.shift) + d - 1) / d);
+    return f;
+}
+
+// SMs of the current device; a kernel's shared-memory limit is raised once per device.
+cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
+{
+    static std::atomic<int> sms_of[kMaxDevices], ready[kMaxDevices];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool cached = dev >= 0 && dev < kMaxDevices;
+    *sms = cached ? sms_of[dev].load(std::memory_order_relaxed) : 0;
+    if (*sms <= 0) {
+        e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        if (cached) sms_of[dev].store(*sms, std::memory_order_relaxed);
+    }
+    if (!cached || !(ready[dev].load(std::memory_order_acquire) >> which & 1)) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        if (e != cudaSuccess) return e;
+        if (cached) ready[dev].fetch_or(1 << which, std::memory_order_release);
+    }
+    return cudaSuccess;
+}
+
+}  // namespace
+
+// The plan by size.  L <= 192: one CTA holds the lattice, in registers for the
+// whole block, and blocks are long (a block of 256 sweeps costs one launch).
+// Above, tiles of full rows: the taller the halo, the fewer launches and the more
+// redundant rows; a tile and its halo are at most 4096 words of a colour (8 rows a
+// thread), so that both shrink as rows get longer.  Measured (us for a call, M/E
+// every tenth sweep), tile and halo:
+//   L =  256, 1000 sweeps: 32 + 64: 352, 32 + 32: 405, 64 + 32: 425, one CTA: 416
+//   L =  512, 1000 sweeps: 32 + 64: 461, 32 + 32: 482, 64 + 32: 558 (every sweep: 32 + 32 is 8 % ahead)
+//   L = 1024,  500 sweeps: 64 + 32: 447, 32 + 32: 470, 32 + 16: 607
+//   L = 2048,  200 sweeps: 64 + 32: 606, 64 + 16: 630, 32 + 16: 659
+//   L = 4096,  200 sweeps: 32 + 16: 2225, 16 + 8: 2399
+// Above 8192 a block would hold fewer than 4 sweeps and its masks 25 times the
+// lattice: the step kernels run there.  min_sweeps: a call has one launch more than
+// it has blocks, and the one-launch forms (L = 64, 128, 256) and two step launches
+// per sweep (above) are as fast on shorter calls.
+AheadPlan ahead_plan(uint64_t L)
+{
+    AheadPlan p{};
+    if (L % 64 != 0 || L < 64 || L > 8192) return p;
+    const uint32_t wc = (uint32_t)(L / 64);
+    if (L <= 192) {
+        p.tile_rows = (uint32_t)L;
+        p.halo = 0;
+    } else {
+        p.tile_rows = L >= 1024 && L <= 2048 ? 64 : L <= 4096 ? 32 : 16;
+        p.halo = L <= 256 ? 64 : L <= 2048 ? 32 : L <= 4096 ? 16 : 8;
+    }
+    p.block_sweeps = p.halo ? p.halo / 2 : 256;
+    p.min_sweeps = L == 64 ? 200 : L == 128 ? 100 : L == 256 ? 10 : L < 2048 ? 3 : 5;
+    const uint32_t rows = p.tile_rows + 2 * p.halo, most = p.halo ? kThreads : kThreads / 2;
+    for (p.kw = 2; rows / p.kw * wc > most;) p.kw *= 2;
+    p.warp = L == 64;
+    p.tiles = (uint32_t)(L / p.tile_rows);
+    p.update_ctas = std::min(p.tiles, 64u);
+    p.mask_bytes = (size_t)2 * p.block_sweeps * L * wc * 8;
+    p.snap_bytes = p.halo ? 0 : (size_t)(p.block_sweeps + 1) * L * wc * 8;
+    return p;
+}
+
+namespace {
+
+cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaStream_t s)
+{
+    const AheadKernel kern = pick_kernel(pl);
+    if (!kern) return cudaErrorInvalidValue;
+    int sms = 0;
+    cudaError_t e = prepare_device(kern, pl.warp ? 0 : pl.kw / 2, &sms);
+    if (e != cudaSuccess) return e;
+    a.update_ctas = a.u_steps ? pl.update_ctas : 0u;
+    const uint32_t per = (a.nwords / pl.kw + 31u) & ~31u;
+    a.count_ctas = a.c_slots ? std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, 32u) : 0u;
+    a.d_four = a.d_sweeps % 4 == 0;
+    a.d_tickets = (a.d_four ? a.d_sweeps / 4 : a.d_sweeps) * 2u * (a.nwords / 32u);
+    const uint32_t early = a.update_ctas + a.count_ctas, warps = kThreads / 32u;
+    const uint32_t grid = std::max(early, std::min<uint32_t>((uint32_t)sms, early + (a.d_tickets + warps - 1) / warps));
+    const size_t smem = !a.u_steps ? 0
+                        : pl.warp  ? kWarpStages * kChunk * 512
+                                   : (stages_of(pl.kw) + 1) * pl.kw * kThreads * 8 + (pl.halo ? (size_t)a.u_slots * 8 : 0);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+}  // namespace
+
+bool ahead_ready(ising_lattice *h, const AheadPlan &pl)
+{
+    const size_t need = kTicketBytes + kBuffers * pl.mask_bytes + 2 * pl.snap_bytes + (pl.halo ? h->bytes : 0);
+    if (h->ahead_bytes >= need) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;  // no allocation while the stream is captured
+    }
+    h->d_ahead = h->alloc.scratch(need, h->stream);
+    h->ahead_bytes = h->d_ahead ? need : 0;
+    return h->d_ahead != nullptr;
+}
+
+cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, uint64_t t0, uint64_t nsweeps, uint32_t record_every,
+                         uint64_t nrec, unsigned int *err, uint32_t hold_step, uint64_t max_block)
+{
+    const uint32_t full = (uint32_t)std::min<uint64_t>(pl.block_sweeps, max_block);
+    unsigned int *const tickets = static_cast<unsigned int *>(h->d_ahead);
+    char *const masks = static_cast<char *>(h->d_ahead) + kTicketBytes;
+    char *const snaps = masks + kBuffers * pl.mask_bytes;
+    uint64_t *const spins = static_cast<uint64_t *>(lattice);
+    uint64_t *const other = pl.halo ? reinterpret_cast<uint64_t *>(snaps + 2 * pl.snap_bytes) : spins;
+    AheadArgs a{};
+    a.key = h->key;
+    a.thr4 = h->thr4;
+    a.thr8 = h->thr8;
+    a.c3base = h->stream_id << 1;
+    a.L = (uint32_t)h->L;
+    a.wc = a.L / 64;
+    a.nwords = a.L * a.wc;
+    a.by_wc = fast_div(a.wc);
+    a.by_group = fast_div(a.nwords / 32);
+    a.tiles = pl.tiles;
+    a.tile_rows = pl.tile_rows;
+    a.halo = pl.halo;
+    a.record_every = record_every;
+    a.acc = h->d_acc;
+    a.final_acc = h->d_acc + 2 * nrec;
+    a.err = err;
+    a.hold_step = hold_step;
+    // Blocks.  Items of 4 sweeps are the cheapest to draw, so a call that is long
+    // enough starts with the rest of a division by 4.  Where an update takes long
+    // (one CTA holds the lattice), blocks start short: nothing overlaps the first
+    // one's draws.
+    uint64_t drawn = 0, done = 0, rec_done = 0, prev = 0, grow = pl.halo ? full : std::min<uint64_t>(full, 32);
+    auto next_block = [&]() -> uint64_t {
+        const uint64_t left = nsweeps - drawn;
+        if (full % 4 != 0 || (left <= 7 && h->L < 2048)) return std::min<uint64_t>(left, full);
+        if (left % 4) return left % 4;
+        if (pl.halo && left % full) return left % full;
+        const uint64_t n = std::min(left, grow);
+        grow = std::min<uint64_t>(full, 4 * grow);
+        return n;
+    };
+    uint64_t nblocks = 0;
+    for (; drawn < nsweeps; ++nblocks) drawn += next_block();
+    drawn = 0;
+    grow = pl.halo ? full : std::min<uint64_t>(full, 32);
+    cudaError_t e = cudaMemsetAsync(tickets, 0, kTicketBytes, h->stream);
+    if (e != cudaSuccess) return e;
+    const uint64_t *src = spins;
+    if (pl.halo && nblocks % 2 == 1) {
+        e = cudaMemcpyAsync(other, spins, h->bytes, cudaMemcpyDeviceToDevice, h->stream);
+        if (e != cudaSuccess) return e;
+        src = other;
+    }
+    // launch b draws block b, updates block b - 1 and counts the snapshots of block b - 2
+    for (uint64_t b = 0; b < nblocks + (pl.halo ? 1 : 2); ++b) {
+        const uint64_t n = drawn < nsweeps ? next_block() : 0;
+        a.c_slots = pl.halo ? 0u : a.u_slots;
+        a.c_recs = a.u_recs;
+        a.c_slot0 = a.u_slot0;
+        a.c_last = a.u_last;
+        a.c_snaps = a.u_snaps;
+        a.u_steps = (uint32_t)(2 * prev);
+        a.u_recs = a.u_slots = a.u_last = 0u;
+        if (prev) {
+            const uint64_t t = t0 + done;
+            a.u_step0 = (uint32_t)(2 * done);
+            a.src = src;
+            a.dst = src == spins ? other : spins;
+            a.u_masks = reinterpret_cast<const uint2 *>(masks + ((b - 1) % kBuffers) * pl.mask_bytes);
+            a.u_snaps = reinterpret_cast<uint32_t *>(snaps + (b % 2) * pl.snap_bytes);
+            a.u_phase = record_every ? (uint32_t)(t % record_every) : 0u;
+            a.u_recs = record_every ? (uint32_t)((t + prev) / record_every - t / record_every) : 0u;
+            a.u_slot0 = (uint32_t)rec_done;
+            a.u_last = done + prev == nsweeps;
+            a.u_slots = a.u_recs + ((a.u_last && !(record_every && (t + prev) % record_every == 0)) ? 1u : 0u);
+            src = a.dst;
+            done += prev;
+            rec_done += a.u_recs;
+        }
+        a.d_t0 = (uint32_t)(t0 + drawn);
+        a.d_sweeps = (uint32_t)n;
+        a.d_masks = reinterpret_cast<uint2 *>(masks + (b % kBuffers) * pl.mask_bytes);
+        a.d_ticket = tickets + b % 4;
+        a.next_ticket = tickets + (b + 2) % 4;
+        if (!a.u_steps && !n && !a.c_slots) break;
+        if ((e = launch_ahead(pl, a, b > 0, h->stream)) != cudaSuccess) return e;
+        drawn += n;
+        prev = n;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace ising

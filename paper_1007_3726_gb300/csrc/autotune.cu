@@ -6,10 +6,12 @@
 // instruction-level parallelism), block size and rows per work item.  The
 // autotuner times each candidate with CUDA events on a scratch copy of the
 // lattice and keeps the fastest per (device, L, storage word width).
+#include "ahead.h"
 #include "handle.h"
 #include "kernels.h"
 #include "runtime.h"
 
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <map>
@@ -20,7 +22,11 @@ using namespace ising;
 
 namespace {
 std::mutex g_tuned_mu;
-std::map<std::tuple<int, uint64_t, uint32_t>, LaunchConfig> g_tuned;
+struct Tuned {
+    LaunchConfig config;
+    bool ahead;  // the draw-ahead form was faster still
+};
+std::map<std::tuple<int, uint64_t, uint32_t>, Tuned> g_tuned;
 
 ising_launch to_abi(const LaunchConfig &c)
 {
@@ -39,7 +45,7 @@ LaunchConfig default_launch(int device, uint64_t L, uint32_t word_bits)
     {
         std::lock_guard<std::mutex> lk(g_tuned_mu);
         auto it = g_tuned.find(std::make_tuple(device, L, word_bits));
-        if (it != g_tuned.end()) return it->second;
+        if (it != g_tuned.end()) return it->second.config;
     }
     // untuned: the shapes the autotuner picked on GB300 at these sizes
     // (fields: proc_bits, regcap, insert, block, rows_per_item, grid)
@@ -53,10 +59,17 @@ LaunchConfig default_launch(int device, uint64_t L, uint32_t word_bits)
     return LaunchConfig{64, 1, 0, 512, 8, 0};
 }
 
-void remember_launch(int device, uint64_t L, uint32_t word_bits, const LaunchConfig &c)
+bool default_ahead(int device, uint64_t L, uint32_t word_bits)
 {
     std::lock_guard<std::mutex> lk(g_tuned_mu);
-    g_tuned[std::make_tuple(device, L, word_bits)] = c;
+    auto it = g_tuned.find(std::make_tuple(device, L, word_bits));
+    return it == g_tuned.end() || it->second.ahead;
+}
+
+void remember_launch(int device, uint64_t L, uint32_t word_bits, const LaunchConfig &c, bool ahead)
+{
+    std::lock_guard<std::mutex> lk(g_tuned_mu);
+    g_tuned[std::make_tuple(device, L, word_bits)] = Tuned{c, ahead};
 }
 
 std::vector<LaunchConfig> launch_candidates(uint64_t L, uint64_t rows)
@@ -130,6 +143,7 @@ ISING_API ising_status ising_set_launch(ising_lattice *h, const ising_launch *cf
         return fail(ISING_ERR_INVALID, "launch configuration not valid for L = %llu",
                     (unsigned long long)h->L);
     h->launch = c;
+    h->ahead = false;
     return ISING_OK;
 }
 
@@ -253,12 +267,35 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
             best_c = c;
         }
     }
+    // the draw-ahead form on the copy, where it applies (the copy is the whole lattice there)
+    const AheadPlan pl = ahead_plan(h->L);
+    bool ahead = false;
+    if (e == cudaSuccess && pl.kw != 0 && rows == h->L && ahead_ready(h, pl)) {
+        const uint32_t n = std::max(8 * reps, 2 * pl.min_sweeps);
+        unsigned int *const flag = reinterpret_cast<unsigned int *>(h->d_acc + 2);  // after the one state slot
+        e = cudaMemsetAsync(flag, 0, 16, h->stream);
+        for (uint32_t k = 0; k < 2 && e == cudaSuccess; ++k) {
+            e = cudaEventRecord(e0, h->stream);
+            if (e == cudaSuccess) e = ahead_sweeps(h, pl, scratch, 0xFFFF0000u, n, 0, 0, flag, 0, 1ull << 30);
+        }
+        if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        float ms = 0;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        unsigned int timeout = 0;
+        if (e == cudaSuccess) e = cudaMemcpy(&timeout, flag, sizeof timeout, cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess && timeout == 0 && (double)ms / (2 * n) < best_step_ms) {
+            ahead = true;
+            best_step_ms = (double)ms / (2 * n);
+        }
+    }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     h->alloc.release(scratch, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "autotune");
     h->launch = best_c;
-    remember_launch(h->device, h->L, h->word_bits, best_c);
+    h->ahead = ahead;
+    remember_launch(h->device, h->L, h->word_bits, best_c, ahead);
     if (best) *best = to_abi(best_c);
     if (best_us_per_step) *best_us_per_step = 1e3 * best_step_ms * ((double)h->L / rows);
     return ISING_OK;

@@ -28,6 +28,9 @@ struct ising_lattice {
     unsigned long long *d_acc = nullptr;  // 2 counters per slot
     unsigned long long *h_acc = nullptr;  // pinned mirror
     size_t acc_slots = 0;
+    void *d_ahead = nullptr;  // scratch of the draw-ahead form (ahead.cu), on first use
+    size_t ahead_bytes = 0;
+    bool ahead = true;        // the draw-ahead form where it applies (no configuration set, none found faster)
     cudaEvent_t ev = nullptr;
     ising::RoundKeys key{};
     ising::LaunchConfig launch{};
@@ -51,7 +54,10 @@ constexpr unsigned char kGuardByte = 0xA5;
 // Launch configuration for a new handle: the autotuned one for (device, L,
 // word width) if there is one, else a fixed default.
 LaunchConfig default_launch(int device, uint64_t L, uint32_t word_bits);
-void remember_launch(int device, uint64_t L, uint32_t word_bits, const LaunchConfig &c);
+// Whether a new handle takes the draw-ahead form where it applies: unless the
+// autotuner found the launch configuration faster.
+bool default_ahead(int device, uint64_t L, uint32_t word_bits);
+void remember_launch(int device, uint64_t L, uint32_t word_bits, const LaunchConfig &c, bool ahead);
 std::vector<LaunchConfig> launch_candidates(uint64_t L, uint64_t rows);
 
 // Shared by the ABI translation units.

@@ -2,6 +2,7 @@
 // thresholds (Sec. 3), memory and stream management, sample bookkeeping and
 // FP64 moments.  All lattice arithmetic runs in the kernels of kernels.cu.
 #include "ising.h"
+#include "ahead.h"
 #include "kernels.h"
 #include "handle.h"
 #include "runtime.h"
@@ -233,6 +234,7 @@ void destroy_all(ising_lattice *h)
     cudaStreamSynchronize(h->stream);
     h->alloc.release(h->d_base, h->stream);
     h->alloc.release(h->d_acc, h->stream);
+    h->alloc.release_scratch(h->d_ahead, h->stream);
     if (h->h_acc) cudaFreeHost(h->h_acc);
     if (h->ev) cudaEventDestroy(h->ev);
     delete h;
@@ -397,6 +399,7 @@ ising_status ising_create(const ising_params *params, void *cuda_stream, ising_l
     if ((st = ensure_acc(h, 64)) != ISING_OK) return bail(st);
 
     h->launch = default_launch(h->device, h->L, wb);
+    h->ahead = default_ahead(h->device, h->L, wb);
 
     // initial state
     switch (params->init) {
@@ -474,6 +477,21 @@ ising_status ising_sweep(ising_lattice *h, uint64_t nsweeps, uint32_t record_eve
     if ((st = ensure_acc(h, nrec + 2)) != ISING_OK) return st;
 
     CK(h, cudaMemsetAsync(h->d_acc, 0, (nrec + 2) * 16, h->stream));
+    unsigned int *const err = reinterpret_cast<unsigned int *>(h->d_acc + 2 * (nrec + 1));
+    // failure-detection testing and testing only (see include/ising.h)
+    const char *hold_env = std::getenv("ISING_TINY_HOLD_STEP"), *max_env = std::getenv("ISING_TINY_MAX_SWEEPS");
+    const uint32_t hold_step = hold_env ? (uint32_t)std::strtoul(hold_env, nullptr, 10) : 0u;
+    uint64_t max_chunk = 1ull << 30;
+    if (max_env) {
+        const uint64_t v = std::strtoull(max_env, nullptr, 10);
+        if (v > 0 && v < max_chunk) max_chunk = v;
+    }
+    const AheadPlan pl = h->ahead && h->H == 0.0 ? ahead_plan(h->L) : AheadPlan{};
+    if (pl.kw != 0 && nsweeps >= pl.min_sweeps && ahead_ready(h, pl)) {
+        CK(h, ahead_sweeps(h, pl, h->d_spins, t0, nsweeps, record_every, nrec, err, hold_step, max_chunk));
+        h->pending_err = true;
+        return finish_sweep_call(h, t0, nsweeps, nrec, M_out, E_out);
+    }
     if (h->launch.proc_bits == kTinyProcBits) {
         // the whole call in one launch of one CTA
         TinyRunArgs ta{};
@@ -494,22 +512,13 @@ ising_status ising_sweep(ising_lattice *h, uint64_t nsweeps, uint32_t record_eve
             ta.k_up = h->field.k_up;
             ta.k_dn = h->field.k_dn;
         }
-        ta.err = reinterpret_cast<unsigned int *>(h->d_acc + 2 * (nrec + 1));
-        {
-            // failure-detection testing only (see include/ising.h)
-            const char *hold = std::getenv("ISING_TINY_HOLD_STEP");
-            ta.hold_step = hold ? (uint32_t)std::strtoul(hold, nullptr, 10) : 0u;
-        }
+        ta.err = err;
+        ta.hold_step = hold_step;
         // A launch counts its checkerboard steps (2 per sweep) in 32 bits: a
         // longer call runs as several launches of at most 2^30 sweeps.  Launch k
         // records its samples from slot rec_done on; its final-state slot is the
         // next launch's first sample slot, cleared in between (some of these
         // kernels add their counts into the slots).
-        uint64_t max_chunk = 1ull << 30;
-        if (const char *mx = std::getenv("ISING_TINY_MAX_SWEEPS")) {  // testing only
-            const uint64_t v = std::strtoull(mx, nullptr, 10);
-            if (v > 0 && v < max_chunk) max_chunk = v;
-        }
         uint64_t done = 0, rec_done = 0;
         while (done < nsweeps) {
             const uint64_t n = std::min(nsweeps - done, max_chunk);
