@@ -47,8 +47,8 @@ namespace ising {
 namespace {
 
 // Steps whose masks an update thread holds or has on the way: their latency (about
-// a microsecond with the L2 busy) against the time of a step, within 128 KiB.
-__host__ __device__ constexpr uint32_t stages_of(uint32_t kw) { return kw == 8 ? 4 : 8; }
+// a microsecond with the L2 busy) against the time of a step, within 160 KiB.
+__host__ __device__ constexpr uint32_t stages_of(uint32_t kw, bool field) { return kw == 8 || (field && kw == 4) ? 4 : 8; }
 
 constexpr uint32_t kThreads = 512;  // per CTA; one CTA per SM, so that an update has an SM to itself
 
@@ -98,15 +98,20 @@ __device__ __forceinline__ uint64_t spread_bits(uint32_t v)
 // pipe, carry chains, funnel shifts, keys in registers: no faster or slower.)
 // The first Philox round, and the half of the second that works on its result,
 // depend on the site and the colour only: they are done once for the K steps.
-template <int K>
+// The mask planes of a step: P4 and P8, or in a field the five of field_planes.
+template <bool FIELD>
+constexpr int kPlanes = FIELD ? 5 : 2;
+
+template <bool FIELD, int K>
 __device__ __forceinline__ void draw_item(const AheadArgs &a, uint32_t p, uint32_t sw, uint32_t idx)
 {
+    constexpr int NP = kPlanes<FIELD>;
     const uint32_t t = a.d_t0 + sw;
     // mask order: pair of rows, word, row of the pair
     const uint32_t pair = a.by_wc.quotient(idx >> 1), w = (idx >> 1) - pair * a.wc;
     const uint32_t g0 = (2u * pair + (idx & 1u)) * (a.L >> 3) + w * 8u;
     const uint32_t x2k = (a.c3base | p) ^ a.key.k1[0];
-    uint32_t c0[K], c2[K], c3[K], m4[K], m8[K];
+    uint32_t c0[K], c2[K], c3[K], m[K][NP];
     {
         // the step's uniform values, lane k those of sweep t + k % K
         const uint64_t pb = (uint64_t)(t + (threadIdx.x & (K - 1u))) * kPhiloxMulB;
@@ -117,7 +122,8 @@ __device__ __forceinline__ void draw_item(const AheadArgs &a, uint32_t p, uint32
             c0[k] = K == 1 ? v0 : __shfl_sync(0xFFFFFFFFu, v0, k);
             c2[k] = K == 1 ? v2 : __shfl_sync(0xFFFFFFFFu, v2, k);
             c3[k] = K == 1 ? (uint32_t)pa : __shfl_sync(0xFFFFFFFFu, (uint32_t)pa, k);
-            m4[k] = m8[k] = 0u;
+#pragma unroll
+            for (int j = 0; j < NP; ++j) m[k][j] = 0u;
         }
     }
 #pragma unroll
@@ -129,23 +135,29 @@ __device__ __forceinline__ void draw_item(const AheadArgs &a, uint32_t p, uint32
             uint32_t u[4] = {(uint32_t)(pb >> 32) ^ c0[k], (uint32_t)pb, (uint32_t)pa ^ c2[k], c3[k]};
             philox_rounds_from<2>(u[0], u[1], u[2], u[3], a.key);
 #pragma unroll
-            for (int l = 0; l < 4; ++l) {
-                asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-                    : "+r"(m4[k])
-                    : "r"(u[l]), "r"(a.thr4), "r"(1u << (4 * q + l)));
-                asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-                    : "+r"(m8[k])
-                    : "r"(u[l]), "r"(a.thr8), "r"(1u << (4 * q + l)));
-            }
+            for (int l = 0; l < 4; ++l)
+#pragma unroll
+                for (int j = 0; j < NP; ++j)
+                    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
+                        : "+r"(m[k][j])
+                        : "r"(u[l]), "r"(a.thr[j]), "r"(1u << (4 * q + l)));
         }
     }
-    uint2 *out = a.d_masks + (size_t)(2u * sw + p) * a.nwords + idx;
 #pragma unroll
-    for (int k = 0; k < K; ++k) out[(size_t)(2 * k) * a.nwords] = make_uint2(m4[k], m8[k]);
+    for (int k = 0; k < K; ++k) {
+        char *const step = a.d_masks + (size_t)(2u * (sw + k) + p) * a.step_bytes;
+        if constexpr (FIELD) {
+            reinterpret_cast<uint4 *>(step)[idx] = make_uint4(m[k][0], m[k][1], m[k][2], m[k][3]);
+            reinterpret_cast<uint32_t *>(step + (size_t)a.nwords * 16u)[idx] = m[k][4];
+        } else {
+            reinterpret_cast<uint2 *>(step)[idx] = make_uint2(m[k][0], m[k][1]);
+        }
+    }
 }
 
 // The warps of the launch take tickets for 32 items each (consecutive words of
 // one colour and group of sweeps: nwords is a multiple of 64).
+template <bool FIELD>
 __device__ __forceinline__ void draw_role(const AheadArgs &a)
 {
     const uint32_t lane = threadIdx.x & 31u, per_group = a.nwords / 32u;
@@ -156,9 +168,9 @@ __device__ __forceinline__ void draw_role(const AheadArgs &a)
         if (lane == 0) next = atomicAdd(a.d_ticket, 1u);  // back before this item is done
         const uint32_t gp = a.by_group.quotient(it), idx = (it - gp * per_group) * 32u + lane;
         if (a.d_four)
-            draw_item<4>(a, gp & 1u, (gp >> 1) * 4u, idx);
+            draw_item<FIELD, 4>(a, gp & 1u, (gp >> 1) * 4u, idx);
         else
-            draw_item<1>(a, gp & 1u, gp >> 1, idx);
+            draw_item<FIELD, 1>(a, gp & 1u, gp >> 1, idx);
     }
 }
 
@@ -168,6 +180,10 @@ __device__ __forceinline__ void draw_role(const AheadArgs &a)
 __device__ __forceinline__ void copy_async16(uint32_t dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async8(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -248,6 +264,36 @@ __device__ __forceinline__ void step_run(uint32_t (&v)[2][KW], const uint32_t (&
         v[P][k] = x;
     }
 }
+// The same in a field H.  With sigma the spin in units of the field's sign, a flip
+// has the class (sigma, c), c the number of anti-aligned neighbours.  Classes sigma =
+// +1 are always taken from c = kA (3, 4 or 5) on, classes sigma = -1 from c = kB on,
+// and kA + kB <= 5 (the neighbour sums n > -|H| and n < -|H| are different ones): five
+// planes hold all draws, P0 .. P2 for sigma = +1, c = 0 .. 2, P3 for (+1, 3) or else
+// (-1, 1), P4 for (+1, 4) or else (-1, 0); a class that is always taken gets an all-one
+// word.  The thresholds of one sigma grow with c, so that "c >= j and below the j-th"
+// for j = 0 .. c adds nothing to "below the c-th".
+template <int KW, int P>
+__device__ __forceinline__ void step_run_field(const AheadArgs &a, uint32_t (&v)[2][KW], const uint32_t (&hz)[KW], uint32_t up,
+                                               uint32_t dn, const uint4 (&m)[KW], const uint2 (&m4)[KW / 2])
+{
+#pragma unroll
+    for (int k = 0; k < KW; ++k) {
+        const uint32_t p4 = (k & 1) ? m4[k / 2].y : m4[k / 2].x;
+        const uint32_t n1 = v[1 - P][k];
+        const uint32_t n2 = ((k + P) & 1) ? __funnelshift_r(n1, hz[k], 1) : __funnelshift_l(hz[k], n1, 1);
+        const uint32_t n3 = k == 0 ? up : v[1 - P][k - 1], n4 = k == KW - 1 ? dn : v[1 - P][k + 1];
+        const uint32_t s3 = n1 ^ n2 ^ n3, m3 = (n1 & n2) | (n3 & (n1 | n2));
+        const uint32_t x = v[P][k];
+        const uint32_t t = (x ^ s3) & (x ^ n4);
+        const uint32_t b0 = s3 ^ n4, b1 = (x ^ m3) ^ t, b2 = (x ^ m3) & t;  // c = b0 + 2 b1 + 4 b2
+        const uint32_t ge1 = b0 | b1 | b2, ge2 = b1 | b2, ge3 = (b0 & b1) | b2;
+        uint32_t plus = m[k].x | (ge1 & m[k].y);
+        plus |= ge2 & m[k].z;
+        plus |= (ge3 & (m[k].w | a.plus3)) | (b2 & (p4 | a.plus4));
+        const uint32_t minus = ge2 | (ge1 & (m[k].w | a.minus1)) | (p4 | a.minus0);
+        v[P][k] = x ^ (((x ^ a.flipped) & plus) | (~(x ^ a.flipped) & minus));
+    }
+}
 // After the step of parity 1: +1 spins of the run, and the anti-aligned bonds of
 // its sites of parity 1 (every bond of the lattice once), by the bit-sliced sum
 // b0 + 2 b1 + 4 b2 of a site's four.
@@ -290,15 +336,20 @@ __device__ __forceinline__ void store_snapshot(const AheadArgs &a, uint32_t slot
 }
 
 // One tile through the block: threads hold KW rows of one column each (a run).
-template <int KW>
+template <int KW, bool FIELD>
 __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, unsigned char *smem)
 {
-    constexpr uint32_t ST = stages_of(KW);
+    constexpr uint32_t ST = stages_of(KW, FIELD);
+    constexpr uint32_t NQ = FIELD ? KW : KW / 2;                  // 16-byte mask units of a run and step
     const uint32_t tid = threadIdx.x, wc = a.wc, L = a.L;
     const uint32_t nruns = (a.tile_rows + 2 * a.halo) / KW, nthr = nruns * wc;  // threads with a run
     const uint32_t nbar = (nthr + 31u) & ~31u;
-    uint4 *const ring = reinterpret_cast<uint4 *>(smem);          // [ST][KW / 2][kThreads]: (P4, P8) of two rows
-    uint32_t *const X = reinterpret_cast<uint32_t *>(ring + ST * (KW / 2) * kThreads);  // [2][KW][kThreads]: the two colours
+    // [ST][NQ][kThreads]: (P4, P8) of two rows, or the first four planes of a row
+    uint4 *const ring = reinterpret_cast<uint4 *>(smem);
+    // in a field [ST][KW / 2][kThreads]: the fifth plane of two rows
+    uint2 *const ring4 = reinterpret_cast<uint2 *>(ring + ST * NQ * kThreads);
+    // [2][KW][kThreads]: the two colours
+    uint32_t *const X = reinterpret_cast<uint32_t *>(ring4 + (FIELD ? ST * (KW / 2) * kThreads : 0u));
     uint32_t *const cnt = X + 2 * KW * kThreads;                   // [samples of the block, last state][2]
     const bool whole = a.halo == 0u;                              // the tile is the lattice
     if (!whole) {
@@ -321,17 +372,27 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
         if (!whole) useful = min(useful, __reduce_max_sync(0xFFFFFFFFu, (min(run, nruns - 1u - run) + 1u) * KW - 1u));
 
         // the masks of the next step not yet asked for, into its stage
-        const uint4 *msrc = reinterpret_cast<const uint4 *>(a.u_masks) + (size_t)(group * (KW / 2)) * wc + w;
-        const uint32_t mdst = shared_addr(ring + c);
+        const size_t first = (size_t)(group * (KW / 2)) * wc + w;   // the run's first pair of rows
+        const char *msrc = a.u_masks + first * (FIELD ? 32u : 16u), *msrc4 = a.u_masks + (size_t)a.nwords * 16u + first * 8u;
+        const uint32_t mdst = shared_addr(ring + c), mdst4 = shared_addr(ring4 + c);
         uint32_t fetched = 0;
         auto fetch = [&]() {
             if (fetched < useful) {
+                const uint32_t st = fetched & (ST - 1u);
 #pragma unroll
-                for (int k = 0; k < KW / 2; ++k)
-                    copy_async16(mdst + ((fetched & (ST - 1u)) * (KW / 2) + k) * kThreads * 16u, msrc + k * wc);
+                for (int k = 0; k < KW / 2; ++k) {
+                    if constexpr (FIELD) {
+                        copy_async16(mdst + (st * NQ + 2 * k) * kThreads * 16u, msrc + (size_t)k * wc * 32u);
+                        copy_async16(mdst + (st * NQ + 2 * k + 1) * kThreads * 16u, msrc + (size_t)k * wc * 32u + 16u);
+                        copy_async8(mdst4 + (st * (KW / 2) + k) * kThreads * 8u, msrc4 + (size_t)k * wc * 8u);
+                    } else {
+                        copy_async16(mdst + (st * NQ + k) * kThreads * 16u, msrc + k * wc * 16u);
+                    }
+                }
             }
             copy_commit();
-            msrc += a.nwords / 2;
+            msrc += a.step_bytes;
+            msrc4 += a.step_bytes;
             ++fetched;
         };
 #pragma unroll
@@ -345,10 +406,19 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
             X[(KW + k) * kThreads + c] = v[1][k];
         }
         Counting cn{a.u_phase, 0u};
-        uint4 m[KW / 2];
-        copy_wait<ST - 1>();
+        uint4 m[NQ];
+        uint2 m4[KW / 2];
+        auto masks_of = [&](uint32_t s) {
+            copy_wait<ST - 1>();
+            const uint32_t st = s & (ST - 1u);
 #pragma unroll
-        for (int k = 0; k < KW / 2; ++k) m[k] = ring[k * kThreads + c];
+            for (int k = 0; k < (int)NQ; ++k) m[k] = ring[(st * NQ + k) * kThreads + c];
+            if constexpr (FIELD) {
+#pragma unroll
+                for (int k = 0; k < KW / 2; ++k) m4[k] = ring4[(st * (KW / 2) + k) * kThreads + c];
+            }
+        };
+        masks_of(0);
         asm volatile("bar.sync 1, %0;" ::"r"(nbar) : "memory");
 
         auto step = [&](auto parity, uint32_t s, bool count) {
@@ -359,14 +429,15 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
 #pragma unroll
                 for (int k = 0; k < KW; ++k) hz[k] = B[k * kThreads + (((k + P) & 1) ? xr : xl)];
                 const uint32_t up = B[xu], dn = B[xd];
-                step_run<KW, P>(v, hz, up, dn, m);
+                if constexpr (FIELD)
+                    step_run_field<KW, P>(a, v, hz, up, dn, m, m4);
+                else
+                    step_run<KW, P>(v, hz, up, dn, m);
 #pragma unroll
                 for (int k = 0; k < KW; ++k) X[(P * KW + k) * kThreads + c] = v[P][k];
                 // the next step's masks, while the others reach the barrier
                 fetch();  // into the stage of this step, whose masks are in registers
-                copy_wait<ST - 1>();
-#pragma unroll
-                for (int k = 0; k < KW / 2; ++k) m[k] = ring[(((s + 1u) & (ST - 1u)) * (KW / 2) + k) * kThreads + c];
+                masks_of(s + 1u);
                 if (P == 1 && count) {
                     if (whole) {
                         if (tid < nthr) store_snapshot<KW>(a, cn.slot, c, nthr, v);
@@ -507,7 +578,7 @@ __device__ __forceinline__ void count_role(const AheadArgs &a, uint32_t cta)
     }
 }
 
-template <int KW, bool WARP>
+template <int KW, bool WARP, bool FIELD>
 __global__ void __launch_bounds__(kThreads, 1) k_ahead(const __grid_constant__ AheadArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -523,19 +594,20 @@ __global__ void __launch_bounds__(kThreads, 1) k_ahead(const __grid_constant__ A
         if constexpr (WARP)
             update_warp(a, smem);
         else
-            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<KW>(a, t, smem);
+            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<KW, FIELD>(a, t, smem);
     } else if (blockIdx.x < early) {
         count_role<KW>(a, blockIdx.x - a.update_ctas);
     }
-    if (a.d_tickets != 0u) draw_role(a);
+    if (a.d_tickets != 0u) draw_role<FIELD>(a);
 }
 
 using AheadKernel = void (*)(AheadArgs);
 
 AheadKernel pick_kernel(const AheadPlan &p)
 {
-    if (p.warp) return k_ahead<2, true>;
-    return p.kw == 2 ? k_ahead<2, false> : p.kw == 4 ? k_ahead<4, false> : p.kw == 8 ? k_ahead<8, false> : nullptr;
+    if (p.field) return p.kw == 2 ? k_ahead<2, false, true> : p.kw == 4 ? k_ahead<4, false, true> : nullptr;
+    if (p.warp) return k_ahead<2, true, false>;
+    return p.kw == 2 ? k_ahead<2, false, false> : p.kw == 4 ? k_ahead<4, false, false> : p.kw == 8 ? k_ahead<8, false, false> : nullptr;
 }
 
 constexpr int kMaxDevices = 64;
@@ -587,13 +659,17 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 //   L = 2048,  200 sweeps: 64 + 32: 606, 64 + 16: 630, 32 + 16: 659
 //   L = 4096,  200 sweeps: 32 + 16: 2225, 16 + 8: 2399
 // Above 8192 a block would hold fewer than 4 sweeps and its masks 25 times the
-// lattice: the step kernels run there.  min_sweeps: a call has one launch more than
+// lattice: the step kernels run there.  In a field (20 bytes of masks a word and step
+// instead of 8, five compares a draw instead of two) L <= 4096.  Measured, 200 sweeps
+// with M/E every sweep, the field step kernel (L = 64 .. 512: the one-launch field
+// kernels) against this form: L = 64 547 -> 102 us, 512 1384 -> 251, 704 5568 -> 357,
+// 2048 5593 -> 991; 20 sweeps of 4096 689 -> 425.  min_sweeps: a call has one launch more than
 // it has blocks, and the one-launch forms (L = 64, 128, 256) and two step launches
 // per sweep (above) are as fast on shorter calls.
-AheadPlan ahead_plan(uint64_t L)
+AheadPlan ahead_plan(uint64_t L, bool field)
 {
     AheadPlan p{};
-    if (L % 64 != 0 || L < 64 || L > 8192) return p;
+    if (L % 64 != 0 || L < 64 || L > (field ? 4096 : 8192)) return p;
     const uint32_t wc = (uint32_t)(L / 64);
     if (L <= 192) {
         p.tile_rows = (uint32_t)L;
@@ -601,15 +677,21 @@ AheadPlan ahead_plan(uint64_t L)
     } else {
         p.tile_rows = L >= 1024 && L <= 2048 ? 64 : L <= 4096 ? 32 : 16;
         p.halo = L <= 256 ? 64 : L <= 2048 ? 32 : L <= 4096 ? 16 : 8;
+        if (field) {  // at most 2048 words of a colour: five planes of masks take the shared memory of 4 rows a thread
+            p.tile_rows = L <= 1024 || L > 2048 ? std::min(p.tile_rows, L <= 1024 ? 64u : 16u) : 32u;
+            p.halo = std::min(p.halo, L <= 1024 ? 32u : L <= 2048 ? 16u : 8u);
+        }
     }
     p.block_sweeps = p.halo ? p.halo / 2 : 256;
-    p.min_sweeps = L == 64 ? 200 : L == 128 ? 100 : L == 256 ? 10 : L < 2048 ? 3 : 5;
+    p.min_sweeps = field ? (L <= 512 && (L & (L - 1)) == 0 ? 5 : L > 2048 ? 3 : 1) : L == 64 ? 200 : L == 128 ? 100 : L == 256 ? 10 : L < 2048 ? 3 : 5;
     const uint32_t rows = p.tile_rows + 2 * p.halo, most = p.halo ? kThreads : kThreads / 2;
     for (p.kw = 2; rows / p.kw * wc > most;) p.kw *= 2;
-    p.warp = L == 64;
+    p.warp = L == 64 && !field;
     p.tiles = (uint32_t)(L / p.tile_rows);
     p.update_ctas = std::min(p.tiles, 64u);
-    p.mask_bytes = (size_t)2 * p.block_sweeps * L * wc * 8;
+    p.field = field;
+    p.step_bytes = (uint32_t)(L * wc * (field ? 20 : 8));
+    p.mask_bytes = (size_t)2 * p.block_sweeps * p.step_bytes;
     p.snap_bytes = p.halo ? 0 : (size_t)(p.block_sweeps + 1) * L * wc * 8;
     return p;
 }
@@ -621,7 +703,7 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
     const AheadKernel kern = pick_kernel(pl);
     if (!kern) return cudaErrorInvalidValue;
     int sms = 0;
-    cudaError_t e = prepare_device(kern, pl.warp ? 0 : pl.kw / 2, &sms);
+    cudaError_t e = prepare_device(kern, pl.warp ? 0 : pl.kw / 2 + (pl.field ? 8 : 0), &sms);
     if (e != cudaSuccess) return e;
     a.update_ctas = a.u_steps ? pl.update_ctas : 0u;
     const uint32_t per = (a.nwords / pl.kw + 31u) & ~31u;
@@ -632,7 +714,7 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
     const uint32_t grid = std::max(early, std::min<uint32_t>((uint32_t)sms, early + (a.d_tickets + warps - 1) / warps));
     const size_t smem = !a.u_steps ? 0
                         : pl.warp  ? kWarpStages * kChunk * 512
-                                   : (stages_of(pl.kw) + 1) * pl.kw * kThreads * 8 + (pl.halo ? (size_t)a.u_slots * 8 : 0);
+                                   : (stages_of(pl.kw, pl.field) * (pl.field ? 20 : 8) + 8) * pl.kw * kThreads + (pl.halo ? (size_t)a.u_slots * 8 : 0);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kThreads);
@@ -657,6 +739,12 @@ bool ahead_ready(ising_lattice *h, const AheadPlan &pl)
         cudaGetLastError();
         return false;  // no allocation while the stream is captured
     }
+    if (h->d_ahead) {  // a smaller one, of the form without a field
+        if (cudaStreamSynchronize(h->stream) != cudaSuccess) return false;
+        h->alloc.release_scratch(h->d_ahead, h->stream);
+        h->d_ahead = nullptr;
+        h->ahead_bytes = 0;
+    }
     h->d_ahead = h->alloc.scratch(need, h->stream);
     h->ahead_bytes = h->d_ahead ? need : 0;
     return h->d_ahead != nullptr;
@@ -673,8 +761,26 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     uint64_t *const other = pl.halo ? reinterpret_cast<uint64_t *>(snaps + 2 * pl.snap_bytes) : spins;
     AheadArgs a{};
     a.key = h->key;
-    a.thr4 = h->thr4;
-    a.thr8 = h->thr8;
+    a.step_bytes = pl.step_bytes;
+    if (pl.field) {
+        // the five planes of step_run_field; i: the spin direction of sigma = +1
+        const FieldTable &ft = h->field;
+        const uint32_t i = h->H > 0.0 ? 1 : 0, kA = i ? ft.k_up : ft.k_dn, kB = i ? ft.k_dn : ft.k_up;
+        const uint32_t *const A = ft.thr + 8 * i, *const B = ft.thr + 8 * (1 - i);
+        a.thr[0] = A[0];
+        a.thr[1] = A[1];
+        a.thr[2] = A[2];
+        a.thr[3] = kA > 3 ? A[3] : kB > 1 ? B[1] : 0u;
+        a.thr[4] = kA > 4 ? A[4] : kB > 0 ? B[0] : 0u;
+        a.plus3 = kA > 3 ? 0u : ~0u;
+        a.plus4 = kA > 4 ? 0u : ~0u;
+        a.minus0 = kB > 0 ? 0u : ~0u;
+        a.minus1 = kB > 1 ? 0u : ~0u;
+        a.flipped = i ? 0u : ~0u;
+    } else {
+        a.thr[0] = h->thr4;
+        a.thr[1] = h->thr8;
+    }
     a.c3base = h->stream_id << 1;
     a.L = (uint32_t)h->L;
     a.wc = a.L / 64;
@@ -730,7 +836,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
             a.u_step0 = (uint32_t)(2 * done);
             a.src = src;
             a.dst = src == spins ? other : spins;
-            a.u_masks = reinterpret_cast<const uint2 *>(masks + ((b - 1) % kBuffers) * pl.mask_bytes);
+            a.u_masks = masks + ((b - 1) % kBuffers) * pl.mask_bytes;
             a.u_snaps = reinterpret_cast<uint32_t *>(snaps + (b % 2) * pl.snap_bytes);
             a.u_phase = record_every ? (uint32_t)(t % record_every) : 0u;
             a.u_recs = record_every ? (uint32_t)((t + prev) / record_every - t / record_every) : 0u;
@@ -743,7 +849,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
         }
         a.d_t0 = (uint32_t)(t0 + drawn);
         a.d_sweeps = (uint32_t)n;
-        a.d_masks = reinterpret_cast<uint2 *>(masks + (b % kBuffers) * pl.mask_bytes);
+        a.d_masks = masks + (b % kBuffers) * pl.mask_bytes;
         a.d_ticket = tickets + b % 4;
         a.next_ticket = tickets + (b + 2) % 4;
         if (!a.u_steps && !n && !a.c_slots) break;

@@ -16,8 +16,10 @@ struct AheadPlan {
     uint32_t tiles;
     uint32_t update_ctas;   // CTAs that share them
     bool warp;              // one warp holds the lattice
+    bool field;             // in a field: five mask planes
     uint32_t block_sweeps;  // sweeps of a block at most (halo / 2 where there is a halo)
     uint32_t min_sweeps;    // shorter calls are as fast without
+    uint32_t step_bytes;    // masks of a step
     size_t mask_bytes;      // one buffer of masks
     size_t snap_bytes;      // one buffer of snapshots
 };
@@ -31,9 +33,11 @@ struct FastDiv {
 // The arguments of one launch.
 struct AheadArgs {
     RoundKeys key;
-    uint32_t thr4, thr8, c3base;
+    uint32_t thr[5], c3base;      // thresholds of the mask planes: P4 and P8, or the five in a field
+    uint32_t plus3, plus4, minus0, minus1, flipped;  // in a field (step_run_field)
     uint32_t L, wc, nwords;       // words per row and in all, of one colour
     FastDiv by_wc, by_group;      // divisions by wc and nwords / 32
+    uint32_t step_bytes;          // of a step's masks
     uint32_t record_every;        // 0: record nothing
     unsigned long long *acc, *final_acc;
     unsigned int *err;            // set when a wait ran out
@@ -43,7 +47,7 @@ struct AheadArgs {
     uint32_t u_steps, u_step0;    // steps; index of the first in the call
     const uint64_t *src;
     uint64_t *dst;
-    const uint2 *u_masks;
+    const char *u_masks;
     uint32_t *u_snaps;            // states after the counted sweeps (where the tile is the lattice)
     uint32_t u_phase;             // sweep index % record_every at the block's start
     uint32_t u_recs, u_slot0;     // samples of the block, slot of the first
@@ -53,11 +57,11 @@ struct AheadArgs {
     const uint32_t *c_snaps;
     // draw: d_sweeps sweeps from sweep index d_t0, in tickets of 32 items of 4 sweeps or of one
     uint32_t d_t0, d_sweeps, d_four, d_tickets;
-    uint2 *d_masks;
+    char *d_masks;
     unsigned int *d_ticket, *next_ticket;  // this launch's counter; the one to clear
 };
 
-AheadPlan ahead_plan(uint64_t L);
+AheadPlan ahead_plan(uint64_t L, bool field);
 
 }  // namespace ising
 

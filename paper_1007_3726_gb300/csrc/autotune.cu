@@ -268,7 +268,7 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
         }
     }
     // the draw-ahead form on the copy, where it applies (the copy is the whole lattice there)
-    const AheadPlan pl = ahead_plan(h->L);
+    const AheadPlan pl = ahead_plan(h->L, false);
     bool ahead = false;
     if (e == cudaSuccess && pl.kw != 0 && rows == h->L && ahead_ready(h, pl)) {
         const uint32_t n = std::max(8 * reps, 2 * pl.min_sweeps);

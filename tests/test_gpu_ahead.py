@@ -74,6 +74,39 @@ def test_temperatures_and_changes_between_calls(P, orc, T):
     lat.close()
 
 
+# neighbour sums strictly inside, on and outside the field's zeros: 0 to 5 thresholds a sign
+@pytest.mark.parametrize("H", [0.1, -0.1, 2.0, -2.0, 3.0, -3.5, 4.0, -4.0, 7.25, 1e-300, -1e3])
+@pytest.mark.parametrize("L", [64, 320])
+def test_field_classes_bit_exact(P, orc, L, H):
+    T, seed, sid = 2.1, 9, 3
+    lat = P.Lattice(L, T, seed=seed, stream_id=sid, init="hot", H=H)
+    s, t = orc.init_hot(L, seed, sid), 0
+    for n, rec in ((205, 1), (34, 3)) if L == 64 else ((34, 1), (37, 3)):
+        M, E = lat.sweep(n, rec, collect=True)
+        Mo, Eo = orc.run_field(s, n, seed, sid, T, H, t0=t)
+        k0 = (rec - 1 - t) % rec
+        assert np.array_equal(M, Mo[k0::rec]) and np.array_equal(E, Eo[k0::rec]), (n, rec)
+        assert np.array_equal(lat.spins(), s)
+        t += n
+    lat.close()
+
+
+@pytest.mark.parametrize("L", [64, 128, 192, 256, 448, 704, 1024, 1088, 2048, 2112, 4096, 4160])
+def test_field_sizes_bit_exact(P, orc, L):
+    T, H, seed = TC, -0.4, L
+    lat = P.Lattice(L, T, seed=seed, init="hot")
+    s, t = orc.init_hot(L, seed, 0), 0
+    n = 210 if L <= 128 else 12
+    _compare(orc, lat, s, 0, n, 2, seed, 0, orc.thresholds(T))  # scratch of the smaller form first
+    lat.set_field(H)
+    M, E = lat.sweep(n + 5, 3, collect=True)
+    Mo, Eo = orc.run_field(s, n + 5, seed, 0, T, H, t0=n)
+    k0 = (2 - n) % 3
+    assert np.array_equal(M, Mo[k0::3]) and np.array_equal(E, Eo[k0::3])
+    assert np.array_equal(lat.spins(), s)
+    lat.close()
+
+
 def test_late_sweep_indices_and_high_stream(P, orc):
     """Sweep indices next to 2^32 and the largest stream id in the Philox counter."""
     L, seed, sid, t = 128, 2 ** 63 + 5, 2 ** 31 - 1, 2 ** 32 - 300
