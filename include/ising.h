@@ -328,6 +328,12 @@ ISING_API ising_status ising_bench_mix(uint32_t form, uint32_t words_per_thread,
  * final states are bit-identical to ising_sweep on each handle: the batch
  * changes where and when sites are updated, never how.
  *
+ * Runs of 8 or more sweeps (12 where no lattice is larger than 128) of lattices up to
+ * L = 4096 (in a field 2048) in a batch without launch options (block .. insert,
+ * wait_ms, hold_strip all zero) take the draw-ahead form of ising_launch instead, over
+ * all lattices at once, if its scratch memory (at least three times a byte per lattice
+ * site, in a field 2.5) is to be had; ising_batch_info still describes the strips.
+ *
  * Options (zero = default):
  *   block          threads per CTA, 128, 256 or 512 (512)
  *   ctas_per_sm    resident CTAs per SM the plan is made for (2); each CTA gets

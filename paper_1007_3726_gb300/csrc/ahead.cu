@@ -50,7 +50,10 @@ namespace {
 // a microsecond with the L2 busy) against the time of a step, within 160 KiB.
 __host__ __device__ constexpr uint32_t stages_of(uint32_t kw, bool field) { return kw == 8 || (field && kw == 4) ? 4 : 8; }
 
-constexpr uint32_t kThreads = 512;  // per CTA; one CTA per SM, so that an update has an SM to itself
+// Threads per CTA.  One lattice: one CTA per SM, so that an update, which the next
+// launch waits for, has an SM to itself.  Several lattices: two CTAs per SM, so that
+// one draws while the other waits for rows and masks.
+constexpr uint32_t kThreads = 512, kBatchThreads = 256;
 
 constexpr uint32_t kChunk = 8;     // steps of a stage of the one-warp form
 constexpr uint32_t kWarpStages = 8;
@@ -102,11 +105,12 @@ __device__ __forceinline__ uint64_t spread_bits(uint32_t v)
 template <bool FIELD>
 constexpr int kPlanes = FIELD ? 5 : 2;
 
-template <bool FIELD, int K>
-__device__ __forceinline__ void draw_item(const AheadArgs &a, uint32_t p, uint32_t sw, uint32_t idx)
+// a: the lattice (AheadArgs or AheadJob); masks, t0: the block's buffer and first sweep index.
+template <bool FIELD, int K, typename A>
+__device__ __forceinline__ void draw_item(const A &a, char *masks, uint32_t t0, uint32_t p, uint32_t sw, uint32_t idx)
 {
     constexpr int NP = kPlanes<FIELD>;
-    const uint32_t t = a.d_t0 + sw;
+    const uint32_t t = t0 + sw;
     // mask order: pair of rows, word, row of the pair
     const uint32_t pair = a.by_wc.quotient(idx >> 1), w = (idx >> 1) - pair * a.wc;
     const uint32_t g0 = (2u * pair + (idx & 1u)) * (a.L >> 3) + w * 8u;
@@ -145,7 +149,7 @@ __device__ __forceinline__ void draw_item(const AheadArgs &a, uint32_t p, uint32
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        char *const step = a.d_masks + (size_t)(2u * (sw + k) + p) * a.step_bytes;
+        char *const step = masks + (size_t)(2u * (sw + k) + p) * a.step_bytes;
         if constexpr (FIELD) {
             reinterpret_cast<uint4 *>(step)[idx] = make_uint4(m[k][0], m[k][1], m[k][2], m[k][3]);
             reinterpret_cast<uint32_t *>(step + (size_t)a.nwords * 16u)[idx] = m[k][4];
@@ -168,9 +172,9 @@ __device__ __forceinline__ void draw_role(const AheadArgs &a)
         if (lane == 0) next = atomicAdd(a.d_ticket, 1u);  // back before this item is done
         const uint32_t gp = a.by_group.quotient(it), idx = (it - gp * per_group) * 32u + lane;
         if (a.d_four)
-            draw_item<FIELD, 4>(a, gp & 1u, (gp >> 1) * 4u, idx);
+            draw_item<FIELD, 4>(a, a.d_masks, a.d_t0, gp & 1u, (gp >> 1) * 4u, idx);
         else
-            draw_item<FIELD, 1>(a, gp & 1u, gp >> 1, idx);
+            draw_item<FIELD, 1>(a, a.d_masks, a.d_t0, gp & 1u, gp >> 1, idx);
     }
 }
 
@@ -336,7 +340,7 @@ __device__ __forceinline__ void store_snapshot(const AheadArgs &a, uint32_t slot
 }
 
 // One tile through the block: threads hold KW rows of one column each (a run).
-template <int KW, bool FIELD>
+template <uint32_t THREADS, int KW, bool FIELD>
 __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, unsigned char *smem)
 {
     constexpr uint32_t ST = stages_of(KW, FIELD);
@@ -344,16 +348,17 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
     const uint32_t tid = threadIdx.x, wc = a.wc, L = a.L;
     const uint32_t nruns = (a.tile_rows + 2 * a.halo) / KW, nthr = nruns * wc;  // threads with a run
     const uint32_t nbar = (nthr + 31u) & ~31u;
-    // [ST][NQ][kThreads]: (P4, P8) of two rows, or the first four planes of a row
+    // [ST][NQ][THREADS]: (P4, P8) of two rows, or the first four planes of a row
     uint4 *const ring = reinterpret_cast<uint4 *>(smem);
-    // in a field [ST][KW / 2][kThreads]: the fifth plane of two rows
-    uint2 *const ring4 = reinterpret_cast<uint2 *>(ring + ST * NQ * kThreads);
-    // [2][KW][kThreads]: the two colours
-    uint32_t *const X = reinterpret_cast<uint32_t *>(ring4 + (FIELD ? ST * (KW / 2) * kThreads : 0u));
-    uint32_t *const cnt = X + 2 * KW * kThreads;                   // [samples of the block, last state][2]
+    // in a field [ST][KW / 2][THREADS]: the fifth plane of two rows
+    uint2 *const ring4 = reinterpret_cast<uint2 *>(ring + ST * NQ * THREADS);
+    // [2][KW][THREADS]: the two colours
+    uint32_t *const X = reinterpret_cast<uint32_t *>(ring4 + (FIELD ? ST * (KW / 2) * THREADS : 0u));
+    uint32_t *const cnt = X + 2 * KW * THREADS;                   // [samples of the block, last state][2]
     const bool whole = a.halo == 0u;                              // the tile is the lattice
-    if (!whole) {
-        for (uint32_t k = tid; k < 2 * a.u_slots; k += kThreads) cnt[k] = 0u;
+    const bool snaps = a.u_snaps != nullptr;                      // counted sweeps go out as snapshots
+    if (!snaps) {
+        for (uint32_t k = tid; k < 2 * a.u_slots; k += THREADS) cnt[k] = 0u;
         __syncthreads();
     }
     if (tid < nbar) {
@@ -364,7 +369,7 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
         while (group >= groups) group -= groups;
         const bool mine = tid < nthr && run >= a.halo / KW && run < (a.halo + a.tile_rows) / KW;
         const uint32_t xl = c - w + (w == 0 ? wc - 1u : w - 1u), xr = c - w + (w + 1u == wc ? 0u : w + 1u);
-        const uint32_t xu = (KW - 1) * kThreads + (run == 0 ? nthr - wc + w : c - wc);
+        const uint32_t xu = (KW - 1) * THREADS + (run == 0 ? nthr - wc + w : c - wc);
         const uint32_t xd = c + wc >= nthr ? w : c + wc;
         // the steps after which this warp's rows are of no more use: a step spoils a
         // row at either end of the tile
@@ -382,11 +387,11 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
 #pragma unroll
                 for (int k = 0; k < KW / 2; ++k) {
                     if constexpr (FIELD) {
-                        copy_async16(mdst + (st * NQ + 2 * k) * kThreads * 16u, msrc + (size_t)k * wc * 32u);
-                        copy_async16(mdst + (st * NQ + 2 * k + 1) * kThreads * 16u, msrc + (size_t)k * wc * 32u + 16u);
-                        copy_async8(mdst4 + (st * (KW / 2) + k) * kThreads * 8u, msrc4 + (size_t)k * wc * 8u);
+                        copy_async16(mdst + (st * NQ + 2 * k) * THREADS * 16u, msrc + (size_t)k * wc * 32u);
+                        copy_async16(mdst + (st * NQ + 2 * k + 1) * THREADS * 16u, msrc + (size_t)k * wc * 32u + 16u);
+                        copy_async8(mdst4 + (st * (KW / 2) + k) * THREADS * 8u, msrc4 + (size_t)k * wc * 8u);
                     } else {
-                        copy_async16(mdst + (st * NQ + k) * kThreads * 16u, msrc + k * wc * 16u);
+                        copy_async16(mdst + (st * NQ + k) * THREADS * 16u, msrc + k * wc * 16u);
                     }
                 }
             }
@@ -402,8 +407,8 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
         load_run<KW>(a.src + (size_t)(group * KW) * wc + w, wc, v);
 #pragma unroll
         for (int k = 0; k < KW; ++k) {
-            X[k * kThreads + c] = v[0][k];
-            X[(KW + k) * kThreads + c] = v[1][k];
+            X[k * THREADS + c] = v[0][k];
+            X[(KW + k) * THREADS + c] = v[1][k];
         }
         Counting cn{a.u_phase, 0u};
         uint4 m[NQ];
@@ -412,10 +417,10 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
             copy_wait<ST - 1>();
             const uint32_t st = s & (ST - 1u);
 #pragma unroll
-            for (int k = 0; k < (int)NQ; ++k) m[k] = ring[(st * NQ + k) * kThreads + c];
+            for (int k = 0; k < (int)NQ; ++k) m[k] = ring[(st * NQ + k) * THREADS + c];
             if constexpr (FIELD) {
 #pragma unroll
-                for (int k = 0; k < KW / 2; ++k) m4[k] = ring4[(st * (KW / 2) + k) * kThreads + c];
+                for (int k = 0; k < KW / 2; ++k) m4[k] = ring4[(st * (KW / 2) + k) * THREADS + c];
             }
         };
         masks_of(0);
@@ -424,22 +429,22 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
         auto step = [&](auto parity, uint32_t s, bool count) {
             constexpr int P = decltype(parity)::value;
             if (s < useful) {
-                const uint32_t *const B = X + (1 - P) * KW * kThreads;
+                const uint32_t *const B = X + (1 - P) * KW * THREADS;
                 uint32_t hz[KW];
 #pragma unroll
-                for (int k = 0; k < KW; ++k) hz[k] = B[k * kThreads + (((k + P) & 1) ? xr : xl)];
+                for (int k = 0; k < KW; ++k) hz[k] = B[k * THREADS + (((k + P) & 1) ? xr : xl)];
                 const uint32_t up = B[xu], dn = B[xd];
                 if constexpr (FIELD)
                     step_run_field<KW, P>(a, v, hz, up, dn, m, m4);
                 else
                     step_run<KW, P>(v, hz, up, dn, m);
 #pragma unroll
-                for (int k = 0; k < KW; ++k) X[(P * KW + k) * kThreads + c] = v[P][k];
+                for (int k = 0; k < KW; ++k) X[(P * KW + k) * THREADS + c] = v[P][k];
                 // the next step's masks, while the others reach the barrier
                 fetch();  // into the stage of this step, whose masks are in registers
                 masks_of(s + 1u);
                 if (P == 1 && count) {
-                    if (whole) {
+                    if (snaps) {
                         if (tid < nthr) store_snapshot<KW>(a, cn.slot, c, nthr, v);
                     } else {
                         uint32_t cu, ca;
@@ -463,7 +468,7 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
         }
         copy_wait<0>();
         // the block's samples (the last counter, if it is none, is the state after the call)
-        for (uint32_t k = tid; !whole && k < a.u_slots; k += nbar) {
+        for (uint32_t k = tid; !snaps && k < a.u_slots; k += nbar) {
             const unsigned long long up = cnt[2 * k], anti = cnt[2 * k + 1];
             if (k < a.u_recs) {
                 atomicAdd(a.acc + 2 * (size_t)(a.u_slot0 + k), up);
@@ -594,11 +599,131 @@ __global__ void __launch_bounds__(kThreads, 1) k_ahead(const __grid_constant__ A
         if constexpr (WARP)
             update_warp(a, smem);
         else
-            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<KW, FIELD>(a, t, smem);
+            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, KW, FIELD>(a, t, smem);
     } else if (blockIdx.x < early) {
         count_role<KW>(a, blockIdx.x - a.update_ctas);
     }
     if (a.d_tickets != 0u) draw_role<FIELD>(a);
+}
+
+// ----------------------------------------------------------------- batch --
+// Bound: the draws, 1.75 per ns (a lattice's keys come from registers here: 1.7), as
+// soon as the lattices together have some 64 M attempts a block; the tiles take the SMs
+// for about a fifth as long.  Measured, strips in one persistent launch (batch.cu) and
+// this: four sizes 256 .. 2048 at 32 temperatures, 100 sweeps 15043 -> 12885 us (1.38
+// attempts per ns); 32 of 512^2, 500 sweeps 10612 -> 3213; one of 2048^2 10998 -> 1554; 128
+// of 64^2 1284 -> 638.
+//
+// Many lattices: launch b draws block b of every lattice that has one and updates
+// block b - 1.  Lattices have blocks of their own length; they are sorted by the
+// number of their blocks, so that those still running come first.
+
+// The job that item `i` of a launch belongs to, by the running sums of the jobs.
+__device__ __forceinline__ uint32_t find_job(const AheadJob *jobs, uint32_t n, uint32_t i, uint32_t AheadJob::*start)
+{
+    uint32_t lo = 0, hi = n;
+    while (hi - lo > 1u) {
+        const uint32_t mid = (lo + hi) / 2u;
+        if (jobs[mid].*start <= i)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
+__device__ __forceinline__ void batch_draw_role(const AheadBatchArgs &a)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t next = lane == 0 ? atomicAdd(a.d_ticket, 1u) : 0u;
+    for (;;) {
+        const uint32_t it = __shfl_sync(0xFFFFFFFFu, next, 0);
+        if (it >= a.d_tickets) return;
+        if (lane == 0) next = atomicAdd(a.d_ticket, 1u);  // back before this item is done
+        const uint32_t ji = find_job(a.jobs, a.d_jobs, it, &AheadJob::ticket_start);
+        const AheadJob j = a.jobs[ji];
+        const uint32_t local = it - j.ticket_start, gp = j.by_group.quotient(local);
+        const uint32_t sw = (gp >> 1) * 4u;
+        if (sw >= j.sweeps - a.block * j.block_sweeps) continue;  // past the lattice's last sweep
+        const uint32_t idx = (local - gp * (j.nwords / 32u)) * 32u + lane;
+        char *const masks = j.masks + (size_t)(a.block % kBuffers) * j.mask_bytes;
+        const uint32_t t0 = a.t0[j.index] + a.block * j.block_sweeps;
+        if (j.field)
+            draw_item<true, 4>(j, masks, t0, gp & 1u, sw, idx);
+        else
+            draw_item<false, 4>(j, masks, t0, gp & 1u, sw, idx);
+    }
+}
+
+// The arguments of a tile's block, as the one-lattice form has them.
+__device__ __forceinline__ void batch_tile_args(const AheadBatchArgs &a, const AheadJob &j, AheadArgs &t)
+{
+    const uint32_t ub = a.block - 1u, done = ub * j.block_sweeps, n = min(j.block_sweeps, j.sweeps - done);
+    const uint32_t t0 = a.t0[j.index], re = j.record_every;
+    t.L = j.L;
+    t.wc = j.wc;
+    t.nwords = j.nwords;
+    t.by_wc = j.by_wc;
+    t.plus3 = j.plus3;
+    t.plus4 = j.plus4;
+    t.minus0 = j.minus0;
+    t.minus1 = j.minus1;
+    t.flipped = j.flipped;
+    t.step_bytes = j.step_bytes;
+    t.record_every = re;
+    t.acc = j.acc;
+    t.final_acc = j.final_acc;
+    t.tile_rows = j.tile_rows;
+    t.halo = j.halo;
+    t.u_steps = 2u * n;
+    t.src = (ub & 1u) ? j.odd : j.even;
+    t.dst = (ub & 1u) ? j.even : j.odd;
+    t.u_masks = j.masks + (size_t)(ub % kBuffers) * j.mask_bytes;
+    t.u_snaps = nullptr;
+    t.u_phase = re ? (t0 + done) % re : 0u;
+    t.u_recs = re ? (t.u_phase + n) / re : 0u;
+    t.u_slot0 = re ? (t0 % re + done) / re : 0u;
+    t.u_last = done + n == j.sweeps ? 1u : 0u;
+    t.u_slots = t.u_recs + ((t.u_last && !(re && (t.u_phase + n) % re == 0u)) ? 1u : 0u);
+}
+
+__global__ void __launch_bounds__(kBatchThreads, 2) k_ahead_batch(const __grid_constant__ AheadBatchArgs a)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ AheadArgs t;
+    // (waits as in k_ahead; the first launch copies the lattices whose last block
+    // would otherwise end in their second buffer)
+    if (blockIdx.x < a.update_ctas || a.block == 0u) dependent_launch_wait();
+    dependent_launch_trigger();
+    if (a.block == 0u) {
+        for (uint32_t k = blockIdx.x; k < a.d_jobs; k += gridDim.x) {
+            const AheadJob &j = a.jobs[k];
+            if (j.copy_from)
+                for (uint32_t i = threadIdx.x; i < j.nwords; i += kBatchThreads) j.even[i] = j.copy_from[i];
+        }
+    } else if (blockIdx.x < a.update_ctas) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *a.next_ticket = 0u;
+        for (uint32_t g = blockIdx.x; g < a.u_tiles; g += a.update_ctas) {
+            const uint32_t ji = find_job(a.jobs, a.u_jobs, g, &AheadJob::tile_start);
+            const AheadJob &j = a.jobs[ji];
+            if (threadIdx.x == 0) batch_tile_args(a, j, t);
+            __syncthreads();
+            const uint32_t tile = g - j.tile_start;
+            if (!j.field) {
+                if (j.kw == 2)
+                    update_tile<kBatchThreads, 2, false>(t, tile, smem);
+                else if (j.kw == 4)
+                    update_tile<kBatchThreads, 4, false>(t, tile, smem);
+                else
+                    update_tile<kBatchThreads, 8, false>(t, tile, smem);
+            } else if (j.kw == 2) {
+                update_tile<kBatchThreads, 2, true>(t, tile, smem);
+            } else {
+                update_tile<kBatchThreads, 4, true>(t, tile, smem);
+            }
+        }
+    }
+    if (a.d_tickets != 0u) batch_draw_role(a);
 }
 
 using AheadKernel = void (*)(AheadArgs);
@@ -698,6 +823,31 @@ AheadPlan ahead_plan(uint64_t L, bool field)
 
 namespace {
 
+// The mask planes' thresholds of a lattice, and in a field what step_run_field needs.
+template <typename A>
+void set_planes(A &a, const ising_lattice *h)
+{
+    if (h->H == 0.0) {
+        a.thr[0] = h->thr4;
+        a.thr[1] = h->thr8;
+        return;
+    }
+    const FieldTable &ft = h->field;
+    const uint32_t i = h->H > 0.0 ? 1 : 0;  // the spin direction of sigma = +1
+    const uint32_t kA = i ? ft.k_up : ft.k_dn, kB = i ? ft.k_dn : ft.k_up;
+    const uint32_t *const plus = ft.thr + 8 * i, *const minus = ft.thr + 8 * (1 - i);
+    a.thr[0] = plus[0];
+    a.thr[1] = plus[1];
+    a.thr[2] = plus[2];
+    a.thr[3] = kA > 3 ? plus[3] : kB > 1 ? minus[1] : 0u;
+    a.thr[4] = kA > 4 ? plus[4] : kB > 0 ? minus[0] : 0u;
+    a.plus3 = kA > 3 ? 0u : ~0u;
+    a.plus4 = kA > 4 ? 0u : ~0u;
+    a.minus0 = kB > 0 ? 0u : ~0u;
+    a.minus1 = kB > 1 ? 0u : ~0u;
+    a.flipped = i ? 0u : ~0u;
+}
+
 cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaStream_t s)
 {
     const AheadKernel kern = pick_kernel(pl);
@@ -762,25 +912,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     AheadArgs a{};
     a.key = h->key;
     a.step_bytes = pl.step_bytes;
-    if (pl.field) {
-        // the five planes of step_run_field; i: the spin direction of sigma = +1
-        const FieldTable &ft = h->field;
-        const uint32_t i = h->H > 0.0 ? 1 : 0, kA = i ? ft.k_up : ft.k_dn, kB = i ? ft.k_dn : ft.k_up;
-        const uint32_t *const A = ft.thr + 8 * i, *const B = ft.thr + 8 * (1 - i);
-        a.thr[0] = A[0];
-        a.thr[1] = A[1];
-        a.thr[2] = A[2];
-        a.thr[3] = kA > 3 ? A[3] : kB > 1 ? B[1] : 0u;
-        a.thr[4] = kA > 4 ? A[4] : kB > 0 ? B[0] : 0u;
-        a.plus3 = kA > 3 ? 0u : ~0u;
-        a.plus4 = kA > 4 ? 0u : ~0u;
-        a.minus0 = kB > 0 ? 0u : ~0u;
-        a.minus1 = kB > 1 ? 0u : ~0u;
-        a.flipped = i ? 0u : ~0u;
-    } else {
-        a.thr[0] = h->thr4;
-        a.thr[1] = h->thr8;
-    }
+    set_planes(a, h);
     a.c3base = h->stream_id << 1;
     a.L = (uint32_t)h->L;
     a.wc = a.L / 64;
@@ -837,7 +969,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
             a.src = src;
             a.dst = src == spins ? other : spins;
             a.u_masks = masks + ((b - 1) % kBuffers) * pl.mask_bytes;
-            a.u_snaps = reinterpret_cast<uint32_t *>(snaps + (b % 2) * pl.snap_bytes);
+            a.u_snaps = pl.halo ? nullptr : reinterpret_cast<uint32_t *>(snaps + (b % 2) * pl.snap_bytes);
             a.u_phase = record_every ? (uint32_t)(t % record_every) : 0u;
             a.u_recs = record_every ? (uint32_t)((t + prev) / record_every - t / record_every) : 0u;
             a.u_slot0 = (uint32_t)rec_done;
@@ -858,6 +990,174 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
         prev = n;
     }
     return cudaSuccess;
+}
+
+// ------------------------------------------------------------ batch, host --
+namespace {
+
+// Lattices up to this many words of a colour are one tile (L <= 256, in a field 192):
+// 128 lattices of 256^2, 500 sweeps, in one tile each 3176 us, in four with halos 3685;
+// 16 of 320^2 877 and 773; 16 of 256^2 in a field (with 16 of 512^2) 2451 and 2287.
+uint32_t whole_words(const AheadJob &j) { return j.field ? 576 : 1024; }
+
+// The tiles of a lattice in a batch for blocks of s sweeps: the lattice, or full rows
+// with halos, at most 8 rows a thread (in a field 4).  False if there are none.
+bool batch_tiles(AheadJob &j, uint32_t s)
+{
+    const uint32_t most = kBatchThreads * (j.field ? 4 : 8);
+    j.block_sweeps = s;
+    if (j.nwords <= whole_words(j)) {
+        j.tile_rows = j.L;
+        j.halo = 0;
+    } else {
+        j.halo = 2 * s;
+        j.tile_rows = 0;
+        for (uint32_t t : {64u, 32u, 16u})
+            if (t >= j.halo && j.L % t == 0 && (t + 2 * j.halo) * j.wc <= most) {
+                j.tile_rows = t;
+                break;
+            }
+        if (!j.tile_rows) return false;
+    }
+    const uint32_t rows = j.tile_rows + 2 * j.halo;
+    for (j.kw = 2; rows / j.kw * j.wc > kBatchThreads;) j.kw *= 2;
+    return rows * j.wc <= most;
+}
+
+}  // namespace
+
+// Blocks: the shortest (4 sweeps) for large lattices; longer ones for small lattices,
+// whose steps take as long but draw less, and where all together would not fill the
+// GPU for some 40 us a launch.
+bool AheadBatch::plan(const std::vector<ising_lattice *> &hs, const std::vector<uint64_t> &sweeps,
+                      const std::vector<uint32_t> &record_every)
+{
+    const size_t n = hs.size();
+    jobs.assign(n, AheadJob{});
+    std::vector<uint32_t> cap(n);
+    double work = 0;
+    for (size_t i = 0; i < n; ++i) {
+        AheadJob &j = jobs[i];
+        const ising_lattice *h = hs[i];
+        if (h->L > 4096) return false;
+        j.key = h->key;
+        set_planes(j, h);
+        j.c3base = h->stream_id << 1;
+        j.L = (uint32_t)h->L;
+        j.wc = j.L / 64;
+        j.nwords = j.L * j.wc;
+        j.by_wc = fast_div(j.wc);
+        j.by_group = fast_div(j.nwords / 32);
+        j.field = h->H != 0.0;
+        j.step_bytes = j.nwords * (j.field ? 20 : 8);
+        j.sweeps = (uint32_t)sweeps[i];
+        j.record_every = record_every[i];
+        j.index = (uint32_t)i;
+        for (cap[i] = j.nwords <= whole_words(j) ? 64 : 16; cap[i] >= 4 && !batch_tiles(j, cap[i]);) cap[i] /= 2;
+        if (cap[i] < 4) return false;
+        uint32_t s = 4;
+        while (s < cap[i] && s < j.sweeps && (uint64_t)2 * s * j.L * j.L <= (4u << 20)) s *= 2;
+        j.block_sweeps = s;
+        work += (double)s * j.L * j.L;
+    }
+    for (bool grown = true; work < (double)(64u << 20) && grown;) {
+        grown = false;
+        for (size_t i = 0; i < n; ++i)
+            if (jobs[i].block_sweeps < cap[i] && jobs[i].block_sweeps < jobs[i].sweeps) {
+                work += (double)jobs[i].block_sweeps * jobs[i].L * jobs[i].L;
+                jobs[i].block_sweeps *= 2;
+                grown = true;
+            }
+    }
+    size_t bytes = 0, cnt_slots = 0;
+    smem = 0;
+    for (AheadJob &j : jobs) {
+        if (!batch_tiles(j, j.block_sweeps)) return false;
+        j.nblocks = (j.sweeps + j.block_sweeps - 1) / j.block_sweeps;
+        j.mask_bytes = (size_t)2 * j.block_sweeps * j.step_bytes;
+        bytes += kBuffers * j.mask_bytes + (j.halo ? (size_t)j.nwords * 8 : 0);
+        cnt_slots = std::max<size_t>(cnt_slots, j.block_sweeps + 1);
+        smem = std::max<size_t>(smem, (size_t)(stages_of(j.kw, j.field) * (j.field ? 20 : 8) + 8) * j.kw * kBatchThreads);
+    }
+    smem += cnt_slots * 8;
+    std::stable_sort(jobs.begin(), jobs.end(), [](const AheadJob &x, const AheadJob &y) { return x.nblocks > y.nblocks; });
+    uint64_t tiles = 0, tickets = 0;
+    for (AheadJob &j : jobs) {
+        j.tile_start = (uint32_t)tiles;
+        j.ticket_start = (uint32_t)tickets;
+        tiles += j.L / j.tile_rows;
+        tickets += (uint64_t)(j.block_sweeps / 4) * 2 * (j.nwords / 32);
+    }
+    if (tickets >= (1ull << 31)) return false;
+    total_tiles = (uint32_t)tiles;
+    total_tickets = (uint32_t)tickets;
+    table_bytes = (kTicketBytes + n * sizeof(AheadJob) + 255) & ~(size_t)255;
+    scratch_bytes = table_bytes + bytes;
+    return true;
+}
+
+cudaError_t AheadBatch::upload(void *scratch, const std::vector<ising_lattice *> &hs,
+                               const std::vector<unsigned long long *> &acc, const std::vector<unsigned long long *> &final_acc,
+                               cudaStream_t s)
+{
+    d_scratch = static_cast<char *>(scratch);
+    char *at = d_scratch + table_bytes;
+    for (AheadJob &j : jobs) {
+        ising_lattice *h = hs[j.index];
+        uint64_t *const spins = static_cast<uint64_t *>(h->d_spins);
+        j.masks = at;
+        at += kBuffers * j.mask_bytes;
+        uint64_t *const other = j.halo ? reinterpret_cast<uint64_t *>(at) : spins;
+        if (j.halo) at += (size_t)j.nwords * 8;
+        const bool swap = j.halo && j.nblocks % 2 == 1;  // the last block ends in the lattice
+        j.even = swap ? other : spins;
+        j.odd = swap ? spins : other;
+        j.copy_from = swap ? spins : nullptr;
+        j.acc = acc[j.index];
+        j.final_acc = final_acc[j.index];
+    }
+    cudaError_t e = cudaMemcpyAsync(d_scratch + kTicketBytes, jobs.data(), jobs.size() * sizeof(AheadJob), cudaMemcpyHostToDevice, s);
+    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
+
+cudaError_t AheadBatch::enqueue(const uint32_t *d_t0, cudaStream_t s)
+{
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ahead_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem / 2);
+    unsigned int *const tickets = reinterpret_cast<unsigned int *>(d_scratch);
+    if (e == cudaSuccess) e = cudaMemsetAsync(tickets, 0, kTicketBytes, s);
+    if (e != cudaSuccess) return e;
+    AheadBatchArgs a{};
+    a.jobs = reinterpret_cast<const AheadJob *>(d_scratch + kTicketBytes);
+    a.t0 = d_t0;
+    size_t drawing = jobs.size(), updating = 0;  // the first so many jobs have a block b, a block b - 1
+    for (uint32_t b = 0;; ++b) {
+        updating = b ? drawing : 0;
+        while (drawing && jobs[drawing - 1].nblocks <= b) --drawing;
+        if (!drawing && !updating) return cudaSuccess;
+        a.block = b;
+        a.d_jobs = (uint32_t)drawing;
+        a.u_jobs = (uint32_t)updating;
+        a.d_tickets = drawing == jobs.size() ? total_tickets : jobs[drawing].ticket_start;
+        a.u_tiles = updating == 0 ? 0u : updating == jobs.size() ? total_tiles : jobs[updating].tile_start;
+        a.update_ctas = std::min<uint32_t>(a.u_tiles, (uint32_t)sms);
+        a.d_ticket = tickets + b % 4;
+        a.next_ticket = tickets + (b + 2) % 4;
+        const uint32_t warps = kBatchThreads / 32;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(std::max(1u, std::min(2 * (uint32_t)sms, a.update_ctas + (a.d_tickets + warps - 1) / warps)));
+        cfg.blockDim = dim3(kBatchThreads);
+        cfg.dynamicSmemBytes = b ? smem : 0;
+        cfg.stream = s;
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = b ? 1 : 0;
+        if ((e = cudaLaunchKernelEx(&cfg, k_ahead_batch, a)) != cudaSuccess) return e;
+    }
 }
 
 }  // namespace ising

@@ -6,6 +6,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <vector>
 
 namespace ising {
 
@@ -63,6 +64,34 @@ struct AheadArgs {
 
 AheadPlan ahead_plan(uint64_t L, bool field);
 
+// One lattice of a batch run (device table).
+struct AheadJob {
+    RoundKeys key;
+    uint32_t thr[5], c3base;
+    uint32_t plus3, plus4, minus0, minus1, flipped;
+    uint32_t L, wc, nwords;
+    FastDiv by_wc, by_group;
+    uint32_t step_bytes, record_every;
+    uint32_t field, kw, tile_rows, halo;
+    uint32_t sweeps, block_sweeps, nblocks;   // of the run; of a block; blocks of the run
+    uint32_t index;                           // of the lattice in the batch
+    uint32_t tile_start, ticket_start;        // tiles and tickets of the jobs before
+    size_t mask_bytes;                        // one buffer of masks
+    char *masks;
+    uint64_t *even, *odd;                     // the lattice before blocks 0, 2, .. and before blocks 1, 3, ..
+    const uint64_t *copy_from;                // where `even` is not the lattice: copied from here first
+    unsigned long long *acc, *final_acc;
+};
+
+struct AheadBatchArgs {
+    const AheadJob *jobs;
+    const uint32_t *t0;           // first sweep index of each lattice
+    uint32_t block;               // drawn by this launch; the one before is updated
+    uint32_t d_jobs, u_jobs;      // jobs that have them
+    uint32_t d_tickets, u_tiles, update_ctas;
+    unsigned int *d_ticket, *next_ticket;
+};
+
 }  // namespace ising
 
 struct ising_lattice;
@@ -77,4 +106,20 @@ bool ahead_ready(ising_lattice *h, const AheadPlan &pl);
 // max_block sweeps.
 cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, uint64_t t0, uint64_t nsweeps,
                          uint32_t record_every, uint64_t nrec, unsigned int *err, uint32_t hold_step, uint64_t max_block);
+
+// A run of many lattices in the draw-ahead form.
+struct AheadBatch {
+    std::vector<AheadJob> jobs;   // by falling number of blocks
+    uint32_t total_tiles = 0, total_tickets = 0;
+    size_t smem = 0, table_bytes = 0, scratch_bytes = 0;
+    char *d_scratch = nullptr;
+    // Plans runs of sweeps[i] sweeps of hs[i]; false if a lattice has no tiles.
+    bool plan(const std::vector<ising_lattice *> &hs, const std::vector<uint64_t> &sweeps,
+              const std::vector<uint32_t> &record_every);
+    // Places the jobs in scratch (scratch_bytes) and uploads their table.
+    cudaError_t upload(void *scratch, const std::vector<ising_lattice *> &hs, const std::vector<unsigned long long *> &acc,
+                       const std::vector<unsigned long long *> &final_acc, cudaStream_t s);
+    // Queues one run; d_t0: the lattices' first sweep indices on the device.
+    cudaError_t enqueue(const uint32_t *d_t0, cudaStream_t s);
+};
 }  // namespace ising

@@ -552,6 +552,13 @@ BatchKernel batch_kernel(uint32_t insert, bool field)
 // ------------------------------------------------------------------ host ---
 namespace {
 
+// Runs whose longest lattice has fewer sweeps (lattices up to 128^2; larger ones) are
+// as fast in strips: 128 of 64^2, 8 sweeps 108 us against 117, 12 sweeps 119 against
+// 111; the four sizes 256 .. 2048 at 32 temperatures, 4 sweeps 703 against 710 us, 8
+// sweeps 1289 against 1202; six of 4096^2, 4 sweeps 374 against 628, 8 sweeps 713
+// against 652.
+constexpr uint64_t kAheadMinSweepsSmall = 12, kAheadMinSweeps = 8;
+
 // Bytes of the per-strip tables at the start of the kernel's shared memory.
 size_t table_entry_bytes() { return sizeof(BatchStrip) + sizeof(HalfSweepArgs) + 6 * 4 + 2 * 4; }
 size_t table_bytes(size_t max_strips) { return (max_strips * table_entry_bytes() + 15) & ~(size_t)15; }
@@ -574,6 +581,7 @@ void free_batch(ising_batch *b)
     if (b->graph) cudaGraphDestroy(b->graph);
     b->alloc.release(b->d_plan, b->stream);
     b->alloc.release(b->d_work, b->stream);
+    b->alloc.release_scratch(b->d_ahead, b->stream);
     if (b->h_counters) cudaFreeHost(b->h_counters);
     if (b->h_t0) cudaFreeHost(b->h_t0);
     if (b->h_error) cudaFreeHost(b->h_error);
@@ -917,6 +925,37 @@ ising_status alloc_batch(ising_batch *b)
     return ISING_OK;
 }
 
+// The draw-ahead form of the runs (ahead.cu) where no launch option asks for the
+// strips, its scratch is to be had and the runs are long enough for it.
+ising_status plan_ahead(ising_batch *b)
+{
+    b->use_ahead = false;
+    const bool small = std::all_of(b->hs.begin(), b->hs.end(), [](const ising_lattice *h) { return h->L <= 128; });
+    if (!b->ahead_allowed || *std::max_element(b->sweeps.begin(), b->sweeps.end()) < (small ? kAheadMinSweepsSmall : kAheadMinSweeps))
+        return ISING_OK;
+    if (!b->ahead.plan(b->hs, b->sweeps, b->record_every)) return ISING_OK;
+    if (b->ahead.scratch_bytes > b->ahead_cap) {
+        cudaStreamSynchronize(b->stream);
+        b->alloc.release_scratch(b->d_ahead, b->stream);
+        b->ahead_cap = b->ahead.scratch_bytes;
+        b->d_ahead = b->alloc.scratch(b->ahead_cap, b->stream);
+        if (!b->d_ahead) {
+            b->ahead_cap = 0;
+            return ISING_OK;
+        }
+    }
+    std::vector<unsigned long long *> acc, final_acc;
+    unsigned long long *const counters = reinterpret_cast<unsigned long long *>(static_cast<char *>(b->d_work) + b->off_counters);
+    for (size_t i = 0; i < b->hs.size(); ++i) {
+        acc.push_back(counters + 2 * b->sample_base[i]);
+        final_acc.push_back(acc.back() + 2 * b->nrec[i]);
+    }
+    const cudaError_t e = b->ahead.upload(b->d_ahead, b->hs, acc, final_acc, b->stream);
+    if (e != cudaSuccess) return bfail(b, e, "batch table upload");
+    b->use_ahead = true;
+    return ISING_OK;
+}
+
 // Work of one run on the batch stream: clear the counters, progress and error
 // flag, copy the lattices' first sweep indices, launch, copy the counters and
 // the error flag back.
@@ -928,6 +967,13 @@ cudaError_t enqueue_run(ising_batch *b)
         e = cudaMemcpyAsync(static_cast<char *>(b->d_plan) + b->off_t0, b->h_t0, b->hs.size() * 4,
                             cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess) return e;
+    if (b->use_ahead) {
+        e = b->ahead.enqueue(b->args.t0, b->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(b->h_counters, work + b->off_counters, b->slots * 16, cudaMemcpyDeviceToHost, b->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(b->h_error, work + b->off_error, 4, cudaMemcpyDeviceToHost, b->stream);
+        return e;
+    }
     void *params[] = {&b->args};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -966,6 +1012,8 @@ ising_status batch_new(int device, const ising_batch_opts *opts, ising_batch **o
         delete b;
         return fail(ISING_ERR_INVALID, "bad batch options");
     }
+    const ising_batch_opts &o = b->opts;
+    b->ahead_allowed = !o.block && !o.ctas_per_sm && !o.rows_per_item && !o.insert && !o.hold_strip && !(o.wait_ms > 0);
     b->device = device;
     b->alloc = current_allocator();
     // a stream of the batch's own (the legacy default stream cannot be captured)
@@ -1010,6 +1058,7 @@ ising_status batch_replan(ising_batch *b, const std::vector<ising_lattice *> &hs
     b->field = std::any_of(hs.begin(), hs.end(), [](const ising_lattice *h) { return h->H != 0.0; });
     ising_status st = make_plan(b);
     if (st == ISING_OK) st = alloc_batch(b);
+    if (st == ISING_OK) st = plan_ahead(b);
     if (st != ISING_OK) b->hs.clear();
     return st;
 }

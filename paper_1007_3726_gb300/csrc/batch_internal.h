@@ -2,6 +2,7 @@
 // with the request server (server.cu), which re-plans one batch per epoch.
 #pragma once
 
+#include "ahead.h"
 #include "handle.h"
 #include "kernels.h"
 #include "runtime.h"
@@ -59,6 +60,11 @@ struct ising_batch {
     cudaGraphExec_t graph_exec = nullptr;
     ising::BatchLaunchArgs args{};
     bool field = false;                     // a lattice is in a field: the field kernel
+    ising::AheadBatch ahead;                // the draw-ahead form of the runs
+    bool ahead_allowed = false;             // no launch option asks for the strips
+    bool use_ahead = false;                 // planned and placed
+    void *d_ahead = nullptr;
+    size_t ahead_cap = 0;
     bool failed = false;
 };
 

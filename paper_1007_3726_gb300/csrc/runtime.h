@@ -39,7 +39,7 @@ struct Allocator {
     void *scratch(size_t bytes, cudaStream_t s) const;
     void release_scratch(void *p, cudaStream_t s) const;
 };
-constexpr size_t kPoolKeeps = 256ull << 20;
+constexpr size_t kPoolKeeps = 1ull << 30;
 Allocator current_allocator();
 
 // floor(2^32 exp(-dE / T)), clamped to [0, 2^32 - 1].

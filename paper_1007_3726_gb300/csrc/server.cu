@@ -61,6 +61,7 @@ struct ising_server {
     std::unordered_map<uint64_t, Request *> kept;   // polled results whose samples are kept
     ising_server_counters stats{};
     ising_batch *batch = nullptr;
+    bool ahead_allowed = false;
     std::vector<uint64_t> plan_ids;     // request ids of the current plan (handle addresses are reused)
     std::vector<uint64_t> plan_sweeps;
     std::string worker_error;
@@ -235,7 +236,7 @@ void run_epoch(ising_server *s)
         }
         batch_free(s->batch);
         s->batch = nullptr;
-        batch_new(s->device, &s->opts.batch, &s->batch);
+        if (batch_new(s->device, &s->opts.batch, &s->batch) == ISING_OK) s->batch->ahead_allowed = s->ahead_allowed;
         s->plan_ids.clear();
         s->plan_sweeps.clear();
         return;
@@ -325,6 +326,10 @@ ISING_API ising_status ising_server_create(const ising_server_opts *opts, ising_
     if (opts) s->opts = *opts;
     if (s->opts.hbm_budget_bytes == 0) s->opts.hbm_budget_bytes = 64ull << 30;
     if (s->opts.epoch_sweeps == 0) s->opts.epoch_sweeps = 1000;
+    // launch options of its own for the strips; without any the batch may take the
+    // draw-ahead form
+    const ising_batch_opts &bo = s->opts.batch;
+    s->ahead_allowed = !bo.block && !bo.ctas_per_sm && !bo.rows_per_item && !bo.insert && !bo.hold_strip && !(bo.wait_ms > 0);
     if (s->opts.batch.block == 0) {
         s->opts.batch.block = 256;
         s->opts.batch.ctas_per_sm = s->opts.batch.ctas_per_sm ? s->opts.batch.ctas_per_sm : 4;
@@ -342,6 +347,7 @@ ISING_API ising_status ising_server_create(const ising_server_opts *opts, ising_
         delete s;
         return st;
     }
+    s->batch->ahead_allowed = s->ahead_allowed;
     s->worker = std::thread(worker_main, s);
     *out = s;
     return ISING_OK;

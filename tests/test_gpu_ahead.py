@@ -195,3 +195,82 @@ def test_handles_on_streams_and_threads(P, orc):
         Mo, Eo = orc.run(s, 660, L, 0, *orc.thresholds(TC))
         M, E, spins = out[L]
         assert np.array_equal(M, Mo[4::5]) and np.array_equal(E, Eo[4::5]) and np.array_equal(spins, s), L
+
+
+# (L, H, sweeps): tiles of every kind, blocks of 4 .. 64 sweeps with remainders, odd and
+# even numbers of blocks, lattices that end before the others
+BATCHES = [
+    [(64, 0.0, 61), (128, 0.0, 9), (192, 0.0, 40), (256, 0.0, 13), (64, 0.0, 8)],
+    [(320, 0.0, 17), (448, 0.0, 24), (512, 0.0, 9), (704, 0.0, 12), (1088, 0.0, 10)],
+    [(1024, 0.0, 21), (2048, 0.0, 9), (4096, 0.0, 8), (2112, 0.0, 11), (960, 0.0, 1)],
+    [(64, 0.3, 30), (192, -2.0, 19), (256, 0.1, 22), (512, 0.0, 14), (320, 4.0, 9), (1024, -0.2, 8), (2048, 0.5, 9)],
+    [(1024, 0.0, 37)],
+]
+
+
+@pytest.mark.parametrize("record_every", [0, 1, 3])
+@pytest.mark.parametrize("k", range(len(BATCHES)))
+def test_batch_equals_the_strips(P, k, record_every):
+    """Runs of a batch without launch options against the same runs in strips."""
+    make = lambda: [P.Lattice(L, 2.0 + 0.05 * i, seed=7 + i, stream_id=i, init="hot", H=H)  # noqa: E731
+                    for i, (L, H, _) in enumerate(BATCHES[k])]
+    a, b = make(), make()
+    sweeps = [n for _, _, n in BATCHES[k]]
+    with P.Batch(a, sweeps, record_every, use_graph=k == 0) as x, P.Batch(b, sweeps, record_every, block=512) as y:
+        x.run(1)
+        y.run(1)
+        a[0].sweep(3, record_every)  # another form in between
+        b[0].sweep(3, record_every)
+        x.run(2)
+        y.run(2)
+    for l, r in zip(a, b):
+        assert np.array_equal(l.spins(), r.spins()), l.L
+        assert np.array_equal(np.stack(l.samples()), np.stack(r.samples())), l.L
+        dl, dr = l.measure(), r.measure()
+        assert (dl["M"], dl["E"], dl["sweeps_done"]) == (dr["M"], dr["E"], dr["sweeps_done"])
+
+
+def test_batch_against_the_oracle(P, orc):
+    specs = [(256, 0.0), (512, 0.2), (1024, 0.0)]
+    lats = [P.Lattice(L, TC, seed=L, stream_id=2, init="hot", H=H) for L, H in specs]
+    with P.Batch(lats, [14, 9, 12], 2) as b:
+        b.run(1)
+    for (L, H), n, lat in zip(specs, (14, 9, 12), lats):
+        s = orc.init_hot(L, L, 2)
+        Mo, Eo = orc.run_field(s, n, L, 2, TC, H) if H else orc.run(s, n, L, 2, *orc.thresholds(TC))
+        M, E = lat.samples()
+        assert np.array_equal(M, Mo[1::2]) and np.array_equal(E, Eo[1::2]) and np.array_equal(lat.spins(), s), L
+
+
+def test_batch_without_scratch_memory_runs_in_strips(P):
+    import torch
+
+    taken, refused = {}, []
+
+    def alloc(n, s):
+        if n > 8 << 20:  # the masks of a block
+            refused.append(n)
+            return None
+        p = torch.cuda.caching_allocator_alloc(n)
+        taken[p] = n
+        return p
+
+    def release(p, s):
+        taken.pop(p)
+        torch.cuda.caching_allocator_delete(p)
+
+    P.ising_set_allocator(alloc, release)
+    try:
+        a = [P.Lattice(512, TC, seed=1, stream_id=i, init="hot") for i in range(4)]
+        with P.Batch(a, [20] * 4, 2) as x:
+            x.run(1)
+        got = [(l.spins(), l.samples()) for l in a]
+        for l in a:
+            l.close()
+        assert refused and not taken
+    finally:
+        P.ising_set_allocator(None)
+    for i, (spins, samples) in enumerate(got):
+        l = P.Lattice(512, TC, seed=1, stream_id=i, init="hot")
+        M, E = l.sweep(20, 2, collect=True)
+        assert np.array_equal(l.spins(), spins) and np.array_equal(samples[0], M) and np.array_equal(samples[1], E)
