@@ -320,6 +320,18 @@ __device__ __forceinline__ void word_draw_masks(const K &a, const S &s, uint64_t
     }
 }
 
+// The accepted flips of sites with spin x, neighbours n1 .. n4 and draws p4 = [u <
+// thr4], p8 = [u < thr8], bit by bit.  With s3 = n1 ^ n2 ^ n3 and m3 = maj(n1, n2, n3),
+// two or more neighbours are anti-aligned where (x ^ m3) | ((x ^ s3) & (x ^ n4)) and one
+// or three where s3 ^ n4; a draw below thr8 is below thr4 too, so Eq. 5 of Sec. 4 needs
+// no "exactly one" and "none": 7 three-input operations per 32 bits.
+template <typename Word>
+__device__ __forceinline__ Word flips(Word x, Word n1, Word n2, Word n3, Word n4, Word p4, Word p8)
+{
+    const Word s3 = n1 ^ n2 ^ n3, m3 = (n1 & n2) | (n3 & (n1 | n2));
+    return (x ^ m3) | ((x ^ s3) & (x ^ n4)) | ((s3 ^ n4) & p4) | p8;
+}
+
 // Update of one word of target sites (Sec. 4): cur is the word, up / dn the
 // words above / below, lw / rw the words left / right of it in its row, mask
 // the target bit positions, off their parity (0 or 1), g the Philox group of
@@ -342,15 +354,6 @@ __device__ __forceinline__ Word update_word(const K &a, const S &s, Word cur, Wo
     const Word right = (cur >> 1) | (rw << (B - 1));  // bit b holds s(x + 1)
     const Word mask = off ? (Word)(Tr::even << 1) : Tr::even;
 
-    // energy variables and their bit-sliced sum c = i1 + i2 + i3 + i4
-    const Word i1 = cur ^ up, i2 = cur ^ dn, i3 = cur ^ left, i4 = cur ^ right;
-    const Word s12 = i1 ^ i2, c12 = i1 & i2;
-    const Word s34 = i3 ^ i4, c34 = i3 & i4;
-    const Word odd = s12 ^ s34;                  // c odd
-    const Word ge2 = c12 | c34 | (s12 & s34);    // c >= 2: dE <= 0, always accepted
-    const Word eq1 = odd & ~ge2;                 // c == 1: dE = 4
-    const Word eq0 = ~(odd | ge2);               // c == 0: dE = 8
-
     // the sites' draws: byte q of the word holds four target sites
     uint32_t h4[(NB + 3) / 4], h8[(NB + 3) / 4];
     word_draw_masks<NB, INS, NQ>(a, s, g, h4, h8, q0);
@@ -358,8 +361,7 @@ __device__ __forceinline__ Word update_word(const K &a, const S &s, Word cur, Wo
     const Word p8 = Tr::from_halves(h8) << off;
     Word sel = mask;
     if constexpr (NQ < NB) sel &= (((Word)1 << (8 * NQ)) - 1) << (8 * q0);  // this thread's bytes
-    const Word flip = sel & (ge2 | (eq1 & p4) | (eq0 & p8));
-    const Word nw = cur ^ flip;
+    const Word nw = cur ^ (sel & flips(cur, up, dn, left, right, p4, p8));
     if (count) {
         // after the step: +1 spins of the word, and the anti-aligned bonds of
         // its target sites (their neighbours are final)
@@ -388,13 +390,6 @@ __device__ __forceinline__ uint32_t update_word32_drawn(uint32_t cur, uint32_t u
     const uint32_t left = (cur << 1) | (lw >> 31);
     const uint32_t right = (cur >> 1) | (rw << 31);
     const uint32_t mask = off ? (even << 1) : even;
-    const uint32_t i1 = cur ^ up, i2 = cur ^ dn, i3 = cur ^ left, i4 = cur ^ right;
-    const uint32_t s12 = i1 ^ i2, c12 = i1 & i2;
-    const uint32_t s34 = i3 ^ i4, c34 = i3 & i4;
-    const uint32_t odd = s12 ^ s34;
-    const uint32_t ge2 = c12 | c34 | (s12 & s34);
-    const uint32_t eq1 = odd & ~ge2;
-    const uint32_t eq0 = ~(odd | ge2);
     const uint32_t p4 = (pk & even) << off;
     const uint32_t p8 = ((pk >> 1) & even) << off;
     uint32_t sel = mask;
@@ -403,7 +398,7 @@ __device__ __forceinline__ uint32_t update_word32_drawn(uint32_t cur, uint32_t u
         own = ((1u << (8 * NQ)) - 1u) << (8 * q0);
         sel &= own;
     }
-    const uint32_t nw = cur ^ (sel & (ge2 | (eq1 & p4) | (eq0 & p8)));
+    const uint32_t nw = cur ^ (sel & flips(cur, up, dn, left, right, p4, p8));
     if (count) {
         cnt_up += __popc(nw & own);
         cnt_anti += __popc(sel & (nw ^ up)) + __popc(sel & (nw ^ dn)) + __popc(sel & (nw ^ left)) +
