@@ -262,8 +262,8 @@ ISING_API const char *ising_last_error(void);
  * persistent = 0 otherwise.
  *
  * The draw-ahead form.  A handle whose configuration was not set runs calls of
- * enough sweeps (200 at L = 64, 100 at 128, 10 at 256, 3 below 2048, 5 up to 8192;
- * in a field 1 to 5) on a lattice of L <= 8192 (in a field 4096) in another form: the acceptance masks of
+ * enough sweeps (200 at L = 64, 100 at 128, 10 at 256, 3 below 1024, 5 below
+ * 2048, 10 up to 8192; in a field 1 to 5) on a lattice of L <= 8192 (in a field 4096) in another form: the acceptance masks of
  * a block of sweeps are drawn by the whole GPU one launch before the tiles of the
  * lattice are updated with them.  It needs scratch memory (three blocks of masks,
  * a second lattice: 3 MB at L = 512, 103 MB at 4096, 210 MB at 8192), which the handle

@@ -48,7 +48,7 @@ namespace {
 
 // Steps whose masks an update thread holds or has on the way: their latency (about
 // a microsecond with the L2 busy) against the time of a step, within 160 KiB.
-__host__ __device__ constexpr uint32_t stages_of(uint32_t kw, bool field) { return kw == 8 || (field && kw == 4) ? 4 : 8; }
+__host__ __device__ constexpr uint32_t stages_of(uint32_t kw, bool field) { return kw == 8 ? 2 : (field && kw == 4) ? 4 : 8; }
 
 // Threads per CTA.  One lattice: one CTA per SM, so that an update, which the next
 // launch waits for, has an SM to itself.  Several lattices: two CTAs per SM, so that
@@ -329,18 +329,22 @@ struct Counting {
     }
 };
 
-// The state of a run after a counted sweep, for the counting CTAs of the next
-// launch: row k of colour q of run c at [(q KW + k) runs + c].
+// The state of a run after a counted sweep, for the counting CTAs of the next launch:
+// row k of colour q of the lattice's run c (row group times wc plus word) at
+// [(q KW + k) runs + c].
 template <int KW>
-__device__ __forceinline__ void store_snapshot(const AheadArgs &a, uint32_t slot, uint32_t c, uint32_t nthr, const uint32_t (&v)[2][KW])
+__device__ __forceinline__ void store_snapshot(const AheadArgs &a, uint32_t slot, uint32_t c, const uint32_t (&v)[2][KW])
 {
+    const uint32_t runs = a.nwords / KW;
     uint32_t *const p = a.u_snaps + (size_t)slot * (2u * a.nwords) + c;
 #pragma unroll
-    for (int k = 0; k < 2 * KW; ++k) p[k * nthr] = v[k / KW][k % KW];
+    for (int k = 0; k < 2 * KW; ++k) p[k * runs] = v[k / KW][k % KW];
 }
 
 // One tile through the block: threads hold KW rows of one column each (a run).
-template <uint32_t THREADS, int KW, bool FIELD>
+// SNAPS: counted sweeps may go out as snapshots (where there is a buffer for them), else
+// the tile counts its own rows.
+template <uint32_t THREADS, int KW, bool FIELD, bool SNAPS>
 __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, unsigned char *smem)
 {
     constexpr uint32_t ST = stages_of(KW, FIELD);
@@ -356,7 +360,7 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
     uint32_t *const X = reinterpret_cast<uint32_t *>(ring4 + (FIELD ? ST * (KW / 2) * THREADS : 0u));
     uint32_t *const cnt = X + 2 * KW * THREADS;                   // [samples of the block, last state][2]
     const bool whole = a.halo == 0u;                              // the tile is the lattice
-    const bool snaps = a.u_snaps != nullptr;                      // counted sweeps go out as snapshots
+    const bool snaps = SNAPS && a.u_snaps != nullptr;
     if (!snaps) {
         for (uint32_t k = tid; k < 2 * a.u_slots; k += THREADS) cnt[k] = 0u;
         __syncthreads();
@@ -445,7 +449,7 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
                 masks_of(s + 1u);
                 if (P == 1 && count) {
                     if (snaps) {
-                        if (tid < nthr) store_snapshot<KW>(a, cn.slot, c, nthr, v);
+                        if (mine) store_snapshot<KW>(a, cn.slot, group * wc + w, v);
                     } else {
                         uint32_t cu, ca;
                         count_run<KW>(v, hz, up, dn, cu, ca);
@@ -539,7 +543,7 @@ __device__ __forceinline__ void update_warp(const AheadArgs &a, unsigned char *s
             for (uint32_t s = 0; s < n; s += 2) {
                 step(Parity<0>{}, true);
                 step(Parity<1>{}, s + 2 < n);
-                if (cn.next(a, a.u_last != 0u && s0 + s + 2 == a.u_steps)) store_snapshot<2>(a, cn.slot++, lane, 32u, v);
+                if (cn.next(a, a.u_last != 0u && s0 + s + 2 == a.u_steps)) store_snapshot<2>(a, cn.slot++, lane, v);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[st]);
@@ -554,22 +558,23 @@ __device__ __forceinline__ void update_warp(const AheadArgs &a, unsigned char *s
 template <int KW>
 __device__ __forceinline__ void count_role(const AheadArgs &a, uint32_t cta)
 {
-    const uint32_t wc = a.wc, nthr = a.nwords / KW, per = (nthr + 31u) & ~31u;  // threads a snapshot: whole warps
+    const uint32_t wc = a.wc, runs = a.nwords / KW, per = (runs + 31u) & ~31u;  // threads a snapshot: whole warps
     for (uint32_t i = cta * kThreads + threadIdx.x; i < a.c_slots * per; i += a.count_ctas * kThreads) {
-        const uint32_t slot = i / per, t = i - slot * per;
-        const uint32_t c = min(t, nthr - 1u), run = a.by_wc.quotient(c), w = c - run * wc;
+        const uint32_t slot = i / per, c = min(i - slot * per, runs - 1u), w = c - a.by_wc.quotient(c) * wc;
+        const bool real = i - slot * per < runs;
         const uint32_t *const B = a.c_snaps + (size_t)slot * (2u * a.nwords);
+        const uint32_t left = c - w + (w == 0 ? wc - 1u : w - 1u), right = c - w + (w + 1u == wc ? 0u : w + 1u);
         uint32_t v[2][KW], hz[KW], cu, ca;
 #pragma unroll
         for (int k = 0; k < KW; ++k) {
-            v[0][k] = B[k * nthr + c];
-            v[1][k] = B[(KW + k) * nthr + c];
-            hz[k] = B[k * nthr + c - w + (((k + 1) & 1) ? (w + 1u == wc ? 0u : w + 1u) : (w == 0 ? wc - 1u : w - 1u))];
+            v[0][k] = B[k * runs + c];
+            v[1][k] = B[(KW + k) * runs + c];
+            hz[k] = B[k * runs + (((k + 1) & 1) ? right : left)];
         }
-        const uint32_t up = B[(KW - 1) * nthr + (run == 0 ? nthr - wc + w : c - wc)], dn = B[c + wc >= nthr ? w : c + wc];
+        const uint32_t up = B[(KW - 1) * runs + (c < wc ? runs - wc + c : c - wc)], dn = B[c + wc >= runs ? c + wc - runs : c + wc];
         count_run<KW>(v, hz, up, dn, cu, ca);
-        cu = __reduce_add_sync(0xFFFFFFFFu, t < nthr ? cu : 0u);
-        ca = __reduce_add_sync(0xFFFFFFFFu, t < nthr ? ca : 0u);
+        cu = __reduce_add_sync(0xFFFFFFFFu, real ? cu : 0u);
+        ca = __reduce_add_sync(0xFFFFFFFFu, real ? ca : 0u);
         if ((threadIdx.x & 31u) == 0u) {
             if (slot < a.c_recs) {
                 atomicAdd(a.acc + 2 * (size_t)(a.c_slot0 + slot), (unsigned long long)cu);
@@ -584,7 +589,7 @@ __device__ __forceinline__ void count_role(const AheadArgs &a, uint32_t cta)
 }
 
 template <int KW, bool WARP, bool FIELD>
-__global__ void __launch_bounds__(kThreads, 1) k_ahead(const __grid_constant__ AheadArgs a)
+__global__ void __launch_bounds__(kThreads, KW == 8 ? 2 : 1) k_ahead(const __grid_constant__ AheadArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     // The first launch of a call (it only draws) starts after all work before it.
@@ -599,7 +604,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ahead(const __grid_constant__ A
         if constexpr (WARP)
             update_warp(a, smem);
         else
-            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, KW, FIELD>(a, t, smem);
+            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, KW, FIELD, true>(a, t, smem);
     } else if (blockIdx.x < early) {
         count_role<KW>(a, blockIdx.x - a.update_ctas);
     }
@@ -679,7 +684,6 @@ __device__ __forceinline__ void batch_tile_args(const AheadBatchArgs &a, const A
     t.src = (ub & 1u) ? j.odd : j.even;
     t.dst = (ub & 1u) ? j.even : j.odd;
     t.u_masks = j.masks + (size_t)(ub % kBuffers) * j.mask_bytes;
-    t.u_snaps = nullptr;
     t.u_phase = re ? (t0 + done) % re : 0u;
     t.u_recs = re ? (t.u_phase + n) / re : 0u;
     t.u_slot0 = re ? (t0 % re + done) / re : 0u;
@@ -711,15 +715,15 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_ahead_batch(const __grid_c
             const uint32_t tile = g - j.tile_start;
             if (!j.field) {
                 if (j.kw == 2)
-                    update_tile<kBatchThreads, 2, false>(t, tile, smem);
+                    update_tile<kBatchThreads, 2, false, false>(t, tile, smem);
                 else if (j.kw == 4)
-                    update_tile<kBatchThreads, 4, false>(t, tile, smem);
+                    update_tile<kBatchThreads, 4, false, false>(t, tile, smem);
                 else
-                    update_tile<kBatchThreads, 8, false>(t, tile, smem);
+                    update_tile<kBatchThreads, 8, false, false>(t, tile, smem);
             } else if (j.kw == 2) {
-                update_tile<kBatchThreads, 2, true>(t, tile, smem);
+                update_tile<kBatchThreads, 2, true, false>(t, tile, smem);
             } else {
-                update_tile<kBatchThreads, 4, true>(t, tile, smem);
+                update_tile<kBatchThreads, 4, true, false>(t, tile, smem);
             }
         }
     }
@@ -784,7 +788,9 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 //   L = 2048,  200 sweeps: 64 + 32: 606, 64 + 16: 630, 32 + 16: 659
 //   L = 4096,  200 sweeps: 32 + 16: 2225, 16 + 8: 2399
 // Above 8192 a block would hold fewer than 4 sweeps and its masks 25 times the
-// lattice: the step kernels run there.  In a field (20 bytes of masks a word and step
+// lattice: the step kernels run there.  Two CTAs of the largest tiles share a SM, and
+// with draws (L = 2048, 200 sweeps: 606 us with one, 585 with two; 4096 2225 and 2137;
+// 8192, 40 sweeps 1848 and 1748).  In a field (20 bytes of masks a word and step
 // instead of 8, five compares a draw instead of two) L <= 4096.  Measured, 200 sweeps
 // with M/E every sweep, the field step kernel (L = 64 .. 512: the one-launch field
 // kernels) against this form: L = 64 547 -> 102 us, 512 1384 -> 251, 704 5568 -> 357,
@@ -808,16 +814,23 @@ AheadPlan ahead_plan(uint64_t L, bool field)
         }
     }
     p.block_sweeps = p.halo ? p.halo / 2 : 256;
-    p.min_sweeps = field ? (L <= 512 && (L & (L - 1)) == 0 ? 5 : L > 2048 ? 3 : 1) : L == 64 ? 200 : L == 128 ? 100 : L == 256 ? 10 : L < 2048 ? 3 : 5;
+    p.min_sweeps = field ? (L <= 512 && (L & (L - 1)) == 0 ? 5 : L > 2048 ? 4 : 1)
+                         : L == 64 ? 200 : L == 128 ? 100 : L == 256 ? 10 : L < 1024 ? 3 : L < 2048 ? 5 : 10;
     const uint32_t rows = p.tile_rows + 2 * p.halo, most = p.halo ? kThreads : kThreads / 2;
     for (p.kw = 2; rows / p.kw * wc > most;) p.kw *= 2;
     p.warp = L == 64 && !field;
     p.tiles = (uint32_t)(L / p.tile_rows);
-    p.update_ctas = std::min(p.tiles, 64u);
+    // one tile a CTA, or several the same number each: of 66 tiles 2 on two CTAs take
+    // twice as long as the others; 128 tiles (L = 4096) on 64 CTAs 2137 us, on 128 2228
+    // (a CTA that updates draws nothing before the launch before has ended: fewer of
+    // them where a CTA has an SM to itself)
+    const uint32_t most_ctas = p.kw == 8 ? 128 : 64;
+    const uint32_t each = p.tiles <= 96 ? 1 : std::max(2u, (p.tiles + most_ctas - 1) / most_ctas);
+    p.update_ctas = (p.tiles + each - 1) / each;
     p.field = field;
     p.step_bytes = (uint32_t)(L * wc * (field ? 20 : 8));
     p.mask_bytes = (size_t)2 * p.block_sweeps * p.step_bytes;
-    p.snap_bytes = p.halo ? 0 : (size_t)(p.block_sweeps + 1) * L * wc * 8;
+    p.snap_bytes = L <= 2048 ? (size_t)p.block_sweeps * L * wc * 8 : 0;
     return p;
 }
 
@@ -857,14 +870,14 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
     if (e != cudaSuccess) return e;
     a.update_ctas = a.u_steps ? pl.update_ctas : 0u;
     const uint32_t per = (a.nwords / pl.kw + 31u) & ~31u;
-    a.count_ctas = a.c_slots ? std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, 32u) : 0u;
+    a.count_ctas = a.c_slots ? std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, pl.kw == 8 ? 64u : 16u) : 0u;
     a.d_four = a.d_sweeps % 4 == 0;
     a.d_tickets = (a.d_four ? a.d_sweeps / 4 : a.d_sweeps) * 2u * (a.nwords / 32u);
     const uint32_t early = a.update_ctas + a.count_ctas, warps = kThreads / 32u;
-    const uint32_t grid = std::max(early, std::min<uint32_t>((uint32_t)sms, early + (a.d_tickets + warps - 1) / warps));
+    const uint32_t grid = std::max(early, std::min<uint32_t>((uint32_t)sms * (pl.kw == 8 ? 2u : 1u), early + (a.d_tickets + warps - 1) / warps));
     const size_t smem = !a.u_steps ? 0
                         : pl.warp  ? kWarpStages * kChunk * 512
-                                   : (stages_of(pl.kw, pl.field) * (pl.field ? 20 : 8) + 8) * pl.kw * kThreads + (pl.halo ? (size_t)a.u_slots * 8 : 0);
+                                   : (stages_of(pl.kw, pl.field) * (pl.field ? 20 : 8) + 8) * pl.kw * kThreads + (a.u_snaps ? 0 : (size_t)a.u_slots * 8);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kThreads);
@@ -927,6 +940,12 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     a.final_acc = h->d_acc + 2 * nrec;
     a.err = err;
     a.hold_step = hold_step;
+    // Counting in the launch after the update takes work off its chain of steps, but
+    // costs a launch at the end and the snapshots' traffic: M/E every sweep, counted by
+    // the tiles and from snapshots, 1000 sweeps of 256 490 and 365 us, 1000 of 512 625 and
+    // 496, 200 of 2048 667 and 618, 200 of 4096 2183 and 2246; 10 sweeps of 4096 165 and
+    // 203.
+    const bool snapshots = pl.warp || (nsweeps >= 32 && h->L <= 2048);
     // Blocks.  Items of 4 sweeps are the cheapest to draw, so a call that is long
     // enough starts with the rest of a division by 4.  Where an update takes long
     // (one CTA holds the lattice), blocks start short: nothing overlaps the first
@@ -954,9 +973,9 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
         src = other;
     }
     // launch b draws block b, updates block b - 1 and counts the snapshots of block b - 2
-    for (uint64_t b = 0; b < nblocks + (pl.halo ? 1 : 2); ++b) {
+    for (uint64_t b = 0; b < nblocks + (snapshots ? 2 : 1); ++b) {
         const uint64_t n = drawn < nsweeps ? next_block() : 0;
-        a.c_slots = pl.halo ? 0u : a.u_slots;
+        a.c_slots = snapshots ? a.u_slots : 0u;
         a.c_recs = a.u_recs;
         a.c_slot0 = a.u_slot0;
         a.c_last = a.u_last;
@@ -969,7 +988,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
             a.src = src;
             a.dst = src == spins ? other : spins;
             a.u_masks = masks + ((b - 1) % kBuffers) * pl.mask_bytes;
-            a.u_snaps = pl.halo ? nullptr : reinterpret_cast<uint32_t *>(snaps + (b % 2) * pl.snap_bytes);
+            a.u_snaps = snapshots ? reinterpret_cast<uint32_t *>(snaps + (b % 2) * pl.snap_bytes) : nullptr;
             a.u_phase = record_every ? (uint32_t)(t % record_every) : 0u;
             a.u_recs = record_every ? (uint32_t)((t + prev) / record_every - t / record_every) : 0u;
             a.u_slot0 = (uint32_t)rec_done;

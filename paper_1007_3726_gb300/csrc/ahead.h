@@ -49,7 +49,7 @@ struct AheadArgs {
     const uint64_t *src;
     uint64_t *dst;
     const char *u_masks;
-    uint32_t *u_snaps;            // states after the counted sweeps (where the tile is the lattice)
+    uint32_t *u_snaps;            // states after the counted sweeps
     uint32_t u_phase;             // sweep index % record_every at the block's start
     uint32_t u_recs, u_slot0;     // samples of the block, slot of the first
     uint32_t u_slots, u_last;     // counted sweeps: u_recs, or one more; the call's last block
