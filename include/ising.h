@@ -262,13 +262,15 @@ ISING_API const char *ising_last_error(void);
  * persistent = 0 otherwise.
  *
  * The draw-ahead form.  A handle whose configuration was not set runs calls of
- * enough sweeps (200 at L = 64, 100 at 128, 10 at 256, 3 below 1024, 5 below
- * 2048, 10 up to 8192; in a field 1 to 5) on a lattice of L <= 8192 (in a field 4096) in another form: the acceptance masks of
- * a block of sweeps are drawn by the whole GPU one launch before the tiles of the
- * lattice are updated with them.  It needs scratch memory (three blocks of masks,
- * a second lattice: 3 MB at L = 512, 103 MB at 4096, 210 MB at 8192), which the handle
- * allocates on its first such call and keeps; where the allocator refuses, or while
- * the stream is captured, the configuration's form runs.  Results are the same.
+ * enough sweeps (200 at L = 64, 100 at 128, 10 at 256, 3 below 1024, 5 below 2048, 10
+ * up to 8192, 4 above; in a field, up to L = 4096, 1 to 5) in another form: the
+ * acceptance masks of a block of sweeps are drawn by the whole GPU one launch before
+ * the tiles of the lattice are updated with them.  It needs scratch memory (three
+ * buffers of masks, a second lattice: 4 MB at L = 512, 103 MB at 4096, 210 MB at 8192,
+ * above 210 to 810 MB and the size of the lattice), which the handle allocates on its
+ * first such call and keeps.  Where the allocator refuses, or more than 1 GiB and half
+ * of the free memory were needed, or while the stream is captured, the configuration's
+ * form runs.  Results are the same.
  * ising_set_launch switches it off for the handle.  (ISING_TINY_HOLD_STEP and
  * ISING_TINY_MAX_SWEEPS, for tests only, also act here: the former at L = 64, where
  * one warp waits for masks on their way, the latter as the longest block.)

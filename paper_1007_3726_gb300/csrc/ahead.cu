@@ -105,15 +105,27 @@ __device__ __forceinline__ uint64_t spread_bits(uint32_t v)
 template <bool FIELD>
 constexpr int kPlanes = FIELD ? 5 : 2;
 
-// a: the lattice (AheadArgs or AheadJob); masks, t0: the block's buffer and first sweep index.
-template <bool FIELD, int K, typename A>
-__device__ __forceinline__ void draw_item(const A &a, char *masks, uint32_t t0, uint32_t p, uint32_t sw, uint32_t idx)
+// a: the lattice (AheadArgs or AheadJob); masks, step_bytes, t0: the block's buffer,
+// its stride and first sweep index.  BAND: the masks are those of the rows from
+// a.d_row0 on, of a lattice whose Philox groups may need the second counter word.
+template <bool FIELD, int K, bool BAND, typename A>
+__device__ __forceinline__ void draw_item(const A &a, char *masks, size_t step_bytes, uint32_t t0, uint32_t p, uint32_t sw,
+                                          uint32_t idx)
 {
     constexpr int NP = kPlanes<FIELD>;
     const uint32_t t = t0 + sw;
     // mask order: pair of rows, word, row of the pair
     const uint32_t pair = a.by_wc.quotient(idx >> 1), w = (idx >> 1) - pair * a.wc;
-    const uint32_t g0 = (2u * pair + (idx & 1u)) * (a.L >> 3) + w * 8u;
+    uint32_t g0, g_hi = 0u;
+    if constexpr (BAND) {
+        uint32_t y = a.d_row0 + 2u * pair + (idx & 1u);
+        if (y >= a.L) y -= a.L;
+        const uint64_t g = (uint64_t)y * (a.L >> 3) + w * 8u;
+        g0 = (uint32_t)g;
+        g_hi = (uint32_t)(g >> 32);
+    } else {
+        g0 = (2u * pair + (idx & 1u)) * (a.L >> 3) + w * 8u;
+    }
     const uint32_t x2k = (a.c3base | p) ^ a.key.k1[0];
     uint32_t c0[K], c2[K], c3[K], m[K][NP];
     {
@@ -129,6 +141,16 @@ __device__ __forceinline__ void draw_item(const A &a, char *masks, uint32_t t0, 
 #pragma unroll
             for (int j = 0; j < NP; ++j) m[k][j] = 0u;
         }
+        if constexpr (BAND)
+            if (a.L > 131072u) {  // the second counter word is not 0 everywhere
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const uint64_t qb = (uint64_t)(t + k) * kPhiloxMulB;
+                    const uint64_t qa = (uint64_t)((uint32_t)(qb >> 32) ^ g_hi ^ a.key.k0[0]) * kPhiloxMulA;
+                    c2[k] = (uint32_t)(qa >> 32) ^ a.key.k1[1];
+                    c3[k] = (uint32_t)qa;
+                }
+            }
     }
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -149,7 +171,7 @@ __device__ __forceinline__ void draw_item(const A &a, char *masks, uint32_t t0, 
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        char *const step = masks + (size_t)(2u * (sw + k) + p) * a.step_bytes;
+        char *const step = masks + (size_t)(2u * (sw + k) + p) * step_bytes;
         if constexpr (FIELD) {
             reinterpret_cast<uint4 *>(step)[idx] = make_uint4(m[k][0], m[k][1], m[k][2], m[k][3]);
             reinterpret_cast<uint32_t *>(step + (size_t)a.nwords * 16u)[idx] = m[k][4];
@@ -161,20 +183,23 @@ __device__ __forceinline__ void draw_item(const A &a, char *masks, uint32_t t0, 
 
 // The warps of the launch take tickets for 32 items each (consecutive words of
 // one colour and group of sweeps: nwords is a multiple of 64).
-template <bool FIELD>
+template <bool FIELD, bool BAND>
 __device__ __forceinline__ void draw_role(const AheadArgs &a)
 {
-    const uint32_t lane = threadIdx.x & 31u, per_group = a.nwords / 32u;
+    const uint32_t lane = threadIdx.x & 31u, per_group = BAND ? (a.d_words + 31u) / 32u : a.nwords / 32u;
+    const size_t step_bytes = BAND ? (size_t)a.d_words * 8u : a.step_bytes;
     uint32_t next = lane == 0 ? atomicAdd(a.d_ticket, 1u) : 0u;
     for (;;) {
         const uint32_t it = __shfl_sync(0xFFFFFFFFu, next, 0);
         if (it >= a.d_tickets) return;
         if (lane == 0) next = atomicAdd(a.d_ticket, 1u);  // back before this item is done
-        const uint32_t gp = a.by_group.quotient(it), idx = (it - gp * per_group) * 32u + lane;
+        const uint32_t gp = a.by_group.quotient(it);
+        uint32_t idx = (it - gp * per_group) * 32u + lane;
+        if constexpr (BAND) idx = min(idx, a.d_words - 1u);  // (the last ticket of a group repeats its last word)
         if (a.d_four)
-            draw_item<FIELD, 4>(a, a.d_masks, a.d_t0, gp & 1u, (gp >> 1) * 4u, idx);
+            draw_item<FIELD, 4, BAND>(a, a.d_masks, step_bytes, a.d_t0, gp & 1u, (gp >> 1) * 4u, idx);
         else
-            draw_item<FIELD, 1>(a, a.d_masks, a.d_t0, gp & 1u, gp >> 1, idx);
+            draw_item<FIELD, 1, BAND>(a, a.d_masks, step_bytes, a.d_t0, gp & 1u, gp >> 1, idx);
     }
 }
 
@@ -344,13 +369,16 @@ __device__ __forceinline__ void store_snapshot(const AheadArgs &a, uint32_t slot
 // One tile through the block: threads hold KW rows of one column each (a run).
 // SNAPS: counted sweeps may go out as snapshots (where there is a buffer for them), else
 // the tile counts its own rows.
-template <uint32_t THREADS, int KW, bool FIELD, bool SNAPS>
+// BAND: the tile is one of a band of rows and holds tile_words words of a row, and one
+// on either side, whose sites of the colour spoil from the far end, one a step.
+template <uint32_t THREADS, int KW, bool FIELD, bool SNAPS, bool BAND>
 __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, unsigned char *smem)
 {
     constexpr uint32_t ST = stages_of(KW, FIELD);
     constexpr uint32_t NQ = FIELD ? KW : KW / 2;                  // 16-byte mask units of a run and step
     const uint32_t tid = threadIdx.x, wc = a.wc, L = a.L;
-    const uint32_t nruns = (a.tile_rows + 2 * a.halo) / KW, nthr = nruns * wc;  // threads with a run
+    const uint32_t tw = BAND ? a.tile_words + 2u : wc;            // words of a row of the tile
+    const uint32_t nruns = (a.tile_rows + 2 * a.halo) / KW, nthr = nruns * tw;  // threads with a run
     const uint32_t nbar = (nthr + 31u) & ~31u;
     // [ST][NQ][THREADS]: (P4, P8) of two rows, or the first four planes of a row
     uint4 *const ring = reinterpret_cast<uint4 *>(smem);
@@ -367,21 +395,36 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
     }
     if (tid < nbar) {
         // (a thread past the last run repeats the last one's work)
-        const uint32_t c = min(tid, nthr - 1u), run = a.by_wc.quotient(c), w = c - run * wc;
+        const uint32_t c = min(tid, nthr - 1u), run = (BAND ? a.by_tw : a.by_wc).quotient(c), w = c - run * tw;
         const uint32_t groups = L / KW;                           // row groups of the lattice
-        uint32_t group = (tile * a.tile_rows + L - a.halo) / KW + run;  // the run's row group
+        uint32_t r0 = tile * a.tile_rows, gw = w;                 // the tile's first own row; the word in the lattice's row
+        bool mine = tid < nthr && run >= a.halo / KW && run < (a.halo + a.tile_rows) / KW;
+        if constexpr (BAND) {
+            const uint32_t ty = tile / a.tiles_x, tx = tile - ty * a.tiles_x, w0 = tx * a.tile_words;
+            r0 = a.u_row0 + ty * a.tile_rows;
+            gw = w0 + w + wc - 1u;
+            while (gw >= wc) gw -= wc;
+            mine = mine && w >= 1u && w <= a.tile_words && w0 + w - 1u < wc;
+        }
+        uint32_t group = (r0 + L - a.halo) / KW + run;            // the run's row group
         while (group >= groups) group -= groups;
-        const bool mine = tid < nthr && run >= a.halo / KW && run < (a.halo + a.tile_rows) / KW;
-        const uint32_t xl = c - w + (w == 0 ? wc - 1u : w - 1u), xr = c - w + (w + 1u == wc ? 0u : w + 1u);
-        const uint32_t xu = (KW - 1) * THREADS + (run == 0 ? nthr - wc + w : c - wc);
-        const uint32_t xd = c + wc >= nthr ? w : c + wc;
+        const uint32_t xl = c - w + (w == 0 ? tw - 1u : w - 1u), xr = c - w + (w + 1u == tw ? 0u : w + 1u);
+        const uint32_t xu = (KW - 1) * THREADS + (run == 0 ? nthr - tw + w : c - tw);
+        const uint32_t xd = c + tw >= nthr ? w : c + tw;
         // the steps after which this warp's rows are of no more use: a step spoils a
         // row at either end of the tile
         uint32_t useful = a.u_steps;
         if (!whole) useful = min(useful, __reduce_max_sync(0xFFFFFFFFu, (min(run, nruns - 1u - run) + 1u) * KW - 1u));
 
         // the masks of the next step not yet asked for, into its stage
-        const size_t first = (size_t)(group * (KW / 2)) * wc + w;   // the run's first pair of rows
+        size_t first = (size_t)(group * (KW / 2)) * wc + gw;      // the run's first pair of rows
+        size_t step_bytes = a.step_bytes;
+        if constexpr (BAND) {
+            uint32_t y = group * KW + L - a.u_mask_row0;          // in the rows that have masks
+            if (y >= L) y -= L;
+            first = (size_t)(y / 2u) * wc + gw;
+            step_bytes = (size_t)a.u_words * 8u;
+        }
         const char *msrc = a.u_masks + first * (FIELD ? 32u : 16u), *msrc4 = a.u_masks + (size_t)a.nwords * 16u + first * 8u;
         const uint32_t mdst = shared_addr(ring + c), mdst4 = shared_addr(ring4 + c);
         uint32_t fetched = 0;
@@ -400,15 +443,15 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
                 }
             }
             copy_commit();
-            msrc += a.step_bytes;
-            msrc4 += a.step_bytes;
+            msrc += step_bytes;
+            msrc4 += step_bytes;
             ++fetched;
         };
 #pragma unroll
         for (uint32_t s = 0; s < ST; ++s) fetch();
 
         uint32_t v[2][KW];
-        load_run<KW>(a.src + (size_t)(group * KW) * wc + w, wc, v);
+        load_run<KW>(a.src + (size_t)(group * KW) * wc + gw, wc, v);
 #pragma unroll
         for (int k = 0; k < KW; ++k) {
             X[k * THREADS + c] = v[0][k];
@@ -483,7 +526,7 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
                 atomicAdd(a.final_acc + 1, anti);
             }
         }
-        if (mine) store_run<KW>(a.dst + (size_t)(group * KW) * wc + w, wc, v);
+        if (mine) store_run<KW>(a.dst + (size_t)(group * KW) * wc + gw, wc, v);
     }
     __syncthreads();  // the tile's shared memory is free again
 }
@@ -604,11 +647,27 @@ __global__ void __launch_bounds__(kThreads, KW == 8 ? 2 : 1) k_ahead(const __gri
         if constexpr (WARP)
             update_warp(a, smem);
         else
-            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, KW, FIELD, true>(a, t, smem);
+            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, KW, FIELD, true, false>(a, t, smem);
     } else if (blockIdx.x < early) {
         count_role<KW>(a, blockIdx.x - a.update_ctas);
     }
-    if (a.d_tickets != 0u) draw_role<FIELD>(a);
+    if (a.d_tickets != 0u) draw_role<FIELD, false>(a);
+}
+
+// Large lattices: a launch draws the masks of a band of rows (and of the rows that the
+// band's tiles spoil) for a block of sweeps and updates the band before from one copy of
+// the lattice to the other.
+__global__ void __launch_bounds__(kThreads, 2) k_ahead_band(const __grid_constant__ AheadArgs a)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    // (waits as in k_ahead)
+    if (blockIdx.x < a.update_ctas || a.update_ctas == 0u) dependent_launch_wait();
+    dependent_launch_trigger();
+    if (blockIdx.x < a.update_ctas) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *a.next_ticket = 0u;
+        for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, 8, false, false, true>(a, t, smem);
+    }
+    if (a.d_tickets != 0u) draw_role<false, true>(a);
 }
 
 // ----------------------------------------------------------------- batch --
@@ -654,9 +713,9 @@ __device__ __forceinline__ void batch_draw_role(const AheadBatchArgs &a)
         char *const masks = j.masks + (size_t)(a.block % kBuffers) * j.mask_bytes;
         const uint32_t t0 = a.t0[j.index] + a.block * j.block_sweeps;
         if (j.field)
-            draw_item<true, 4>(j, masks, t0, gp & 1u, sw, idx);
+            draw_item<true, 4, false>(j, masks, j.step_bytes, t0, gp & 1u, sw, idx);
         else
-            draw_item<false, 4>(j, masks, t0, gp & 1u, sw, idx);
+            draw_item<false, 4, false>(j, masks, j.step_bytes, t0, gp & 1u, sw, idx);
     }
 }
 
@@ -715,15 +774,15 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_ahead_batch(const __grid_c
             const uint32_t tile = g - j.tile_start;
             if (!j.field) {
                 if (j.kw == 2)
-                    update_tile<kBatchThreads, 2, false, false>(t, tile, smem);
+                    update_tile<kBatchThreads, 2, false, false, false>(t, tile, smem);
                 else if (j.kw == 4)
-                    update_tile<kBatchThreads, 4, false, false>(t, tile, smem);
+                    update_tile<kBatchThreads, 4, false, false, false>(t, tile, smem);
                 else
-                    update_tile<kBatchThreads, 8, false, false>(t, tile, smem);
+                    update_tile<kBatchThreads, 8, false, false, false>(t, tile, smem);
             } else if (j.kw == 2) {
-                update_tile<kBatchThreads, 2, true, false>(t, tile, smem);
+                update_tile<kBatchThreads, 2, true, false, false>(t, tile, smem);
             } else {
-                update_tile<kBatchThreads, 4, true, false>(t, tile, smem);
+                update_tile<kBatchThreads, 4, true, false, false>(t, tile, smem);
             }
         }
     }
@@ -734,6 +793,7 @@ using AheadKernel = void (*)(AheadArgs);
 
 AheadKernel pick_kernel(const AheadPlan &p)
 {
+    if (p.band_rows) return k_ahead_band;
     if (p.field) return p.kw == 2 ? k_ahead<2, false, true> : p.kw == 4 ? k_ahead<4, false, true> : nullptr;
     if (p.warp) return k_ahead<2, true, false>;
     return p.kw == 2 ? k_ahead<2, false, false> : p.kw == 4 ? k_ahead<4, false, false> : p.kw == 8 ? k_ahead<8, false, false> : nullptr;
@@ -787,8 +847,10 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 //   L = 1024,  500 sweeps: 64 + 32: 447, 32 + 32: 470, 32 + 16: 607
 //   L = 2048,  200 sweeps: 64 + 32: 606, 64 + 16: 630, 32 + 16: 659
 //   L = 4096,  200 sweeps: 32 + 16: 2225, 16 + 8: 2399
-// Above 8192 a block would hold fewer than 4 sweeps and its masks 25 times the
-// lattice: the step kernels run there.  Two CTAs of the largest tiles share a SM, and
+// Above 8192 tiles are parts of rows and a launch takes a band of rows: the masks of
+// all would be 64 times the lattice a block.  Measured against the step kernels (two
+// launches a sweep): L = 65536, 4 sweeps 12252 -> 11083 us (1.55 attempts per ns), 8 sweeps
+// 24481 -> 21766; 16384, 40 sweeps 8510 -> 6808; 8256, 40 sweeps 2456 -> 1804.  Two CTAs of the largest tiles share a SM, and
 // with draws (L = 2048, 200 sweeps: 606 us with one, 585 with two; 4096 2225 and 2137;
 // 8192, 40 sweeps 1848 and 1748).  In a field (20 bytes of masks a word and step
 // instead of 8, five compares a draw instead of two) L <= 4096.  Measured, 200 sweeps
@@ -800,8 +862,24 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 AheadPlan ahead_plan(uint64_t L, bool field)
 {
     AheadPlan p{};
-    if (L % 64 != 0 || L < 64 || L > (field ? 4096 : 8192)) return p;
+    if (L % 64 != 0 || L < 64 || (field && L > 4096)) return p;
     const uint32_t wc = (uint32_t)(L / 64);
+    if (L > 8192) {
+        // tiles of 64 rows (80 with the halo of a block of 4 sweeps, 10 runs of 8) and as
+        // many words as fill 512 threads with two more, in equal parts of a row; bands
+        // of about 2^20 words, at least 512 rows (16 more are drawn twice)
+        p.kw = 8;
+        p.tile_rows = 64;
+        p.halo = 8;
+        p.block_sweeps = 4;
+        p.min_sweeps = 4;
+        const uint32_t words = kThreads / ((p.tile_rows + 2 * p.halo) / p.kw) - 2;
+        p.tiles_x = (wc + words - 1) / words;
+        p.tile_words = (wc + p.tiles_x - 1) / p.tiles_x;
+        p.band_rows = std::min((uint32_t)L, std::max(512u, (1u << 20) / wc / 64 * 64));
+        p.mask_bytes = (size_t)2 * p.block_sweeps * std::min<uint64_t>(L, p.band_rows + 2 * p.halo) * wc * 8;
+        return p;
+    }
     if (L <= 192) {
         p.tile_rows = (uint32_t)L;
         p.halo = 0;
@@ -866,9 +944,10 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
     const AheadKernel kern = pick_kernel(pl);
     if (!kern) return cudaErrorInvalidValue;
     int sms = 0;
-    cudaError_t e = prepare_device(kern, pl.warp ? 0 : pl.kw / 2 + (pl.field ? 8 : 0), &sms);
+    cudaError_t e = prepare_device(kern, pl.band_rows ? 16 : pl.warp ? 0 : pl.kw / 2 + (pl.field ? 8 : 0), &sms);
     if (e != cudaSuccess) return e;
-    a.update_ctas = a.u_steps ? pl.update_ctas : 0u;
+    if (pl.band_rows) a.nwords = (a.d_words + 31) / 32 * 32;  // for the tickets
+    a.update_ctas = !a.u_steps ? 0u : pl.band_rows ? std::min(a.tiles, (uint32_t)sms) : pl.update_ctas;
     const uint32_t per = (a.nwords / pl.kw + 31u) & ~31u;
     a.count_ctas = a.c_slots ? std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, pl.kw == 8 ? 64u : 16u) : 0u;
     a.d_four = a.d_sweeps % 4 == 0;
@@ -893,9 +972,9 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
 
 }  // namespace
 
-bool ahead_ready(ising_lattice *h, const AheadPlan &pl)
+bool ahead_ready(ising_lattice *h, const AheadPlan &pl, uint64_t L)
 {
-    const size_t need = kTicketBytes + kBuffers * pl.mask_bytes + 2 * pl.snap_bytes + (pl.halo ? h->bytes : 0);
+    const size_t need = kTicketBytes + kBuffers * pl.mask_bytes + 2 * pl.snap_bytes + (pl.halo ? (size_t)(L * L / 8) : 0);
     if (h->ahead_bytes >= need) return true;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
@@ -908,15 +987,85 @@ bool ahead_ready(ising_lattice *h, const AheadPlan &pl)
         h->d_ahead = nullptr;
         h->ahead_bytes = 0;
     }
+    // a second copy of a lattice that fills the GPU would take what its user may need:
+    // at most half of what is free
+    size_t free_bytes = 0, total_bytes = 0;
+    if (need > kPoolKeeps && (cudaMemGetInfo(&free_bytes, &total_bytes) != cudaSuccess || need > free_bytes / 2)) {
+        cudaGetLastError();
+        return false;
+    }
     h->d_ahead = h->alloc.scratch(need, h->stream);
     h->ahead_bytes = h->d_ahead ? need : 0;
     return h->d_ahead != nullptr;
 }
 
-cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, uint64_t t0, uint64_t nsweeps, uint32_t record_every,
+// Blocks of 4 sweeps (the rest of a division by 4 first), each in bands of rows.
+static cudaError_t band_sweeps(const AheadPlan &pl, AheadArgs a, char *masks, unsigned int *tickets, uint64_t *spins, uint64_t *other,
+                               size_t bytes, uint64_t t0, uint64_t nsweeps, uint64_t full, cudaStream_t s)
+{
+    const uint32_t L = a.L, halo = pl.halo, bands = (L + pl.band_rows - 1) / pl.band_rows;
+    const uint64_t first = nsweeps % full ? nsweeps % full : full, nblocks = 1 + (nsweeps - first + full - 1) / full;
+    uint64_t *src = spins, *dst = other;
+    cudaError_t e = cudaSuccess;
+    if (nblocks % 2 == 1) {
+        e = cudaMemcpyAsync(other, spins, bytes, cudaMemcpyDeviceToDevice, s);
+        std::swap(src, dst);
+    }
+    a.tile_words = pl.tile_words;
+    a.tiles_x = pl.tiles_x;
+    a.by_tw = fast_div(pl.tile_words + 2);
+    const uint32_t re = a.record_every;
+    uint64_t i = 0, rec_done = 0, done = 0;  // items before; samples and sweeps of the blocks before the one updated
+    for (uint64_t b = 0; b <= nblocks; ++b) {
+        const uint64_t drawn = b == 0 ? 0 : first + (b - 1) * full;
+        for (uint32_t k = 0; k < bands && e == cudaSuccess; ++k, ++i) {
+            // draw band k of block b, update the band before
+            if (i > 0) {
+                const uint64_t ub = k ? b : b - 1, t = t0 + done, n = ub == 0 ? first : full;
+                const uint32_t uk = k ? k - 1 : bands - 1, rows = std::min(pl.band_rows, L - uk * pl.band_rows);
+                a.u_steps = (uint32_t)(2 * n);
+                a.src = src;
+                a.dst = dst;
+                a.u_masks = masks + ((i - 1) % kBuffers) * pl.mask_bytes;
+                a.u_row0 = uk * pl.band_rows;
+                a.u_mask_row0 = bands == 1 ? 0u : (a.u_row0 + L - halo) % L;
+                a.u_words = (bands == 1 ? L : rows + 2 * halo) * a.wc;
+                a.tiles = rows / pl.tile_rows * pl.tiles_x;
+                a.u_phase = re ? (uint32_t)(t % re) : 0u;
+                a.u_recs = re ? (uint32_t)((t + n) / re - t / re) : 0u;
+                a.u_slot0 = (uint32_t)rec_done;
+                a.u_last = done + n == nsweeps;
+                a.u_slots = a.u_recs + ((a.u_last && !(re && (t + n) % re == 0)) ? 1u : 0u);
+                if (uk == bands - 1) {  // the block's last band
+                    std::swap(src, dst);
+                    done += n;
+                    rec_done += a.u_recs;
+                }
+            }
+            if (b == nblocks && k > 0) return e;
+            a.d_sweeps = b == nblocks ? 0u : (uint32_t)(b == 0 ? first : full);
+            if (a.d_sweeps) {
+                const uint32_t row0 = k * pl.band_rows, rows = std::min(pl.band_rows, L - row0);
+                a.d_t0 = (uint32_t)(t0 + drawn);
+                a.d_row0 = bands == 1 ? 0u : (row0 + L - halo) % L;
+                a.d_words = (bands == 1 ? L : rows + 2 * halo) * a.wc;
+                a.by_group = fast_div((a.d_words + 31) / 32);
+            }
+            a.d_masks = masks + (i % kBuffers) * pl.mask_bytes;
+            a.d_ticket = tickets + i % 4;
+            a.next_ticket = tickets + (i + 2) % 4;
+            e = launch_ahead(pl, a, i > 0, s);
+        }
+        if (e != cudaSuccess) break;
+    }
+    return e;
+}
+
+cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, uint64_t L, uint64_t t0, uint64_t nsweeps, uint32_t record_every,
                          uint64_t nrec, unsigned int *err, uint32_t hold_step, uint64_t max_block)
 {
     const uint32_t full = (uint32_t)std::min<uint64_t>(pl.block_sweeps, max_block);
+    const size_t bytes = (size_t)(L * L / 8);
     unsigned int *const tickets = static_cast<unsigned int *>(h->d_ahead);
     char *const masks = static_cast<char *>(h->d_ahead) + kTicketBytes;
     char *const snaps = masks + kBuffers * pl.mask_bytes;
@@ -927,11 +1076,13 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     a.step_bytes = pl.step_bytes;
     set_planes(a, h);
     a.c3base = h->stream_id << 1;
-    a.L = (uint32_t)h->L;
+    a.L = (uint32_t)L;
     a.wc = a.L / 64;
-    a.nwords = a.L * a.wc;
     a.by_wc = fast_div(a.wc);
-    a.by_group = fast_div(a.nwords / 32);
+    if (!pl.band_rows) {
+        a.nwords = a.L * a.wc;
+        a.by_group = fast_div(a.nwords / 32);
+    }
     a.tiles = pl.tiles;
     a.tile_rows = pl.tile_rows;
     a.halo = pl.halo;
@@ -940,12 +1091,16 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     a.final_acc = h->d_acc + 2 * nrec;
     a.err = err;
     a.hold_step = hold_step;
+    if (pl.band_rows) {
+        const cudaError_t e = cudaMemsetAsync(tickets, 0, kTicketBytes, h->stream);
+        return e != cudaSuccess ? e : band_sweeps(pl, a, masks, tickets, spins, other, bytes, t0, nsweeps, full, h->stream);
+    }
     // Counting in the launch after the update takes work off its chain of steps, but
     // costs a launch at the end and the snapshots' traffic: M/E every sweep, counted by
     // the tiles and from snapshots, 1000 sweeps of 256 490 and 365 us, 1000 of 512 625 and
     // 496, 200 of 2048 667 and 618, 200 of 4096 2183 and 2246; 10 sweeps of 4096 165 and
     // 203.
-    const bool snapshots = pl.warp || (nsweeps >= 32 && h->L <= 2048);
+    const bool snapshots = pl.warp || (nsweeps >= 32 && L <= 2048);
     // Blocks.  Items of 4 sweeps are the cheapest to draw, so a call that is long
     // enough starts with the rest of a division by 4.  Where an update takes long
     // (one CTA holds the lattice), blocks start short: nothing overlaps the first
@@ -953,7 +1108,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     uint64_t drawn = 0, done = 0, rec_done = 0, prev = 0, grow = pl.halo ? full : std::min<uint64_t>(full, 32);
     auto next_block = [&]() -> uint64_t {
         const uint64_t left = nsweeps - drawn;
-        if (full % 4 != 0 || (left <= 7 && h->L < 2048)) return std::min<uint64_t>(left, full);
+        if (full % 4 != 0 || (left <= 7 && L < 2048)) return std::min<uint64_t>(left, full);
         if (left % 4) return left % 4;
         if (pl.halo && left % full) return left % full;
         const uint64_t n = std::min(left, grow);
@@ -968,7 +1123,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     if (e != cudaSuccess) return e;
     const uint64_t *src = spins;
     if (pl.halo && nblocks % 2 == 1) {
-        e = cudaMemcpyAsync(other, spins, h->bytes, cudaMemcpyDeviceToDevice, h->stream);
+        e = cudaMemcpyAsync(other, spins, bytes, cudaMemcpyDeviceToDevice, h->stream);
         if (e != cudaSuccess) return e;
         src = other;
     }

@@ -18,6 +18,8 @@ struct AheadPlan {
     uint32_t update_ctas;   // CTAs that share them
     bool warp;              // one warp holds the lattice
     bool field;             // in a field: five mask planes
+    uint32_t band_rows;     // rows that a launch takes (0: all)
+    uint32_t tile_words, tiles_x;  // words of a tile's rows and tiles of a row, where a launch takes a band
     uint32_t block_sweeps;  // sweeps of a block at most (halo / 2 where there is a halo)
     uint32_t min_sweeps;    // shorter calls are as fast without
     uint32_t step_bytes;    // masks of a step
@@ -53,11 +55,16 @@ struct AheadArgs {
     uint32_t u_phase;             // sweep index % record_every at the block's start
     uint32_t u_recs, u_slot0;     // samples of the block, slot of the first
     uint32_t u_slots, u_last;     // counted sweeps: u_recs, or one more; the call's last block
+    // a band of rows: its first; the first row and the words of a step with masks
+    uint32_t u_row0, u_mask_row0, u_words;
+    uint32_t tile_words, tiles_x;
+    FastDiv by_tw;                // division by tile_words + 2
     // count: the snapshots of the block before
     uint32_t count_ctas, c_slots, c_recs, c_slot0, c_last;
     const uint32_t *c_snaps;
     // draw: d_sweeps sweeps from sweep index d_t0, in tickets of 32 items of 4 sweeps or of one
     uint32_t d_t0, d_sweeps, d_four, d_tickets;
+    uint32_t d_row0, d_words;     // a band: the first row drawn, words of a step
     char *d_masks;
     unsigned int *d_ticket, *next_ticket;  // this launch's counter; the one to clear
 };
@@ -97,15 +104,15 @@ struct AheadBatchArgs {
 struct ising_lattice;
 
 namespace ising {
-// The handle's scratch for the plan (masks, snapshots, a second lattice), allocated
+// The handle's scratch for the plan of size L (masks, snapshots, a second lattice), allocated
 // on first use and kept; false when there is none to be had (the allocator refuses,
 // or the stream is being captured): the caller then takes another path.
-bool ahead_ready(ising_lattice *h, const AheadPlan &pl);
-// Queues nsweeps sweeps of `lattice` (the handle's, or a copy of it) from sweep
+bool ahead_ready(ising_lattice *h, const AheadPlan &pl, uint64_t L);
+// Queues nsweeps sweeps of `lattice` (the handle's, or scratch of L^2 sites) from sweep
 // index t0 on the handle's stream; counters as TinyRunArgs.  A block holds at most
 // max_block sweeps.
-cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, uint64_t t0, uint64_t nsweeps,
-                         uint32_t record_every, uint64_t nrec, unsigned int *err, uint32_t hold_step, uint64_t max_block);
+cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, uint64_t L, uint64_t t0,
+                         uint64_t nsweeps, uint32_t record_every, uint64_t nrec, unsigned int *err, uint32_t hold_step, uint64_t max_block);
 
 // A run of many lattices in the draw-ahead form.
 struct AheadBatch {

@@ -267,16 +267,19 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
             best_c = c;
         }
     }
-    // the draw-ahead form on the copy, where it applies (the copy is the whole lattice there)
-    const AheadPlan pl = ahead_plan(h->L, false);
+    // the draw-ahead form on the copy, or where that is not the whole lattice on a
+    // lattice of 32768^2 of the copy's words: the time per site of a large lattice
+    // does not depend on its size
+    const uint64_t La = rows == h->L ? h->L : 32768;
+    const AheadPlan pl = ahead_plan(La, false);
     bool ahead = false;
-    if (e == cudaSuccess && pl.kw != 0 && rows == h->L && ahead_ready(h, pl)) {
+    if (e == cudaSuccess && pl.kw != 0 && La * La / 8 <= rows * row_bytes && ahead_ready(h, pl, La)) {
         const uint32_t n = std::max(8 * reps, 2 * pl.min_sweeps);
         unsigned int *const flag = reinterpret_cast<unsigned int *>(h->d_acc + 2);  // after the one state slot
         e = cudaMemsetAsync(flag, 0, 16, h->stream);
         for (uint32_t k = 0; k < 2 && e == cudaSuccess; ++k) {
             e = cudaEventRecord(e0, h->stream);
-            if (e == cudaSuccess) e = ahead_sweeps(h, pl, scratch, 0xFFFF0000u, n, 0, 0, flag, 0, 1ull << 30);
+            if (e == cudaSuccess) e = ahead_sweeps(h, pl, scratch, La, 0xFFFF0000u, n, 0, 0, flag, 0, 1ull << 30);
         }
         if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
@@ -284,9 +287,11 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
         unsigned int timeout = 0;
         if (e == cudaSuccess) e = cudaMemcpy(&timeout, flag, sizeof timeout, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess && timeout == 0 && (double)ms / (2 * n) < best_step_ms) {
+        // (best_step_ms: for `rows` rows)
+        const double step_ms = (double)ms / (2 * n) * ((double)rows * (double)h->L / ((double)La * (double)La));
+        if (e == cudaSuccess && timeout == 0 && step_ms < best_step_ms) {
             ahead = true;
-            best_step_ms = (double)ms / (2 * n);
+            best_step_ms = step_ms;
         }
     }
     if (e0) cudaEventDestroy(e0);

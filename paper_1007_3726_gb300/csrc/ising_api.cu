@@ -487,8 +487,8 @@ ising_status ising_sweep(ising_lattice *h, uint64_t nsweeps, uint32_t record_eve
         if (v > 0 && v < max_chunk) max_chunk = v;
     }
     const AheadPlan pl = h->ahead ? ahead_plan(h->L, h->H != 0.0) : AheadPlan{};
-    if (pl.kw != 0 && nsweeps >= pl.min_sweeps && ahead_ready(h, pl)) {
-        CK(h, ahead_sweeps(h, pl, h->d_spins, t0, nsweeps, record_every, nrec, err, hold_step, max_chunk));
+    if (pl.kw != 0 && nsweeps >= pl.min_sweeps && ahead_ready(h, pl, h->L)) {
+        CK(h, ahead_sweeps(h, pl, h->d_spins, h->L, t0, nsweeps, record_every, nrec, err, hold_step, max_chunk));
         h->pending_err = true;
         return finish_sweep_call(h, t0, nsweeps, nrec, M_out, E_out);
     }

@@ -42,7 +42,8 @@ LARGE = ((10, 1), (12, 3), (18, 0), (23, 1), (33, 5))
 @pytest.mark.parametrize("L,calls", [(64, SMALL), (128, SMALL), (192, SMALL + MIDDLE), (256, MIDDLE), (320, MIDDLE),
                                      (448, MIDDLE), (512, MIDDLE), (704, MIDDLE), (960, MIDDLE), (1024, MIDDLE),
                                      (1088, MIDDLE), (2048, LARGE), (2112, LARGE), (4096, LARGE), (4160, LARGE),
-                                     (8192, ((10, 1), (13, 2)))])
+                                     (8192, ((10, 1), (13, 2))), (8256, ((4, 1), (11, 2))), (9984, ((9, 1), (8, 0))),
+                                     (16384, ((7, 3), (4, 1)))])
 def test_sizes_blocks_and_records_bit_exact(P, orc, L, calls):
     T, seed, sid = TC, L + 3, 5
     lat = P.Lattice(L, T, seed=seed, stream_id=sid, init="hot", word_bits=64 if L % 128 == 0 else 32)
