@@ -174,7 +174,7 @@ __device__ __forceinline__ void draw_item(const A &a, char *masks, size_t step_b
         char *const step = masks + (size_t)(2u * (sw + k) + p) * step_bytes;
         if constexpr (FIELD) {
             reinterpret_cast<uint4 *>(step)[idx] = make_uint4(m[k][0], m[k][1], m[k][2], m[k][3]);
-            reinterpret_cast<uint32_t *>(step + (size_t)a.nwords * 16u)[idx] = m[k][4];
+            reinterpret_cast<uint32_t *>(step + step_bytes / 5u * 4u)[idx] = m[k][4];  // behind 16 bytes a word
         } else {
             reinterpret_cast<uint2 *>(step)[idx] = make_uint2(m[k][0], m[k][1]);
         }
@@ -187,7 +187,7 @@ template <bool FIELD, bool BAND>
 __device__ __forceinline__ void draw_role(const AheadArgs &a)
 {
     const uint32_t lane = threadIdx.x & 31u, per_group = BAND ? (a.d_words + 31u) / 32u : a.nwords / 32u;
-    const size_t step_bytes = BAND ? (size_t)a.d_words * 8u : a.step_bytes;
+    const size_t step_bytes = BAND ? (size_t)a.d_words * (FIELD ? 20u : 8u) : a.step_bytes;
     uint32_t next = lane == 0 ? atomicAdd(a.d_ticket, 1u) : 0u;
     for (;;) {
         const uint32_t it = __shfl_sync(0xFFFFFFFFu, next, 0);
@@ -196,8 +196,10 @@ __device__ __forceinline__ void draw_role(const AheadArgs &a)
         const uint32_t gp = a.by_group.quotient(it);
         uint32_t idx = (it - gp * per_group) * 32u + lane;
         if constexpr (BAND) idx = min(idx, a.d_words - 1u);  // (the last ticket of a group repeats its last word)
-        if (a.d_four)
+        if (a.d_k == 4u)
             draw_item<FIELD, 4, BAND>(a, a.d_masks, step_bytes, a.d_t0, gp & 1u, (gp >> 1) * 4u, idx);
+        else if (a.d_k == 2u)
+            draw_item<FIELD, 2, BAND>(a, a.d_masks, step_bytes, a.d_t0, gp & 1u, (gp >> 1) * 2u, idx);
         else
             draw_item<FIELD, 1, BAND>(a, a.d_masks, step_bytes, a.d_t0, gp & 1u, gp >> 1, idx);
     }
@@ -423,9 +425,9 @@ __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, u
             uint32_t y = group * KW + L - a.u_mask_row0;          // in the rows that have masks
             if (y >= L) y -= L;
             first = (size_t)(y / 2u) * wc + gw;
-            step_bytes = (size_t)a.u_words * 8u;
+            step_bytes = (size_t)a.u_words * (FIELD ? 20u : 8u);
         }
-        const char *msrc = a.u_masks + first * (FIELD ? 32u : 16u), *msrc4 = a.u_masks + (size_t)a.nwords * 16u + first * 8u;
+        const char *msrc = a.u_masks + first * (FIELD ? 32u : 16u), *msrc4 = a.u_masks + step_bytes / 5u * 4u + first * 8u;
         const uint32_t mdst = shared_addr(ring + c), mdst4 = shared_addr(ring4 + c);
         uint32_t fetched = 0;
         auto fetch = [&]() {
@@ -657,7 +659,8 @@ __global__ void __launch_bounds__(kThreads, KW == 8 ? 2 : 1) k_ahead(const __gri
 // Large lattices: a launch draws the masks of a band of rows (and of the rows that the
 // band's tiles spoil) for a block of sweeps and updates the band before from one copy of
 // the lattice to the other.
-__global__ void __launch_bounds__(kThreads, 2) k_ahead_band(const __grid_constant__ AheadArgs a)
+template <bool FIELD>
+__global__ void __launch_bounds__(kThreads, FIELD ? 1 : 2) k_ahead_band(const __grid_constant__ AheadArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     // (waits as in k_ahead)
@@ -665,9 +668,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_ahead_band(const __grid_constan
     dependent_launch_trigger();
     if (blockIdx.x < a.update_ctas) {
         if (blockIdx.x == 0 && threadIdx.x == 0) *a.next_ticket = 0u;
-        for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, 8, false, false, true>(a, t, smem);
+        for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, FIELD ? 4 : 8, FIELD, false, true>(a, t, smem);
     }
-    if (a.d_tickets != 0u) draw_role<false, true>(a);
+    if (a.d_tickets != 0u) draw_role<FIELD, true>(a);
 }
 
 // ----------------------------------------------------------------- batch --
@@ -793,7 +796,7 @@ using AheadKernel = void (*)(AheadArgs);
 
 AheadKernel pick_kernel(const AheadPlan &p)
 {
-    if (p.band_rows) return k_ahead_band;
+    if (p.band_rows) return p.field ? k_ahead_band<true> : k_ahead_band<false>;
     if (p.field) return p.kw == 2 ? k_ahead<2, false, true> : p.kw == 4 ? k_ahead<4, false, true> : nullptr;
     if (p.warp) return k_ahead<2, true, false>;
     return p.kw == 2 ? k_ahead<2, false, false> : p.kw == 4 ? k_ahead<4, false, false> : p.kw == 8 ? k_ahead<8, false, false> : nullptr;
@@ -850,10 +853,13 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 // Above 8192 tiles are parts of rows and a launch takes a band of rows: the masks of
 // all would be 64 times the lattice a block.  Measured against the step kernels (two
 // launches a sweep): L = 65536, 4 sweeps 12252 -> 11083 us (1.55 attempts per ns), 8 sweeps
-// 24481 -> 21766; 16384, 40 sweeps 8510 -> 6808; 8256, 40 sweeps 2456 -> 1804.  Two CTAs of the largest tiles share a SM, and
-// with draws (L = 2048, 200 sweeps: 606 us with one, 585 with two; 4096 2225 and 2137;
-// 8192, 40 sweeps 1848 and 1748).  In a field (20 bytes of masks a word and step
-// instead of 8, five compares a draw instead of two) L <= 4096.  Measured, 200 sweeps
+// 24481 -> 21766; 16384, 40 sweeps 8510 -> 6808; 8256, 40 sweeps 2456 -> 1804; in a field
+// (five compares a draw instead of two: the draws are the more of the work) 65536, 8 sweeps
+// 38787 -> 36216; 16384, 40 sweeps 12538 -> 11360; 8256, 40 sweeps 3769 -> 3256, but 6 sweeps
+// 596 and 615.  Two CTAs of the largest tiles share a SM, and with draws (L = 2048,
+// 200 sweeps: 606 us with one, 585 with two; 4096 2225 and 2137; 8192, 40 sweeps 1848
+// and 1748).  In a field (20 bytes of masks a word and step instead of 8) the bands
+// start above 4096, for tiles of half the words.  Measured, 200 sweeps
 // with M/E every sweep, the field step kernel (L = 64 .. 512: the one-launch field
 // kernels) against this form: L = 64 547 -> 102 us, 512 1384 -> 251, 704 5568 -> 357,
 // 2048 5593 -> 991; 20 sweeps of 4096 689 -> 425.  min_sweeps: a call has one launch more than
@@ -862,22 +868,24 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 AheadPlan ahead_plan(uint64_t L, bool field)
 {
     AheadPlan p{};
-    if (L % 64 != 0 || L < 64 || (field && L > 4096)) return p;
+    if (L % 64 != 0 || L < 64) return p;
     const uint32_t wc = (uint32_t)(L / 64);
-    if (L > 8192) {
-        // tiles of 64 rows (80 with the halo of a block of 4 sweeps, 10 runs of 8) and as
-        // many words as fill 512 threads with two more, in equal parts of a row; bands
+    p.field = field;
+    if (L > (field ? 4096 : 8192)) {
+        // tiles of 64 rows (80 with the halo of a block of 4 sweeps, 10 runs of 8; in a field
+        // 32 rows, 12 runs of 4) and as many words as fill 512 threads with two more, in
+        // equal parts of a row; bands
         // of about 2^20 words, at least 512 rows (16 more are drawn twice)
-        p.kw = 8;
-        p.tile_rows = 64;
+        p.kw = field ? 4 : 8;
+        p.tile_rows = field ? 32 : 64;
         p.halo = 8;
         p.block_sweeps = 4;
-        p.min_sweeps = 4;
+        p.min_sweeps = field && L < 16384 ? 12 : 4;
         const uint32_t words = kThreads / ((p.tile_rows + 2 * p.halo) / p.kw) - 2;
         p.tiles_x = (wc + words - 1) / words;
         p.tile_words = (wc + p.tiles_x - 1) / p.tiles_x;
         p.band_rows = std::min((uint32_t)L, std::max(512u, (1u << 20) / wc / 64 * 64));
-        p.mask_bytes = (size_t)2 * p.block_sweeps * std::min<uint64_t>(L, p.band_rows + 2 * p.halo) * wc * 8;
+        p.mask_bytes = (size_t)2 * p.block_sweeps * std::min<uint64_t>(L, p.band_rows + 2 * p.halo) * wc * (field ? 20 : 8);
         return p;
     }
     if (L <= 192) {
@@ -905,7 +913,6 @@ AheadPlan ahead_plan(uint64_t L, bool field)
     const uint32_t most_ctas = p.kw == 8 ? 128 : 64;
     const uint32_t each = p.tiles <= 96 ? 1 : std::max(2u, (p.tiles + most_ctas - 1) / most_ctas);
     p.update_ctas = (p.tiles + each - 1) / each;
-    p.field = field;
     p.step_bytes = (uint32_t)(L * wc * (field ? 20 : 8));
     p.mask_bytes = (size_t)2 * p.block_sweeps * p.step_bytes;
     p.snap_bytes = L <= 2048 ? (size_t)p.block_sweeps * L * wc * 8 : 0;
@@ -944,14 +951,15 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
     const AheadKernel kern = pick_kernel(pl);
     if (!kern) return cudaErrorInvalidValue;
     int sms = 0;
-    cudaError_t e = prepare_device(kern, pl.band_rows ? 16 : pl.warp ? 0 : pl.kw / 2 + (pl.field ? 8 : 0), &sms);
+    cudaError_t e = prepare_device(kern, pl.band_rows ? 16 + pl.field : pl.warp ? 0 : pl.kw / 2 + (pl.field ? 8 : 0), &sms);
     if (e != cudaSuccess) return e;
     if (pl.band_rows) a.nwords = (a.d_words + 31) / 32 * 32;  // for the tickets
-    a.update_ctas = !a.u_steps ? 0u : pl.band_rows ? std::min(a.tiles, (uint32_t)sms) : pl.update_ctas;
+    a.update_ctas = !a.u_steps ? 0u : pl.band_rows ? std::min(a.tiles, pl.field ? 64u : (uint32_t)sms) : pl.update_ctas;
     const uint32_t per = (a.nwords / pl.kw + 31u) & ~31u;
     a.count_ctas = a.c_slots ? std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, pl.kw == 8 ? 64u : 16u) : 0u;
-    a.d_four = a.d_sweeps % 4 == 0;
-    a.d_tickets = (a.d_four ? a.d_sweeps / 4 : a.d_sweeps) * 2u * (a.nwords / 32u);
+    // 1756 attempts/ns in items of 4 sweeps, 1708 in items of 2, 1616 one by one
+    a.d_k = a.d_sweeps % 4 == 0 ? 4 : a.d_sweeps % 2 == 0 ? 2 : 1;
+    a.d_tickets = a.d_sweeps / a.d_k * 2u * (a.nwords / 32u);
     const uint32_t early = a.update_ctas + a.count_ctas, warps = kThreads / 32u;
     const uint32_t grid = std::max(early, std::min<uint32_t>((uint32_t)sms * (pl.kw == 8 ? 2u : 1u), early + (a.d_tickets + warps - 1) / warps));
     const size_t smem = !a.u_steps ? 0

@@ -62,8 +62,8 @@ struct AheadArgs {
     // count: the snapshots of the block before
     uint32_t count_ctas, c_slots, c_recs, c_slot0, c_last;
     const uint32_t *c_snaps;
-    // draw: d_sweeps sweeps from sweep index d_t0, in tickets of 32 items of 4 sweeps or of one
-    uint32_t d_t0, d_sweeps, d_four, d_tickets;
+    // draw: d_sweeps sweeps from sweep index d_t0, in tickets of 32 items of d_k sweeps
+    uint32_t d_t0, d_sweeps, d_k, d_tickets;
     uint32_t d_row0, d_words;     // a band: the first row drawn, words of a step
     char *d_masks;
     unsigned int *d_ticket, *next_ticket;  // this launch's counter; the one to clear

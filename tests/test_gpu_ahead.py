@@ -36,11 +36,12 @@ def _compare(orc, lat, s, t, n, rec, seed, sid, thr):
 # remainder of 4, sample spacings that cross the calls, none
 SMALL = ((200, 1), (203, 3), (321, 0), (514, 7))
 MIDDLE = ((10, 1), (33, 3), (64, 0), (71, 7))
+LONG = MIDDLE + ((130, 1), (203, 3))
 LARGE = ((10, 1), (12, 3), (18, 0), (23, 1), (33, 5))
 
 
-@pytest.mark.parametrize("L,calls", [(64, SMALL), (128, SMALL), (192, SMALL + MIDDLE), (256, MIDDLE), (320, MIDDLE),
-                                     (448, MIDDLE), (512, MIDDLE), (704, MIDDLE), (960, MIDDLE), (1024, MIDDLE),
+@pytest.mark.parametrize("L,calls", [(64, SMALL), (128, SMALL), (192, SMALL + MIDDLE), (256, LONG), (320, LONG),
+                                     (448, LONG), (512, LONG), (704, LONG), (960, LONG), (1024, LONG),
                                      (1088, MIDDLE), (2048, LARGE), (2112, LARGE), (4096, LARGE), (4160, LARGE),
                                      (8192, ((10, 1), (13, 2))), (8256, ((4, 1), (11, 2))), (9984, ((9, 1), (8, 0))),
                                      (16384, ((7, 3), (4, 1)))])
@@ -92,7 +93,7 @@ def test_field_classes_bit_exact(P, orc, L, H):
     lat.close()
 
 
-@pytest.mark.parametrize("L", [64, 128, 192, 256, 448, 704, 1024, 1088, 2048, 2112, 4096, 4160])
+@pytest.mark.parametrize("L", [64, 128, 192, 256, 448, 704, 1024, 1088, 2048, 2112, 4096, 4160, 8256])
 def test_field_sizes_bit_exact(P, orc, L):
     T, H, seed = TC, -0.4, L
     lat = P.Lattice(L, T, seed=seed, init="hot")
@@ -275,3 +276,17 @@ def test_batch_without_scratch_memory_runs_in_strips(P):
         l = P.Lattice(512, TC, seed=1, stream_id=i, init="hot")
         M, E = l.sweep(20, 2, collect=True)
         assert np.array_equal(l.spins(), spins) and np.array_equal(samples[0], M) and np.array_equal(samples[1], E)
+
+
+def test_second_counter_word_within_a_row(P):
+    """Above 2^35 sites the Philox group index needs its second word, which changes
+    inside a row of this size: the band form against the step kernels."""
+    L = 185408
+    out = []
+    for legacy in (True, False):
+        with P.Lattice(L, TC, seed=5, init="hot") as lat:
+            if legacy:
+                lat.set_launch(**lat.launch)
+            out.append(lat.sweep(6, 1, collect=True))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    np.testing.assert_array_equal(out[0][1], out[1][1])
