@@ -57,6 +57,7 @@ constexpr uint32_t kThreads = 512, kBatchThreads = 256;
 
 constexpr uint32_t kChunk = 8;     // steps of a stage of the one-warp form
 constexpr uint32_t kWarpStages = 8;
+constexpr uint32_t kClusterThreads = 256, kClusterChunk = 4, kClusterStages = 8;  // of the cluster form: update threads, steps of a stage, stages
 constexpr uint32_t kBuffers = 3;   // mask buffers, used in turn
 constexpr uint32_t kWaitLimit = 1u << 22;  // polls of a wait for masks on their way into shared memory
 
@@ -709,6 +710,266 @@ __global__ void __launch_bounds__(kThreads, KW == 8 ? 2 : 1) k_ahead(const __gri
     if (a.d_tickets != 0u) draw_role<FIELD, false>(a);
 }
 
+// --------------------------------------------------------------- cluster --
+// A lattice of 320^2 .. 512^2 held by the CTAs of one cluster: each has its tile of rows and
+// a halo of a.halo rows on either side, which its neighbours' boundary rows refresh every
+// a.halo steps through distributed shared memory, so that a block of many sweeps is one
+// launch and the halo is short.
+//
+// Bound: the chain of steps, 290 cycles each (a barrier 70, shared memory 35, 45
+// dependent instructions; an exchange 600 every 16 steps), with the draws beside it.  The
+// tiles of separate launches need 230 cycles a step and 2.8 us a launch: 1000
+// sweeps of 512 486 -> 390 us, 500 of 320 230 -> 215, M/E every sweep and every tenth about the
+// same; 256 (2 us of 32 sweeps a launch) is no faster than with tiles, 1024 is bound by its
+// draws.  One row a thread, 8 rows of halo, and 4 rows a lane with shuffles in place of
+// the barrier took as long within 5 %.
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The address of a shared variable of this CTA in the one of the given rank.
+__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// 16 bytes into a peer's shared memory; the peer's barrier counts them.
+__device__ __forceinline__ void store_peer16(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "r"(x),
+                 "r"(y), "r"(z), "r"(w), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t *bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(shared_addr(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copy_bulk_part(uint32_t dst, const void *src, uint32_t bytes, uint64_t *bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+                 "r"(bytes), "r"(shared_addr(bar))
+                 : "memory");
+}
+
+// Shared memory of update_cluster: the masks of a.stages chunks of kClusterChunk steps, the
+// two colours of the rows, two inboxes of halo rows.
+__host__ __device__ inline uint32_t cluster_step_bytes(uint32_t rows, uint32_t wc) { return rows * wc * 8u; }
+__host__ __device__ inline uint32_t cluster_smem(uint32_t rows, uint32_t halo, uint32_t wc, uint32_t stages)
+{
+    return stages * kClusterChunk * cluster_step_bytes(rows, wc) + 4u * kClusterThreads * 4u + 2u * (2u * halo * wc * 8u);
+}
+
+__device__ __forceinline__ void update_cluster(const AheadArgs &a, unsigned char *smem)
+{
+    constexpr uint32_t CH = kClusterChunk, T = kClusterThreads;
+    constexpr int KW = 2;                                              // rows of a run
+    __shared__ __align__(8) uint64_t full[kClusterStages], empty[kClusterStages], inbox_bar[2];
+    const uint32_t tid = threadIdx.x, wc = a.wc, L = a.L, rank = blockIdx.x, ranks = a.update_ctas;
+    const uint32_t R = a.tile_rows, H = a.halo, rows = R + 2 * H;
+    const uint32_t nthr = rows / KW * wc, nbar = (nthr + 31u) & ~31u;  // threads with a run; in whole warps
+    const uint32_t sb = cluster_step_bytes(rows, wc), ST = a.stages;
+    unsigned char *const ring = smem;                                  // [ST][CH][pair of rows][word][row of the pair]
+    uint32_t *const X = reinterpret_cast<uint32_t *>(smem + ST * CH * sb);  // [2][KW][T]: the two colours
+    uint4 *const inbox = reinterpret_cast<uint4 *>(X + 2 * KW * T);    // [2][runs of both halos]
+    const uint32_t inbox_bytes = 2u * H * wc * 8u;
+    if (tid == 0) {
+        for (uint32_t k = 0; k < ST; ++k) {
+            mbar_init(&full[k]);
+            mbar_init(&empty[k]);
+        }
+        mbar_init(&inbox_bar[0]);
+        mbar_init(&inbox_bar[1]);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    const uint32_t limit = a.hold_step ? 1u << 12 : kWaitLimit;
+    const uint32_t r0 = rank * R;
+    if (tid >= nbar) {
+        // the warp that fetches masks
+        cluster_sync();
+        if (tid == nbar) {
+            const uint32_t y0 = r0 >= H ? r0 - H : r0 + L - H;  // the first row with masks; the rows may go on at row 0
+            const uint32_t bytes1 = min(rows, L - y0) * wc * 8u, bytes2 = sb - bytes1;
+            uint32_t f = 0;
+            const char *from = a.u_masks;
+            for (uint32_t s = 0; s < a.u_steps; s += CH, ++f) {
+                const uint32_t st = f % ST, n = min(CH, a.u_steps - s);
+                if (f >= ST && !mbar_wait(&empty[st], (f / ST - 1u) & 1u, 4 * limit)) break;
+                // (failure testing, as in update_warp)
+                if (a.hold_step != 0u && a.hold_step - 1u < a.u_step0 + s + CH) break;
+                mbar_expect(&full[st], n * sb);
+                uint32_t dst = shared_addr(ring + st * CH * sb);
+                for (uint32_t j = 0; j < n; ++j, from += a.step_bytes, dst += sb) {
+                    copy_bulk_part(dst, from + (size_t)y0 * wc * 8u, bytes1, &full[st]);
+                    if (bytes2) copy_bulk_part(dst + bytes1, from, bytes2, &full[st]);
+                }
+            }
+            // no copy is on its way when the CTA goes on
+            for (uint32_t k = f > ST ? f - ST : 0u; k < f; ++k) (void)mbar_wait(&full[k % ST], k / ST & 1u, limit);
+        }
+        __syncwarp();
+    } else {
+        // (a thread past the last run repeats the last one's work)
+        const uint32_t c = min(tid, nthr - 1u), run = a.by_wc.quotient(c), w = c - run * wc;
+        const uint32_t groups = L / KW, hr = H / KW, rr = R / KW;
+        uint32_t group = (r0 + L - H) / KW + run;                      // the run's row group
+        while (group >= groups) group -= groups;
+        const bool own = run >= hr && run < hr + rr, mine = own && tid < nthr;
+        const uint32_t xl = c - w + (w == 0 ? wc - 1u : w - 1u), xr = c - w + (w + 1u == wc ? 0u : w + 1u);
+        const uint32_t xu = (KW - 1) * T + (run == 0 ? nthr - wc + w : c - wc);
+        const uint32_t xd = c + wc >= nthr ? w : c + wc;
+        uint32_t v[2][KW];
+        load_run<KW>(a.src + (size_t)(group * KW) * wc + w, wc, v);
+#pragma unroll
+        for (int k = 0; k < KW; ++k) {
+            X[k * T + c] = v[0][k];
+            X[(KW + k) * T + c] = v[1][k];
+        }
+        // where this run's rows go in the peers' inboxes, and come from in this one's
+        const uint32_t up_rank = rank == 0 ? ranks - 1u : rank - 1u, dn_rank = rank + 1u == ranks ? 0u : rank + 1u;
+        const bool to_up = mine && run < 2u * hr, to_dn = mine && run >= rr;
+        const uint32_t put_up = peer_addr(shared_addr(inbox + run * wc + w), up_rank), bar_up = peer_addr(shared_addr(inbox_bar), up_rank);
+        const uint32_t put_dn = peer_addr(shared_addr(inbox + (to_dn ? run - rr : 0u) * wc + w), dn_rank),
+                       bar_dn = peer_addr(shared_addr(inbox_bar), dn_rank);
+        const uint32_t take = (run < hr ? run : run >= rr ? run - rr : 0u) * wc + w;
+        // no peer writes here before the barriers are ready; every peer has loaded its rows
+        cluster_sync();
+
+        // after a wait for masks has run out the others hardly wait; rows of peers always
+        // come, if late
+        uint32_t patience = limit;
+        bool good = true, received = true;
+        auto wait_masks = [&](uint64_t *bar, uint32_t parity) {
+            if (!mbar_wait(bar, parity, patience)) {
+                good = false;
+                patience = 1u;
+            }
+        };
+        // the masks of a chunk's steps, read while the threads gather at the barrier before it
+        uint4 m[CH][1];
+        const unsigned char *const mp = ring + c * 16u;
+        auto masks_of = [&](uint32_t stage) {
+            const unsigned char *p = mp + stage * (CH * sb);
+#pragma unroll
+            for (uint32_t j = 0; j < CH; ++j, p += sb) m[j][0] = *reinterpret_cast<const uint4 *>(p);
+        };
+        wait_masks(&full[0], 0u);
+        masks_of(0);
+        asm volatile("bar.sync 1, %0;" ::"r"(nbar) : "memory");
+        // steps for which this warp's rows are right after an exchange: a step spoils a
+        // row at either end of the tile
+        const uint32_t useful = __reduce_max_sync(0xFFFFFFFFu, (min(run, rows / KW - 1u - run) + 1u) * KW - 1u);
+        uint32_t phase = 0, exchanges = 0;                             // steps since the last exchange; exchanges
+        uint32_t st = 0, turn = 0;                                     // the chunk's stage and its parity
+        uint32_t until = a.record_every - a.u_phase;                   // sweeps to the next recorded one (0: none)
+        uint32_t *snap = a.u_snaps + (size_t)(group * wc + w) * (2 * KW);
+        if (tid == 0 && a.u_steps > H) mbar_expect(&inbox_bar[0], inbox_bytes);
+        auto step = [&](auto parity, const uint4 (&mj)[1]) {
+            constexpr int P = decltype(parity)::value;
+            const uint32_t *const B = X + (1 - P) * KW * T;
+            uint32_t hz[KW];
+#pragma unroll
+            for (int k = 0; k < KW; ++k) hz[k] = B[k * T + (((k + P) & 1) ? xr : xl)];
+            const uint32_t up = B[xu], dn = B[xd];
+            step_run<KW, P>(v, hz, up, dn, mj);
+#pragma unroll
+            for (int k = 0; k < KW; ++k) X[(P * KW + k) * T + c] = v[P][k];
+        };
+        auto record = [&]() {
+            if (mine) store_snapshot<KW>(snap, v);
+            snap += 2 * a.nwords;
+        };
+        for (uint32_t left = a.u_steps;;) {
+            // a chunk is 4 steps, the last one 2 or 4
+            const bool active = phase < useful;
+            if (active) step(Parity<0>{}, m[0]);
+            asm volatile("bar.sync 1, %0;" ::"r"(nbar) : "memory");
+            if (active) step(Parity<1>{}, m[1]);
+            if (--until == 0u) {
+                record();
+                until = a.record_every;
+            }
+            if (left <= 2u) break;
+            asm volatile("bar.sync 1, %0;" ::"r"(nbar) : "memory");
+            if (active) step(Parity<0>{}, m[2]);
+            asm volatile("bar.sync 1, %0;" ::"r"(nbar) : "memory");
+            if (active) step(Parity<1>{}, m[3]);
+            if (--until == 0u) {
+                record();
+                until = a.record_every;
+            }
+            if (left <= 4u) break;
+            left -= CH;
+            phase += CH;
+            uint32_t next_st = st + 1u;
+            if (next_st == ST) {
+                next_st = 0u;
+                turn ^= 1u;
+            }
+            if (phase == H) {
+                // exchange: boundary rows out, halo rows in
+                phase = 0u;
+                const uint32_t e = exchanges & 1u, off = e * inbox_bytes;
+                if (to_up) store_peer16(put_up + off, v[0][0], v[0][1], v[1][0], v[1][1], bar_up + e * 8u);
+                if (to_dn) store_peer16(put_dn + off, v[0][0], v[0][1], v[1][0], v[1][1], bar_dn + e * 8u);
+                // (the next exchange's bytes may come as soon as this one's have gone)
+                if (tid == 0 && received) mbar_expect(&inbox_bar[1u - e], inbox_bytes);
+                asm volatile("bar.sync 1, %0;" ::"r"(nbar) : "memory");
+                if (!own) {
+                    received = received && mbar_wait(&inbox_bar[e], exchanges >> 1 & 1u, 4 * limit);
+                    const uint4 q = inbox[e * (inbox_bytes / 16u) + take];
+                    v[0][0] = q.x;
+                    v[0][1] = q.y;
+                    v[1][0] = q.z;
+                    v[1][1] = q.w;
+#pragma unroll
+                    for (int k = 0; k < KW; ++k) {
+                        X[k * T + c] = v[0][k];
+                        X[(KW + k) * T + c] = v[1][k];
+                    }
+                }
+                ++exchanges;
+            }
+            wait_masks(&full[next_st], turn);
+            masks_of(next_st);
+            asm volatile("bar.sync 1, %0;" ::"r"(nbar) : "memory");
+            if (tid == 0) mbar_arrive(&empty[st]);
+            st = next_st;
+        }
+        if (a.u_slots > a.u_recs) record();                            // the state after the call
+        if (!(good && received) && a.err) atomicExch(a.err, 1u);
+        if (mine) store_run<KW>(a.dst + (size_t)(group * KW) * wc + w, wc, v);
+    }
+    cluster_sync();  // no peer writes into a CTA that has ended
+}
+
+// The launches of a call take turns: draws of block b and counts of block b - 2, and the
+// update of block b.  The update starts when the draws have ended; it lets the next draws
+// start at once, which need not wait for it: what they write was read, and what they
+// count was written, by launches that ended before the update began.  One CTA of the draws
+// stays until the update before has ended, for the next update, which waits for the
+// draws alone.
+__global__ void __launch_bounds__(kThreads, 1) k_ahead_draw(const __grid_constant__ AheadArgs a)
+{
+    if (a.c_wait != 0u) dependent_launch_wait();  // the call's last counts, or its first draws
+    dependent_launch_trigger();
+    if (blockIdx.x < a.count_ctas) count_role<2>(a, blockIdx.x);
+    if (a.d_tickets != 0u) draw_role<false, false>(a);
+    if (blockIdx.x + 1u == gridDim.x) {
+        dependent_launch_wait();
+        if (threadIdx.x == 0) *a.next_ticket = 0u;
+    }
+}
+
+__global__ void __launch_bounds__(kClusterThreads + 32, 1) k_ahead_cluster(const __grid_constant__ AheadArgs a)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    dependent_launch_wait();
+    dependent_launch_trigger();
+    update_cluster(a, smem);
+}
+
 // Large lattices: a launch draws the masks of a band of rows (and of the rows that the
 // band's tiles spoil) for a block of sweeps and updates the band before from one copy of
 // the lattice to the other.
@@ -1035,7 +1296,7 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
 
 bool ahead_ready(ising_lattice *h, const AheadPlan &pl, uint64_t L)
 {
-    const size_t need = kTicketBytes + kBuffers * pl.mask_bytes + 2 * pl.snap_bytes + (pl.halo ? (size_t)(L * L / 8) : 0);
+    const size_t need = kTicketBytes + kBuffers * pl.mask_bytes + 2 * pl.snap_bytes + (pl.halo && !pl.cluster ? (size_t)(L * L / 8) : 0);
     if (h->ahead_bytes >= need) return true;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
@@ -1122,6 +1383,146 @@ static cudaError_t band_sweeps(const AheadPlan &pl, AheadArgs a, char *masks, un
     return e;
 }
 
+static uint32_t cluster_threads(const AheadPlan &p, uint32_t wc) { return (((p.tile_rows + 2 * p.halo) / 2 * wc + 31u) & ~31u) + 32u; }
+static uint32_t cluster_smem_of(const AheadPlan &p, uint32_t wc) { return cluster_smem(p.tile_rows + 2 * p.halo, p.halo, wc, p.stages); }
+
+// Whether this GPU (a partition may not) has room for a cluster of the plan.
+static bool cluster_fits(const AheadPlan &pl, uint32_t wc)
+{
+    static std::atomic<signed char> known[kMaxDevices][17];  // by device, CTAs
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+    std::atomic<signed char> &fits = known[dev][pl.tiles];
+    if (fits.load(std::memory_order_acquire) == 0) {
+        const AheadKernel kern = k_ahead_cluster;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(pl.tiles);
+        cfg.blockDim = dim3(cluster_threads(pl, wc));
+        cfg.dynamicSmemBytes = cluster_smem_of(pl, wc);
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = pl.tiles;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) == cudaSuccess &&
+                        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n >= 1;
+        if (!ok) cudaGetLastError();
+        fits.store(ok ? 1 : -1, std::memory_order_release);
+    }
+    return fits.load(std::memory_order_acquire) > 0;
+}
+
+// Calls of 192 sweeps and more: the first block's draws overlap nothing and the blocks
+// start short, so that calls of 64 and 128 take 72 and 100 us at 512 and with tiles
+// 65 and 93.
+AheadPlan cluster_plan(uint64_t L, uint64_t nsweeps)
+{
+    AheadPlan p{};
+    if (L % 64 != 0 || L < 320 || L > 512 || nsweeps < 192) return p;
+    const uint32_t wc = (uint32_t)(L / 64);
+    p.cluster = true;
+    p.kw = 2;
+    p.tile_rows = 32;
+    p.halo = 16;
+    p.tiles = p.update_ctas = (uint32_t)(L / p.tile_rows);
+    p.stages = kClusterStages;
+    p.block_sweeps = 256;
+    p.min_sweeps = 192;
+    p.step_bytes = (uint32_t)(L * wc * 8);
+    p.mask_bytes = (size_t)2 * p.block_sweeps * p.step_bytes;
+    p.snap_bytes = (size_t)p.block_sweeps * L * wc * 8;
+    if (!cluster_fits(p, wc)) p.kw = 0;
+    return p;
+}
+
+// The launches of the cluster form (k_ahead_draw and k_ahead_cluster in turn).
+static cudaError_t cluster_sweeps(const AheadPlan &pl, AheadArgs a, char *masks, char *snaps, unsigned int *tickets, uint64_t *spins,
+                                  uint64_t t0, uint64_t nsweeps, uint64_t full, cudaStream_t s)
+{
+    const AheadKernel kern = k_ahead_cluster, draw = k_ahead_draw;
+    int sms = 0;
+    cudaError_t e = prepare_device(draw, 18, &sms);
+    if (e != cudaSuccess) return e;
+    a.stages = pl.stages;
+    a.src = a.dst = spins;
+    a.update_ctas = pl.tiles;
+    cudaLaunchAttribute attr[2]{};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = pl.tiles;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t dc{}, uc{};
+    dc.blockDim = dim3(kThreads);
+    uc.gridDim = dim3(pl.tiles);
+    uc.blockDim = dim3(cluster_threads(pl, a.wc));
+    uc.dynamicSmemBytes = cluster_smem_of(pl, a.wc);
+    dc.stream = uc.stream = s;
+    dc.attrs = uc.attrs = attr;
+    uc.numAttrs = 2;
+    // Blocks start short, since nothing overlaps the first one's draws, and with the rest of
+    // a division by 4 (items of 4 sweeps are the cheapest to draw).
+    uint64_t left = nsweeps, done = 0, rec_done = 0, grow = std::min<uint64_t>(full, 32);
+    struct Counted {
+        uint32_t slots = 0, recs = 0, slot0 = 0, last = 0;
+        const uint32_t *snaps = nullptr;
+    } counted[2];  // of the blocks before
+    const uint32_t re = a.record_every, per = (a.nwords / pl.kw + 31u) & ~31u;
+    for (uint64_t b = 0;; ++b) {
+        uint64_t n = std::min(left, grow);
+        if (left % 4 && n < left && n > 4) n -= 4 - left % 4;
+        grow = std::min<uint64_t>(full, 2 * grow);
+        left -= n;
+        const Counted c = counted[0];
+        if (n == 0 && c.slots == 0) {
+            if (counted[1].slots == 0) return cudaSuccess;
+            counted[0] = counted[1];
+            counted[1] = Counted{};
+            continue;
+        }
+        a.c_slots = c.slots;
+        a.c_recs = c.recs;
+        a.c_slot0 = c.slot0;
+        a.c_last = c.last;
+        a.c_snaps = c.snaps;
+        a.c_wait = n == 0;
+        a.count_ctas = std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, 64u);  // (fewer than SMs)
+        a.d_t0 = (uint32_t)(t0 + done);
+        a.d_sweeps = (uint32_t)n;
+        a.d_masks = masks + (b % 2) * pl.mask_bytes;
+        a.d_ticket = tickets + b % 4;
+        a.next_ticket = tickets + (b + 2) % 4;
+        a.d_k = n % 4 == 0 ? 4 : n % 2 == 0 ? 2 : 1;
+        a.d_tickets = a.d_sweeps / a.d_k * 2u * (a.nwords / 32u);
+        dc.gridDim = dim3(std::max(1u, std::min<uint32_t>((uint32_t)sms, a.count_ctas + (a.d_tickets + kThreads / 32u - 1) / (kThreads / 32u))));
+        dc.numAttrs = b > 0 ? 1 : 0;
+        if ((e = cudaLaunchKernelEx(&dc, draw, a)) != cudaSuccess) return e;
+        counted[0] = counted[1];
+        counted[1] = Counted{};
+        if (n == 0) continue;
+        const uint64_t t = t0 + done;
+        a.u_steps = (uint32_t)(2 * n);
+        a.u_step0 = (uint32_t)(2 * done);
+        a.u_masks = a.d_masks;
+        a.u_snaps = reinterpret_cast<uint32_t *>(snaps + (b % 2) * pl.snap_bytes);
+        a.u_phase = re ? (uint32_t)(t % re) : 0u;
+        a.u_recs = re ? (uint32_t)((t + n) / re - t / re) : 0u;
+        a.u_last = left == 0;
+        a.u_slots = a.u_recs + ((a.u_last && !(re && (t + n) % re == 0)) ? 1u : 0u);
+        counted[1].slots = a.u_slots;
+        counted[1].recs = a.u_recs;
+        counted[1].slot0 = (uint32_t)rec_done;
+        counted[1].last = a.u_last;
+        counted[1].snaps = a.u_snaps;
+        if ((e = cudaLaunchKernelEx(&uc, kern, a)) != cudaSuccess) return e;
+        done += n;
+        rec_done += a.u_recs;
+    }
+}
+
 cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, uint64_t L, uint64_t t0, uint64_t nsweeps, uint32_t record_every,
                          uint64_t nrec, unsigned int *err, uint32_t hold_step, uint64_t max_block)
 {
@@ -1152,6 +1553,10 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     a.final_acc = h->d_acc + 2 * nrec;
     a.err = err;
     a.hold_step = hold_step;
+    if (pl.cluster) {
+        const cudaError_t e = cudaMemsetAsync(tickets, 0, kTicketBytes, h->stream);
+        return e != cudaSuccess ? e : cluster_sweeps(pl, a, masks, snaps, tickets, spins, t0, nsweeps, full, h->stream);
+    }
     if (pl.band_rows) {
         const cudaError_t e = cudaMemsetAsync(tickets, 0, kTicketBytes, h->stream);
         return e != cudaSuccess ? e : band_sweeps(pl, a, masks, tickets, spins, other, bytes, t0, nsweeps, full, h->stream);

@@ -17,6 +17,8 @@ struct AheadPlan {
     uint32_t tiles;
     uint32_t update_ctas;   // CTAs that share them
     bool warp;              // one warp holds the lattice
+    bool cluster;           // the CTAs of one cluster hold it
+    uint32_t stages;        // and have the masks of that many chunks of steps in shared memory
     bool field;             // in a field: five mask planes
     uint32_t band_rows;     // rows that a launch takes (0: all)
     uint32_t tile_words, tiles_x;  // words of a tile's rows and tiles of a row, where a launch takes a band
@@ -47,6 +49,7 @@ struct AheadArgs {
     uint32_t hold_step;           // failure testing: 1 + a step whose masks never arrive
     // update: u_steps steps (0: none) from src to dst
     uint32_t update_ctas, tiles, tile_rows, halo;
+    uint32_t stages;              // chunks of masks in shared memory (cluster form)
     uint32_t u_steps, u_step0;    // steps; index of the first in the call
     const uint64_t *src;
     uint64_t *dst;
@@ -61,6 +64,7 @@ struct AheadArgs {
     FastDiv by_tw;                // division by tile_words + 2
     // count: the snapshots of the block before
     uint32_t count_ctas, c_slots, c_recs, c_slot0, c_last;
+    uint32_t c_wait;              // they are those of the launch before
     const uint32_t *c_snaps;
     // draw: d_sweeps sweeps from sweep index d_t0, in tickets of 32 items of d_k sweeps
     uint32_t d_t0, d_sweeps, d_k, d_tickets;
@@ -70,6 +74,9 @@ struct AheadArgs {
 };
 
 AheadPlan ahead_plan(uint64_t L, bool field);
+// The cluster form, for the sizes and calls where it is the faster one (no field; kw 0: not
+// here).
+AheadPlan cluster_plan(uint64_t L, uint64_t nsweeps);
 
 // One lattice of a batch run (device table).
 struct AheadJob {

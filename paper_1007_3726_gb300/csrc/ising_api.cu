@@ -486,7 +486,8 @@ ising_status ising_sweep(ising_lattice *h, uint64_t nsweeps, uint32_t record_eve
         const uint64_t v = std::strtoull(max_env, nullptr, 10);
         if (v > 0 && v < max_chunk) max_chunk = v;
     }
-    const AheadPlan pl = h->ahead ? ahead_plan(h->L, h->H != 0.0) : AheadPlan{};
+    AheadPlan pl = h->ahead && h->H == 0.0 ? cluster_plan(h->L, nsweeps) : AheadPlan{};
+    if (pl.kw == 0 || !ahead_ready(h, pl, h->L)) pl = h->ahead ? ahead_plan(h->L, h->H != 0.0) : AheadPlan{};
     if (pl.kw != 0 && nsweeps >= pl.min_sweeps && ahead_ready(h, pl, h->L)) {
         CK(h, ahead_sweeps(h, pl, h->d_spins, h->L, t0, nsweeps, record_every, nrec, err, hold_step, max_chunk));
         h->pending_err = true;

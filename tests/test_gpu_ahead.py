@@ -36,12 +36,12 @@ def _compare(orc, lat, s, t, n, rec, seed, sid, thr):
 # remainder of 4, sample spacings that cross the calls, none
 SMALL = ((200, 1), (203, 3), (321, 0), (514, 7))
 MIDDLE = ((10, 1), (33, 3), (64, 0), (71, 7))
-LONG = MIDDLE + ((130, 1), (203, 3))
+LONG = MIDDLE + ((130, 1), (203, 3), (514, 1), (193, 0))
 LARGE = ((10, 1), (12, 3), (18, 0), (23, 1), (33, 5))
 
 
-@pytest.mark.parametrize("L,calls", [(64, SMALL), (128, SMALL), (192, SMALL + MIDDLE), (256, LONG), (320, LONG),
-                                     (448, LONG), (512, LONG), (704, LONG), (960, LONG), (1024, LONG),
+@pytest.mark.parametrize("L,calls", [(64, SMALL), (128, SMALL), (192, SMALL + MIDDLE), (256, MIDDLE), (320, LONG),
+                                     (384, LONG), (448, LONG), (512, LONG), (704, MIDDLE), (960, MIDDLE), (1024, MIDDLE),
                                      (1088, MIDDLE), (2048, LARGE), (2112, LARGE), (4096, LARGE), (4160, LARGE),
                                      (8192, ((10, 1), (13, 2))), (8256, ((4, 1), (11, 2))), (9984, ((9, 1), (8, 0))),
                                      (16384, ((7, 3), (4, 1)))])
@@ -118,11 +118,12 @@ def test_late_sweep_indices_and_high_stream(P, orc):
     lat.close()
 
 
-@pytest.mark.parametrize("hold", [6, 390, 400])
-def test_masks_that_never_arrive_are_reported(P, monkeypatch, hold):
-    """L = 64 waits for masks on their way: a step whose masks never arrive ends the
-    wait, the call reports ISING_ERR_TIMEOUT and the GPU stays usable."""
-    lat = P.Lattice(64, 2.0, seed=1, init="hot")
+@pytest.mark.parametrize("L,hold", [(64, 6), (64, 390), (64, 400), (448, 6), (512, 390), (512, 400)])
+def test_masks_that_never_arrive_are_reported(P, monkeypatch, L, hold):
+    """L = 64 and the clusters (L = 320 .. 512) wait for masks on their way: a step whose
+    masks never arrive ends the wait, the call reports ISING_ERR_TIMEOUT and the GPU stays
+    usable."""
+    lat = P.Lattice(L, 2.0, seed=1, init="hot")
     monkeypatch.setenv("ISING_TINY_HOLD_STEP", str(hold))
     with pytest.raises(P.IsingError) as ei:
         lat.sweep(200, 1, collect=True)
@@ -132,7 +133,7 @@ def test_masks_that_never_arrive_are_reported(P, monkeypatch, hold):
         lat.sweep(1, 1)
     assert ei.value.status == P.ERR_STATE
     lat.close()
-    ok = P.Lattice(64, 2.0, seed=1, init="hot")
+    ok = P.Lattice(L, 2.0, seed=1, init="hot")
     ok.sweep(200, 1)
     assert ok.measure()["sweeps_done"] == 200
     ok.close()
