@@ -263,17 +263,20 @@ ISING_API const char *ising_last_error(void);
  *
  * The draw-ahead form.  A handle whose configuration was not set runs calls of
  * enough sweeps (200 at L = 64, 100 at 128, 10 at 256, 3 below 1024, 5 below 2048, 10
- * up to 8192, 4 above; in a field, up to L = 4096, 1 to 5) in another form: the
- * acceptance masks of a block of sweeps are drawn by the whole GPU one launch before
- * the tiles of the lattice are updated with them.  It needs scratch memory (three
- * buffers of masks, a second lattice: 4 MB at L = 512, 103 MB at 4096, 210 MB at 8192,
- * above 210 to 810 MB and the size of the lattice), which the handle allocates on its
- * first such call and keeps.  Where the allocator refuses, or more than 1 GiB and half
- * of the free memory were needed, or while the stream is captured, the configuration's
- * form runs.  Results are the same.
+ * up to 8192, 4 above; in a field 1 to 5 up to L = 4096, 4 above) in
+ * another form: the acceptance masks of a block of sweeps are drawn by the whole GPU
+ * one launch before the tiles of the lattice are updated with them (L = 320 .. 512, 192
+ * sweeps and more: tiles that are the CTAs of one thread-block cluster).  It needs
+ * scratch memory (buffers of masks, a second lattice: 4 MB at L = 512, in the cluster
+ * 25 MB; 103 MB at 4096, 210 MB at 8192, above 210 to 810 MB, in a field up to 2 GB, and
+ * the size of the lattice), which the handle allocates on its first such call and
+ * keeps.  Where the allocator refuses, or more than 1 GiB and half of the free memory
+ * were needed, or while the stream is captured before the scratch is there, the
+ * configuration's form runs.  Results are the same.
  * ising_set_launch switches it off for the handle.  (ISING_TINY_HOLD_STEP and
- * ISING_TINY_MAX_SWEEPS, for tests only, also act here: the former at L = 64, where
- * one warp waits for masks on their way, the latter as the longest block.)
+ * ISING_TINY_MAX_SWEEPS, for tests only, also act here: the former where an update waits
+ * for masks on their way, at L = 64 and in the cluster, the latter as the longest
+ * block.)
  */
 typedef struct {
     uint32_t proc_bits, regcap, block, rows_per_item, grid, insert;

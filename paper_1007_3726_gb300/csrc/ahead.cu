@@ -16,13 +16,14 @@
 // synchronisation between CTAs.
 //
 // Bound: draws at 1.75 per ns on the whole GPU (below); where the lattice is small,
-// the chain of steps of a tile (80 ns a step at L = 64, 110 .. 220 ns above) and 2 to
+// the chain of steps of a tile (62 ns a step at L = 64, 110 .. 220 ns above) and 2 to
 // 3 us per launch.  Measured, one call, before (step launches or one-launch forms)
-// and with this form: L = 64, 1000 sweeps 239 -> 179 us; 256, 1000: 1072 -> 342;
-// 320, 500: 2996 -> 299; 512, 1000: 4887 -> 470; 1024, 500: 2766 -> 443; 2048, 200:
-// 1446 -> 606; 4096, 200: 3548 -> 2332 (1.44 attempts per ns of 0.95).  Persistent
-// CTAs that wait for one another on flags instead of launches were no faster (a
-// block's hand-over costs them 3.4 us).
+// and with this form: L = 64, 1000 sweeps 239 -> 170 us; 256, 1000: 1072 -> 316;
+// 320, 500: 2985 -> 221; 512, 1000: 4885 -> 376; 1024, 500: 2850 -> 460; 2048, 200:
+// 1446 -> 606; 4096, 200: 3546 -> 2193 (1.53 attempts per ns of 0.95); 65536, 4: 12449 ->
+// 11120 (1.54 of 1.38).  Persistent CTAs that wait for one another on flags instead
+// of launches were no faster (a block's hand-over costs them 3.4 us); CTAs of one
+// cluster are, where they can hold the lattice.
 //
 // Layout of a tile: the two checkerboard colours of a row are kept apart, 32
 // sites of one colour per word, so that a step works on full words: bit k of
@@ -48,7 +49,8 @@ namespace {
 
 // Steps whose masks an update thread holds or has on the way: their latency (about
 // a microsecond with the L2 busy) against the time of a step, within 160 KiB.
-__host__ __device__ constexpr uint32_t stages_of(uint32_t kw, bool field) { return kw == 8 ? 2 : (field && kw == 4) ? 4 : 8; }
+// (two CTAs a SM: 98 KiB).
+__host__ __device__ constexpr uint32_t stages_of(uint32_t kw, bool field, bool two) { return two ? 2 : (field && kw == 4) ? 4 : 8; }
 
 // Threads per CTA.  One lattice: one CTA per SM, so that an update, which the next
 // launch waits for, has an SM to itself.  Several lattices: two CTAs per SM, so that
@@ -58,7 +60,7 @@ constexpr uint32_t kThreads = 512, kBatchThreads = 256;
 constexpr uint32_t kChunk = 8;     // steps of a stage of the one-warp form
 constexpr uint32_t kWarpStages = 8;
 constexpr uint32_t kClusterThreads = 256, kClusterChunk = 4, kClusterStages = 8;  // of the cluster form: update threads, steps of a stage, stages
-constexpr uint32_t kBuffers = 3;   // mask buffers, used in turn
+constexpr uint32_t kBuffers = 3, kClusterBuffers = 2;  // mask buffers, used in turn
 constexpr uint32_t kWaitLimit = 1u << 22;  // polls of a wait for masks on their way into shared memory
 
 template <int V>
@@ -184,7 +186,7 @@ __device__ __forceinline__ void draw_item(const A &a, char *masks, size_t step_b
 
 // The warps of the launch take tickets for 32 items each (consecutive words of
 // one colour and group of sweeps: nwords is a multiple of 64).
-template <bool FIELD, bool BAND>
+template <bool FIELD, bool BAND, bool TWO>
 __device__ __forceinline__ void draw_role(const AheadArgs &a)
 {
     const uint32_t lane = threadIdx.x & 31u, per_group = BAND ? (a.d_words + 31u) / 32u : a.nwords / 32u;
@@ -197,7 +199,7 @@ __device__ __forceinline__ void draw_role(const AheadArgs &a)
         const uint32_t gp = a.by_group.quotient(it);
         uint32_t idx = (it - gp * per_group) * 32u + lane;
         if constexpr (BAND) idx = min(idx, a.d_words - 1u);  // (the last ticket of a group repeats its last word)
-        if (a.d_k == 4u)
+        if (!(FIELD && TWO) && a.d_k == 4u)
             draw_item<FIELD, 4, BAND>(a, a.d_masks, step_bytes, a.d_t0, gp & 1u, (gp >> 1) * 4u, idx);
         else if (a.d_k == 2u)
             draw_item<FIELD, 2, BAND>(a, a.d_masks, step_bytes, a.d_t0, gp & 1u, (gp >> 1) * 2u, idx);
@@ -392,10 +394,10 @@ __device__ __forceinline__ void store_snapshot(const AheadArgs &a, uint32_t slot
 // the tile counts its own rows.
 // BAND: the tile is one of a band of rows and holds tile_words words of a row, and one
 // on either side, whose sites of the colour spoil from the far end, one a step.
-template <uint32_t THREADS, int KW, bool FIELD, bool SNAPS, bool BAND>
+template <uint32_t THREADS, int KW, bool FIELD, bool SNAPS, bool BAND, bool TWO>
 __device__ __forceinline__ void update_tile(const AheadArgs &a, uint32_t tile, unsigned char *smem)
 {
-    constexpr uint32_t ST = stages_of(KW, FIELD);
+    constexpr uint32_t ST = stages_of(KW, FIELD, TWO);
     constexpr uint32_t NQ = FIELD ? KW : KW / 2;                  // 16-byte mask units of a run and step
     const uint32_t tid = threadIdx.x, wc = a.wc, L = a.L;
     const uint32_t tw = BAND ? a.tile_words + 2u : wc;            // words of a row of the tile
@@ -687,8 +689,9 @@ __device__ __forceinline__ void count_role(const AheadArgs &a, uint32_t cta)
     }
 }
 
-template <int KW, bool WARP, bool FIELD>
-__global__ void __launch_bounds__(kThreads, KW == 8 ? 2 : 1) k_ahead(const __grid_constant__ AheadArgs a)
+// TWO: two CTAs share a SM (8 rows a thread, and 4 in a field).
+template <int KW, bool WARP, bool FIELD, bool TWO>
+__global__ void __launch_bounds__(kThreads, TWO ? 2 : 1) k_ahead(const __grid_constant__ AheadArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     // The first launch of a call (it only draws) starts after all work before it.
@@ -703,11 +706,11 @@ __global__ void __launch_bounds__(kThreads, KW == 8 ? 2 : 1) k_ahead(const __gri
         if constexpr (WARP)
             update_warp(a, smem);
         else
-            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, KW, FIELD, true, false>(a, t, smem);
+            for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, KW, FIELD, true, false, TWO>(a, t, smem);
     } else if (blockIdx.x < early) {
         count_role<KW>(a, blockIdx.x - a.update_ctas);
     }
-    if (a.d_tickets != 0u) draw_role<FIELD, false>(a);
+    if (a.d_tickets != 0u) draw_role<FIELD, false, TWO>(a);
 }
 
 // --------------------------------------------------------------- cluster --
@@ -955,7 +958,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ahead_draw(const __grid_constan
     if (a.c_wait != 0u) dependent_launch_wait();  // the call's last counts, or its first draws
     dependent_launch_trigger();
     if (blockIdx.x < a.count_ctas) count_role<2>(a, blockIdx.x);
-    if (a.d_tickets != 0u) draw_role<false, false>(a);
+    if (a.d_tickets != 0u) draw_role<false, false, false>(a);
     if (blockIdx.x + 1u == gridDim.x) {
         dependent_launch_wait();
         if (threadIdx.x == 0) *a.next_ticket = 0u;
@@ -974,7 +977,7 @@ __global__ void __launch_bounds__(kClusterThreads + 32, 1) k_ahead_cluster(const
 // band's tiles spoil) for a block of sweeps and updates the band before from one copy of
 // the lattice to the other.
 template <bool FIELD>
-__global__ void __launch_bounds__(kThreads, FIELD ? 1 : 2) k_ahead_band(const __grid_constant__ AheadArgs a)
+__global__ void __launch_bounds__(kThreads, 2) k_ahead_band(const __grid_constant__ AheadArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     // (waits as in k_ahead)
@@ -982,9 +985,9 @@ __global__ void __launch_bounds__(kThreads, FIELD ? 1 : 2) k_ahead_band(const __
     dependent_launch_trigger();
     if (blockIdx.x < a.update_ctas) {
         if (blockIdx.x == 0 && threadIdx.x == 0) *a.next_ticket = 0u;
-        for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, FIELD ? 4 : 8, FIELD, false, true>(a, t, smem);
+        for (uint32_t t = blockIdx.x; t < a.tiles; t += a.update_ctas) update_tile<kThreads, FIELD ? 4 : 8, FIELD, false, true, true>(a, t, smem);
     }
-    if (a.d_tickets != 0u) draw_role<FIELD, true>(a);
+    if (a.d_tickets != 0u) draw_role<FIELD, true, true>(a);
 }
 
 // ----------------------------------------------------------------- batch --
@@ -1091,15 +1094,15 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_ahead_batch(const __grid_c
             const uint32_t tile = g - j.tile_start;
             if (!j.field) {
                 if (j.kw == 2)
-                    update_tile<kBatchThreads, 2, false, false, false>(t, tile, smem);
+                    update_tile<kBatchThreads, 2, false, false, false, false>(t, tile, smem);
                 else if (j.kw == 4)
-                    update_tile<kBatchThreads, 4, false, false, false>(t, tile, smem);
+                    update_tile<kBatchThreads, 4, false, false, false, false>(t, tile, smem);
                 else
-                    update_tile<kBatchThreads, 8, false, false, false>(t, tile, smem);
+                    update_tile<kBatchThreads, 8, false, false, false, true>(t, tile, smem);
             } else if (j.kw == 2) {
-                update_tile<kBatchThreads, 2, true, false, false>(t, tile, smem);
+                update_tile<kBatchThreads, 2, true, false, false, false>(t, tile, smem);
             } else {
-                update_tile<kBatchThreads, 4, true, false, false>(t, tile, smem);
+                update_tile<kBatchThreads, 4, true, false, false, false>(t, tile, smem);
             }
         }
     }
@@ -1111,9 +1114,16 @@ using AheadKernel = void (*)(AheadArgs);
 AheadKernel pick_kernel(const AheadPlan &p)
 {
     if (p.band_rows) return p.field ? k_ahead_band<true> : k_ahead_band<false>;
-    if (p.field) return p.kw == 2 ? k_ahead<2, false, true> : p.kw == 4 ? k_ahead<4, false, true> : nullptr;
-    if (p.warp) return k_ahead<2, true, false>;
-    return p.kw == 2 ? k_ahead<2, false, false> : p.kw == 4 ? k_ahead<4, false, false> : p.kw == 8 ? k_ahead<8, false, false> : nullptr;
+    if (p.field)
+        return p.kw == 2 ? k_ahead<2, false, true, false>
+               : p.kw != 4 ? nullptr
+               : p.two     ? k_ahead<4, false, true, true>
+                           : k_ahead<4, false, true, false>;
+    if (p.warp) return k_ahead<2, true, false, false>;
+    return p.kw == 2   ? k_ahead<2, false, false, false>
+           : p.kw == 4 ? k_ahead<4, false, false, false>
+           : p.kw == 8 ? k_ahead<8, false, false, true>
+                       : nullptr;
 }
 
 constexpr int kMaxDevices = 64;
@@ -1167,17 +1177,18 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 // Above 8192 tiles are parts of rows and a launch takes a band of rows: the masks of
 // all would be 64 times the lattice a block.  Measured against the step kernels (two
 // launches a sweep): L = 65536, 4 sweeps 12252 -> 11083 us (1.55 attempts per ns), 8 sweeps
-// 24481 -> 21766; 16384, 40 sweeps 8510 -> 6808; 8256, 40 sweeps 2456 -> 1804; in a field
-// (five compares a draw instead of two: the draws are the more of the work) 65536, 8 sweeps
-// 38787 -> 36216; 16384, 40 sweeps 12538 -> 11360; 8256, 40 sweeps 3769 -> 3256, but 6 sweeps
-// 596 and 615.  Two CTAs of the largest tiles share a SM, and with draws (L = 2048,
-// 200 sweeps: 606 us with one, 585 with two; 4096 2225 and 2137; 8192, 40 sweeps 1848
-// and 1748).  In a field (20 bytes of masks a word and step instead of 8) the bands
-// start above 4096, for tiles of half the words.  Measured, 200 sweeps
-// with M/E every sweep, the field step kernel (L = 64 .. 512: the one-launch field
-// kernels) against this form: L = 64 547 -> 102 us, 512 1384 -> 251, 704 5568 -> 357,
-// 2048 5593 -> 991; 20 sweeps of 4096 689 -> 425.  min_sweeps: a call has one launch more than
-// it has blocks, and the one-launch forms (L = 64, 128, 256) and two step launches
+// 24481 -> 21766; 16384, 40 sweeps 8510 -> 6808; 8256, 40 sweeps 2456 -> 1804.  Two CTAs
+// of the largest tiles share a SM, and with draws (L = 2048, 200 sweeps: 606 us with
+// one, 585 with two; 4096 2225 and 2137; 8192, 40 sweeps 1848 and 1748).  In a field (20
+// bytes of masks a word and step instead of 8) the bands start above 4096, for tiles of
+// half the words.  Measured with M/E every sweep, the field step kernel (L = 64 .. 512:
+// the one-launch field kernels) against this form: 200 sweeps of L = 64 547 -> 102 us, 512
+// 1384 -> 249, 704 5568 -> 347, 2048 5593 -> 922, 20 of 4096 689 -> 335, 40 of 8256 3769 ->
+// 2620, 8 of 32768 9718 -> 7849.  There too two CTAs share a SM above L = 1024 (with one,
+// and items of 4 sweeps: 2048 1018, 4096 200 sweeps 3745 and 3225, 32768 9119; below, where
+// the chain of steps counts, one CTA is faster: 1024 567 and 622).  min_sweeps: a call
+// has one launch more than it has blocks, and the one-launch forms (L = 64, 128, 256) and
+// two step launches
 // per sweep (above) are as fast on shorter calls.
 AheadPlan ahead_plan(uint64_t L, bool field)
 {
@@ -1188,13 +1199,14 @@ AheadPlan ahead_plan(uint64_t L, bool field)
     if (L > (field ? 4096 : 8192)) {
         // tiles of 64 rows (80 with the halo of a block of 4 sweeps, 10 runs of 8; in a field
         // 32 rows, 12 runs of 4) and as many words as fill 512 threads with two more, in
-        // equal parts of a row; bands
-        // of about 2^20 words, at least 512 rows (16 more are drawn twice)
+        // equal parts of a row; bands of about 2^20 words, at least 512 rows (16 more are
+        // drawn twice)
         p.kw = field ? 4 : 8;
+        p.two = true;
         p.tile_rows = field ? 32 : 64;
         p.halo = 8;
         p.block_sweeps = 4;
-        p.min_sweeps = field && L < 16384 ? 12 : 4;
+        p.min_sweeps = 4;
         const uint32_t words = kThreads / ((p.tile_rows + 2 * p.halo) / p.kw) - 2;
         p.tiles_x = (wc + words - 1) / words;
         p.tile_words = (wc + p.tiles_x - 1) / p.tiles_x;
@@ -1218,13 +1230,14 @@ AheadPlan ahead_plan(uint64_t L, bool field)
                          : L == 64 ? 200 : L == 128 ? 100 : L == 256 ? 10 : L < 1024 ? 3 : L < 2048 ? 5 : 10;
     const uint32_t rows = p.tile_rows + 2 * p.halo, most = p.halo ? kThreads : kThreads / 2;
     for (p.kw = 2; rows / p.kw * wc > most;) p.kw *= 2;
+    p.two = p.kw == 8 || (field && p.kw == 4 && L > 1024);
     p.warp = L == 64 && !field;
     p.tiles = (uint32_t)(L / p.tile_rows);
     // one tile a CTA, or several the same number each: of 66 tiles 2 on two CTAs take
     // twice as long as the others; 128 tiles (L = 4096) on 64 CTAs 2137 us, on 128 2228
     // (a CTA that updates draws nothing before the launch before has ended: fewer of
     // them where a CTA has an SM to itself)
-    const uint32_t most_ctas = p.kw == 8 ? 128 : 64;
+    const uint32_t most_ctas = p.two ? 128 : 64;
     const uint32_t each = p.tiles <= 96 ? 1 : std::max(2u, (p.tiles + most_ctas - 1) / most_ctas);
     p.update_ctas = (p.tiles + each - 1) / each;
     p.step_bytes = (uint32_t)(L * wc * (field ? 20 : 8));
@@ -1265,20 +1278,21 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
     const AheadKernel kern = pick_kernel(pl);
     if (!kern) return cudaErrorInvalidValue;
     int sms = 0;
-    cudaError_t e = prepare_device(kern, pl.band_rows ? 16 + pl.field : pl.warp ? 0 : pl.kw / 2 + (pl.field ? 8 : 0), &sms);
+    cudaError_t e = prepare_device(kern, pl.band_rows ? 16 + pl.field : pl.warp ? 0 : pl.kw / 2 + (pl.field ? 8 : 0) + (pl.field && pl.two ? 1 : 0), &sms);
     if (e != cudaSuccess) return e;
     if (pl.band_rows) a.nwords = (a.d_words + 31) / 32 * 32;  // for the tickets
-    a.update_ctas = !a.u_steps ? 0u : pl.band_rows ? std::min(a.tiles, pl.field ? 64u : (uint32_t)sms) : pl.update_ctas;
+    a.update_ctas = !a.u_steps ? 0u : pl.band_rows ? std::min(a.tiles, (uint32_t)sms) : pl.update_ctas;
     const uint32_t per = (a.nwords / pl.kw + 31u) & ~31u;
-    a.count_ctas = a.c_slots ? std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, pl.kw == 8 ? 64u : 16u) : 0u;
-    // 1756 attempts/ns in items of 4 sweeps, 1708 in items of 2, 1616 one by one
-    a.d_k = a.d_sweeps % 4 == 0 ? 4 : a.d_sweeps % 2 == 0 ? 2 : 1;
+    a.count_ctas = a.c_slots ? std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, pl.two ? 64u : 16u) : 0u;
+    // 1756 attempts/ns in items of 4 sweeps, 1708 in items of 2, 1616 one by one; the masks
+    // of 4 sweeps in a field do not fit the registers of two CTAs a SM
+    a.d_k = a.d_sweeps % 4 == 0 && !(pl.field && pl.two) ? 4 : a.d_sweeps % 2 == 0 ? 2 : 1;
     a.d_tickets = a.d_sweeps / a.d_k * 2u * (a.nwords / 32u);
     const uint32_t early = a.update_ctas + a.count_ctas, warps = kThreads / 32u;
-    const uint32_t grid = std::max(early, std::min<uint32_t>((uint32_t)sms * (pl.kw == 8 ? 2u : 1u), early + (a.d_tickets + warps - 1) / warps));
+    const uint32_t grid = std::max(early, std::min<uint32_t>((uint32_t)sms * (pl.two ? 2u : 1u), early + (a.d_tickets + warps - 1) / warps));
     const size_t smem = !a.u_steps ? 0
                         : pl.warp  ? kWarpStages * kChunk * 512
-                                   : (stages_of(pl.kw, pl.field) * (pl.field ? 20 : 8) + 8) * pl.kw * kThreads + (a.u_snaps ? 0 : (size_t)a.u_slots * 8);
+                                   : (stages_of(pl.kw, pl.field, pl.two) * (pl.field ? 20 : 8) + 8) * pl.kw * kThreads + (a.u_snaps ? 0 : (size_t)a.u_slots * 8);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kThreads);
@@ -1296,7 +1310,7 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
 
 bool ahead_ready(ising_lattice *h, const AheadPlan &pl, uint64_t L)
 {
-    const size_t need = kTicketBytes + kBuffers * pl.mask_bytes + 2 * pl.snap_bytes + (pl.halo && !pl.cluster ? (size_t)(L * L / 8) : 0);
+    const size_t need = kTicketBytes + (pl.cluster ? kClusterBuffers : kBuffers) * pl.mask_bytes + 2 * pl.snap_bytes + (pl.halo && !pl.cluster ? (size_t)(L * L / 8) : 0);
     if (h->ahead_bytes >= need) return true;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
@@ -1429,7 +1443,7 @@ AheadPlan cluster_plan(uint64_t L, uint64_t nsweeps)
     p.halo = 16;
     p.tiles = p.update_ctas = (uint32_t)(L / p.tile_rows);
     p.stages = kClusterStages;
-    p.block_sweeps = 256;
+    p.block_sweeps = 128;  // (256: 1 % faster at 512 with twice the scratch; 64: 8 % slower)
     p.min_sweeps = 192;
     p.step_bytes = (uint32_t)(L * wc * 8);
     p.mask_bytes = (size_t)2 * p.block_sweeps * p.step_bytes;
@@ -1492,7 +1506,7 @@ static cudaError_t cluster_sweeps(const AheadPlan &pl, AheadArgs a, char *masks,
         a.count_ctas = std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, 64u);  // (fewer than SMs)
         a.d_t0 = (uint32_t)(t0 + done);
         a.d_sweeps = (uint32_t)n;
-        a.d_masks = masks + (b % 2) * pl.mask_bytes;
+        a.d_masks = masks + (b % kClusterBuffers) * pl.mask_bytes;
         a.d_ticket = tickets + b % 4;
         a.next_ticket = tickets + (b + 2) % 4;
         a.d_k = n % 4 == 0 ? 4 : n % 2 == 0 ? 2 : 1;
@@ -1530,7 +1544,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     const size_t bytes = (size_t)(L * L / 8);
     unsigned int *const tickets = static_cast<unsigned int *>(h->d_ahead);
     char *const masks = static_cast<char *>(h->d_ahead) + kTicketBytes;
-    char *const snaps = masks + kBuffers * pl.mask_bytes;
+    char *const snaps = masks + (pl.cluster ? kClusterBuffers : kBuffers) * pl.mask_bytes;
     uint64_t *const spins = static_cast<uint64_t *>(lattice);
     uint64_t *const other = pl.halo ? reinterpret_cast<uint64_t *>(snaps + 2 * pl.snap_bytes) : spins;
     AheadArgs a{};
@@ -1717,7 +1731,7 @@ bool AheadBatch::plan(const std::vector<ising_lattice *> &hs, const std::vector<
         j.mask_bytes = (size_t)2 * j.block_sweeps * j.step_bytes;
         bytes += kBuffers * j.mask_bytes + (j.halo ? (size_t)j.nwords * 8 : 0);
         cnt_slots = std::max<size_t>(cnt_slots, j.block_sweeps + 1);
-        smem = std::max<size_t>(smem, (size_t)(stages_of(j.kw, j.field) * (j.field ? 20 : 8) + 8) * j.kw * kBatchThreads);
+        smem = std::max<size_t>(smem, (size_t)(stages_of(j.kw, j.field, j.kw == 8) * (j.field ? 20 : 8) + 8) * j.kw * kBatchThreads);
     }
     smem += cnt_slots * 8;
     std::stable_sort(jobs.begin(), jobs.end(), [](const AheadJob &x, const AheadJob &y) { return x.nblocks > y.nblocks; });

@@ -20,6 +20,7 @@ struct AheadPlan {
     bool cluster;           // the CTAs of one cluster hold it
     uint32_t stages;        // and have the masks of that many chunks of steps in shared memory
     bool field;             // in a field: five mask planes
+    bool two;               // two CTAs share a SM
     uint32_t band_rows;     // rows that a launch takes (0: all)
     uint32_t tile_words, tiles_x;  // words of a tile's rows and tiles of a row, where a launch takes a band
     uint32_t block_sweeps;  // sweeps of a block at most (halo / 2 where there is a halo)
