@@ -24,8 +24,8 @@ One JSON line on rank 0:
   e2e            the same through the C ABI from pinned host memory: each step
                  creates the lattice from the host copy (H2D), sweeps, reads
                  the M/E samples back (D2H) and destroys it
-  roofline       the dominant kernel (the half-sweep) against the integer-ALU
-                 bound (16 int32 ops per attempt at 128 lanes per SM per clock),
+  roofline       the dominant kernel (the band kernel of the draw-ahead form, or the
+                 half-sweep) against the integer-ALU bound (16 int32 ops per attempt at 128 lanes per SM per clock),
                  with the measured draw-generation rates beside it
   cpu_baseline   the oracle on this host's cores (all, and one) on a bounded
                  light-cone sample of the same lattice (rank 0, N = 1 only)
@@ -186,12 +186,12 @@ class ClockSampler:
 
 
 # ---------------------------------------------------------------- profiles --
-KERNEL_SOURCES = ("kernels.cu", "sweep_device.cuh")
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "half_sweep_traffic.json")
+KERNEL_SOURCES = ("ahead.cu", "ahead.h", "sweep_device.cuh")
+TRAFFIC_FILE = os.path.join(ROOT, "profiles", "ahead_band_traffic.json")
 
 
 def kernel_source_hash() -> str:
-    """sha256[:16] of the half-sweep kernel's sources, concatenated in order."""
+    """sha256[:16] of the band kernel's sources, concatenated in order."""
     h = hashlib.sha256()
     for name in KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_1007_3726_gb300", "csrc", name), "rb") as f:
@@ -200,8 +200,8 @@ def kernel_source_hash() -> str:
 
 
 def profiled_kernel():
-    """The committed ncu figures of the half-sweep (DRAM bytes per launch at the
-    captured size, thread instructions per attempt), if they were taken on the
+    """The committed ncu figures of the band kernel (DRAM bytes and thread
+    instructions per attempt at the captured size), if they were taken on the
     current kernel source; else None."""
     try:
         with open(TRAFFIC_FILE) as f:
@@ -211,6 +211,17 @@ def profiled_kernel():
     if d.get("kernel_sources_sha16") != kernel_source_hash():
         return None
     return d
+
+
+def launches_of_step(strips: bool, ahead: bool) -> int:
+    """Kernel launches of one step (a call of SWEEPS_PER_STEP sweeps).  Step kernels: two a
+    sweep.  The band form of the library (csrc/ahead.cu): blocks of 4 sweeps, the first
+    with the rest of the division, a launch per band of rows and block, and one more; a
+    band is 2^20 words of 32 sites, at least 512 rows."""
+    if strips or not ahead:
+        return 2 * SWEEPS_PER_STEP
+    bands = -(-L // max(512, 2 ** 20 // (L // 64) // 64 * 64))
+    return -(-SWEEPS_PER_STEP // 4) * bands + 1
 
 
 def measured_peaks():
@@ -483,9 +494,8 @@ def extras(P, stream, peaks, mix):
     timed_sweeps(P, lat, stream, 20)
     t = timed_sweeps(P, lat, stream, w["sweeps"], reps=2)
     rate = w["L"] ** 2 * w["sweeps"] / t / 1e9
-    mean_launch = t / (2 * w["sweeps"])
     out["L32768_1000_sweeps"] = {
-        "attempts_per_ns": rate, "launch": cfg, "mean_launch_us": mean_launch * 1e6,
+        "attempts_per_ns": rate, "launch": cfg, "us_per_half_sweep": t / (2 * w["sweeps"]) * 1e6,
         "frac_nominal_int32": OPS_PER_ATTEMPT * rate * 1e9 / (peaks["int32_tops"] * 1e12),
         "frac_of_measured_draw_rate": rate / mix["kernel_philox_form"],
         "frac_of_measured_draws_with_masks": rate / mix["kernel_form_with_masks"],
@@ -501,31 +511,26 @@ def extras(P, stream, peaks, mix):
         lat.measure()
         return time.perf_counter() - t
 
-    # small lattices: one CTA (L = 64) and an 8-CTA cluster (L = 256)
+    # small lattices
     for Ls in (64, 128, 256, 512):
         name = "L%d_1000_sweeps" % Ls
         a = P.Lattice(Ls, 2.269185, seed=1, init="cold_up")
         ta = min(wall_call(a, 1000) for _ in range(3))
         n = Ls * Ls * 1000
-        d = {"attempts_per_ns": n / ta / 1e9, "launch": a.launch,
+        d = {"attempts_per_ns": n / ta / 1e9,
              "note": "wall time of one ising_sweep call (launch, 1000 sweeps, read-back of 1000 M/E samples), "
                      "best of 3"}
         s = P.Lattice(Ls, 2.269185, seed=1, init="cold_up")
         s.set_launch(proc_bits=32, regcap=0, insert=0, block=128, rows_per_item=4, grid=0)
         d["step_launches_attempts_per_ns"] = n / wall_call(s, 1000) / 1e9
-        ctas = max(1, a.launch["grid"])
-        d["issue_bound_attempts_per_ns"] = ctas * INT32_LANES_PER_SM * peaks["sm_max_ghz"] / OPS_PER_ATTEMPT
-        # the SMs that draw the acceptance masks (the warp-specialised form
-        # draws in all CTAs but the first) at the measured per-SM draw rate
-        drawing = ctas - 1 if a.launch["block"] == 1024 and ctas > 1 else ctas
-        d["draw_bound_attempts_per_ns"] = drawing * mix["kernel_form_with_masks"] / torch.cuda.get_device_properties(
-            torch.cuda.current_device()).multi_processor_count
-        d["frac_of_draw_bound"] = d["attempts_per_ns"] / d["draw_bound_attempts_per_ns"]
+        # bound by the chain of 2000 steps, not by draws (which the whole GPU makes)
+        d["ns_per_step"] = ta / 2000 * 1e9
         out[name] = d
         a.close()
         s.close()
 
-    # the 128-lattice finite-size-scaling batch: one tuned persistent launch
+    # the 128-lattice finite-size-scaling batch: the default form, and the strips of one
+    # tuned persistent launch
     specs = WL.fss_batch()
     lats = [P.Lattice(**WL.lattice_kwargs(sp)) for sp in specs]
     sweeps = [sp["sweeps"] for sp in specs]
@@ -536,6 +541,10 @@ def extras(P, stream, peaks, mix):
         info = b.info()
         t = time.perf_counter()
         b.run(1)
+        t_s = time.perf_counter() - t
+    with P.Batch(lats, sweeps, specs[0]["record_every"]) as b:
+        t = time.perf_counter()
+        b.run(1)
         t_b = time.perf_counter() - t
     t = time.perf_counter()
     for lat in lats:
@@ -544,10 +553,12 @@ def extras(P, stream, peaks, mix):
         lat.measure()
     t_p = time.perf_counter() - t
     out["fss_batch_128_lattices"] = {
-        "persistent_attempts_per_ns": N * sweeps[0] / t_b / 1e9,
+        "attempts_per_ns": N * sweeps[0] / t_b / 1e9,
+        "strips_attempts_per_ns": N * sweeps[0] / t_s / 1e9,
         "sequential_plain_attempts_per_ns": N * 200 / t_p / 1e9,
-        "seconds": t_b, "plan": info, "options": opts,
-        "note": "10^4 sweeps of 128 lattices in one launch (wall time incl. sample read-back); "
+        "seconds": t_b, "strips_plan": info, "strips_options": opts,
+        "note": "10^4 sweeps of 128 lattices in one run (wall time incl. sample read-back), draws ahead; "
+                "strips: one persistent launch with tuned options; "
                 "plain: each lattice's default launch, 200 sweeps each, one after another"}
     for lat in lats:
         lat.close()
@@ -649,7 +660,7 @@ def run_ours(args, ws, rank, local):
     for i in range(args.steps):
         with torch.cuda.stream(stream):
             ev[i][0].record(stream)
-            lat.sweep(SWEEPS_PER_STEP, 1)   # 2 half-sweep launches per sweep
+            lat.sweep(SWEEPS_PER_STEP, 1)
             ev[i][1].record(stream)
         if not strips:
             lat.measure()                   # harvests the samples, FP64 moments on the host
@@ -661,9 +672,12 @@ def run_ours(args, ws, rank, local):
     t_dev = max_over_ranks(sum(step_ms) / 1e3)
     value = units_per_step * args.steps / t_dev / 1e9
     obs = None if strips else lat.measure()
+    # the draw-ahead form holds a second copy of the lattice
+    free, total = torch.cuda.mem_get_info()
+    ahead = not strips and total - free > 1.9 * (N // 8)
     lat.close()
-    launches = 2 * SWEEPS_PER_STEP * args.steps
-    mean_launch_s = sum(step_ms) / 1e3 / launches
+    launches = launches_of_step(strips, ahead) * args.steps
+    step_s = sum(step_ms) / 1e3 / args.steps
 
     # ---------------- end to end through the C ABI from pinned host memory
     nbytes = N // 8
@@ -761,31 +775,32 @@ def run_ours(args, ws, rank, local):
     sms = props.multi_processor_count
     sm_max_ghz = (peaks.get("sm_max_mhz") or 2070.0) / 1e3
     peak_tops = sms * INT32_LANES_PER_SM * sm_max_ghz * 1e9 / 1e12
-    per_rank_attempts = N / 2 / (ws if strips else 1)
-    achieved_tops = OPS_PER_ATTEMPT * per_rank_attempts / mean_launch_s / 1e12
-    rate_per_gpu = per_rank_attempts / mean_launch_s / 1e9  # attempts/ns of one GPU's launches
+    per_rank_attempts = N * SWEEPS_PER_STEP / (ws if strips else 1)  # of a step
+    achieved_tops = OPS_PER_ATTEMPT * per_rank_attempts / step_s / 1e12
+    rate_per_gpu = per_rank_attempts / step_s / 1e9  # attempts/ns of one GPU
     mix = mix_peaks(P, stream) if ws == 1 else None
     prof = profiled_kernel()
     traffic = None
-    if prof and not strips:
-        # DRAM bytes of one launch at the captured size, scaled by the sites of this one
-        traffic = prof["dram_bytes_per_launch"] * (N / float(prof["L"]) ** 2)
+    if prof and ahead:
+        traffic = prof["dram_bytes_per_attempt"] * per_rank_attempts
     roof = {
         "bound": "alu", "achieved": achieved_tops, "peak": peak_tops, "unit": "Tops/s (int32)",
         "frac": achieved_tops / peak_tops, "traffic": traffic,
-        "kernel": "k_half_sweep (proc_bits=%s, regcap=%s)" % (
+        "kernel": "k_ahead_band (draws of a band of rows for 4 sweeps beside the update of the band before)" if ahead
+        else "k_half_sweep (proc_bits=%s, regcap=%s)" % (
             tuned["proc_bits"] if tuned else "default", tuned["regcap"] if tuned else "default"),
         "peak_basis": "%d SMs x %d int32 lanes x %.2f GHz (max SM clock), derived" % (
             sms, INT32_LANES_PER_SM, sm_max_ghz),
-        "achieved_basis": "%d ops/attempt x %d attempts per launch / mean launch time %.1f us (CUDA events "
-                          "over the timed region)" % (OPS_PER_ATTEMPT, per_rank_attempts, mean_launch_s * 1e6),
-        "hbm_view": {"bytes_per_launch_algorithmic": per_rank_attempts * 2 / 8 * 2,
-                     "achieved_gbs": per_rank_attempts * 2 / 8 * 2 / mean_launch_s / 1e9,
-                     "peak_gbs": peaks.get("hbm_gbs"), "peak_note": "of measured"},
+        "achieved_basis": "%d ops/attempt x %d attempts per step / mean step time %.1f us (CUDA events "
+                          "over the timed region)" % (OPS_PER_ATTEMPT, per_rank_attempts, step_s * 1e6),
+        "hbm_view": {"bytes_per_step_algorithmic": per_rank_attempts / 4,
+                     "achieved_gbs": per_rank_attempts / 4 / step_s / 1e9,
+                     "peak_gbs": peaks.get("hbm_gbs"), "peak_note": "of measured",
+                     "basis": "the lattice read and written once per sweep"},
     }
     if traffic is not None:
-        roof["traffic_basis"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per launch at L=%d, "
-                                 "scaled by the sites per launch (%s)" % (prof["L"], prof["source"]))
+        roof["traffic_basis"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per attempt at L=%d, times the "
+                                 "attempts of a step (%s)" % (prof["L"], prof["source"]))
         roof["ncu_thread_instructions_per_attempt"] = prof.get("thread_inst_per_attempt")
     if mix:
         roof["measured_mix"] = dict(mix, unit="draws/ns", how="ising_bench_mix: one wave of resident 512-thread "

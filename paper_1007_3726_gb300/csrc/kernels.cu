@@ -14,8 +14,9 @@
 // variables i_n = s0 ^ s_n (Sec. 4, Eq. 4) are summed bit-parallel with a
 // carry-save adder into "two or more anti-aligned", "exactly one" and "none".
 // The acceptance i1 + i2 + i3 + i4 + 2 exp8 + exp4 >= 2 of Sec. 4, Eq. 5 then
-// reads flip = ge2 | (eq1 & P4) | (eq0 & P8), with P4 / P8 the bit masks of
-// u < thr4 / u < thr8 for the sites' own Philox draws.
+// reads flip = ge2 | (odd & P4) | P8 (flips in sweep_device.cuh), with odd "one or
+// three" and P4 / P8 the bit masks of u < thr4 / u < thr8 for the sites' own Philox
+// draws (a draw below thr8 is below thr4 too).
 //
 // Each Philox4x32-10 call yields the draws of four consecutive target sites,
 // which in every row occupy one byte of the packed row (x = 8q .. 8q + 7).

@@ -6,7 +6,7 @@
 // buffers to plug-ins and forbids them the CUDA allocator, or a loop that
 // cannot afford the device-wide synchronisation a cudaMalloc / cudaFree may
 // bring.  For them this entry point runs ising_sweep's kernels on a lattice the
-// caller owns (the one-CTA or cluster kernel where ising_sweep's default takes
+// caller owns (the one-CTA or cluster kernel where the handle's configuration names
 // it, the half-sweep step kernels otherwise), and keeps the kernels' scratch
 // (the per-sweep M/E counters) in a fixed array compiled into the library
 // instead of allocating it.
