@@ -1484,7 +1484,7 @@ static cudaError_t cluster_sweeps(const AheadPlan &pl, AheadArgs a, char *masks,
         uint32_t slots = 0, recs = 0, slot0 = 0, last = 0;
         const uint32_t *snaps = nullptr;
     } counted[2];  // of the blocks before
-    const uint32_t re = a.record_every, per = (a.nwords / pl.kw + 31u) & ~31u;
+    const uint32_t re = a.record_every;
     for (uint64_t b = 0;; ++b) {
         uint64_t n = std::min(left, grow);
         if (left % 4 && n < left && n > 4) n -= 4 - left % 4;
@@ -1503,7 +1503,6 @@ static cudaError_t cluster_sweeps(const AheadPlan &pl, AheadArgs a, char *masks,
         a.c_last = c.last;
         a.c_snaps = c.snaps;
         a.c_wait = n == 0;
-        a.count_ctas = std::min<uint32_t>((a.c_slots * per + kThreads - 1) / kThreads, 64u);  // (fewer than SMs)
         a.d_t0 = (uint32_t)(t0 + done);
         a.d_sweeps = (uint32_t)n;
         a.d_masks = masks + (b % kClusterBuffers) * pl.mask_bytes;
@@ -1511,7 +1510,9 @@ static cudaError_t cluster_sweeps(const AheadPlan &pl, AheadArgs a, char *masks,
         a.next_ticket = tickets + (b + 2) % 4;
         a.d_k = n % 4 == 0 ? 4 : n % 2 == 0 ? 2 : 1;
         a.d_tickets = a.d_sweeps / a.d_k * 2u * (a.nwords / 32u);
-        dc.gridDim = dim3(std::max(1u, std::min<uint32_t>((uint32_t)sms, a.count_ctas + (a.d_tickets + kThreads / 32u - 1) / (kThreads / 32u))));
+        const DrawGrid g = draw_grid((uint32_t)sms, kThreads, a.c_slots, a.nwords / pl.kw, a.d_tickets);
+        a.count_ctas = g.count_ctas;
+        dc.gridDim = dim3(g.grid);
         dc.numAttrs = b > 0 ? 1 : 0;
         if ((e = cudaLaunchKernelEx(&dc, draw, a)) != cudaSuccess) return e;
         counted[0] = counted[1];

@@ -4,6 +4,7 @@
 
 #include "kernels.h"
 
+#include <algorithm>
 #include <cstddef>
 #include <cstdint>
 #include <vector>
@@ -73,6 +74,22 @@ struct AheadArgs {
     char *d_masks;
     unsigned int *d_ticket, *next_ticket;  // this launch's counter; the one to clear
 };
+
+// A launch of the cluster form's draws and counts.
+struct DrawGrid {
+    uint32_t count_ctas, grid;  // CTAs that count (the first ones), and in all
+};
+// For `slots` snapshots of `runs` runs and `tickets` items, with CTAs of `threads` threads
+// on `sms` SMs (one CTA each).  The counting CTAs share the snapshots by their number, so
+// that all of them have to be in the grid, also on a partition with few SMs.
+inline DrawGrid draw_grid(uint32_t sms, uint32_t threads, uint32_t slots, uint32_t runs, uint32_t tickets)
+{
+    const uint32_t per = (runs + 31u) & ~31u;  // threads a snapshot: whole warps
+    DrawGrid g;
+    g.count_ctas = std::min({(slots * per + threads - 1) / threads, 64u, sms});
+    g.grid = std::max(1u, std::min(sms, g.count_ctas + (tickets + threads / 32u - 1) / (threads / 32u)));
+    return g;
+}
 
 AheadPlan ahead_plan(uint64_t L, bool field);
 // The cluster form, for the sizes and calls where it is the faster one (no field; kw 0: not
