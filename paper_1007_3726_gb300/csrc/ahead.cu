@@ -62,6 +62,7 @@ constexpr uint32_t kWarpStages = 8;
 constexpr uint32_t kClusterThreads = 256, kClusterChunk = 4, kClusterStages = 8;  // of the cluster form: update threads, steps of a stage, stages
 constexpr uint32_t kBuffers = 3, kClusterBuffers = 2;  // mask buffers, used in turn
 constexpr uint32_t kWaitLimit = 1u << 22;  // polls of a wait for masks on their way into shared memory
+constexpr uint32_t kPublishedLimit = 1u << 12;  // polls for a word that is there already
 
 template <int V>
 struct Parity {
@@ -947,18 +948,43 @@ __device__ __forceinline__ void update_cluster(const AheadArgs &a, unsigned char
     cluster_sync();  // no peer writes into a CTA that has ended
 }
 
+// How many updates' writes are visible here: published with release order by a thread that
+// has waited for them, read with acquire order (and then a CTA barrier) by one that has not.
+__device__ __forceinline__ void publish(unsigned int *done, uint32_t n)
+{
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(done), "r"(n) : "memory");
+}
+__device__ __forceinline__ bool published(const unsigned int *done, uint32_t n, uint32_t limit)
+{
+    for (uint32_t k = 0; k < limit; ++k) {
+        uint32_t v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
+        if (v >= n) return true;
+    }
+    return false;
+}
+
 // The launches of a call take turns: draws of block b and counts of block b - 2, and the
 // update of block b.  The update starts when the draws have ended; it lets the next draws
 // start at once, which need not wait for it: what they write was read, and what they
-// count was written, by launches that ended before the update began.  One CTA of the draws
-// stays until the update before has ended, for the next update, which waits for the
-// draws alone.
+// count was written, by launches that ended before the update began.  That they have ended
+// does not make their writes visible to a launch that did not wait for them, and the
+// buffers are used again every other block: so the update publishes, before it lets the
+// draws start, what it has waited for, and the draws acquire that (it is there when they
+// start).  One CTA of the draws stays until the update before has ended, for the next
+// update, which waits for the draws alone.
 __global__ void __launch_bounds__(kThreads, 1) k_ahead_draw(const __grid_constant__ AheadArgs a)
 {
-    if (a.c_wait != 0u) dependent_launch_wait();  // the call's last counts, or its first draws
+    if (a.c_wait != 0u) dependent_launch_wait();  // the call's last counts
     dependent_launch_trigger();
-    if (blockIdx.x < a.count_ctas) count_role<2>(a, blockIdx.x);
-    if (a.d_tickets != 0u) draw_role<false, false, false>(a);
+    bool go = true;
+    if (a.d_after != 0u) {
+        const bool late = threadIdx.x == 0 && !published(a.done, a.d_after, kPublishedLimit);
+        if (late && a.err) atomicExch(a.err, 1u);
+        go = __syncthreads_or(late) == 0;
+    }
+    if (go && blockIdx.x < a.count_ctas) count_role<2>(a, blockIdx.x);
+    if (go && a.d_tickets != 0u) draw_role<false, false, false>(a);
     if (blockIdx.x + 1u == gridDim.x) {
         dependent_launch_wait();
         if (threadIdx.x == 0) *a.next_ticket = 0u;
@@ -969,7 +995,11 @@ __global__ void __launch_bounds__(kClusterThreads + 32, 1) k_ahead_cluster(const
 {
     extern __shared__ __align__(128) unsigned char smem[];
     dependent_launch_wait();
-    dependent_launch_trigger();
+    // (the last thread, of the warp that fetches masks: the others need not wait for it)
+    const bool last = threadIdx.x + 1u == blockDim.x;
+    if (blockIdx.x == 0 && last) publish(a.done, a.u_before);
+    if (blockIdx.x != 0 || last) dependent_launch_trigger();
+    __syncwarp();
     update_cluster(a, smem);
 }
 
@@ -1129,6 +1159,7 @@ AheadKernel pick_kernel(const AheadPlan &p)
 constexpr int kMaxDevices = 64;
 constexpr int kMaxSmem = 200 * 1024;
 constexpr size_t kTicketBytes = 256;  // the ticket counters at the start of the scratch
+constexpr size_t kDoneWord = 32;      // and the cluster form's count of updates, on a line of its own
 
 FastDiv fast_div(uint32_t d)
 {
@@ -1463,6 +1494,7 @@ static cudaError_t cluster_sweeps(const AheadPlan &pl, AheadArgs a, char *masks,
     a.stages = pl.stages;
     a.src = a.dst = spins;
     a.update_ctas = pl.tiles;
+    a.done = tickets + kDoneWord;
     cudaLaunchAttribute attr[2]{};
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1503,6 +1535,8 @@ static cudaError_t cluster_sweeps(const AheadPlan &pl, AheadArgs a, char *masks,
         a.c_last = c.last;
         a.c_snaps = c.snaps;
         a.c_wait = n == 0;
+        // block b - 2: its counts, and the buffer of masks that its update read
+        a.d_after = n != 0 && b >= 2 ? (uint32_t)(b - 1) : 0u;
         a.d_t0 = (uint32_t)(t0 + done);
         a.d_sweeps = (uint32_t)n;
         a.d_masks = masks + (b % kClusterBuffers) * pl.mask_bytes;
@@ -1521,6 +1555,7 @@ static cudaError_t cluster_sweeps(const AheadPlan &pl, AheadArgs a, char *masks,
         const uint64_t t = t0 + done;
         a.u_steps = (uint32_t)(2 * n);
         a.u_step0 = (uint32_t)(2 * done);
+        a.u_before = (uint32_t)b;
         a.u_masks = a.d_masks;
         a.u_snaps = reinterpret_cast<uint32_t *>(snaps + (b % 2) * pl.snap_bytes);
         a.u_phase = re ? (uint32_t)(t % re) : 0u;

@@ -67,6 +67,10 @@ struct AheadArgs {
     // count: the snapshots of the block before
     uint32_t count_ctas, c_slots, c_recs, c_slot0, c_last;
     uint32_t c_wait;              // they are those of the launch before
+    // cluster form: updates of the call whose writes are visible (each publishes those before
+    // it); those before this update; those that a draw launch needs (0: it waits, or none)
+    unsigned int *done;
+    uint32_t u_before, d_after;
     const uint32_t *c_snaps;
     // draw: d_sweeps sweeps from sweep index d_t0, in tickets of 32 items of d_k sweeps
     uint32_t d_t0, d_sweeps, d_k, d_tickets;

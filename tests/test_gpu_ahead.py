@@ -291,3 +291,17 @@ def test_second_counter_word_within_a_row(P):
             out.append(lat.sweep(6, 1, collect=True))
     np.testing.assert_array_equal(out[0][0], out[1][0])
     np.testing.assert_array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("L", [320, 448, 512])
+def test_cluster_counts_every_sweep_while_its_buffers_turn(P, orc, L):
+    """Calls of many blocks with M/E after every sweep: both snapshot buffers and both
+    mask buffers are used over and over, by launches that start beside the update before,
+    and what an earlier call left in them is counted by none."""
+    seed, calls = 5, (1030, 700)
+    lat = P.Lattice(L, TC, seed=seed, init="cold_up")
+    s, t = orc.init_cold(L, 1), 0
+    for n in calls:
+        _compare(orc, lat, s, t, n, 1, seed, 0, orc.thresholds(TC))
+        t += n
+    lat.close()
