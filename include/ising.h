@@ -62,6 +62,7 @@ extern "C" {
 #endif
 
 typedef struct ising_lattice ising_lattice; /* opaque; owned by the caller until ising_destroy */
+typedef struct ising_batch ising_batch;     /* opaque, see below */
 
 typedef enum {
     ISING_OK = 0,
@@ -283,6 +284,21 @@ typedef struct {
     uint32_t persistent;
 } ising_launch;
 
+/* What ran: the form that the handle's last ising_sweep call took (NONE before the first),
+ * and the one that runs of a batch take as it is planned now. */
+typedef enum {
+    ISING_FORM_NONE = 0,
+    ISING_FORM_STEPS = 1,         /* two launches per sweep */
+    ISING_FORM_ONE_LAUNCH = 2,    /* one CTA or cluster, proc_bits = 8 */
+    ISING_FORM_COOPERATIVE = 3,   /* persistent = 1 */
+    ISING_FORM_AHEAD = 4,         /* draw-ahead, tiles or the whole lattice per launch */
+    ISING_FORM_AHEAD_CLUSTER = 5, /* draw-ahead, the lattice in one cluster */
+    ISING_FORM_AHEAD_BANDS = 6,   /* draw-ahead, a band of rows per launch */
+    ISING_FORM_STRIPS = 7         /* a batch in strips, one persistent launch */
+} ising_form;
+ISING_API ising_status ising_last_form(const ising_lattice *h, ising_form *form);
+ISING_API ising_status ising_batch_form(const ising_batch *b, ising_form *form);
+
 /* The handle's current configuration. */
 ISING_API ising_status ising_get_launch(const ising_lattice *h, ising_launch *out);
 /* Replaces it (ISING_ERR_INVALID if not valid for the handle's L). */
@@ -354,7 +370,6 @@ ISING_API ising_status ising_bench_mix(uint32_t form, uint32_t words_per_thread,
  *                  never announces its steps, so that its neighbours' waits
  *                  run out (0 = none)
  */
-typedef struct ising_batch ising_batch;
 typedef struct {
     uint32_t block, ctas_per_sm, rows_per_item, insert, use_graph;
     double wait_ms;

@@ -22,14 +22,15 @@ __all__ = [
     "IsingError", "Lattice", "build", "load", "thresholds", "ising_create", "ising_sweep",
     "ising_measure", "ising_measure_from", "ising_destroy", "ising_get_spins", "ising_get_packed", "ising_recount", "ising_get_samples",
     "ising_thresholds", "ising_last_error", "ising_set_allocator", "ising_info",
-    "ising_device_spins", "ising_check_guards", "ising_sweep_noalloc", "ising_bench_mix", "ising_strip_init", "ising_strip_step", "ising_strip_observables", "ising_get_launch", "ising_set_launch",
+    "ising_device_spins", "ising_check_guards", "ising_sweep_noalloc", "ising_bench_mix", "ising_strip_init", "ising_strip_step", "ising_strip_observables", "ising_get_launch", "ising_set_launch", "ising_last_form", "ising_batch_form",
     "ising_launch_candidates", "ising_autotune", "ising_sweep_batch", "ising_batch_tune", "Batch", "Server", "IsingBatchOpts",
-    "IsingParams", "IsingLaunch", "IsingObs", "INIT_MODES", "STATUS_NAMES",
+    "IsingParams", "IsingLaunch", "IsingObs", "INIT_MODES", "STATUS_NAMES", "FORM_NAMES",
 ]
 
 OK, ERR_INVALID, ERR_OOM, ERR_CUDA, ERR_TIMEOUT, ERR_STATE, ERR_CANCELLED = range(7)
 STATUS_NAMES = {0: "ISING_OK", 1: "ISING_ERR_INVALID", 2: "ISING_ERR_OOM", 3: "ISING_ERR_CUDA",
                 4: "ISING_ERR_TIMEOUT", 5: "ISING_ERR_STATE", 6: "ISING_ERR_CANCELLED"}
+FORM_NAMES = ("none", "steps", "one_launch", "cooperative", "ahead", "ahead_cluster", "ahead_bands", "strips")
 INIT_MODES = {"cold_up": 0, "cold": 0, "cold_down": 1, "hot": 2, "buffer": 3, "packed": 4}
 
 
@@ -179,6 +180,8 @@ def load(path: str | None = None):
         "ising_get_params": ([H, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double)],
                              ctypes.c_int),
         "ising_check_guards": ([H, _u32p], ctypes.c_int),
+        "ising_last_form": ([H, ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
+        "ising_batch_form": ([H, ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
         "ising_strip_observables": ([ctypes.c_uint64, ctypes.c_uint64, ctypes.c_uint64, _i64p, _i64p],
                                     ctypes.c_int),
         "ising_bench_mix": ([ctypes.c_uint32, ctypes.c_uint32, ctypes.POINTER(ctypes.c_double),
@@ -352,6 +355,20 @@ def ising_set_launch(h, cfg: dict):
     _check(load().ising_set_launch(h, ctypes.byref(IsingLaunch(**cfg))))
 
 
+def ising_last_form(h) -> str:
+    """The form that the handle's last sweep call took (one of FORM_NAMES)."""
+    v = ctypes.c_int()
+    _check(load().ising_last_form(h, ctypes.byref(v)))
+    return FORM_NAMES[v.value]
+
+
+def ising_batch_form(b) -> str:
+    """The form that runs of a batch take (one of FORM_NAMES)."""
+    v = ctypes.c_int()
+    _check(load().ising_batch_form(b, ctypes.byref(v)))
+    return FORM_NAMES[v.value]
+
+
 def ising_launch_candidates(L: int) -> list[dict]:
     n = load().ising_launch_candidates(L, None, 0)
     arr = (IsingLaunch * max(n, 1))()
@@ -412,6 +429,11 @@ class Batch:
         _check(load().ising_batch_info(self._b, ctypes.byref(g), ctypes.byref(b), ctypes.byref(st),
                                        ctypes.byref(sm)))
         return {"grid": g.value, "block": b.value, "strips": st.value, "smem_bytes": sm.value}
+
+    @property
+    def form(self) -> str:
+        """What run() runs: "ahead" or "strips"."""
+        return ising_batch_form(self._b)
 
     def close(self):
         if self._b is not None and self._b.value:
@@ -638,6 +660,11 @@ class Lattice:
     @property
     def launch(self) -> dict:
         return ising_get_launch(self._h)
+
+    @property
+    def form(self) -> str:
+        """What the last sweep() ran (one of FORM_NAMES)."""
+        return ising_last_form(self._h)
 
     def set_launch(self, **cfg):
         """Replace the launch configuration; fields not given keep their current

@@ -1183,6 +1183,14 @@ ISING_API ising_status ising_batch_info(const ising_batch *b, uint32_t *grid, ui
     return ISING_OK;
 }
 
+ISING_API ising_status ising_batch_form(const ising_batch *b, ising_form *form)
+{
+    clear_error();
+    if (!b || !form) return fail(ISING_ERR_INVALID, "null argument");
+    *form = b->hs.empty() ? ISING_FORM_NONE : b->use_ahead ? ISING_FORM_AHEAD : ISING_FORM_STRIPS;
+    return ISING_OK;
+}
+
 ISING_API ising_status ising_batch_destroy(ising_batch *b)
 {
     clear_error();

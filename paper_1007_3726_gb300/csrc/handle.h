@@ -31,6 +31,7 @@ struct ising_lattice {
     void *d_ahead = nullptr;  // scratch of the draw-ahead form (ahead.cu), on first use
     size_t ahead_bytes = 0;
     bool ahead = true;        // the draw-ahead form where it applies (no configuration set, none found faster)
+    ising_form form = ISING_FORM_NONE;  // of the last ising_sweep call
     cudaEvent_t ev = nullptr;
     ising::RoundKeys key{};
     ising::LaunchConfig launch{};

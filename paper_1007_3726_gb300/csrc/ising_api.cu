@@ -489,12 +489,14 @@ ising_status ising_sweep(ising_lattice *h, uint64_t nsweeps, uint32_t record_eve
     AheadPlan pl = h->ahead && h->H == 0.0 ? cluster_plan(h->L, nsweeps) : AheadPlan{};
     if (pl.kw == 0 || !ahead_ready(h, pl, h->L)) pl = h->ahead ? ahead_plan(h->L, h->H != 0.0) : AheadPlan{};
     if (pl.kw != 0 && nsweeps >= pl.min_sweeps && ahead_ready(h, pl, h->L)) {
+        h->form = pl.cluster ? ISING_FORM_AHEAD_CLUSTER : pl.band_rows ? ISING_FORM_AHEAD_BANDS : ISING_FORM_AHEAD;
         CK(h, ahead_sweeps(h, pl, h->d_spins, h->L, t0, nsweeps, record_every, nrec, err, hold_step, max_chunk));
         h->pending_err = true;
         return finish_sweep_call(h, t0, nsweeps, nrec, M_out, E_out);
     }
     if (h->launch.proc_bits == kTinyProcBits) {
         // the whole call in one launch of one CTA
+        h->form = ISING_FORM_ONE_LAUNCH;
         TinyRunArgs ta{};
         ta.spins = h->d_spins;
         ta.L = h->L;
@@ -539,6 +541,7 @@ ising_status ising_sweep(ising_lattice *h, uint64_t nsweeps, uint32_t record_eve
     }
     if (h->launch.persistent && h->H == 0.0) {
         // the whole call in one cooperative launch
+        h->form = ISING_FORM_COOPERATIVE;
         HalfSweepArgs a{};
         a.spins = h->d_spins;
         a.L = h->L;
@@ -555,6 +558,7 @@ ising_status ising_sweep(ising_lattice *h, uint64_t nsweeps, uint32_t record_eve
         CK(h, launch_sweeps(a, h->launch, sr, h->stream));
         return finish_sweep_call(h, t0, nsweeps, nrec, M_out, E_out);
     }
+    h->form = ISING_FORM_STEPS;
     HalfSweepArgs a{};
     a.spins = h->d_spins;
     a.L = h->L;
@@ -741,6 +745,14 @@ ising_status ising_info(const ising_lattice *h, uint32_t *word_bits, uint64_t *L
     if (word_bits) *word_bits = h->word_bits;
     if (L) *L = h->L;
     if (sweeps_done) *sweeps_done = h->sweeps_done;
+    return ISING_OK;
+}
+
+ising_status ising_last_form(const ising_lattice *h, ising_form *form)
+{
+    clear_error();
+    if (!h || !form) return fail(ISING_ERR_INVALID, "null argument");
+    *form = h->form;
     return ISING_OK;
 }
 

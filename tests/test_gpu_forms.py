@@ -1,0 +1,125 @@
+"""Which form a call takes, and the forms that the draw-ahead form has replaced as the
+default: they remain what runs where it does not apply, and what a set configuration runs."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+TC = 2.269185
+
+
+@pytest.fixture(scope="module")
+def P():
+    import paper_1007_3726_gb300 as P
+
+    P.build()
+    P.load()
+    return P
+
+
+# the edges of the plans' ranges: (L, H, sweeps) and the form
+DEFAULTS = [
+    (64, 0.0, 199, "one_launch"), (64, 0.0, 200, "ahead"), (128, 0.0, 99, "one_launch"), (128, 0.0, 100, "ahead"),
+    (192, 0.0, 2, "steps"), (192, 0.0, 3, "ahead"), (256, 0.0, 9, "one_launch"), (256, 0.0, 10, "ahead"),
+    (320, 0.0, 191, "ahead"), (320, 0.0, 192, "ahead_cluster"), (512, 0.0, 2, "one_launch"), (512, 0.0, 3, "ahead"),
+    (512, 0.0, 192, "ahead_cluster"), (576, 0.0, 200, "ahead"), (1024, 0.0, 4, "steps"), (1024, 0.0, 5, "ahead"),
+    (2048, 0.0, 9, "steps"), (2048, 0.0, 10, "ahead"), (8192, 0.0, 10, "ahead"), (8256, 0.0, 3, "steps"),
+    (8256, 0.0, 4, "ahead_bands"), (185408, 0.0, 6, "ahead_bands"),
+    (64, 0.3, 4, "one_launch"), (64, 0.3, 5, "ahead"), (320, 0.3, 1, "ahead"), (512, -2.0, 200, "ahead"),
+    (2048, 0.3, 1, "ahead"), (4096, 0.3, 3, "steps"), (4096, 0.3, 4, "ahead"),
+]
+
+
+@pytest.mark.parametrize("L,H,n,form", DEFAULTS)
+def test_form_of_a_default_call(P, L, H, n, form):
+    with P.Lattice(L, TC, seed=1, init="hot", H=H) as lat:
+        assert lat.form == "none"
+        lat.sweep(n, 1)
+        assert lat.form == form
+
+
+def test_a_set_configuration_is_what_runs(P):
+    with P.Lattice(512, TC, seed=1) as lat:
+        for cfg, form in ((dict(lat.launch), "one_launch"),
+                          (dict(proc_bits=32, regcap=0, insert=0, block=256, rows_per_item=4, grid=0), "steps"),
+                          (dict(proc_bits=32, regcap=0, insert=0, block=256, rows_per_item=4, grid=0, persistent=1), "cooperative")):
+            lat.set_launch(**cfg)
+            lat.sweep(200, 1)
+            assert lat.form == form
+
+
+def test_form_of_a_batch(P):
+    lats = [P.Lattice(L, TC, seed=L) for L in (64, 512)]
+    for n, opts, form in ((20, {}, "ahead"), (20, dict(use_graph=True), "ahead"), (4, {}, "strips"), (20, dict(block=512), "strips"),
+                          (20, dict(wait_ms=100.0), "strips")):
+        with P.Batch(lats, [n, n], 1, **opts) as b:
+            assert b.form == form
+            b.run(1)
+
+
+# one-launch forms on whole calls of the plain method's length, as they were the default
+@pytest.mark.parametrize("L,n", [(64, 1000), (128, 400), (256, 200), (512, 60)])
+def test_one_launch_forms_on_long_calls(P, orc, L, n):
+    lat = P.Lattice(L, TC, seed=1, init="cold_up")
+    lat.set_launch(**lat.launch)
+    M, E = lat.sweep(n, 1, collect=True)
+    assert lat.form == "one_launch"
+    s = orc.init_cold(L, 1)
+    Mo, Eo = orc.run(s, n, 1, 0, *orc.thresholds(TC))
+    assert np.array_equal(M, Mo) and np.array_equal(E, Eo) and np.array_equal(lat.spins(), s)
+    lat.close()
+
+
+@pytest.mark.parametrize("L,H", [(64, 0.0), (128, 0.0), (256, 0.0), (512, 0.0), (64, 0.3), (256, -2.0)])
+def test_one_launch_forms_in_several_launches(P, orc, monkeypatch, L, H):
+    """Calls longer than a launch's bound: a launch hands its sample slots to the next."""
+    T, seed, sid, t = 2.1, 23, 2, 0
+    lat = P.Lattice(L, T, seed=seed, stream_id=sid, init="hot", H=H)
+    lat.set_launch(**lat.launch)
+    monkeypatch.setenv("ISING_TINY_MAX_SWEEPS", "7")
+    s = orc.init_hot(L, seed, sid)
+    for n, rec in ((50, 3), (15, 0), (22, 1)):
+        got = lat.sweep(n, rec, collect=bool(rec))
+        assert lat.form == "one_launch"
+        Mo, Eo = orc.run_field(s, n, seed, sid, T, H, t0=t) if H else orc.run(s, n, seed, sid, *orc.thresholds(T), t0=t)
+        if rec:
+            k0 = (rec - 1 - t) % rec
+            assert np.array_equal(got[0], Mo[k0::rec]) and np.array_equal(got[1], Eo[k0::rec]), (n, rec)
+        d = lat.measure()
+        assert (d["M"], d["E"]) == (Mo[-1], Eo[-1])
+        t += n
+    assert np.array_equal(lat.spins(), s)
+    lat.close()
+
+
+@pytest.mark.parametrize("L,H,n", [(4096, 0.0, 12), (4096, 0.25, 6), (32768, 0.0, 6)])
+def test_step_kernels_on_larger_lattices(P, orc, L, H, n):
+    """The whole lattice and every sample, in the step kernels' default configuration."""
+    lat = P.Lattice(L, TC, seed=7, init="hot", H=H)
+    lat.set_launch(**lat.launch)
+    M, E = lat.sweep(n, 1, collect=True)
+    assert lat.form == "steps"
+    s = orc.init_hot(L, 7, 0)
+    Mo, Eo = orc.run_field(s, n, 7, 0, TC, H) if H else orc.run(s, n, 7, 0, *orc.thresholds(TC), check=False)
+    assert np.array_equal(M, Mo) and np.array_equal(E, Eo) and np.array_equal(lat.spins(), s)
+    lat.close()
+
+
+def test_step_kernels_on_L524288(P, orc):
+    """Rows of four windows (both ends, the middle) after 5 sweeps, against the oracle's
+    light-cone evolution, and the fused M/E against a recount."""
+    import torch
+
+    if torch.cuda.mem_get_info()[0] < 40 * 2 ** 30:
+        pytest.skip("needs 40 GiB of free device memory")
+    L, T, seed, k = 524288, 2.0, 5, 5
+    lat = P.Lattice(L, T, seed=seed, init="cold_up", word_bits=64)
+    lat.set_launch(**lat.launch)
+    M, E = lat.sweep(k, 1, collect=True)
+    assert lat.form == "steps"
+    margin = 2 * k + 1
+    for row0 in (0, L - 40, L // 2 + 17, 123456):
+        w = np.ones((64 + 2 * margin, L), dtype=np.int8)
+        orc.run_window(w, L, (row0 - margin) % L, k, seed, 0, *orc.thresholds(T))
+        assert np.array_equal(lat.spins(row0, 64), w[margin:margin + 64]), row0
+    assert (int(M[-1]), int(E[-1])) == lat.recount()
+    lat.close()
