@@ -308,12 +308,15 @@ ISING_API ising_status ising_set_launch(ising_lattice *h, const ising_launch *cf
 ISING_API uint32_t ising_launch_candidates(uint64_t L, ising_launch *out, uint32_t cap);
 /*
  * Times every candidate (reps timed step pairs each, after one untimed pair;
- * a one-CTA candidate: one launch of 8 reps sweeps after a one-sweep launch)
- * and the draw-ahead form, on a scratch copy of up to 256 MiB of the handle's rows,
- * installs the fastest candidate on the handle (and keeps the draw-ahead form in
- * use only where that is faster still), remembers it for later handles of the same L and
- * word width on this device, and returns it with its mean time per step in
- * microseconds.  The lattice itself is not changed.  Waits for the GPU.
+ * a one-CTA or cooperative candidate: one launch of 8 reps sweeps after a one-sweep
+ * launch) and the draw-ahead form without a field, with M/E counted every sweep, on a
+ * scratch copy of up to 256 MiB of the handle's rows.  Installs the fastest candidate on
+ * the handle, remembers it for later handles of the same L and word width on this
+ * device, and returns it with its mean time per step in microseconds.  It is the
+ * configuration of the calls that do not take the draw-ahead form; that form is left, for
+ * calls without a field, only where it was timed to the end and took longer (where its
+ * scratch was refused, nothing changes; the cluster form and the form in a field, which
+ * are not timed, stay).  The lattice itself is not changed.  Waits for the GPU.
  */
 ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_launch *best,
                                       double *best_us_per_step);

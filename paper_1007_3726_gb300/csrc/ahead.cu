@@ -1281,9 +1281,9 @@ namespace {
 
 // The mask planes' thresholds of a lattice, and in a field what step_run_field needs.
 template <typename A>
-void set_planes(A &a, const ising_lattice *h)
+void set_planes(A &a, const ising_lattice *h, bool field)
 {
-    if (h->H == 0.0) {
+    if (!field) {
         a.thr[0] = h->thr4;
         a.thr[1] = h->thr8;
         return;
@@ -1586,7 +1586,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     AheadArgs a{};
     a.key = h->key;
     a.step_bytes = pl.step_bytes;
-    set_planes(a, h);
+    set_planes(a, h, pl.field);
     a.c3base = h->stream_id << 1;
     a.L = (uint32_t)L;
     a.wc = a.L / 64;
@@ -1731,7 +1731,7 @@ bool AheadBatch::plan(const std::vector<ising_lattice *> &hs, const std::vector<
         const ising_lattice *h = hs[i];
         if (h->L > 4096) return false;
         j.key = h->key;
-        set_planes(j, h);
+        set_planes(j, h, h->H != 0.0);
         j.c3base = h->stream_id << 1;
         j.L = (uint32_t)h->L;
         j.wc = j.L / 64;

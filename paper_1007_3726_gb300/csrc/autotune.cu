@@ -24,7 +24,7 @@ namespace {
 std::mutex g_tuned_mu;
 struct Tuned {
     LaunchConfig config;
-    bool ahead;  // the draw-ahead form was faster still
+    bool ahead_slower;  // than the configuration, timed without a field and to the end
 };
 std::map<std::tuple<int, uint64_t, uint32_t>, Tuned> g_tuned;
 
@@ -59,17 +59,17 @@ LaunchConfig default_launch(int device, uint64_t L, uint32_t word_bits)
     return LaunchConfig{64, 1, 0, 512, 8, 0};
 }
 
-bool default_ahead(int device, uint64_t L, uint32_t word_bits)
+bool default_ahead_slower(int device, uint64_t L, uint32_t word_bits)
 {
     std::lock_guard<std::mutex> lk(g_tuned_mu);
     auto it = g_tuned.find(std::make_tuple(device, L, word_bits));
-    return it == g_tuned.end() || it->second.ahead;
+    return it != g_tuned.end() && it->second.ahead_slower;
 }
 
-void remember_launch(int device, uint64_t L, uint32_t word_bits, const LaunchConfig &c, bool ahead)
+void remember_launch(int device, uint64_t L, uint32_t word_bits, const LaunchConfig &c, bool ahead_slower)
 {
     std::lock_guard<std::mutex> lk(g_tuned_mu);
-    g_tuned[std::make_tuple(device, L, word_bits)] = Tuned{c, ahead};
+    g_tuned[std::make_tuple(device, L, word_bits)] = Tuned{c, ahead_slower};
 }
 
 std::vector<LaunchConfig> launch_candidates(uint64_t L, uint64_t rows)
@@ -143,7 +143,7 @@ ISING_API ising_status ising_set_launch(ising_lattice *h, const ising_launch *cf
         return fail(ISING_ERR_INVALID, "launch configuration not valid for L = %llu",
                     (unsigned long long)h->L);
     h->launch = c;
-    h->ahead = false;
+    h->configured = true;
     return ISING_OK;
 }
 
@@ -169,6 +169,12 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
     rows = rows - rows % 64;
     if (rows < 64) rows = 64;
     if (rows > h->L) rows = h->L;
+    // everything is timed with M/E counted after every sweep: the step kernels into one
+    // slot, a call in one launch and the draw-ahead form into a slot per sweep
+    const uint64_t La = rows == h->L ? h->L : 32768;
+    const AheadPlan pl = ahead_plan(La, false);
+    const uint64_t n_ahead = std::max<uint64_t>(8ull * reps, 2 * pl.min_sweeps), n_rec = 8ull * reps;
+    if ((st = ensure_acc(h, std::max(n_ahead, n_rec) + 2)) != ISING_OK) return st;
     void *scratch = h->alloc.allocate(rows * row_bytes, h->stream);
     if (!scratch) return fail(ISING_ERR_OOM, "cannot allocate the autotuning scratch");
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -202,13 +208,13 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
             pa.thr4 = h->thr4;
             pa.thr8 = h->thr8;
             SweepsRun sr{};
-            sr.t0 = 0xFFFFF000u;  // any value: the scratch is thrown away
-            sr.nsweeps = 1;
+            sr.t0 = 0;  // any value: the scratch is thrown away
+            sr.nsweeps = sr.nrec = sr.record_every = 1;
             sr.c3base = h->stream_id << 1;
             sr.acc = h->d_acc;
             e = launch_sweeps(pa, c, sr, h->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-            sr.nsweeps = 8 * reps;
+            sr.nsweeps = sr.nrec = 8 * reps;
             if (e == cudaSuccess) e = launch_sweeps(pa, c, sr, h->stream);
             steps = 16 * reps;
         } else if (c.proc_bits == kTinyProcBits) {
@@ -220,16 +226,15 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
             ta.thr4 = h->thr4;
             ta.thr8 = h->thr8;
             ta.c3base = h->stream_id << 1;
-            ta.t0 = 0xFFFFF000u;  // any value: the scratch is thrown away
-            ta.record_every = 0;
-            ta.nrec = 0;
+            ta.t0 = 0;  // any value: the scratch is thrown away
+            ta.record_every = 1;
             ta.acc = h->d_acc;
-            ta.err = reinterpret_cast<unsigned int *>(h->d_acc + 2);  // after the one state slot
-            ta.nsweeps = 1;
-            e = cudaMemsetAsync(h->d_acc + 2, 0, 16, h->stream);
+            ta.err = reinterpret_cast<unsigned int *>(h->d_acc + 2 * (n_rec + 1));  // after the samples and the state
+            ta.nsweeps = ta.nrec = 1;
+            e = cudaMemsetAsync(h->d_acc, 0, 16 * (n_rec + 2), h->stream);
             if (e == cudaSuccess) e = launch_tiny(ta, c.block, c.rows_per_item, c.grid, h->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-            ta.nsweeps = 8 * reps;
+            ta.nsweeps = ta.nrec = 8 * reps;
             if (e == cudaSuccess) e = launch_tiny(ta, c.block, c.rows_per_item, c.grid, h->stream);
             steps = 16 * reps;
         }
@@ -246,7 +251,7 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         if (e == cudaSuccess && c.proc_bits == kTinyProcBits) {
             unsigned int flag = 0;
-            e = cudaMemcpy(&flag, h->d_acc + 2, sizeof flag, cudaMemcpyDeviceToHost);
+            e = cudaMemcpy(&flag, h->d_acc + 2 * (n_rec + 1), sizeof flag, cudaMemcpyDeviceToHost);
             if (e == cudaSuccess && flag) {
                 if (e0) cudaEventDestroy(e0);
                 if (e1) cudaEventDestroy(e1);
@@ -269,17 +274,14 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
     }
     // the draw-ahead form on the copy, or where that is not the whole lattice on a
     // lattice of 32768^2 of the copy's words: the time per site of a large lattice
-    // does not depend on its size
-    const uint64_t La = rows == h->L ? h->L : 32768;
-    const AheadPlan pl = ahead_plan(La, false);
-    bool ahead = false;
+    // does not depend on its size.  Where it could not be timed it stays what it is.
+    bool ahead_slower = h->ahead_slower;
     if (e == cudaSuccess && pl.kw != 0 && La * La / 8 <= rows * row_bytes && ahead_ready(h, pl, La)) {
-        const uint32_t n = std::max(8 * reps, 2 * pl.min_sweeps);
-        unsigned int *const flag = reinterpret_cast<unsigned int *>(h->d_acc + 2);  // after the one state slot
-        e = cudaMemsetAsync(flag, 0, 16, h->stream);
+        unsigned int *const flag = reinterpret_cast<unsigned int *>(h->d_acc + 2 * (n_ahead + 1));
+        e = cudaMemsetAsync(h->d_acc, 0, 16 * (n_ahead + 2), h->stream);
         for (uint32_t k = 0; k < 2 && e == cudaSuccess; ++k) {
             e = cudaEventRecord(e0, h->stream);
-            if (e == cudaSuccess) e = ahead_sweeps(h, pl, scratch, La, 0xFFFF0000u, n, 0, 0, flag, 0, 1ull << 30);
+            if (e == cudaSuccess) e = ahead_sweeps(h, pl, scratch, La, 0, n_ahead, 1, n_ahead, flag, 0, 1ull << 30);
         }
         if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
@@ -288,19 +290,19 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
         unsigned int timeout = 0;
         if (e == cudaSuccess) e = cudaMemcpy(&timeout, flag, sizeof timeout, cudaMemcpyDeviceToHost);
         // (best_step_ms: for `rows` rows)
-        const double step_ms = (double)ms / (2 * n) * ((double)rows * (double)h->L / ((double)La * (double)La));
-        if (e == cudaSuccess && timeout == 0 && step_ms < best_step_ms) {
-            ahead = true;
-            best_step_ms = step_ms;
-        }
+        const double step_ms = (double)ms / (2 * n_ahead) * ((double)rows * (double)h->L / ((double)La * (double)La));
+        if (e == cudaSuccess && log)
+            std::fprintf(stderr, "autotune L=%llu draw-ahead: %.2f us/step\n", (unsigned long long)h->L, 1e3 * step_ms);
+        if (e == cudaSuccess && timeout == 0) ahead_slower = step_ms >= best_step_ms;
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     h->alloc.release(scratch, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "autotune");
     h->launch = best_c;
-    h->ahead = ahead;
-    remember_launch(h->device, h->L, h->word_bits, best_c, ahead);
+    h->configured = false;
+    h->ahead_slower = ahead_slower;
+    remember_launch(h->device, h->L, h->word_bits, best_c, ahead_slower);
     if (best) *best = to_abi(best_c);
     if (best_us_per_step) *best_us_per_step = 1e3 * best_step_ms * ((double)h->L / rows);
     return ISING_OK;

@@ -30,7 +30,8 @@ struct ising_lattice {
     size_t acc_slots = 0;
     void *d_ahead = nullptr;  // scratch of the draw-ahead form (ahead.cu), on first use
     size_t ahead_bytes = 0;
-    bool ahead = true;        // the draw-ahead form where it applies (no configuration set, none found faster)
+    bool configured = false;    // ising_set_launch: that configuration runs, not the draw-ahead form
+    bool ahead_slower = false;  // autotuned: without a field the configuration is faster than its tiles or bands
     ising_form form = ISING_FORM_NONE;  // of the last ising_sweep call
     cudaEvent_t ev = nullptr;
     ising::RoundKeys key{};
@@ -55,10 +56,11 @@ constexpr unsigned char kGuardByte = 0xA5;
 // Launch configuration for a new handle: the autotuned one for (device, L,
 // word width) if there is one, else a fixed default.
 LaunchConfig default_launch(int device, uint64_t L, uint32_t word_bits);
-// Whether a new handle takes the draw-ahead form where it applies: unless the
-// autotuner found the launch configuration faster.
-bool default_ahead(int device, uint64_t L, uint32_t word_bits);
-void remember_launch(int device, uint64_t L, uint32_t word_bits, const LaunchConfig &c, bool ahead);
+// Whether the autotuner found the launch configuration faster than the draw-ahead form of
+// calls without a field (one launch after another: the cluster form and the field have not
+// been timed).
+bool default_ahead_slower(int device, uint64_t L, uint32_t word_bits);
+void remember_launch(int device, uint64_t L, uint32_t word_bits, const LaunchConfig &c, bool ahead_slower);
 std::vector<LaunchConfig> launch_candidates(uint64_t L, uint64_t rows);
 
 // Shared by the ABI translation units.

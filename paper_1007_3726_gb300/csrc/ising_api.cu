@@ -399,7 +399,7 @@ ising_status ising_create(const ising_params *params, void *cuda_stream, ising_l
     if ((st = ensure_acc(h, 64)) != ISING_OK) return bail(st);
 
     h->launch = default_launch(h->device, h->L, wb);
-    h->ahead = default_ahead(h->device, h->L, wb);
+    h->ahead_slower = default_ahead_slower(h->device, h->L, wb);
 
     // initial state
     switch (params->init) {
@@ -486,8 +486,10 @@ ising_status ising_sweep(ising_lattice *h, uint64_t nsweeps, uint32_t record_eve
         const uint64_t v = std::strtoull(max_env, nullptr, 10);
         if (v > 0 && v < max_chunk) max_chunk = v;
     }
-    AheadPlan pl = h->ahead && h->H == 0.0 ? cluster_plan(h->L, nsweeps) : AheadPlan{};
-    if (pl.kw == 0 || !ahead_ready(h, pl, h->L)) pl = h->ahead ? ahead_plan(h->L, h->H != 0.0) : AheadPlan{};
+    const bool field = h->H != 0.0;
+    AheadPlan pl = !h->configured && !field ? cluster_plan(h->L, nsweeps) : AheadPlan{};
+    if (pl.kw == 0 || !ahead_ready(h, pl, h->L))
+        pl = !h->configured && (field || !h->ahead_slower) ? ahead_plan(h->L, field) : AheadPlan{};
     if (pl.kw != 0 && nsweeps >= pl.min_sweeps && ahead_ready(h, pl, h->L)) {
         h->form = pl.cluster ? ISING_FORM_AHEAD_CLUSTER : pl.band_rows ? ISING_FORM_AHEAD_BANDS : ISING_FORM_AHEAD;
         CK(h, ahead_sweeps(h, pl, h->d_spins, h->L, t0, nsweeps, record_every, nrec, err, hold_step, max_chunk));

@@ -123,3 +123,46 @@ def test_step_kernels_on_L524288(P, orc):
         assert np.array_equal(lat.spins(row0, 64), w[margin:margin + 64]), row0
     assert (int(M[-1]), int(E[-1])) == lat.recount()
     lat.close()
+
+
+def test_autotune_without_scratch_leaves_the_default_form(P):
+    """Where the draw-ahead form's scratch is refused while a handle is tuned, the form is
+    not timed and stays the default, for the handle and for later ones."""
+    import torch
+
+    L, refused = 832, []
+
+    def alloc(n, s):
+        if n > 1 << 20:  # the masks, not the lattice or its copy
+            refused.append(n)
+            return None
+        return torch.cuda.caching_allocator_alloc(n)
+
+    P.ising_set_allocator(alloc, lambda p, s: torch.cuda.caching_allocator_delete(p))
+    try:
+        with P.Lattice(L, TC, seed=1) as lat:
+            lat.autotune(reps=1)
+            assert refused
+            lat.sweep(20, 1)
+            assert lat.form != "ahead"  # refused here too
+    finally:
+        P.ising_set_allocator(None)
+    with P.Lattice(L, TC, seed=1) as lat:
+        lat.sweep(20, 1)
+        assert lat.form == "ahead"
+
+
+def test_autotune_returns_the_time_of_the_configuration_it_returns(P, monkeypatch, capfd):
+    monkeypatch.setenv("ISING_AUTOTUNE_LOG", "1")
+    with P.Lattice(448, TC, seed=1) as lat:
+        cfg, us = lat.autotune(reps=2)
+        log = [ln for ln in capfd.readouterr().err.splitlines() if ln.startswith("autotune L=448")]
+        times = [float(ln.split(": ")[1].split()[0]) for ln in log if "draw-ahead" not in ln]
+        assert len(times) == len(P.ising_launch_candidates(448)) and len(log) == len(times) + 1
+        assert abs(us - min(times)) < 0.01
+        # what was not timed stays: calls in a field, and long ones in a cluster
+        lat.sweep(200, 1)
+        assert lat.form == "ahead_cluster"
+        lat.set_field(0.2)
+        lat.sweep(20, 1)
+        assert lat.form == "ahead"
