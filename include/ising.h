@@ -274,7 +274,7 @@ ISING_API const char *ising_last_error(void);
  * keeps.  Where the allocator refuses, or more than 1 GiB and half of the free memory
  * were needed, or while the stream is captured before the scratch is there, the
  * configuration's form runs.  Results are the same.
- * ising_set_launch switches it off for the handle.  (ISING_TINY_HOLD_STEP and
+ * ising_set_launch switches it off for the handle, ising_clear_launch on again.  (ISING_TINY_HOLD_STEP and
  * ISING_TINY_MAX_SWEEPS, for tests only, also act here: the former where an update waits
  * for masks on their way, at L = 64 and in the cluster, the latter as the longest
  * block.)
@@ -301,8 +301,14 @@ ISING_API ising_status ising_batch_form(const ising_batch *b, ising_form *form);
 
 /* The handle's current configuration. */
 ISING_API ising_status ising_get_launch(const ising_lattice *h, ising_launch *out);
-/* Replaces it (ISING_ERR_INVALID if not valid for the handle's L). */
+/* Replaces it (ISING_ERR_INVALID if not valid for the handle's L).  Every later call of the
+ * handle runs that configuration, also where the draw-ahead form would be faster, until
+ * ising_clear_launch or ising_autotune; so does one that ising_get_launch or
+ * ising_autotune has returned. */
 ISING_API ising_status ising_set_launch(ising_lattice *h, const ising_launch *cfg);
+/* Back to what a new handle of this L and word width has: the default configuration (or
+ * the autotuned one), and the draw-ahead form where it applies. */
+ISING_API ising_status ising_clear_launch(ising_lattice *h);
 /* Writes up to cap candidate configurations for lattices of size L to out and
  * returns how many there are in total (out may be NULL to count). */
 ISING_API uint32_t ising_launch_candidates(uint64_t L, ising_launch *out, uint32_t cap);

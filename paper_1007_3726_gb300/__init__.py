@@ -22,7 +22,7 @@ __all__ = [
     "IsingError", "Lattice", "build", "load", "thresholds", "ising_create", "ising_sweep",
     "ising_measure", "ising_measure_from", "ising_destroy", "ising_get_spins", "ising_get_packed", "ising_recount", "ising_get_samples",
     "ising_thresholds", "ising_last_error", "ising_set_allocator", "ising_info",
-    "ising_device_spins", "ising_check_guards", "ising_sweep_noalloc", "ising_bench_mix", "ising_strip_init", "ising_strip_step", "ising_strip_observables", "ising_get_launch", "ising_set_launch", "ising_last_form", "ising_batch_form",
+    "ising_device_spins", "ising_check_guards", "ising_sweep_noalloc", "ising_bench_mix", "ising_strip_init", "ising_strip_step", "ising_strip_observables", "ising_get_launch", "ising_set_launch", "ising_clear_launch", "ising_last_form", "ising_batch_form",
     "ising_launch_candidates", "ising_autotune", "ising_sweep_batch", "ising_batch_tune", "Batch", "Server", "IsingBatchOpts",
     "IsingParams", "IsingLaunch", "IsingObs", "INIT_MODES", "STATUS_NAMES", "FORM_NAMES",
 ]
@@ -146,6 +146,7 @@ def load(path: str | None = None):
         "ising_set_allocator": ([ALLOC_FN, FREE_FN, ctypes.c_void_p], ctypes.c_int),
         "ising_get_launch": ([H, ctypes.POINTER(IsingLaunch)], ctypes.c_int),
         "ising_set_launch": ([H, ctypes.POINTER(IsingLaunch)], ctypes.c_int),
+        "ising_clear_launch": ([H], ctypes.c_int),
         "ising_launch_candidates": ([ctypes.c_uint64, ctypes.POINTER(IsingLaunch), ctypes.c_uint32],
                                     ctypes.c_uint32),
         "ising_autotune": ([H, ctypes.c_uint32, ctypes.POINTER(IsingLaunch),
@@ -353,6 +354,10 @@ def ising_get_launch(h) -> dict:
 
 def ising_set_launch(h, cfg: dict):
     _check(load().ising_set_launch(h, ctypes.byref(IsingLaunch(**cfg))))
+
+
+def ising_clear_launch(h):
+    _check(load().ising_clear_launch(h))
 
 
 def ising_last_form(h) -> str:
@@ -668,12 +673,17 @@ class Lattice:
 
     def set_launch(self, **cfg):
         """Replace the launch configuration; fields not given keep their current
-        values, except that naming proc_bits without persistent means persistent = 0."""
+        values, except that naming proc_bits without persistent means persistent = 0.
+        The handle then runs that configuration until clear_launch() or autotune()."""
         full = dict(self.launch)
         if "proc_bits" in cfg and "persistent" not in cfg:
             full["persistent"] = 0
         full.update(cfg)
         ising_set_launch(self._h, full)
+
+    def clear_launch(self):
+        """Back to the default (or autotuned) configuration and the draw-ahead form."""
+        ising_clear_launch(self._h)
 
     def autotune(self, reps: int = 3) -> tuple[dict, float]:
         """Pick the fastest launch configuration (results do not depend on it)."""

@@ -147,6 +147,16 @@ ISING_API ising_status ising_set_launch(ising_lattice *h, const ising_launch *cf
     return ISING_OK;
 }
 
+ISING_API ising_status ising_clear_launch(ising_lattice *h)
+{
+    clear_error();
+    if (!h) return fail(ISING_ERR_INVALID, "null argument");
+    h->launch = default_launch(h->device, h->L, h->word_bits);
+    h->ahead_slower = default_ahead_slower(h->device, h->L, h->word_bits);
+    h->configured = false;
+    return ISING_OK;
+}
+
 ISING_API uint32_t ising_launch_candidates(uint64_t L, ising_launch *out, uint32_t cap)
 {
     const std::vector<LaunchConfig> v = launch_candidates(L, L);

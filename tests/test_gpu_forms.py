@@ -47,6 +47,21 @@ def test_a_set_configuration_is_what_runs(P):
             assert lat.form == form
 
 
+def test_the_way_back_to_the_default_form(P, orc):
+    with P.Lattice(512, TC, seed=3, init="hot") as lat:
+        default = lat.launch
+        M, forms = [], []
+        for change in (lambda: None, lambda: lat.set_launch(**default), lat.clear_launch,
+                       lambda: lat.set_launch(proc_bits=32, regcap=0, insert=0, block=128, rows_per_item=4, grid=0), lat.clear_launch):
+            change()
+            M.append(lat.sweep(30, 1, collect=True)[0])
+            forms.append(lat.form)
+        assert forms == ["ahead", "one_launch", "ahead", "steps", "ahead"] and lat.launch == default
+        s = orc.init_hot(512, 3, 0)
+        Mo, _ = orc.run(s, 150, 3, 0, *orc.thresholds(TC))
+        assert np.array_equal(np.concatenate(M), Mo) and np.array_equal(lat.spins(), s)
+
+
 def test_form_of_a_batch(P):
     lats = [P.Lattice(L, TC, seed=L) for L in (64, 512)]
     for n, opts, form in ((20, {}, "ahead"), (20, dict(use_graph=True), "ahead"), (4, {}, "strips"), (20, dict(block=512), "strips"),
