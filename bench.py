@@ -535,7 +535,7 @@ def extras(P, stream, peaks, mix):
     lats = [P.Lattice(**WL.lattice_kwargs(sp)) for sp in specs]
     sweeps = [sp["sweeps"] for sp in specs]
     N = sum(sp["L"] ** 2 for sp in specs)
-    opts, _ = P.ising_batch_tune(lats, sweeps, 20)
+    opts, _ = P.ising_batch_tune(lats, sweeps, 20, wait_ms=2000.0)  # (a wait limit: strips only)
     torch.cuda.synchronize()
     with P.Batch(lats, sweeps, specs[0]["record_every"], **opts) as b:
         info = b.info()

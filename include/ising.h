@@ -402,7 +402,8 @@ ISING_API ising_status ising_batch_info(const ising_batch *b, uint32_t *grid, ui
                                         uint32_t *strips, size_t *smem_bytes);
 ISING_API ising_status ising_batch_destroy(ising_batch *b);
 /* Times a few batch configurations (threads per CTA, CTAs per SM, rows per
- * item) on probe runs of about probe_sweeps sweeps (0 = 20) and writes the
+ * item; and none, block = ctas_per_sm = rows_per_item = 0, where the runs would then take
+ * the draw-ahead form) on probe runs of about probe_sweeps sweeps (0 = 20) and writes the
  * fastest into *best (its other fields are kept from *best on entry); the
  * lattices are saved before and restored after, the handles' counters and
  * samples are untouched.  best_ms receives the probe run's time. */

@@ -925,13 +925,23 @@ ising_status alloc_batch(ising_batch *b)
     return ISING_OK;
 }
 
+// No launch option asks for the strips.
+bool default_options(const ising_batch_opts &o)
+{
+    return !o.block && !o.ctas_per_sm && !o.rows_per_item && !o.insert && !o.hold_strip && !(o.wait_ms > 0);
+}
+// Sweeps that the longest of a run's lattices needs for the draw-ahead form.
+uint64_t ahead_min_sweeps(ising_lattice *const *hs, size_t n)
+{
+    return std::all_of(hs, hs + n, [](const ising_lattice *h) { return h->L <= 128; }) ? kAheadMinSweepsSmall : kAheadMinSweeps;
+}
+
 // The draw-ahead form of the runs (ahead.cu) where no launch option asks for the
 // strips, its scratch is to be had and the runs are long enough for it.
 ising_status plan_ahead(ising_batch *b)
 {
     b->use_ahead = false;
-    const bool small = std::all_of(b->hs.begin(), b->hs.end(), [](const ising_lattice *h) { return h->L <= 128; });
-    if (!b->ahead_allowed || *std::max_element(b->sweeps.begin(), b->sweeps.end()) < (small ? kAheadMinSweepsSmall : kAheadMinSweeps))
+    if (!b->ahead_allowed || *std::max_element(b->sweeps.begin(), b->sweeps.end()) < ahead_min_sweeps(b->hs.data(), b->hs.size()))
         return ISING_OK;
     if (!b->ahead.plan(b->hs, b->sweeps, b->record_every)) return ISING_OK;
     if (b->ahead.scratch_bytes > b->ahead_cap) {
@@ -1012,8 +1022,7 @@ ising_status batch_new(int device, const ising_batch_opts *opts, ising_batch **o
         delete b;
         return fail(ISING_ERR_INVALID, "bad batch options");
     }
-    const ising_batch_opts &o = b->opts;
-    b->ahead_allowed = !o.block && !o.ctas_per_sm && !o.rows_per_item && !o.insert && !o.hold_strip && !(o.wait_ms > 0);
+    b->ahead_allowed = default_options(b->opts);
     b->device = device;
     b->alloc = current_allocator();
     // a stream of the batch's own (the legacy default stream cannot be captured)
@@ -1229,13 +1238,19 @@ ISING_API ising_status ising_batch_tune(ising_lattice *const *hs, uint32_t n, co
     // probe sweeps in proportion to the requested ones (at least one each)
     uint64_t maxn = 1;
     for (uint32_t i = 0; i < n; ++i) maxn = std::max<uint64_t>(maxn, nsweeps[i]);
+    // where the runs would take the draw-ahead form without options, so do the probes
+    ising_batch_opts plain = *best;
+    plain.block = plain.ctas_per_sm = plain.rows_per_item = plain.use_graph = plain.hold_strip = 0;
+    const uint64_t ahead_min = ahead_min_sweeps(hs, n);
+    const bool ahead = default_options(plain) && maxn >= ahead_min;
+    if (ahead) probe_sweeps = (uint32_t)std::max<uint64_t>(probe_sweeps, ahead_min);
     std::vector<uint64_t> probe(n);
     for (uint32_t i = 0; i < n; ++i)
         probe[i] = std::max<uint64_t>(1, (uint64_t)((double)probe_sweeps * nsweeps[i] / maxn + 0.5));
     struct Cand {
         uint32_t block, ctas, rows;
     };
-    const Cand cands[] = {{256, 4, 4}, {256, 4, 8}, {256, 3, 4}, {256, 2, 4}, {512, 2, 4},
+    const Cand cands[] = {{0, 0, 0}, {256, 4, 4}, {256, 4, 8}, {256, 3, 4}, {256, 2, 4}, {512, 2, 4},
                           {512, 2, 8}, {512, 1, 4}, {256, 8, 4}, {128, 8, 4}, {128, 16, 4}};
     double best_t = 1e300;
     bool found = false;
@@ -1244,6 +1259,7 @@ ISING_API ising_status ising_batch_tune(ising_lattice *const *hs, uint32_t n, co
     if (e == cudaSuccess) e = cudaEventCreate(&t1);
     for (const Cand &c : cands) {
         if (e != cudaSuccess) break;
+        if (c.block == 0 && !ahead) continue;
         ising_batch_opts o = *best;
         o.block = c.block;
         o.ctas_per_sm = c.ctas;
@@ -1252,6 +1268,10 @@ ISING_API ising_status ising_batch_tune(ising_lattice *const *hs, uint32_t n, co
         o.hold_strip = 0;
         ising_batch *b = nullptr;
         if (ising_batch_create(hs, n, probe.data(), 0, &o, &b) != ISING_OK) continue;  // plan does not fit
+        if (c.block == 0 && !b->use_ahead) {  // (no scratch, or a lattice without tiles: it is a form of the others)
+            ising_batch_destroy(b);
+            continue;
+        }
         for (uint32_t i = 0; i < n; ++i) b->h_t0[i] = (uint32_t)hs[i]->sweeps_done;
         float ms = 0;
         e = enqueue_run(b);  // warm-up

@@ -181,3 +181,23 @@ def test_autotune_returns_the_time_of_the_configuration_it_returns(P, monkeypatc
         lat.set_field(0.2)
         lat.sweep(20, 1)
         assert lat.form == "ahead"
+
+
+@pytest.mark.parametrize("probe", [0, 4])
+def test_batch_tune_weighs_the_default_form_too(P, probe):
+    """Where the runs take the draw-ahead form without options, it is one of the
+    candidates (and by far the fastest on 32 of 512^2); with an option that asks for the
+    strips, or for runs too short for it, it is none."""
+    lats = [P.Lattice(512, 2.0 + 0.02 * i, seed=i) for i in range(32)]
+    before = [l.packed() for l in lats]
+    opts, ms = P.ising_batch_tune(lats, [1000] * 32, probe)
+    assert opts["block"] == opts["ctas_per_sm"] == opts["rows_per_item"] == 0 and ms > 0
+    with P.Batch(lats, [20] * 32, 1, **opts) as b:
+        assert b.form == "ahead"
+    for kw, n in ((dict(wait_ms=500.0), 1000), ({}, 6)):
+        opts, _ = P.ising_batch_tune(lats, [n] * 32, probe, **kw)
+        assert opts["block"] in (128, 256, 512) and opts["wait_ms"] == kw.get("wait_ms", 0.0)
+        with P.Batch(lats, [n] * 32, 1, **opts) as b:
+            assert b.form == "strips"
+    for l, p in zip(lats, before):
+        assert np.array_equal(l.packed(), p) and l.sweeps_done == 0
