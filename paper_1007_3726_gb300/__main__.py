@@ -2,7 +2,7 @@
 
     python -m paper_1007_3726_gb300 --L 32768 --T 2.269185 --seed 7 --init hot \
         --sweeps 1000 --record-every 1 [--word-bits 32] [--H 0.1] [--time]
-    python -m paper_1007_3726_gb300 fss-batch --sweeps 10000   (128 lattices, one launch)
+    python -m paper_1007_3726_gb300 fss-batch --sweeps 10000   (128 lattices)
 """
 import argparse
 import json
@@ -11,13 +11,14 @@ import time
 
 
 def fss_batch(argv):
-    """The 128-lattice finite-size-scaling batch in one persistent launch."""
+    """The 128-lattice finite-size-scaling batch: the default form, or with a launch option
+    (256 threads, 4 CTAs a SM, 4 rows an item are the fastest) strips in one persistent launch."""
     ap = argparse.ArgumentParser(prog="python -m paper_1007_3726_gb300 fss-batch")
     ap.add_argument("--sweeps", type=int, default=10000)
     ap.add_argument("--record-every", type=int, default=10)
-    ap.add_argument("--block", type=int, default=256)
-    ap.add_argument("--ctas-per-sm", type=int, default=4)
-    ap.add_argument("--rows-per-item", type=int, default=4)
+    ap.add_argument("--block", type=int, default=0)
+    ap.add_argument("--ctas-per-sm", type=int, default=0)
+    ap.add_argument("--rows-per-item", type=int, default=0)
     a = ap.parse_args(argv)
 
     import paper_1007_3726_gb300 as P
@@ -29,11 +30,11 @@ def fss_batch(argv):
     t0 = time.perf_counter()
     with P.Batch(lats, [a.sweeps] * len(lats), a.record_every, block=a.block, ctas_per_sm=a.ctas_per_sm,
                  rows_per_item=a.rows_per_item) as b:
-        info = b.info()
+        info, form = b.info(), b.form
         b.run(1)
     el = time.perf_counter() - t0
     N = sum(sp["L"] ** 2 for sp in specs)
-    print(json.dumps({"lattices": len(lats), "sweeps": a.sweeps, "plan": info, "seconds": el,
+    print(json.dumps({"lattices": len(lats), "sweeps": a.sweeps, "form": form, "plan": info, "seconds": el,
                       "attempts_per_ns": N * a.sweeps / el / 1e9}))
     return 0
 

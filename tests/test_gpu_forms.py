@@ -201,3 +201,13 @@ def test_batch_tune_weighs_the_default_form_too(P, probe):
             assert b.form == "strips"
     for l, p in zip(lats, before):
         assert np.array_equal(l.packed(), p) and l.sweeps_done == 0
+
+
+def test_command_line_batch_runs_the_default_form(P, capsys):
+    import json
+
+    from paper_1007_3726_gb300 import __main__ as cli
+
+    for argv, form in (([], "ahead"), (["--block", "256", "--ctas-per-sm", "4"], "strips")):
+        assert cli.main(["fss-batch", "--sweeps", "20", *argv]) == 0
+        assert json.loads(capsys.readouterr().out)["form"] == form
