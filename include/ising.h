@@ -207,6 +207,11 @@ ISING_API ising_status ising_device_spins(const ising_lattice *h, void **dptr, s
  * factor rounds to 1.0 gives 2^32 - 1. */
 ISING_API ising_status ising_thresholds(double T, uint32_t *thr4, uint32_t *thr8);
 
+/* Gives back the scratch memory that idle handles of the current device keep for their next
+ * call, and what the pool of scratch memory keeps (see the draw-ahead form below).  Waits
+ * for the streams of those handles. */
+ISING_API ising_status ising_release_scratch(void);
+
 /* Thread-local text of the last failure on this thread ("" if none). */
 ISING_API const char *ising_last_error(void);
 
@@ -271,7 +276,11 @@ ISING_API const char *ising_last_error(void);
  * scratch memory (buffers of masks, a second lattice: 4 MB at L = 512, in the cluster
  * 25 MB; 103 MB at 4096, 210 MB at 8192, above 210 to 810 MB, in a field up to 2 GB, and
  * the size of the lattice), which the handle allocates on its first such call and
- * keeps.  Where the allocator refuses, or more than 1 GiB and half of the free memory
+ * keeps for the next one while nobody else needs it: idle scratch is given back, the longest
+ * unused first, when the handles of a device would together keep more than a quarter of
+ * its memory, when an allocation of the library would fail, and by ising_release_scratch.
+ * Without an allocator hook it comes from a pool that keeps up to 1 GiB of what was given
+ * back.  Where the allocator refuses, or more than 1 GiB and half of the free memory
  * were needed, or while the stream is captured before the scratch is there, the
  * configuration's form runs.  Results are the same.
  * ising_set_launch switches it off for the handle, ising_clear_launch on again.  (ISING_TINY_HOLD_STEP and
@@ -550,7 +559,8 @@ ISING_API ising_status ising_sweep_noalloc(void *d_spins, uint64_t L, uint32_t w
  * Optional device allocator for every later allocation of the library (for
  * example PyTorch's caching allocator).  alloc(bytes, stream, ctx) returns a
  * device pointer or NULL (reported as ISING_ERR_OOM); release(ptr, stream,
- * ctx) frees it.  Passing NULL functions restores cudaMalloc / cudaFree.  Must
+ * ctx) frees it, also a handle's idle scratch during a call on another handle (that
+ * handle's stream has been waited for).  Passing NULL functions restores cudaMalloc / cudaFree.  Must
  * not be changed while handles created under another allocator are alive.
  */
 typedef void *(*ising_alloc_fn)(size_t bytes, void *cuda_stream, void *ctx);

@@ -22,7 +22,7 @@ __all__ = [
     "IsingError", "Lattice", "build", "load", "thresholds", "ising_create", "ising_sweep",
     "ising_measure", "ising_measure_from", "ising_destroy", "ising_get_spins", "ising_get_packed", "ising_recount", "ising_get_samples",
     "ising_thresholds", "ising_last_error", "ising_set_allocator", "ising_info",
-    "ising_device_spins", "ising_check_guards", "ising_sweep_noalloc", "ising_bench_mix", "ising_strip_init", "ising_strip_step", "ising_strip_observables", "ising_get_launch", "ising_set_launch", "ising_clear_launch", "ising_last_form", "ising_batch_form",
+    "ising_device_spins", "ising_check_guards", "ising_sweep_noalloc", "ising_bench_mix", "ising_strip_init", "ising_strip_step", "ising_strip_observables", "ising_get_launch", "ising_set_launch", "ising_clear_launch", "ising_release_scratch", "ising_last_form", "ising_batch_form",
     "ising_launch_candidates", "ising_autotune", "ising_sweep_batch", "ising_batch_tune", "Batch", "Server", "IsingBatchOpts",
     "IsingParams", "IsingLaunch", "IsingObs", "INIT_MODES", "STATUS_NAMES", "FORM_NAMES",
 ]
@@ -147,6 +147,7 @@ def load(path: str | None = None):
         "ising_get_launch": ([H, ctypes.POINTER(IsingLaunch)], ctypes.c_int),
         "ising_set_launch": ([H, ctypes.POINTER(IsingLaunch)], ctypes.c_int),
         "ising_clear_launch": ([H], ctypes.c_int),
+        "ising_release_scratch": ([], ctypes.c_int),
         "ising_launch_candidates": ([ctypes.c_uint64, ctypes.POINTER(IsingLaunch), ctypes.c_uint32],
                                     ctypes.c_uint32),
         "ising_autotune": ([H, ctypes.c_uint32, ctypes.POINTER(IsingLaunch),
@@ -354,6 +355,11 @@ def ising_get_launch(h) -> dict:
 
 def ising_set_launch(h, cfg: dict):
     _check(load().ising_set_launch(h, ctypes.byref(IsingLaunch(**cfg))))
+
+
+def ising_release_scratch():
+    """Give back the scratch memory that idle handles keep for their next call."""
+    _check(load().ising_release_scratch())
 
 
 def ising_clear_launch(h):

@@ -1339,31 +1339,9 @@ cudaError_t launch_ahead(const AheadPlan &pl, AheadArgs a, bool dependent, cudaS
 
 }  // namespace
 
-bool ahead_ready(ising_lattice *h, const AheadPlan &pl, uint64_t L)
+size_t ahead_bytes(const AheadPlan &pl, uint64_t L)
 {
-    const size_t need = kTicketBytes + (pl.cluster ? kClusterBuffers : kBuffers) * pl.mask_bytes + 2 * pl.snap_bytes + (pl.halo && !pl.cluster ? (size_t)(L * L / 8) : 0);
-    if (h->ahead_bytes >= need) return true;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return false;  // no allocation while the stream is captured
-    }
-    if (h->d_ahead) {  // a smaller one, of the form without a field
-        if (cudaStreamSynchronize(h->stream) != cudaSuccess) return false;
-        h->alloc.release_scratch(h->d_ahead, h->stream);
-        h->d_ahead = nullptr;
-        h->ahead_bytes = 0;
-    }
-    // a second copy of a lattice that fills the GPU would take what its user may need:
-    // at most half of what is free
-    size_t free_bytes = 0, total_bytes = 0;
-    if (need > kPoolKeeps && (cudaMemGetInfo(&free_bytes, &total_bytes) != cudaSuccess || need > free_bytes / 2)) {
-        cudaGetLastError();
-        return false;
-    }
-    h->d_ahead = h->alloc.scratch(need, h->stream);
-    h->ahead_bytes = h->d_ahead ? need : 0;
-    return h->d_ahead != nullptr;
+    return kTicketBytes + (pl.cluster ? kClusterBuffers : kBuffers) * pl.mask_bytes + 2 * pl.snap_bytes + (pl.halo && !pl.cluster ? (size_t)(L * L / 8) : 0);
 }
 
 // Blocks of 4 sweeps (the rest of a division by 4 first), each in bands of rows.
@@ -1578,8 +1556,8 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
 {
     const uint32_t full = (uint32_t)std::min<uint64_t>(pl.block_sweeps, max_block);
     const size_t bytes = (size_t)(L * L / 8);
-    unsigned int *const tickets = static_cast<unsigned int *>(h->d_ahead);
-    char *const masks = static_cast<char *>(h->d_ahead) + kTicketBytes;
+    unsigned int *const tickets = static_cast<unsigned int *>(h->scratch.p);
+    char *const masks = static_cast<char *>(h->scratch.p) + kTicketBytes;
     char *const snaps = masks + (pl.cluster ? kClusterBuffers : kBuffers) * pl.mask_bytes;
     uint64_t *const spins = static_cast<uint64_t *>(lattice);
     uint64_t *const other = pl.halo ? reinterpret_cast<uint64_t *>(snaps + 2 * pl.snap_bytes) : spins;

@@ -133,12 +133,10 @@ struct AheadBatchArgs {
 struct ising_lattice;
 
 namespace ising {
-// The handle's scratch for the plan of size L (masks, snapshots, a second lattice), allocated
-// on first use and kept; false when there is none to be had (the allocator refuses,
-// or the stream is being captured): the caller then takes another path.
-bool ahead_ready(ising_lattice *h, const AheadPlan &pl, uint64_t L);
+// Bytes of scratch that the plan of size L works in (masks, snapshots, a second lattice).
+size_t ahead_bytes(const AheadPlan &pl, uint64_t L);
 // Queues nsweeps sweeps of `lattice` (the handle's, or scratch of L^2 sites) from sweep
-// index t0 on the handle's stream; counters as TinyRunArgs.  A block holds at most
+// index t0 on the handle's stream, in its scratch; counters as TinyRunArgs.  A block holds at most
 // max_block sweeps.
 cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, uint64_t L, uint64_t t0,
                          uint64_t nsweeps, uint32_t record_every, uint64_t nrec, unsigned int *err, uint32_t hold_step, uint64_t max_block);

@@ -286,7 +286,8 @@ ISING_API ising_status ising_autotune(ising_lattice *h, uint32_t reps, ising_lau
     // lattice of 32768^2 of the copy's words: the time per site of a large lattice
     // does not depend on its size.  Where it could not be timed it stays what it is.
     bool ahead_slower = h->ahead_slower;
-    if (e == cudaSuccess && pl.kw != 0 && La * La / 8 <= rows * row_bytes && ahead_ready(h, pl, La)) {
+    ScratchUse use;
+    if (e == cudaSuccess && pl.kw != 0 && La * La / 8 <= rows * row_bytes && use.begin(h->scratch, ahead_bytes(pl, La))) {
         unsigned int *const flag = reinterpret_cast<unsigned int *>(h->d_acc + 2 * (n_ahead + 1));
         e = cudaMemsetAsync(h->d_acc, 0, 16 * (n_ahead + 2), h->stream);
         for (uint32_t k = 0; k < 2 && e == cudaSuccess; ++k) {

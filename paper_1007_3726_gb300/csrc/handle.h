@@ -28,8 +28,7 @@ struct ising_lattice {
     unsigned long long *d_acc = nullptr;  // 2 counters per slot
     unsigned long long *h_acc = nullptr;  // pinned mirror
     size_t acc_slots = 0;
-    void *d_ahead = nullptr;  // scratch of the draw-ahead form (ahead.cu), on first use
-    size_t ahead_bytes = 0;
+    ising::Scratch scratch;   // of the draw-ahead form (ahead.cu)
     bool configured = false;    // ising_set_launch: that configuration runs, not the draw-ahead form
     bool ahead_slower = false;  // autotuned: without a field the configuration is faster than its tiles or bands
     ising_form form = ISING_FORM_NONE;  // of the last ising_sweep call

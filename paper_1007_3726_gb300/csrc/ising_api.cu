@@ -54,85 +54,6 @@ Allocator current_allocator()
     return Allocator{g_alloc, g_free, g_alloc_ctx};
 }
 
-namespace {
-constexpr int kMaxDevices = 64;
-std::mutex g_pool_mu;
-cudaMemPool_t g_pool[kMaxDevices] = {};
-
-// The scratch pool of the current device, made on first use; nullptr if there is none.
-cudaMemPool_t device_pool()
-{
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-    std::lock_guard<std::mutex> lk(g_pool_mu);
-    if (!g_pool[dev]) {
-        cudaMemPoolProps props{};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        uint64_t keeps = kPoolKeeps;
-        cudaMemPool_t pool = nullptr;
-        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
-            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keeps) != cudaSuccess) {
-            cudaGetLastError();
-            if (pool) cudaMemPoolDestroy(pool);
-            return nullptr;
-        }
-        g_pool[dev] = pool;
-    }
-    return g_pool[dev];
-}
-
-// Gives back what the pools of all devices keep unused.
-void trim_pools()
-{
-    std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (cudaMemPool_t p : g_pool)
-        if (p) cudaMemPoolTrimTo(p, 0);
-}
-}  // namespace
-
-void *Allocator::allocate(size_t bytes, cudaStream_t s) const
-{
-    if (bytes == 0) bytes = 16;
-    if (alloc) return alloc(bytes, (void *)s, ctx);
-    void *p = nullptr;
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
-        cudaGetLastError();  // clear the (non-sticky) allocation error
-        if (attempt == 0) trim_pools();
-    }
-    return nullptr;
-}
-
-void Allocator::release(void *p, cudaStream_t s) const
-{
-    if (!p) return;
-    if (free_fn)
-        free_fn(p, (void *)s, ctx);
-    else
-        cudaFree(p);
-}
-
-void *Allocator::scratch(size_t bytes, cudaStream_t s) const
-{
-    if (alloc) return allocate(bytes, s);
-    const cudaMemPool_t pool = device_pool();
-    void *p = nullptr;
-    if (pool && cudaMallocFromPoolAsync(&p, bytes ? bytes : 16, pool, s) == cudaSuccess) return p;
-    cudaGetLastError();
-    return nullptr;
-}
-
-void Allocator::release_scratch(void *p, cudaStream_t s) const
-{
-    if (!p) return;
-    if (free_fn)
-        free_fn(p, (void *)s, ctx);
-    else
-        cudaFreeAsync(p, s);
-}
-
 // ------------------------------------------------------------ thresholds ---
 // floor(2^32 exp(-dE / T)) in FP64 (Sec. 3: the acceptance factors of the two
 // positive energy changes are fixed on the CPU for each temperature).
@@ -234,7 +155,7 @@ void destroy_all(ising_lattice *h)
     cudaStreamSynchronize(h->stream);
     h->alloc.release(h->d_base, h->stream);
     h->alloc.release(h->d_acc, h->stream);
-    h->alloc.release_scratch(h->d_ahead, h->stream);
+    scratch_drop(h->scratch);
     if (h->h_acc) cudaFreeHost(h->h_acc);
     if (h->ev) cudaEventDestroy(h->ev);
     delete h;
@@ -346,6 +267,13 @@ ising_status ising_set_allocator(ising_alloc_fn alloc, ising_free_fn release, vo
     return ISING_OK;
 }
 
+ising_status ising_release_scratch(void)
+{
+    clear_error();
+    scratch_give_back();
+    return ISING_OK;
+}
+
 ising_status ising_create(const ising_params *params, void *cuda_stream, ising_lattice **out)
 {
     clear_error();
@@ -370,6 +298,8 @@ ising_status ising_create(const ising_params *params, void *cuda_stream, ising_l
     h->bytes = (size_t)(params->L * params->L / 8);
     h->stream = (cudaStream_t)cuda_stream;
     h->alloc = current_allocator();
+    h->scratch.alloc = h->alloc;
+    h->scratch.stream = h->stream;
     h->key = make_round_keys(params->seed);
     h->sweeps_done = params->first_sweep;
     cudaError_t e = cudaGetDevice(&h->device);
@@ -377,6 +307,7 @@ ising_status ising_create(const ising_params *params, void *cuda_stream, ising_l
         delete h;
         return fail(ISING_ERR_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
     }
+    h->scratch.device = h->device;
     auto bail = [&](ising_status s) {
         std::string msg = g_last_error;
         destroy_all(h);
@@ -487,10 +418,13 @@ ising_status ising_sweep(ising_lattice *h, uint64_t nsweeps, uint32_t record_eve
         if (v > 0 && v < max_chunk) max_chunk = v;
     }
     const bool field = h->H != 0.0;
+    ScratchUse use;
     AheadPlan pl = !h->configured && !field ? cluster_plan(h->L, nsweeps) : AheadPlan{};
-    if (pl.kw == 0 || !ahead_ready(h, pl, h->L))
+    if (pl.kw == 0 || !use.begin(h->scratch, ahead_bytes(pl, h->L))) {
         pl = !h->configured && (field || !h->ahead_slower) ? ahead_plan(h->L, field) : AheadPlan{};
-    if (pl.kw != 0 && nsweeps >= pl.min_sweeps && ahead_ready(h, pl, h->L)) {
+        if (pl.kw != 0 && (nsweeps < pl.min_sweeps || !use.begin(h->scratch, ahead_bytes(pl, h->L)))) pl.kw = 0;
+    }
+    if (pl.kw != 0) {
         h->form = pl.cluster ? ISING_FORM_AHEAD_CLUSTER : pl.band_rows ? ISING_FORM_AHEAD_BANDS : ISING_FORM_AHEAD;
         CK(h, ahead_sweeps(h, pl, h->d_spins, h->L, t0, nsweeps, record_every, nrec, err, hold_step, max_chunk));
         h->pending_err = true;

@@ -90,3 +90,89 @@ def test_invalid_first_sweep_and_counter_limit(P):
     with pytest.raises(P.IsingError) as ei:
         lat.sweep(1)
     assert ei.value.status == P.ERR_INVALID
+
+
+def test_scratch_of_many_handles_is_bounded_and_given_back(P, orc, monkeypatch):
+    """Handles swept in turn keep scratch up to a bound together (here 100 MB; one of these
+    takes 25 MB): all run the draw-ahead form, and lattices and samples are the oracle's
+    although a handle's scratch was another's a call before.  Scratch also gives way to a
+    lattice that would not fit beside it."""
+    import torch
+
+    monkeypatch.setenv("ISING_SCRATCH_MB", "100")
+    taken, most, room = {}, [0], [1 << 40]
+
+    def alloc(n, s):
+        if sum(taken.values()) + n > room[0]:
+            return None
+        p = torch.cuda.caching_allocator_alloc(n)
+        taken[p] = n
+        most[0] = max(most[0], sum(v for v in taken.values() if v > 20 << 20))
+        return p
+
+    def release(p, s):
+        taken.pop(p)
+        torch.cuda.caching_allocator_delete(p)
+
+    L, n, k = 512, 200, 7
+    for hook in (True, False):
+        if hook:
+            P.ising_set_allocator(alloc, release)
+        try:
+            streams = [torch.cuda.Stream() for _ in range(k)]
+            lats = [P.Lattice(L, 2.2 + 0.02 * i, seed=i, init="hot", stream=streams[i]) for i in range(k)]
+            for _ in range(2):
+                for lat in lats:
+                    lat.sweep(n, 4)  # queued only
+                    assert lat.form == "ahead_cluster"
+            for i, lat in enumerate(lats):
+                s = orc.init_hot(L, i, 0)
+                Mo, Eo = orc.run(s, 2 * n, i, 0, *orc.thresholds(2.2 + 0.02 * i))
+                M, E = lat.samples()
+                assert np.array_equal(M, Mo[3::4]) and np.array_equal(E, Eo[3::4]) and np.array_equal(lat.spins(), s)
+            if hook:
+                assert 20 << 20 < most[0] <= 100 << 20
+                room[0] = sum(taken.values()) + (20 << 20)
+                with P.Lattice(16384, 2.0, seed=1) as big:  # 32 MB
+                    assert big.sweeps_done == 0
+                room[0] = 1 << 40
+            P.ising_release_scratch()
+            assert not hook or not any(v > 20 << 20 for v in taken.values())
+            lats[0].sweep(n, 4)
+            assert lats[0].form == "ahead_cluster"
+            for lat in lats:
+                lat.close()
+            assert not taken
+        finally:
+            if hook:
+                P.ising_set_allocator(None)
+
+
+def test_scratch_is_taken_from_handles_on_other_threads(P, orc, monkeypatch):
+    """Threads with a handle each, on streams of their own, that take one another's idle
+    scratch all the time (a bound of two)."""
+    import threading
+
+    import torch
+
+    monkeypatch.setenv("ISING_SCRATCH_MB", "52")
+    L, n, out = 512, 192, {}
+
+    def work(i):
+        st = torch.cuda.Stream()
+        with P.Lattice(L, 2.25, seed=i, init="hot", stream=st) as lat:
+            r = []
+            for _ in range(6):
+                r.append(lat.sweep(n, 3, collect=True))
+            out[i] = (np.concatenate([m for m, _ in r]), np.concatenate([e for _, e in r]), lat.spins())
+
+    th = [threading.Thread(target=work, args=(i,)) for i in range(5)]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    assert len(out) == 5
+    for i, (M, E, spins) in out.items():
+        s = orc.init_hot(L, i, 0)
+        Mo, Eo = orc.run(s, 6 * n, i, 0, *orc.thresholds(2.25))
+        assert np.array_equal(M, Mo[2::3]) and np.array_equal(E, Eo[2::3]) and np.array_equal(spins, s)
