@@ -16,6 +16,7 @@ namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {};
+std::set<void *> g_plain;  // staging memory from cudaMalloc
 
 // The scratch pool of the current device, made on first use; nullptr if there is none.
 cudaMemPool_t device_pool()
@@ -185,7 +186,13 @@ void Allocator::release(void *p, cudaStream_t s) const
 void *Allocator::scratch(size_t bytes, cudaStream_t s) const
 {
     if (alloc) return allocate(bytes, s);
-    return from_pool(bytes, s);
+    if (void *p = from_pool(bytes, s)) return p;
+    void *p = allocate(bytes, s);  // no pool, or it is full: what is idle goes, the pools are trimmed
+    if (p) {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        g_plain.insert(p);
+    }
+    return p;
 }
 
 void Allocator::release_scratch(void *p, cudaStream_t s) const
@@ -195,7 +202,12 @@ void Allocator::release_scratch(void *p, cudaStream_t s) const
         free_fn(p, (void *)s, ctx);
         return;
     }
-    if (cudaFreeAsync(p, s) == cudaSuccess) return;
+    bool plain;
+    {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        plain = g_plain.erase(p) != 0;
+    }
+    if (!plain && cudaFreeAsync(p, s) == cudaSuccess) return;
     cudaGetLastError();
     cudaFree(p);
 }

@@ -34,7 +34,8 @@ struct Allocator {
     void release(void *p, cudaStream_t s) const;
     // Scratch and staging memory, used in the order of stream s: from the hook, or
     // from a pool per device that keeps at most kPoolKeeps bytes of what was
-    // released, so that a handle that comes and goes does not map and unmap its scratch.
+    // released, so that a handle that comes and goes does not map and unmap its scratch
+    // (where there is no pool, or it has no room, from cudaMalloc).
     void *scratch(size_t bytes, cudaStream_t s) const;
     void release_scratch(void *p, cudaStream_t s) const;
 };

@@ -177,6 +177,15 @@ int main()
     CHECK(!call(s[3], 20 * MB) && !s[3].p);
     al.release(big, nullptr);
     CHECK(call(s[3], 20 * MB));
+    // staging memory that the pool has no piece for comes from elsewhere, once what the
+    // pool keeps has been trimmed, and goes back there
+    pool_reserved = 900 * MB;
+    fragmented = true;
+    void *st = al.scratch(400 * MB, nullptr);
+    CHECK(st && sum(plain) == 400 * MB && pool_reserved == 60 * MB && !s[3].p);
+    al.release_scratch(st, nullptr);
+    CHECK(plain.empty());
+    fragmented = false;
     // hooks: released without the lock, after their stream has been waited for
     Scratch h[3];
     for (int k = 0; k < 3; ++k) { h[k].alloc = Allocator{hook_alloc, hook_free, nullptr}; h[k].stream = stream(100 + k); }
@@ -220,3 +229,24 @@ int main()
 
 def test_scratch_is_bounded_and_given_back(tmp_path):
     _run(tmp_path, SCRATCH_BOOK, "memory.cu")
+
+
+NO_POOL = FAKE_CUDART + r"""
+int main()
+{
+    // a device without memory pools: staging memory still comes, scratch does not
+    pools = false;
+    Allocator al;
+    void *st = al.scratch(100 * MB, nullptr);
+    CHECK(st && sum(plain) == 100 * MB);
+    al.release_scratch(st, nullptr);
+    CHECK(plain.empty());
+    Scratch s;
+    CHECK(!scratch_begin(s, MB) && !s.p && plain.empty());
+    return 0;
+}
+"""
+
+
+def test_staging_memory_without_memory_pools(tmp_path):
+    _run(tmp_path, NO_POOL, "memory.cu")
