@@ -581,7 +581,7 @@ void free_batch(ising_batch *b)
     if (b->graph) cudaGraphDestroy(b->graph);
     b->alloc.release(b->d_plan, b->stream);
     b->alloc.release(b->d_work, b->stream);
-    b->alloc.release_scratch(b->d_ahead, b->stream);
+    scratch_drop(b->scratch);
     if (b->h_counters) cudaFreeHost(b->h_counters);
     if (b->h_t0) cudaFreeHost(b->h_t0);
     if (b->h_error) cudaFreeHost(b->h_error);
@@ -936,34 +936,39 @@ uint64_t ahead_min_sweeps(ising_lattice *const *hs, size_t n)
     return std::all_of(hs, hs + n, [](const ising_lattice *h) { return h->L <= 128; }) ? kAheadMinSweepsSmall : kAheadMinSweeps;
 }
 
+// The scratch of the draw-ahead form, with the plan's table in it (again, if it was given
+// back in between); without it the runs go in strips.
+ising_status place_ahead(ising_batch *b, ScratchUse &use)
+{
+    b->use_ahead = false;
+    if (!b->ahead_planned || !use.begin(b->scratch, b->ahead.scratch_bytes)) return ISING_OK;
+    if (b->placed != b->scratch.made) {
+        std::vector<unsigned long long *> acc, final_acc;
+        unsigned long long *const counters = reinterpret_cast<unsigned long long *>(static_cast<char *>(b->d_work) + b->off_counters);
+        for (size_t i = 0; i < b->hs.size(); ++i) {
+            acc.push_back(counters + 2 * b->sample_base[i]);
+            final_acc.push_back(acc.back() + 2 * b->nrec[i]);
+        }
+        const cudaError_t e = b->ahead.upload(b->scratch.p, b->hs, acc, final_acc, b->stream);
+        if (e != cudaSuccess) return bfail(b, e, "batch table upload");
+        b->placed = b->scratch.made;
+    }
+    b->use_ahead = true;
+    return ISING_OK;
+}
+
 // The draw-ahead form of the runs (ahead.cu) where no launch option asks for the
 // strips, its scratch is to be had and the runs are long enough for it.
 ising_status plan_ahead(ising_batch *b)
 {
     b->use_ahead = false;
-    if (!b->ahead_allowed || *std::max_element(b->sweeps.begin(), b->sweeps.end()) < ahead_min_sweeps(b->hs.data(), b->hs.size()))
-        return ISING_OK;
-    if (!b->ahead.plan(b->hs, b->sweeps, b->record_every)) return ISING_OK;
-    if (b->ahead.scratch_bytes > b->ahead_cap) {
-        cudaStreamSynchronize(b->stream);
-        b->alloc.release_scratch(b->d_ahead, b->stream);
-        b->ahead_cap = b->ahead.scratch_bytes;
-        b->d_ahead = b->alloc.scratch(b->ahead_cap, b->stream);
-        if (!b->d_ahead) {
-            b->ahead_cap = 0;
-            return ISING_OK;
-        }
-    }
-    std::vector<unsigned long long *> acc, final_acc;
-    unsigned long long *const counters = reinterpret_cast<unsigned long long *>(static_cast<char *>(b->d_work) + b->off_counters);
-    for (size_t i = 0; i < b->hs.size(); ++i) {
-        acc.push_back(counters + 2 * b->sample_base[i]);
-        final_acc.push_back(acc.back() + 2 * b->nrec[i]);
-    }
-    const cudaError_t e = b->ahead.upload(b->d_ahead, b->hs, acc, final_acc, b->stream);
-    if (e != cudaSuccess) return bfail(b, e, "batch table upload");
-    b->use_ahead = true;
-    return ISING_OK;
+    b->placed = 0;
+    b->ahead_planned = b->ahead_allowed &&
+                       *std::max_element(b->sweeps.begin(), b->sweeps.end()) >= ahead_min_sweeps(b->hs.data(), b->hs.size()) &&
+                       b->ahead.plan(b->hs, b->sweeps, b->record_every) && b->ahead.scratch_bytes <= b->ahead_budget;
+    if (scratch_bytes(b->scratch) > b->ahead_budget) scratch_drop(b->scratch);
+    ScratchUse use;
+    return place_ahead(b, use);
 }
 
 // Work of one run on the batch stream: clear the counters, progress and error
@@ -1024,7 +1029,8 @@ ising_status batch_new(int device, const ising_batch_opts *opts, ising_batch **o
     }
     b->ahead_allowed = default_options(b->opts);
     b->device = device;
-    b->alloc = current_allocator();
+    b->alloc = b->scratch.alloc = current_allocator();
+    b->scratch.device = device;
     // a stream of the batch's own (the legacy default stream cannot be captured)
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
@@ -1032,6 +1038,7 @@ ising_status batch_new(int device, const ising_batch_opts *opts, ising_batch **o
         return fail(ISING_ERR_CUDA, "stream creation failed");
     }
     b->own_stream = true;
+    b->scratch.stream = b->stream;
     if (cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         batch_free(b);
@@ -1061,6 +1068,7 @@ ising_status batch_replan(ising_batch *b, const std::vector<ising_lattice *> &hs
     if (b->graph) cudaGraphDestroy(b->graph);
     b->graph_exec = nullptr;
     b->graph = nullptr;
+    scratch_pin(b->scratch, false);
     b->hs = hs;
     b->sweeps = sweeps;
     b->record_every = record_every;
@@ -1125,6 +1133,11 @@ ISING_API ising_status ising_batch_run(ising_batch *b, uint32_t runs)
     cudaError_t e = cudaSetDevice(b->device);
     if (e != cudaSuccess) return bfail(b, e, "cudaSetDevice");
     const size_t n = b->hs.size();
+    ScratchUse use;
+    if (!b->graph_exec) {  // (a captured run keeps its form and its scratch)
+        ising_status st = place_ahead(b, use);
+        if (st != ISING_OK) return st;
+    }
     for (uint32_t r = 0; r < runs; ++r) {
         for (size_t i = 0; i < n; ++i) {
             ising_lattice *h = b->hs[i];
@@ -1150,6 +1163,7 @@ ISING_API ising_status ising_batch_run(ising_batch *b, uint32_t runs)
                 }
                 if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph_exec, b->graph, 0);
                 if (e != cudaSuccess) return bfail(b, e, "batch graph capture");
+                scratch_pin(b->scratch, b->use_ahead);
             }
             e = cudaGraphLaunch(b->graph_exec, b->stream);
         } else {
@@ -1274,13 +1288,17 @@ ISING_API ising_status ising_batch_tune(ising_lattice *const *hs, uint32_t n, co
         }
         for (uint32_t i = 0; i < n; ++i) b->h_t0[i] = (uint32_t)hs[i]->sweeps_done;
         float ms = 0;
-        e = enqueue_run(b);  // warm-up
-        if (e == cudaSuccess) e = cudaEventRecord(t0, b->stream);
-        if (e == cudaSuccess) e = enqueue_run(b);
-        if (e == cudaSuccess) e = cudaEventRecord(t1, b->stream);
-        if (e == cudaSuccess) e = cudaEventSynchronize(t1);
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, t0, t1);
-        const bool ok = e == cudaSuccess && *b->h_error == 0u;
+        {
+            ScratchUse use;
+            if (place_ahead(b, use) != ISING_OK) e = cudaErrorUnknown;
+            if (e == cudaSuccess) e = enqueue_run(b);  // warm-up
+            if (e == cudaSuccess) e = cudaEventRecord(t0, b->stream);
+            if (e == cudaSuccess) e = enqueue_run(b);
+            if (e == cudaSuccess) e = cudaEventRecord(t1, b->stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(t1);
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, t0, t1);
+        }
+        const bool ok = e == cudaSuccess && *b->h_error == 0u && (c.block != 0 || b->use_ahead);
         b->hs.clear();  // the handles are not part of the probe's failure
         free_batch(b);
         if (ok && ms < best_t) {

@@ -62,9 +62,11 @@ struct ising_batch {
     bool field = false;                     // a lattice is in a field: the field kernel
     ising::AheadBatch ahead;                // the draw-ahead form of the runs
     bool ahead_allowed = false;             // no launch option asks for the strips
-    bool use_ahead = false;                 // planned and placed
-    void *d_ahead = nullptr;
-    size_t ahead_cap = 0;
+    bool ahead_planned = false;             // the runs can take it
+    bool use_ahead = false;                 // and have the scratch
+    ising::Scratch scratch;
+    uint64_t placed = 0;                    // the allocation that the plan's table is in (0: none)
+    size_t ahead_budget = ~(size_t)0;       // bytes that the scratch may take
     bool failed = false;
 };
 

@@ -79,7 +79,7 @@ void *from_pool(size_t bytes, cudaStream_t s)
 // ---------------------------------------------------------------- the book --
 std::mutex g_book_mu;
 std::set<Scratch *> g_held;  // owners with memory
-uint64_t g_use = 0;
+uint64_t g_use = 0;          // uses and allocations, counted
 
 struct HookFree {
     Allocator alloc;
@@ -274,6 +274,7 @@ bool scratch_begin(Scratch &s, size_t need)
     std::lock_guard<std::mutex> lk(g_book_mu);
     s.p = p;
     s.bytes = need;
+    s.made = ++g_use;
     s.busy = true;
     g_held.insert(&s);
     return true;
@@ -303,6 +304,12 @@ void scratch_drop(Scratch &s)
         s.busy = s.pinned = false;
     }
     s.alloc.release_scratch(p, s.stream);
+}
+
+size_t scratch_bytes(const Scratch &s)
+{
+    std::lock_guard<std::mutex> lk(g_book_mu);
+    return s.bytes;
 }
 
 void scratch_give_back()

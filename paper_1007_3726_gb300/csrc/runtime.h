@@ -54,6 +54,7 @@ struct Scratch {
     int device = 0;
     void *p = nullptr;
     size_t bytes = 0;
+    uint64_t made = 0;      // which allocation it is: another number, other contents
     // under the book's lock
     bool busy = false;      // a call is queueing work that uses it
     bool pinned = false;    // a captured graph holds its address: never given back
@@ -65,6 +66,7 @@ bool scratch_begin(Scratch &s, size_t need);
 void scratch_end(Scratch &s);                // all work that uses it is queued
 void scratch_pin(Scratch &s, bool pinned);
 void scratch_drop(Scratch &s);               // the owner ends; its stream's work is done
+size_t scratch_bytes(const Scratch &s);      // that it holds now
 void scratch_give_back();                    // all idle scratch of the current device, and the pools
 size_t scratch_limit(int device);
 

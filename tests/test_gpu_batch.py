@@ -213,3 +213,54 @@ def test_binder_crossing_small_lattices(P):
     tc = 2.0 / math.log(1.0 + math.sqrt(2.0))
     assert cr["T_cross"] is not None
     assert abs(cr["T_cross"] - tc) < max(0.02, 5 * (cr["err"] or 0.0))
+
+
+def test_batch_whose_scratch_is_given_back_between_runs(P):
+    """A batch keeps scratch between runs as a handle does: a run after it was given back
+    places its tables again, one that gets none runs in strips, and a captured run keeps
+    what its graph holds."""
+    specs = [(512, 2.2, 1), (1024, 2.3, 2), (256, 2.4, 3)]
+    sweeps = [16, 12, 20]
+    ref = [P.Lattice(L, T, seed=s, init="hot") for L, T, s in specs]
+    for l, n in zip(ref, sweeps):
+        l.sweep(4 * n, 1)
+    held, refuse = {}, []
+    import torch
+
+    def alloc(n, s):
+        if refuse and n > 1 << 20:
+            return None
+        p = torch.cuda.caching_allocator_alloc(n)
+        held[p] = n
+        return p
+
+    def release(p, s):
+        held.pop(p)
+        torch.cuda.caching_allocator_delete(p)
+
+    P.ising_set_allocator(alloc, release)
+    try:
+        for graph in (False, True):
+            lats = [P.Lattice(L, T, seed=s, init="hot") for L, T, s in specs]
+            with P.Batch(lats, sweeps, 1, use_graph=graph) as b:
+                big = lambda: sum(v for v in held.values() if v > 1 << 20)  # noqa: E731
+                assert b.form == "ahead" and big()
+                P.ising_release_scratch()
+                assert not big()
+                b.run(1)
+                assert b.form == "ahead" and big()
+                P.ising_release_scratch()
+                assert bool(big()) == graph
+                refuse.append(1)
+                b.run(1)
+                assert b.form == ("ahead" if graph else "strips")
+                refuse.clear()
+                b.run(2)
+                assert b.form == "ahead"
+            for l, r in zip(lats, ref):
+                assert np.array_equal(l.spins(), r.spins())
+                assert np.array_equal(np.stack(l.samples()), np.stack(r.samples()))
+                l.close()
+            assert not held
+    finally:
+        P.ising_set_allocator(None)
