@@ -371,7 +371,9 @@ ISING_API ising_status ising_bench_mix(uint32_t form, uint32_t words_per_thread,
  * L = 4096 (in a field 2048) in a batch without launch options (block .. insert,
  * wait_ms, hold_strip all zero) take the draw-ahead form of ising_launch instead, over
  * all lattices at once, if its scratch memory (at least three times a byte per lattice
- * site, in a field 2.5) is to be had; ising_batch_info still describes the strips.
+ * site, in a field 2.5) is to be had; ising_batch_info still describes the strips.  The
+ * scratch is kept between runs as a handle's is (a batch that has captured its run keeps it
+ * until it is destroyed), and a run whose scratch is not to be had any more runs in strips.
  *
  * Options (zero = default):
  *   block          threads per CTA, 128, 256 or 512 (512)
@@ -436,7 +438,9 @@ ISING_API ising_status ising_sweep_batch(ising_lattice *const *hs, uint32_t n, c
  */
 typedef struct ising_server ising_server;
 typedef struct {
-    uint64_t hbm_budget_bytes;  /* device memory of resident lattices (0 = 64 GiB) */
+    uint64_t hbm_budget_bytes;  /* device memory of resident lattices and of the scratch that
+                                   their launches work in (0 = 64 GiB); lattices come first:
+                                   where no room is left for the scratch, launches run in strips */
     uint32_t epoch_sweeps;      /* sweeps per lattice per launch at most (0 = 1000) */
     uint32_t max_active;        /* lattices per launch at most (0 = as shared memory allows) */
     uint32_t keep_samples;      /* 1: keep each request's M/E samples for ising_server_samples */
@@ -458,7 +462,7 @@ typedef struct {
 } ising_result;
 typedef struct {
     uint64_t submitted, admitted, completed, failed, cancelled, queued, resident;
-    uint64_t epochs, mem_used, peak_mem, attempts;
+    uint64_t epochs, mem_used, peak_mem, attempts;  /* mem_*: lattices and scratch */
     double busy_seconds;        /* time inside launches */
     double now;                 /* seconds since the server started */
 } ising_server_counters;

@@ -62,6 +62,7 @@ struct ising_server {
     ising_server_counters stats{};
     ising_batch *batch = nullptr;
     bool ahead_allowed = false;
+    size_t scratch = 0;                 // bytes of the batch's scratch, as of the last admission or plan
     std::vector<uint64_t> plan_ids;     // request ids of the current plan (handle addresses are reused)
     std::vector<uint64_t> plan_sweeps;
     std::string worker_error;
@@ -102,6 +103,13 @@ void finish(ising_server *s, Request *r, ising_status st)
     s->cv_done.notify_all();
 }
 
+// The budget is for the lattices and for what the batch works in besides (under the lock).
+void note_memory(ising_server *s)
+{
+    s->scratch = s->batch ? scratch_bytes(s->batch->scratch) : 0;
+    s->stats.peak_mem = std::max<uint64_t>(s->stats.peak_mem, s->stats.mem_used + s->scratch);
+}
+
 // Admits queued requests, in arrival order, while the budget allows.
 void admit(ising_server *s)
 {
@@ -125,6 +133,13 @@ void admit(ising_server *s)
             finish(s, r, ISING_ERR_OOM);
             continue;
         }
+        // (the worker's own batch: nothing of it runs now)
+        if (s->batch && s->stats.mem_used + r->bytes + scratch_bytes(s->batch->scratch) > s->opts.hbm_budget_bytes) {
+            // lattices come first: the batch is planned again, with less scratch or none
+            scratch_drop(s->batch->scratch);
+            s->plan_ids.clear();
+            s->plan_sweeps.clear();
+        }
         ising_lattice *h = nullptr;
         ising_status st = ising_create(&r->req.params, (void *)s->stream, &h);
         if (st != ISING_OK) {
@@ -135,7 +150,7 @@ void admit(ising_server *s)
         r->res.t_admit = s->now();
         std::lock_guard<std::mutex> lk(s->mu);
         s->stats.mem_used += r->bytes;
-        s->stats.peak_mem = std::max(s->stats.peak_mem, s->stats.mem_used);
+        note_memory(s);
         ++s->stats.admitted;
         s->resident.push_back(r);
     }
@@ -187,6 +202,11 @@ void run_epoch(ising_server *s)
     }
     ising_status st = ISING_OK;
     if (ids != s->plan_ids || sw != s->plan_sweeps) {
+        {
+            std::lock_guard<std::mutex> lk(s->mu);
+            const uint64_t budget = s->opts.hbm_budget_bytes;
+            s->batch->ahead_budget = budget > s->stats.mem_used ? budget - s->stats.mem_used : 0;
+        }
         // shrink the set until it plans (shared memory is the limit)
         while (true) {
             st = batch_replan(s->batch, hs, sw, re);
@@ -212,6 +232,8 @@ void run_epoch(ising_server *s)
         }
         s->plan_ids = ids;
         s->plan_sweeps = sw;
+        std::lock_guard<std::mutex> lk(s->mu);
+        note_memory(s);
     }
     const double t_start = s->now();
     for (Request *r : act)
@@ -446,6 +468,7 @@ ISING_API ising_status ising_server_stats(ising_server *s, ising_server_counters
     if (!s || !out) return fail(ISING_ERR_INVALID, "null argument");
     std::lock_guard<std::mutex> lk(s->mu);
     *out = s->stats;
+    out->mem_used += s->scratch;
     out->queued = s->incoming.size() + s->queue.size();
     out->resident = s->resident.size();
     out->now = s->now();

@@ -117,3 +117,48 @@ def test_served_requests_equal_the_oracle(P, orc):
             ref = orc.moments(Mo[k - 1::k], Eo[k - 1::k], N=r["L"] ** 2, T=r["T"])
             for key in ("mean_abs_m", "mean_m2", "mean_m4", "U4", "chi"):
                 assert abs(obs[key] - ref[key]) <= 1e-12 * max(1.0, abs(ref[key])), (i, key)
+
+
+def test_budget_covers_the_scratch_of_the_launches(P):
+    """What the library holds on the device stays within the server's budget (and what the
+    batch's own plan takes), whether or not the draw-ahead form's scratch fits beside the
+    lattices; results are those of the requests alone."""
+    import torch
+
+    reqs = [dict(L=1024, T=1.8 + 0.1 * i, nsweeps=20 + 3 * i, seed=100 + i, record_every=5) for i in range(10)]
+    alone = [_alone(P, r) for r in reqs]
+    taken, most = {}, [0]
+
+    def alloc(n, s):
+        p = torch.cuda.caching_allocator_alloc(n)
+        taken[p] = n
+        most[0] = max(most[0], sum(taken.values()))
+        return p
+
+    def release(p, s):
+        taken.pop(p)
+        torch.cuda.caching_allocator_delete(p)
+
+    # lattices: 10 of 128 KiB; scratch of all together: some 65 MB
+    for budget, scratch in ((4 << 20, False), (96 << 20, True)):
+        P.ising_set_allocator(alloc, release)
+        most[0] = 0
+        try:
+            with P.Server(hbm_budget_bytes=budget, keep_samples=True) as srv:
+                ids = [srv.submit(r["L"], r["T"], r["nsweeps"], seed=r["seed"], record_every=r["record_every"], tag=i)
+                       for i, r in enumerate(reqs)]
+                got = {}
+                while len(got) < len(reqs):
+                    for res in srv.poll(wait_s=1.0):
+                        got[res["tag"]] = res
+                st = srv.stats()
+                assert st["completed"] == len(reqs) and st["peak_mem"] <= budget
+                assert most[0] <= budget + (8 << 20)  # the plan: borders, counters, tables
+                assert (st["peak_mem"] > 4 << 20) == scratch
+                for i, r in enumerate(reqs):
+                    M, E = srv.samples(ids[i])
+                    assert np.array_equal(M, alone[i][0]) and np.array_equal(E, alone[i][1])
+                    assert got[i]["obs"] == alone[i][2]
+        finally:
+            P.ising_set_allocator(None)
+        assert not taken
