@@ -268,8 +268,8 @@ ISING_API const char *ising_last_error(void);
  * persistent = 0 otherwise.
  *
  * The draw-ahead form.  A handle whose configuration was not set runs calls of
- * enough sweeps (200 at L = 64, 100 at 128, 10 at 256, 3 below 1024, 5 below 2048, 10
- * up to 8192, 4 above; in a field 1 to 5 up to L = 4096, 4 above) in
+ * enough sweeps (200 at L = 64, 100 at 128, 10 at 256, 3 below 1024, 5 below 1536,
+ * 6 or 9 below 2048, 10 up to 8192, 4 above; in a field 1 to 5 up to L = 4096, 4 above) in
  * another form: the acceptance masks of a block of sweeps are drawn by the whole GPU
  * one launch before the tiles of the lattice are updated with them (L = 320 .. 512, 192
  * sweeps and more: tiles that are the CTAs of one thread-block cluster).  It needs

@@ -1219,8 +1219,13 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 // and items of 4 sweeps: 2048 1018, 4096 200 sweeps 3745 and 3225, 32768 9119; below, where
 // the chain of steps counts, one CTA is faster: 1024 567 and 622).  min_sweeps: a call
 // has one launch more than it has blocks, and the one-launch forms (L = 64, 128, 256) and
-// two step launches
-// per sweep (above) are as fast on shorter calls.
+// two step launches per sweep (above) are as fast on shorter calls.  Measured at the edges,
+// form of the configuration and this form, M/E every sweep (and none): L = 1024, 5 sweeps 60
+// -> 46 us (45 -> 34); 1536, 5 57 -> 57 (45 -> 46), 6 69 -> 65 (51 -> 50); 1984, 6 73 -> 77
+// (60 -> 60), 7 85 -> 78 (67 -> 69), 9 96 -> 78 (82 -> 81); 2048, 10 100 -> 88; 8256, 4 273
+// -> 255; 32768, 5 3867 -> 3671.  In a field: 2048, 1 54 -> 52 (42 -> 44), 2 83 -> 59; 4096, 4
+// 161 -> 128; 4160, 4 165 -> 134, 6 225 -> 166; 8256, 4 407 -> 402, 6 600 -> 477; 32768, 4
+// 4882 -> 4012.
 AheadPlan ahead_plan(uint64_t L, bool field)
 {
     AheadPlan p{};
@@ -1258,7 +1263,7 @@ AheadPlan ahead_plan(uint64_t L, bool field)
     }
     p.block_sweeps = p.halo ? p.halo / 2 : 256;
     p.min_sweeps = field ? (L <= 512 && (L & (L - 1)) == 0 ? 5 : L > 2048 ? 4 : 1)
-                         : L == 64 ? 200 : L == 128 ? 100 : L == 256 ? 10 : L < 1024 ? 3 : L < 2048 ? 5 : 10;
+                         : L == 64 ? 200 : L == 128 ? 100 : L == 256 ? 10 : L < 1024 ? 3 : L < 1536 ? 5 : L < 1856 ? 6 : L < 2048 ? 9 : 10;
     const uint32_t rows = p.tile_rows + 2 * p.halo, most = p.halo ? kThreads : kThreads / 2;
     for (p.kw = 2; rows / p.kw * wc > most;) p.kw *= 2;
     p.two = p.kw == 8 || (field && p.kw == 4 && L > 1024);

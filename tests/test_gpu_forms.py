@@ -22,10 +22,11 @@ DEFAULTS = [
     (192, 0.0, 2, "steps"), (192, 0.0, 3, "ahead"), (256, 0.0, 9, "one_launch"), (256, 0.0, 10, "ahead"),
     (320, 0.0, 191, "ahead"), (320, 0.0, 192, "ahead_cluster"), (512, 0.0, 2, "one_launch"), (512, 0.0, 3, "ahead"),
     (512, 0.0, 192, "ahead_cluster"), (576, 0.0, 200, "ahead"), (1024, 0.0, 4, "steps"), (1024, 0.0, 5, "ahead"),
+    (1472, 0.0, 5, "ahead"), (1536, 0.0, 5, "steps"), (1536, 0.0, 6, "ahead"), (1856, 0.0, 8, "steps"), (1856, 0.0, 9, "ahead"),
     (2048, 0.0, 9, "steps"), (2048, 0.0, 10, "ahead"), (8192, 0.0, 10, "ahead"), (8256, 0.0, 3, "steps"),
     (8256, 0.0, 4, "ahead_bands"), (185408, 0.0, 6, "ahead_bands"),
     (64, 0.3, 4, "one_launch"), (64, 0.3, 5, "ahead"), (320, 0.3, 1, "ahead"), (512, -2.0, 200, "ahead"),
-    (2048, 0.3, 1, "ahead"), (4096, 0.3, 3, "steps"), (4096, 0.3, 4, "ahead"),
+    (2048, 0.3, 1, "ahead"), (4096, 0.3, 3, "steps"), (4096, 0.3, 4, "ahead"), (4160, 0.3, 3, "steps"), (4160, 0.3, 4, "ahead_bands"),
 ]
 
 
