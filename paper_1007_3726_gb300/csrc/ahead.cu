@@ -1109,10 +1109,14 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_ahead_batch(const __grid_c
     if (blockIdx.x < a.update_ctas || a.block == 0u) dependent_launch_wait();
     dependent_launch_trigger();
     if (a.block == 0u) {
-        for (uint32_t k = blockIdx.x; k < a.d_jobs; k += gridDim.x) {
+        // groups of CTAs, each for every so many-th lattice (one CTA a lattice took 200 us for
+        // one of 4096^2)
+        const uint32_t parts = max(1u, gridDim.x / a.d_jobs), groups = gridDim.x / parts, group = blockIdx.x / parts;
+        for (uint32_t k = group; group < groups && k < a.d_jobs; k += groups) {
             const AheadJob &j = a.jobs[k];
             if (j.copy_from)
-                for (uint32_t i = threadIdx.x; i < j.nwords; i += kBatchThreads) j.even[i] = j.copy_from[i];
+                for (uint32_t i = blockIdx.x % parts * kBatchThreads + threadIdx.x; i < j.nwords; i += parts * kBatchThreads)
+                    j.even[i] = j.copy_from[i];
         }
     } else if (blockIdx.x < a.update_ctas) {
         if (blockIdx.x == 0 && threadIdx.x == 0) *a.next_ticket = 0u;

@@ -264,3 +264,20 @@ def test_batch_whose_scratch_is_given_back_between_runs(P):
             assert not held
     finally:
         P.ising_set_allocator(None)
+
+
+@pytest.mark.parametrize("L,count,sweeps", [(4096, 1, 12), (1088, 3, 36), (320, 320, 12), (512, 200, 20)])
+def test_batch_with_an_odd_number_of_blocks(P, L, count, sweeps):
+    """Lattices whose last block would end in their second buffer are copied first, by one
+    or many CTAs each (fewer and more lattices than CTAs)."""
+    lats = [P.Lattice(L, 2.2 + 0.001 * i, seed=3, stream_id=i, init="hot") for i in range(count)]
+    with P.Batch(lats, [sweeps] * count, 4) as b:
+        assert b.form == "ahead"
+        b.run(1)
+    for i in list(range(0, count, 37)) + [count - 1]:
+        with P.Lattice(L, 2.2 + 0.001 * i, seed=3, stream_id=i, init="hot") as one:
+            one.sweep(sweeps, 4)
+            assert np.array_equal(lats[i].packed(), one.packed())
+            assert np.array_equal(np.stack(lats[i].samples()), np.stack(one.samples()))
+    for l in lats:
+        l.close()
