@@ -111,7 +111,8 @@ ising_status harvest(ising_lattice *h)
         h->pending = false;
         h->pending_err = false;
         h->failed = true;
-        return fail(ISING_ERR_TIMEOUT, "a wait inside the one-CTA kernel ran out; the lattice is lost");
+        return fail(ISING_ERR_TIMEOUT, "a wait inside the %s ran out; the lattice is lost",
+                    h->form == ISING_FORM_ONE_LAUNCH ? "one-launch kernel" : "draw-ahead form");
     }
     h->pending_err = false;
     for (size_t i = 0; i < h->pending_rec; ++i) {

@@ -212,3 +212,12 @@ def test_command_line_batch_runs_the_default_form(P, capsys):
     for argv, form in (([], "ahead"), (["--block", "256", "--ctas-per-sm", "4"], "strips")):
         assert cli.main(["fss-batch", "--sweeps", "20", *argv]) == 0
         assert json.loads(capsys.readouterr().out)["form"] == form
+
+
+@pytest.mark.parametrize("L,n,what", [(64, 20, "one-launch"), (64, 200, "draw-ahead"), (512, 200, "draw-ahead")])
+def test_a_wait_that_runs_out_names_the_form(P, monkeypatch, L, n, what):
+    with P.Lattice(L, 2.0, seed=1) as lat:
+        monkeypatch.setenv("ISING_TINY_HOLD_STEP", "6")
+        with pytest.raises(P.IsingError) as ei:
+            lat.sweep(n, 1, collect=True)
+        assert ei.value.status == P.ERR_TIMEOUT and what in str(ei.value)
