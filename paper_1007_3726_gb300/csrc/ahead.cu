@@ -15,13 +15,13 @@
 // The next launch updates what this one drew; a launch boundary is the only
 // synchronisation between CTAs.
 //
-// Bound: draws at 1.75 per ns on the whole GPU (below); where the lattice is small,
+// Bound: draws at 1750 per ns on the whole GPU (below); where the lattice is small,
 // the chain of steps of a tile (62 ns a step at L = 64, 110 .. 220 ns above) and 2 to
 // 3 us per launch.  Measured, one call, before (step launches or one-launch forms)
 // and with this form: L = 64, 1000 sweeps 239 -> 170 us; 256, 1000: 1072 -> 316;
-// 320, 500: 2985 -> 221; 512, 1000: 4885 -> 376; 1024, 500: 2850 -> 460; 2048, 200:
-// 1446 -> 606; 4096, 200: 3546 -> 2193 (1.53 attempts per ns of 0.95); 65536, 4: 12449 ->
-// 11120 (1.54 of 1.38).  Persistent CTAs that wait for one another on flags instead
+// 320, 500: 2985 -> 223; 512, 1000: 4885 -> 383; 1024, 500: 2850 -> 460; 2048, 200:
+// 1446 -> 585; 4096, 200: 3546 -> 2193 (1530 attempts per ns of 946); 65536, 4: 12449 ->
+// 11150 (1540 of 1380).  Persistent CTAs that wait for one another on flags instead
 // of launches were no faster (a block's hand-over costs them 3.4 us); CTAs of one
 // cluster are, where they can hold the lattice.
 //
@@ -723,8 +723,7 @@ __global__ void __launch_bounds__(kThreads, TWO ? 2 : 1) k_ahead(const __grid_co
 // Bound: the chain of steps, 290 cycles each (a barrier 70, shared memory 35, 45
 // dependent instructions; an exchange 600 every 16 steps), with the draws beside it.  The
 // tiles of separate launches need 230 cycles a step and 2.8 us a launch: 1000
-// sweeps of 512 486 -> 390 us, 500 of 320 230 -> 215, M/E every sweep and every tenth about the
-// same; 256 (2 us of 32 sweeps a launch) is no faster than with tiles, 1024 is bound by its
+// sweeps of 512 478 -> 383 us (M/E every hundredth), 500 of 320 237 -> 223 (every sweep); 256 (2 us of 32 sweeps a launch) is no faster than with tiles, 1024 is bound by its
 // draws.  One row a thread, 8 rows of halo, and 4 rows a lane with shuffles in place of
 // the barrier took as long within 5 %.
 
@@ -1021,10 +1020,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_ahead_band(const __grid_constan
 }
 
 // ----------------------------------------------------------------- batch --
-// Bound: the draws, 1.75 per ns (a lattice's keys come from registers here: 1.7), as
+// Bound: the draws, 1750 per ns (a lattice's keys come from registers here: 1700), as
 // soon as the lattices together have some 64 M attempts a block; the tiles take the SMs
 // for about a fifth as long.  Measured, strips in one persistent launch (batch.cu) and
-// this: four sizes 256 .. 2048 at 32 temperatures, 100 sweeps 15043 -> 12885 us (1.38
+// this: four sizes 256 .. 2048 at 32 temperatures, 100 sweeps 15043 -> 12885 us (1380
 // attempts per ns); 32 of 512^2, 500 sweeps 10612 -> 3213; one of 2048^2 10998 -> 1554; 128
 // of 64^2 1284 -> 638.
 //
@@ -1211,7 +1210,7 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 //   L = 4096,  200 sweeps: 32 + 16: 2225, 16 + 8: 2399
 // Above 8192 tiles are parts of rows and a launch takes a band of rows: the masks of
 // all would be 64 times the lattice a block.  Measured against the step kernels (two
-// launches a sweep): L = 65536, 4 sweeps 12252 -> 11083 us (1.55 attempts per ns), 8 sweeps
+// launches a sweep): L = 65536, 4 sweeps 12252 -> 11083 us (1550 attempts per ns), 8 sweeps
 // 24481 -> 21766; 16384, 40 sweeps 8510 -> 6808; 8256, 40 sweeps 2456 -> 1804.  Two CTAs
 // of the largest tiles share a SM, and with draws (L = 2048, 200 sweeps: 606 us with
 // one, 585 with two; 4096 2225 and 2137; 8192, 40 sweeps 1848 and 1748).  In a field (20
