@@ -199,10 +199,10 @@ def kernel_source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-def profiled_kernel():
-    """The committed ncu figures of the band kernel (DRAM bytes and thread
-    instructions per attempt at the captured size), if they were taken on the
-    current kernel source; else None."""
+def profiled_kernel(size: int):
+    """The committed ncu figures of the band kernel on a lattice of this size (DRAM bytes
+    per attempt: they depend on whether the masks of a band stay in the L2), if they were
+    taken on the current kernel source; else None."""
     try:
         with open(TRAFFIC_FILE) as f:
             d = json.load(f)
@@ -210,7 +210,7 @@ def profiled_kernel():
         return None
     if d.get("kernel_sources_sha16") != kernel_source_hash():
         return None
-    return d
+    return next((c for c in d["captures"] if c["L"] == size), None)
 
 
 def launches_of_step(strips: bool, ahead: bool) -> int:
@@ -779,7 +779,7 @@ def run_ours(args, ws, rank, local):
     achieved_tops = OPS_PER_ATTEMPT * per_rank_attempts / step_s / 1e12
     rate_per_gpu = per_rank_attempts / step_s / 1e9  # attempts/ns of one GPU
     mix = mix_peaks(P, stream) if ws == 1 else None
-    prof = profiled_kernel()
+    prof = profiled_kernel(L)
     traffic = None
     if prof and ahead:
         traffic = prof["dram_bytes_per_attempt"] * per_rank_attempts
@@ -799,9 +799,10 @@ def run_ours(args, ws, rank, local):
                      "basis": "the lattice read and written once per sweep"},
     }
     if traffic is not None:
-        roof["traffic_basis"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per attempt at L=%d, times the "
-                                 "attempts of a step (%s)" % (prof["L"], prof["source"]))
-        roof["ncu_thread_instructions_per_attempt"] = prof.get("thread_inst_per_attempt")
+        roof["traffic_basis"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per attempt of a band in a block of 4 "
+                                 "sweeps at L=%d, times the attempts of a step (%s)" % (prof["L"], prof["source"]))
+        small = profiled_kernel(32768)
+        roof["ncu_thread_instructions_per_attempt"] = small["thread_inst_per_attempt"] if small else None
     if mix:
         roof["measured_mix"] = dict(mix, unit="draws/ns", how="ising_bench_mix: one wave of resident 512-thread "
                                     "blocks, 32 draws per thread per word, CUDA events",
