@@ -1198,7 +1198,9 @@ cudaError_t prepare_device(AheadKernel kern, uint32_t which, int *sms)
 }  // namespace
 
 // The plan by size.  L <= 192: one CTA holds the lattice, in registers for the
-// whole block, and blocks are long (a block of 256 sweeps costs one launch).
+// whole block, and blocks are long: 256 sweeps a launch, at L = 64 1024, whose draws take
+// the whole GPU 2 us (256: calls queued on 8 streams of their own, 1000 sweeps 0.30 ms and
+// 0.22, 10^5 16.1 and 12.2; one stream 11.6 and 11.0).
 // Above, tiles of full rows: the taller the halo, the fewer launches and the more
 // redundant rows; a tile and its halo are at most 4096 words of a colour (8 rows a
 // thread), so that both shrink as rows get longer.  Measured (us for a call, M/E
@@ -1264,13 +1266,13 @@ AheadPlan ahead_plan(uint64_t L, bool field)
             p.halo = std::min(p.halo, L <= 1024 ? 32u : L <= 2048 ? 16u : 8u);
         }
     }
-    p.block_sweeps = p.halo ? p.halo / 2 : 256;
+    p.warp = L == 64 && !field;
+    p.block_sweeps = p.halo ? p.halo / 2 : p.warp ? 1024 : 256;
     p.min_sweeps = field ? (L <= 512 && (L & (L - 1)) == 0 ? 5 : L > 2048 ? 4 : 1)
                          : L == 64 ? 200 : L == 128 ? 100 : L == 256 ? 10 : L < 1024 ? 3 : L < 1536 ? 5 : L < 1856 ? 6 : L < 2048 ? 9 : 10;
     const uint32_t rows = p.tile_rows + 2 * p.halo, most = p.halo ? kThreads : kThreads / 2;
     for (p.kw = 2; rows / p.kw * wc > most;) p.kw *= 2;
     p.two = p.kw == 8 || (field && p.kw == 4 && L > 1024);
-    p.warp = L == 64 && !field;
     p.tiles = (uint32_t)(L / p.tile_rows);
     // one tile a CTA, or several the same number each: of 66 tiles 2 on two CTAs take
     // twice as long as the others; 128 tiles (L = 4096) on 64 CTAs 2137 us, on 128 2228
@@ -1605,9 +1607,9 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     const bool snapshots = pl.warp || (nsweeps >= 32 && L <= 2048);
     // Blocks.  Items of 4 sweeps are the cheapest to draw, so a call that is long
     // enough starts with the rest of a division by 4.  Where an update takes long
-    // (one CTA holds the lattice), blocks start short: nothing overlaps the first
-    // one's draws.
-    uint64_t drawn = 0, done = 0, rec_done = 0, prev = 0, grow = pl.halo ? full : std::min<uint64_t>(full, 32);
+    // (one CTA holds the lattice), blocks start short, but for the cheap draws of L = 64:
+    // nothing overlaps the first one's draws.
+    uint64_t drawn = 0, done = 0, rec_done = 0, prev = 0, grow = pl.halo || pl.warp ? full : std::min<uint64_t>(full, 32);
     auto next_block = [&]() -> uint64_t {
         const uint64_t left = nsweeps - drawn;
         if (full % 4 != 0 || (left <= 7 && L < 2048)) return std::min<uint64_t>(left, full);
@@ -1620,7 +1622,7 @@ cudaError_t ahead_sweeps(ising_lattice *h, const AheadPlan &pl, void *lattice, u
     uint64_t nblocks = 0;
     for (; drawn < nsweeps; ++nblocks) drawn += next_block();
     drawn = 0;
-    grow = pl.halo ? full : std::min<uint64_t>(full, 32);
+    grow = pl.halo || pl.warp ? full : std::min<uint64_t>(full, 32);
     cudaError_t e = cudaMemsetAsync(tickets, 0, kTicketBytes, h->stream);
     if (e != cudaSuccess) return e;
     const uint64_t *src = spins;

@@ -221,3 +221,50 @@ def test_a_wait_that_runs_out_names_the_form(P, monkeypatch, L, n, what):
         with pytest.raises(P.IsingError) as ei:
             lat.sweep(n, 1, collect=True)
         assert ei.value.status == P.ERR_TIMEOUT and what in str(ei.value)
+
+
+def test_small_lattices_in_blocks_of_a_thousand_sweeps(P, orc):
+    """L = 64, calls of several blocks, whole and partial ones."""
+    s, t, lat = orc.init_hot(64, 3, 0), 0, P.Lattice(64, TC, seed=3, init="hot")
+    for n, rec in ((1030, 1), (2500, 7), (1024, 0), (203, 3), (2049, 1)):
+        got = lat.sweep(n, rec, collect=bool(rec))
+        assert lat.form == "ahead"
+        Mo, Eo = orc.run(s, n, 3, 0, *orc.thresholds(TC), t0=t)
+        if rec:
+            k0 = (rec - 1 - t) % rec
+            assert np.array_equal(got[0], Mo[k0::rec]) and np.array_equal(got[1], Eo[k0::rec]), n
+        d = lat.measure()
+        assert (d["M"], d["E"]) == (Mo[-1], Eo[-1]) and np.array_equal(lat.spins(), s)
+        t += n
+    lat.close()
+
+
+def test_small_lattices_on_many_streams(P, orc):
+    """L = 64: calls of handles on more than eight streams are one launch each, whatever was
+    queued before; lattices and samples do not depend on it."""
+    import torch
+
+    streams = [torch.cuda.Stream() for _ in range(9)]
+    lats = [P.Lattice(64, 2.2, seed=i, init="hot", stream=streams[i % 8]) for i in range(10)]
+
+    def call(form):
+        for lat in lats:
+            lat.sweep(250, 5)
+            assert lat.form == form
+
+    call("ahead")
+    lats.append(P.Lattice(64, 2.2, seed=10, init="hot", stream=streams[8]))
+    call("one_launch")
+    with P.Lattice(64, 2.2, seed=1, H=0.1) as f, P.Lattice(128, 2.2, seed=1) as g:
+        f.sweep(200)
+        g.sweep(200)
+        assert f.form == g.form == "ahead"
+    last = lats.pop()
+    last.close()  # while its call may still run
+    call("ahead")
+    for i, lat in enumerate(lats):
+        s = orc.init_hot(64, i, 0)
+        Mo, Eo = orc.run(s, 750, i, 0, *orc.thresholds(2.2))
+        M, E = lat.samples()
+        assert np.array_equal(M, Mo[4::5]) and np.array_equal(E, Eo[4::5]) and np.array_equal(lat.spins(), s)
+        lat.close()
