@@ -698,7 +698,9 @@ __global__ void __launch_bounds__(kThreads, TWO ? 2 : 1) k_ahead(const __grid_co
     // The first launch of a call (it only draws) starts after all work before it.
     // A later one draws into a buffer, and takes tickets from a counter, that no
     // launch still running uses (three and four in turn), so its draws need not
-    // wait; updates and counts need what the launch before wrote.
+    // wait: of what the stream has written they read the counter alone, by atomics in the
+    // L2, which a launch that has ended has cleared.  Updates and counts need what the
+    // launch before wrote.
     const uint32_t early = a.update_ctas + a.count_ctas;
     if (blockIdx.x < early || early == 0u) dependent_launch_wait();
     dependent_launch_trigger();
@@ -1045,10 +1047,19 @@ __device__ __forceinline__ uint32_t find_job(const AheadJob *jobs, uint32_t n, u
     return lo;
 }
 
-__device__ __forceinline__ void batch_draw_role(const AheadBatchArgs &a)
+// early: this CTA has not waited for the launch before.  It reads the table of the lattices
+// and the run's first sweep indices, which the copies before the run wrote where an earlier
+// run's were: that the launch before has waited for them is acquired here, beside the first
+// ticket (it published that before it let this one start).
+__device__ __forceinline__ void batch_draw_role(const AheadBatchArgs &a, bool early)
 {
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t next = lane == 0 ? atomicAdd(a.d_ticket, 1u) : 0u;
+    if (early && lane == 0 && !published(a.done, a.block, kPublishedLimit)) {
+        atomicExch(a.err, 1u);
+        next = a.d_tickets;
+    }
+    __syncwarp();
     for (;;) {
         const uint32_t it = __shfl_sync(0xFFFFFFFFu, next, 0);
         if (it >= a.d_tickets) return;
@@ -1105,8 +1116,10 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_ahead_batch(const __grid_c
     __shared__ AheadArgs t;
     // (waits as in k_ahead; the first launch copies the lattices whose last block
     // would otherwise end in their second buffer)
-    if (blockIdx.x < a.update_ctas || a.block == 0u) dependent_launch_wait();
-    dependent_launch_trigger();
+    const bool early = blockIdx.x >= a.update_ctas && a.block != 0u;
+    if (!early) dependent_launch_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) publish(a.done, a.block + 1u);
+    if (blockIdx.x != 0 || threadIdx.x == 0) dependent_launch_trigger();
     if (a.block == 0u) {
         // groups of CTAs, each for every so many-th lattice (one CTA a lattice took 200 us for
         // one of 4096^2)
@@ -1139,7 +1152,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_ahead_batch(const __grid_c
             }
         }
     }
-    if (a.d_tickets != 0u) batch_draw_role(a);
+    if (a.d_tickets != 0u) batch_draw_role(a, early);
 }
 
 using AheadKernel = void (*)(AheadArgs);
@@ -1798,7 +1811,7 @@ cudaError_t AheadBatch::upload(void *scratch, const std::vector<ising_lattice *>
     return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
-cudaError_t AheadBatch::enqueue(const uint32_t *d_t0, cudaStream_t s)
+cudaError_t AheadBatch::enqueue(const uint32_t *d_t0, unsigned int *d_err, cudaStream_t s)
 {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1810,6 +1823,8 @@ cudaError_t AheadBatch::enqueue(const uint32_t *d_t0, cudaStream_t s)
     AheadBatchArgs a{};
     a.jobs = reinterpret_cast<const AheadJob *>(d_scratch + kTicketBytes);
     a.t0 = d_t0;
+    a.done = tickets + kDoneWord;
+    a.err = d_err;
     size_t drawing = jobs.size(), updating = 0;  // the first so many jobs have a block b, a block b - 1
     for (uint32_t b = 0;; ++b) {
         updating = b ? drawing : 0;

@@ -126,6 +126,8 @@ struct AheadBatchArgs {
     uint32_t d_jobs, u_jobs;      // jobs that have them
     uint32_t d_tickets, u_tiles, update_ctas;
     unsigned int *d_ticket, *next_ticket;
+    unsigned int *done;           // launches of the run that have waited for what was before them
+    unsigned int *err;
 };
 
 }  // namespace ising
@@ -153,7 +155,8 @@ struct AheadBatch {
     // Places the jobs in scratch (scratch_bytes) and uploads their table.
     cudaError_t upload(void *scratch, const std::vector<ising_lattice *> &hs, const std::vector<unsigned long long *> &acc,
                        const std::vector<unsigned long long *> &final_acc, cudaStream_t s);
-    // Queues one run; d_t0: the lattices' first sweep indices on the device.
-    cudaError_t enqueue(const uint32_t *d_t0, cudaStream_t s);
+    // Queues one run; d_t0: the lattices' first sweep indices on the device, d_err: its error
+    // flag.
+    cudaError_t enqueue(const uint32_t *d_t0, unsigned int *d_err, cudaStream_t s);
 };
 }  // namespace ising

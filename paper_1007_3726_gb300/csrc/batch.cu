@@ -983,7 +983,7 @@ cudaError_t enqueue_run(ising_batch *b)
                             cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess) return e;
     if (b->use_ahead) {
-        e = b->ahead.enqueue(b->args.t0, b->stream);
+        e = b->ahead.enqueue(b->args.t0, b->args.error_flag, b->stream);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(b->h_counters, work + b->off_counters, b->slots * 16, cudaMemcpyDeviceToHost, b->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(b->h_error, work + b->off_error, 4, cudaMemcpyDeviceToHost, b->stream);
@@ -1175,7 +1175,8 @@ ISING_API ising_status ising_batch_run(ising_batch *b, uint32_t runs)
         if (*b->h_error != 0u) {
             b->failed = true;
             for (ising_lattice *h : b->hs) h->failed = true;
-            return fail(ISING_ERR_TIMEOUT, "a strip waited longer than the limit; the lattices are lost");
+            return fail(ISING_ERR_TIMEOUT, b->use_ahead ? "a wait inside the draw-ahead form ran out; the lattices are lost"
+                                                        : "a strip waited longer than the limit; the lattices are lost");
         }
         for (size_t i = 0; i < n; ++i) {
             ising_lattice *h = b->hs[i];

@@ -281,3 +281,26 @@ def test_batch_with_an_odd_number_of_blocks(P, L, count, sweeps):
             assert np.array_equal(np.stack(lats[i].samples()), np.stack(one.samples()))
     for l in lats:
         l.close()
+
+
+def test_batch_runs_draw_for_their_own_sweep_indices(P):
+    """Run after run of small batches (fewer CTAs than SMs) whose lattices are swept alone in
+    between, and a second batch's table where the first one's was: every launch draws with
+    the indices and the lattices of its own run."""
+    specs = [(64, 2.1, 1), (128, 2.2, 2), (320, 2.3, 3), (64, 2.4, 4)]
+    mk = lambda: [P.Lattice(L, T, seed=s, init="hot") for L, T, s in specs]  # noqa: E731
+    lats, ref = mk(), mk()
+    for k in range(6):
+        which = [0, 1, 2, 3] if k % 2 == 0 else [3, 2, 0]
+        n = [24 + 4 * k, 16, 13, 40][:len(which)]
+        with P.Batch([lats[i] for i in which], n, 1) as b:
+            assert b.form == "ahead"
+            for r in range(5):
+                b.run(1)
+                lats[which[0]].sweep(r + 1, 1)
+        for r in range(5):
+            for i, m in zip(which, n):
+                ref[i].sweep(m, 1)
+            ref[which[0]].sweep(r + 1, 1)
+    for l, r in zip(lats, ref):
+        assert np.array_equal(l.spins(), r.spins()) and np.array_equal(np.stack(l.samples()), np.stack(r.samples()))
