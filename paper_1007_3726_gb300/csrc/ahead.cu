@@ -1049,13 +1049,13 @@ __device__ __forceinline__ uint32_t find_job(const AheadJob *jobs, uint32_t n, u
 
 // early: this CTA has not waited for the launch before.  It reads the table of the lattices
 // and the run's first sweep indices, which the copies before the run wrote where an earlier
-// run's were: that the launch before has waited for them is acquired here, beside the first
-// ticket (it published that before it let this one start).
+// run's were: that the run's first launch has waited for them is acquired here, beside the
+// first ticket (it published that before it let the next one start).
 __device__ __forceinline__ void batch_draw_role(const AheadBatchArgs &a, bool early)
 {
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t next = lane == 0 ? atomicAdd(a.d_ticket, 1u) : 0u;
-    if (early && lane == 0 && !published(a.done, a.block, kPublishedLimit)) {
+    if (early && lane == 0 && !published(a.done, 1u, kPublishedLimit)) {
         atomicExch(a.err, 1u);
         next = a.d_tickets;
     }
@@ -1118,8 +1118,9 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_ahead_batch(const __grid_c
     // would otherwise end in their second buffer)
     const bool early = blockIdx.x >= a.update_ctas && a.block != 0u;
     if (!early) dependent_launch_wait();
-    if (blockIdx.x == 0 && threadIdx.x == 0) publish(a.done, a.block + 1u);
-    if (blockIdx.x != 0 || threadIdx.x == 0) dependent_launch_trigger();
+    const bool first = a.block == 0u && blockIdx.x == 0;
+    if (first && threadIdx.x == 0) publish(a.done, 1u);
+    if (!first || threadIdx.x == 0) dependent_launch_trigger();
     if (a.block == 0u) {
         // groups of CTAs, each for every so many-th lattice (one CTA a lattice took 200 us for
         // one of 4096^2)

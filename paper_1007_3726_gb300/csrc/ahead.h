@@ -126,7 +126,7 @@ struct AheadBatchArgs {
     uint32_t d_jobs, u_jobs;      // jobs that have them
     uint32_t d_tickets, u_tiles, update_ctas;
     unsigned int *d_ticket, *next_ticket;
-    unsigned int *done;           // launches of the run that have waited for what was before them
+    unsigned int *done;           // 1 once the run's first launch has waited for what was before it
     unsigned int *err;
 };
 
