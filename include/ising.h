@@ -285,10 +285,11 @@ ISING_API const char *ising_last_error(void);
  * configuration's form runs.  Results are the same.
  * While handles of L = 64 live on more than eight streams of the device, those without a
  * field run the configuration's form, whose calls are one launch each.
- * ising_set_launch switches it off for the handle, ising_clear_launch on again.  (ISING_TINY_HOLD_STEP and
- * ISING_TINY_MAX_SWEEPS, for tests only, also act here: the former where an update waits
- * for masks on their way, at L = 64 and in the cluster, the latter as the longest
- * block.)
+ * ising_set_launch switches it off for the handle, ising_clear_launch on again.
+ * (ISING_TINY_HOLD_STEP and ISING_TINY_MAX_SWEEPS, for tests only, also act here: the
+ * former where an update waits for masks on their way, at L = 64 and in the cluster, the
+ * latter as the longest block.  ISING_SCRATCH_MB, for tests only, is the bound on what
+ * handles keep together.)
  */
 typedef struct {
     uint32_t proc_bits, regcap, block, rows_per_item, grid, insert;
